@@ -114,14 +114,16 @@ struct p2p_plan {
     unsigned int* status;   // device status word
     long long* scratch64;   // small device scratch (pair count)
     // tensor-core path (plans with max_nrhs >= 16)
-    int32_t* tc_gstart;     // [nb + 1] first 16-source group of every box (exclusive scan of ceil(n_b / 16))
-    int32_t tc_groups;      // number of 16-source groups
-    int32_t* tc_glist_off;  // [nb + 1] offsets of the per-box group lists
-    int32_t* tc_glist;      // per box: the groups of its neighbour boxes (ascending box id), -1 padding to a
-                            // multiple of 4 entries
-    int32_t* tc_gcount;     // [nb] groups in the list of every box (without padding)
-    unsigned char* tc_pack; // per-apply group records: BF16 hi/lo strength images (one per block of 64 RHS)
-                            // followed by the group's 16 source coordinates
+    int32_t* tc_off;        // [blocks + 1] first entry of every block of 32 target boxes (p2p_tc.cu)
+    int32_t* tc_ustart;     // [blocks + 1] first unit (window of at most 128 targets) of every block
+    int32_t* tc_ecount;     // [blocks] entries of every block
+    int32_t* tc_unit_block; // [units] block of every unit
+    int32_t* tc_gid;        // per entry: group of 16 consecutive sorted sources
+    uint32_t* tc_bits;      // per entry: bit per box of the block that has a neighbour source in the group
+    uint32_t* tc_masks;     // per entry: 32 16-bit masks, the neighbour sources of every box of the block
+    uint8_t* tc_member;     // [n] box number in its block of every sorted target
+    unsigned int* tc_counter;  // [2] unit counter and CTA count of a running launch, zero between launches
+    unsigned char* tc_pack; // per-apply group records: BF16 part images of the strengths, source coordinates
     int32_t tc_wait_polls;  // poll bound of the tensor-core pipeline's waits, -1: the default (a self-check
                             // lowers it to make the abort path run)
     // box-group kernel (p2p_group.cu; indexed layout, one right-hand side): kGroupBoxes consecutive target boxes
@@ -141,12 +143,13 @@ struct p2p_plan {
     int4* g_copy;           // [n_groups * kGroupBoxes * 27] union copies: source start, buffer offset, length
 };
 
-// Bytes of the tensor-core group records for n points in nb boxes (0 when max_nrhs < 16).
-size_t p2p_tc_pack_bytes(int64_t n, int32_t nb, int32_t max_nrhs);
-// Entries of the tensor-core group lists: at most sources / 16 + nnz + 3 nb.
-inline size_t p2p_tc_list_bound(int64_t sources, int64_t nnz, int32_t nb) {
-    return (size_t)(sources / 16 + nnz + 3 * (int64_t)nb + 4);
-}
+// Tensor-core path (p2p_tc.cu): bytes of the group records for n sources (0 when max_nrhs < 16), blocks of target
+// boxes, a bound of the units, and a bound of the list entries (a neighbour box of m sources touches at most
+// m / 16 + 2 groups).
+size_t p2p_tc_pack_bytes(int64_t n, int32_t max_nrhs);
+int32_t p2p_tc_block_count(int32_t nb);
+int64_t p2p_tc_unit_bound(int64_t n, int32_t nb);
+inline size_t p2p_tc_entry_bound(int64_t sources, int64_t nnz) { return (size_t)(sources / 16 + 2 * nnz + 4); }
 
 namespace p2p_detail {
 

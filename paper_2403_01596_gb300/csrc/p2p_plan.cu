@@ -27,6 +27,9 @@ cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* 
                             int32_t* vals, uint64_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
                             cudaStream_t s, int32_t* cap);
 
+// Tensor-core lists (p2p_tc.cu).
+cudaError_t p2p_tc_build(p2p_plan* p, int32_t* bound, int32_t* units, void* scan_ws, cudaStream_t s);
+
 namespace {
 
 constexpr int kThreads = 256;
@@ -293,42 +296,6 @@ __global__ void k_direct_items(const int32_t* __restrict__ box_ptr, const int32_
     recs[b] = r;
     keys[b] = 0xFFFFFFFFull - (uint64_t)min((int64_t)nt * S, (int64_t)0xFFFFFFFF);
     vals[b] = b;
-}
-
-// Source groups of the tensor-core path: ceil(n_b / 16) per box.
-__global__ void k_tc_groups(const int32_t* __restrict__ box_ptr, int32_t nb, int32_t* __restrict__ groups) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb) groups[b] = (box_ptr[b + 1] - box_ptr[b] + 15) / 16;
-}
-
-// Length of every box's group list: the groups of its neighbour boxes, and that
-// count padded to a multiple of 4.
-__global__ void k_tc_list_len(const int32_t* __restrict__ nbr_ptr, const int32_t* __restrict__ nbr_idx,
-                              const int32_t* __restrict__ gstart, int32_t nb, int32_t* __restrict__ count,
-                              int32_t* __restrict__ padded) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    int g = 0;
-    for (int e = nbr_ptr[b]; e < nbr_ptr[b + 1]; ++e) {
-        const int c = nbr_idx[e];
-        g += gstart[c + 1] - gstart[c];
-    }
-    count[b] = g;
-    padded[b] = (g + 3) & ~3;
-}
-
-// Group lists: neighbour boxes in ascending id, each box's groups in order, -1 padding.
-__global__ void k_tc_list_fill(const int32_t* __restrict__ nbr_ptr, const int32_t* __restrict__ nbr_idx,
-                               const int32_t* __restrict__ gstart, const int32_t* __restrict__ off, int32_t nb,
-                               int32_t* __restrict__ list) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    int o = off[b];
-    for (int e = nbr_ptr[b]; e < nbr_ptr[b + 1]; ++e) {
-        const int c = nbr_idx[e];
-        for (int g = gstart[c]; g < gstart[c + 1]; ++g) list[o++] = g;
-    }
-    while (o < off[b + 1]) list[o++] = -1;
 }
 
 // One warp per target box: writes the box's source list -- the sources of its
@@ -663,12 +630,20 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     const size_t lam_bytes = lam_rows * (size_t)max_nrhs * sizeof(float2);
     L.p.lam_buf = c.take<float2>(lam_rows * (size_t)max_nrhs);
     L.p.g_buf = two_sets ? nullptr : c.take<float2>(m * (size_t)max_nrhs);
-    const size_t tc_bytes = p2p_tc_pack_bytes((int64_t)ms, (int32_t)mbs, max_nrhs);
-    L.p.tc_gstart = tc_bytes ? c.take<int32_t>(mbs + 1) : nullptr;
-    L.p.tc_glist_off = tc_bytes ? c.take<int32_t>(mb + 1) : nullptr;
-    L.p.tc_gcount = tc_bytes ? c.take<int32_t>(mb) : nullptr;
-    L.p.tc_glist = tc_bytes ? c.take<int32_t>(p2p_tc_list_bound(sources, nnz, (int32_t)mb)) : nullptr;
-    L.p.tc_pack = tc_bytes ? c.take<unsigned char>(tc_bytes) : nullptr;
+    const size_t tc_bytes = p2p_tc_pack_bytes((int64_t)ms, max_nrhs);
+    if (tc_bytes) {
+        const size_t blocks = (size_t)p2p_tc_block_count((int32_t)mb), entries = p2p_tc_entry_bound(sources, nnz);
+        L.p.tc_off = c.take<int32_t>(blocks + 1);
+        L.p.tc_ustart = c.take<int32_t>(blocks + 1);
+        L.p.tc_ecount = c.take<int32_t>(blocks);
+        L.p.tc_unit_block = c.take<int32_t>((size_t)p2p_tc_unit_bound((int64_t)m, (int32_t)mb));
+        L.p.tc_gid = c.take<int32_t>(entries);
+        L.p.tc_bits = c.take<uint32_t>(entries);
+        L.p.tc_masks = c.take<uint32_t>(entries * 16);
+        L.p.tc_member = c.take<uint8_t>(m);
+        L.p.tc_counter = c.take<unsigned int>(2);
+        L.p.tc_pack = c.take<unsigned char>(tc_bytes);
+    }
     const size_t mx = mb > mbs ? mb : mbs;
     L.n_chunks = c.take<int32_t>(mx);
     L.list_len = c.take<int32_t>(mb);
@@ -1070,34 +1045,14 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
                                                                  L.self_len, p->pk_off, nb, t.chunk, t.target_group,
                                                                  p->two_sets, L.recs, L.keys, L.vals);
     FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/items");
-    if (p->tc_gstart && p->nbs > 0) {
-        // 16-source groups of the tensor-core path over the source boxes (n_chunks is free once the items are
-        // built), then every target box's list of its neighbourhood's groups
-        k_tc_groups<<<blocks_for(p->nbs, kThreads), kThreads, 0, s>>>(p->src_box_ptr, p->nbs, L.n_chunks);
-        FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/tc_groups");
-        FAIL_CUDA(scan_exclusive_i32(L.n_chunks, p->tc_gstart, p->nbs, p->tc_gstart + p->nbs, L.scan_ws, s),
-                  "p2p_plan_create/tc_scan");
-        k_tc_list_len<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(in.nbr_ptr, in.nbr_idx, p->tc_gstart, nb,
-                                                                    p->tc_gcount, L.n_chunks);
-        FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/tc_lists");
-        FAIL_CUDA(scan_exclusive_i32(L.n_chunks, p->tc_glist_off, nb, p->tc_glist_off + nb, L.scan_ws, s),
-                  "p2p_plan_create/tc_scan");
-        k_tc_list_fill<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(in.nbr_ptr, in.nbr_idx, p->tc_gstart,
-                                                                     p->tc_glist_off, nb, p->tc_glist);
-        FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/tc_lists");
-    }
     int32_t host[4] = {0, 0, 0, 0};
     unsigned int status = 0;
     int32_t packed = 0;
-    int32_t tc_groups = 0;
     FAIL_CUDA(cudaMemcpyAsync(host, L.maxes, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
     FAIL_CUDA(cudaMemcpyAsync(host + 2, L.small, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
     FAIL_CUDA(cudaMemcpyAsync(&status, p->status, sizeof(status), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
     FAIL_CUDA(cudaMemcpyAsync(&packed, p->pk_off + nb, sizeof(int32_t), cudaMemcpyDeviceToHost, s),
               "p2p_plan_create");
-    if (p->tc_gstart && p->nbs > 0)
-        FAIL_CUDA(cudaMemcpyAsync(&tc_groups, p->tc_gstart + p->nbs, sizeof(int32_t), cudaMemcpyDeviceToHost, s),
-                  "p2p_plan_create");
     FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
     if (!status) {
         const int64_t items = host[2];
@@ -1115,6 +1070,8 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
         free(p);
         return P2P_ERR_INVALID;
     }
+    if (p->tc_pack)  // n_chunks and padded are free once the items are built
+        FAIL_CUDA(p2p_tc_build(p, L.n_chunks, L.padded, L.scan_ws, s), "p2p_plan_create/tc_lists");
     // direct kernel: one item per target box (the item-sort scratch is free again)
     p->direct_k = 0;
     if (layout != P2P_LAYOUT_SYMMETRIC && layout != P2P_LAYOUT_REPETITION) {
@@ -1161,7 +1118,6 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     p->max_box = host[1];
     p->n_items = host[2];
     p->packed = packed;
-    p->tc_groups = tc_groups;
     FAIL_CUDA(p2p_pair_configure(p), "p2p_plan_create/occupancy");
 #undef FAIL_CUDA
     *plan = p;

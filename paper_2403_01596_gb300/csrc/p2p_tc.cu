@@ -1,56 +1,74 @@
-// Multi-RHS P2P on the 5th-generation tensor cores (tcgen05, TMEM accumulator).
+// Multi-RHS P2P on the 5th-generation tensor cores (tcgen05, TMEM operands).
 //
-// Contraction.  A unit of work is one target box b and a group of nt <= TG of
-// its targets (T = nt rounded up to 8).  For every group of 16 consecutive
-// box-sorted sources of a neighbour box, one real MMA chain adds
+// Contraction.  A unit of work is a window of up to 128 box-sorted targets (the
+// rows of one MMA), an entry one group of 16 consecutive box-sorted sources.  For
+// every entry with a source near one of the unit's targets two real MMA chains add
 //
-//     D[128 x 2T] += A[128 x 16] . B[16 x 2T],
-//     A[r, s] = Re lambda[s, r],  A[64 + r, s] = Im lambda[s, r]   (r: RHS within a block of 64)
-//     B[s, t] = Re G(x_t, y_s),   B[s, T + t]  = Im G(x_t, y_s),
+//     D1[128 x 2R] += Gr[128 x 16] . [Lr | Li][16 x 2R]
+//     D2[128 x 2R] += Gi[128 x 16] . [Lr | Li][16 x 2R]
 //
-// so that Re out[t, r] = D[r, t] - D[64 + r, T + t] and Im out[t, r] =
-// D[r, T + t] + D[64 + r, t] (the four real products of a complex product; no
-// padded M rows and no negated copy).  G is formed on the CUDA cores in FP32
-// (rsqrt, sincos), both operands are split x = hi + lo into BF16, and three MMAs
-// (hi.hi + hi.lo + lo.hi, kind::f16, FP32 accumulation in TMEM) keep the product
-// error near 2^-16.  With NP = 3 parts (hi + mid + lo, ~24 bits) six MMAs take
-// every part product p.q with p + q < 3, and the product error is near 2^-24.
+// with Gr, Gi = Re, Im G(x_t, y_s) (0 where s is not in t's neighbourhood or r = 0)
+// and Lr, Li = Re, Im lambda[s, r], so that Re out[t, r] = D1[t, r] - D2[t, R + r]
+// and Im out[t, r] = D1[t, R + r] + D2[t, r].  The Laplace kernel needs D1 alone.
+// G is formed on the CUDA cores in FP32 (rsqrt, sincos), both operands are split
+// x = hi + lo into BF16, and three products (hi.hi + hi.lo + lo.hi, kind::f16,
+// FP32 accumulation in TMEM) keep the product error near 2^-16.  With NP = 3 parts
+// (hi + mid + lo, ~24 bits) six products take every p.q with p + q < 3, and the
+// product error is near 2^-24.
 //
-// Group records.  The A operand of a source group does not depend on the target
-// box, so a pass per apply (k_tc_pack) writes every group's hi and lo images,
-// already in the operand's shared-memory layout, followed by the group's source
-// coordinates; the main kernel moves a record with one TMA bulk copy.  The plan
-// keeps, per box, the list of the groups of its neighbour boxes (ascending box
-// id), padded with -1 to a multiple of four entries.
+// Why this shape.  G is the MMA's A operand and goes from registers straight into
+// tensor memory: a thread owns one target (one TMEM lane), reads the entry's
+// sources as broadcasts and forms 16 pairs per stage, so the per-stage hand-offs
+// are paid once per 128 x 16 pairs, and no proxy fence or shared-memory tile is on
+// the way.  The strengths are the B operand: one record per entry serves every
+// target box of the unit.  (An earlier kernel had one target box per unit, T <= 32
+// or 64 targets on the MMA's N side and both operands in shared memory: 3.7 M
+// stages on the 2^21-point ellipsoid against 1.27 M entries here, every stage
+// bound by its hand-offs; DESIGN has both sides measured.)
 //
-// Main kernel (k_p2p_tc): persistent, one CTA per SM, units (box, target group)
-// round robin over the CTAs in Morton order (neighbouring CTAs share records in
-// L2).  Warp roles:
-//   warps 0-3    one producer per G set: walks a unit's group list four entries (a quad) at a time and
-//                issues entry 4q + s into a slot of set s (metadata, TMA bulk copy of the record, the
-//                unit's targets with the first quad)
-//   warps 4-19   four G sets of four warps: G tile in FP32, BF16 hi/lo split into the slot's B operand
-//   warps 20-23  one MMA issuer per set (one thread): once the set has written B, the three MMAs (per RHS
-//                block) into the set's own accumulator, committed to the slot's release barrier
-//   warps 24-27  epilogue: sums the sets' accumulators (TMEM -> registers), combines Re/Im through
-//                shared memory and writes out[perm[t]]
-// (with P2P_TC_SETS = 2: two producers, two sets of eight warps, entries taken in pairs)
-// Four independent issue chains (one per set) keep the tensor core fed with the
-// small (N = 2T) MMAs.  With the hi/lo split (units of up to 32 targets) two TMEM
-// buffers alternate between a CTA's units so the epilogue of one unit overlaps
-// the MMAs of the next; the three-part split takes units of up to 64 targets in
-// one buffer.
+// Group records.  The B operand of a source group does not depend on the targets,
+// so a pass per apply (k_tc_pack) writes every group's part images, already in the
+// operand's shared-memory layout, followed by the group's source coordinates and
+// markers of non-finite strengths; the main kernel moves a record with one TMA bulk
+// copy.  Groups ignore box boundaries (n / 16 of them): which of the 16 sources a
+// target meets is a 16-bit mask per (entry, target box).
+//
+// Lists (k_tc_fill, at plan time).  Blocks of 32 consecutive target boxes hold the
+// union of their neighbour boxes' groups, ascending: the group, a bit per box of
+// the block that has a neighbour source in it, and the boxes' 16-bit masks.  A
+// block's targets are cut into near-equal windows of at most 128; a window takes
+// the entries whose bits meet its own boxes.
+//
+// Main kernel (k_p2p_tc): persistent, one CTA per SM, units from a counter in
+// Morton order (neighbouring CTAs share records in L2).  Warp roles:
+//   warp 3       scout: takes units from the counter and reads their headers ahead of the producer
+//   warp 0       producer: picks the unit's entries out of its block's list and issues entry e
+//                into slot e % 16 (e % 8 where records are large): metadata, TMA bulk copies of the
+//                record and of the masks
+//   warps 1-2    MMA issuers (an elected lane each): D1 and D2 of every entry in order
+//   warps 4-7    epilogue: TMEM -> a tile in shared memory, the complex combination, out[perm[t]]
+//   warps 8-23   four G sets of four warps: entry e goes to set e % 4, which writes the BF16
+//                parts of G into TMEM operand slot e % (operand slots)
+// D occupies columns 0..255, the operand slots the other 256.  With at most 32
+// right-hand sides the small products (all but hi.hi) have accumulators of their
+// own.  The tensor core's FP32 accumulation truncates, ~2^-26 of the accumulator
+// per MMA in the same direction, so chains are kept short: a unit's list is cut
+// into near-equal segments (segment_entries), and the epilogue adds the segments in
+// FP32.
 //
 // Every wait is bounded: a wait that runs out sets the plan's status word and an
-// abort flag; every role then stops (the epilogue warps decide together through
-// a barrier reduction), the producer waits (bounded) for the bulk copies it
-// issued, each MMA issuer for its MMAs, and the CTA frees its TMEM and returns.
+// abort flag; every role then stops, the producer waits (bounded) for the bulk
+// copies it issued, each MMA issuer for its MMAs, and the CTA frees its TMEM and
+// returns.
 //
-// Operands use the canonical K-major layout without swizzle: 8-row x 16-byte
+// The B operand uses the canonical K-major layout without swizzle: 8-row x 16-byte
 // core matrices, the two K-adjacent cores of a 16-wide K slice 128 bytes apart
-// (leading byte offset) and 8-row groups 256 bytes apart (stride byte offset).
+// (leading byte offset) and 8-row groups 256 bytes apart (stride byte offset).  A
+// part of G is 8 TMEM columns, two consecutive sources per 32-bit column.
 #include <cuda_bf16.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "p2p_internal.cuh"
 
@@ -63,20 +81,18 @@ constexpr int kSrcGroup = 16;          // sources per stage (MMA K)
 constexpr int kPart = 4096;            // one BF16 image of a 128 x 16 A operand
 constexpr int kImage = 2 * kPart;      // hi + lo images (the operand self-check)
 constexpr int kLbo = 128, kSbo = 256;  // core-matrix strides (K direction, 8-row groups)
-constexpr int kSetCols = 256;          // TMEM columns of a unit buffer of 32-target units (an accumulator per set)
-// G sets (independent producer -> G -> MMA chains; 2 or 4, the group lists are
-// padded to multiples of 4).  On the 2^21-point ellipsoid at 64 RHS four sets of
-// four warps measured 5.1 ms against 5.3 for two sets of eight with units of up
-// to 64 targets; two sets would also halve the accumulators of the three-part
-// split, whose error grows with the accumulation chains.
-#ifndef P2P_TC_SETS
-#define P2P_TC_SETS 4
-#endif
-constexpr int kSets = P2P_TC_SETS;     // G sets; set s takes list entries s, s + kSets, ... of a unit
-constexpr int kSetWarps = 16 / kSets;  // warps of one G set
-constexpr int kSetThreads = 32 * kSetWarps;
-constexpr int kGWarp0 = kSets, kMmaWarp0 = kGWarp0 + kSetWarps * kSets, kEpiWarp0 = kMmaWarp0 + kSets;
-constexpr int kWarps = kEpiWarp0 + 4;
+constexpr int kRows = 128;             // targets per unit (MMA M)
+constexpr int kBlockBoxes = 32;        // target boxes per list block (a bit each)
+constexpr int kSets = 4;               // G sets; set s takes entries s, s + kSets, ...
+// Entries added up in one accumulator chain at most.  With accumulators of their own for the small products (at most
+// 32 right-hand sides) a chain takes one truncated addition per entry, otherwise every product of the split: 3 for
+// hi / lo, whose products are far less exact than that, and 6 for the three-part split, which at 48 entries measured
+// 1.3e-6 of S_i on boxes of ~140 points (the split promises 2^-20) and at 16 still 1.4 times the relative error of
+// chains of ~55 additions (1.1e-6 against 7.8e-7).
+__host__ __device__ inline int segment_entries(int rhs, int np) { return np == 3 && rhs > 32 ? 10 : 48; }
+constexpr int kAColumn = 256;          // first TMEM column of the operand slots
+constexpr int kMmaWarp0 = 1, kScoutWarp = 3, kEpiWarp0 = 4, kGWarp0 = 8;
+constexpr int kWarps = kGWarp0 + 4 * kSets;
 constexpr int kThreads = kWarps * 32;
 // A waiting thread is suspended (up to kSuspendNs per poll) until the phase
 // completes, so idle roles do not take issue slots from the working warps.
@@ -117,9 +133,24 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
     return done != 0;
 }
 
-// Bounded wait; gives up early once *abort is set.
+// One poll without suspension.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
+// Bounded wait; gives up early once *abort is set.  The first poll is the plain one: a barrier that has completed
+// costs ~15 cycles with it, ~50 with the suspending one.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           uint32_t limit = kWaitLimit) {
+    if (limit > 0u && mbar_test(bar, parity)) return true;
     for (uint32_t i = 0; i < limit; ++i) {
         if (mbar_try(bar, parity)) return true;
         if (abort && (i & 15u) == 15u && *abort) return false;
@@ -162,40 +193,57 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
         : "memory");
 }
 
+// The A operand in tensor memory (128 lanes x 8 columns for K = 16).
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
 }
 
+// One lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t e;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(e));
+    return e != 0;
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// Named barrier 5 for the epilogue warps (0 is __syncthreads).
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 5, 128;" ::: "memory"); }
-// Barrier of the 128 epilogue threads that also ORs a condition over them.
-__device__ __forceinline__ bool epi_any(bool c) {
-    int r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.s32 q, %1, 0;\n\t"
-        "bar.red.or.pred p, 5, 128, q;\n\t"
-        "selp.s32 %0, 1, 0, p;\n\t}"
-        : "=r"(r)
-        : "r"((int)c)
-        : "memory");
-    return r != 0;
-}
-
-// 32 lanes x 8 consecutive 32-bit columns of TMEM into registers.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
+// 32 lanes x 8 consecutive 32-bit columns of TMEM into registers; valid after tmem_ld_wait.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+                 : "r"(taddr)
+                 : "memory");
 }
+// Orders the uses of v after every earlier load of this thread.
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+                 :
+                 : "memory");
+}
+
+// Registers into 4 consecutive 32-bit columns of the warp's 32 lanes; complete after tmem_st_wait.
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(a), "r"(b), "r"(c),
+                 "r"(d)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 32 lanes x 16 consecutive 32-bit columns of TMEM into registers.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
@@ -211,34 +259,32 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// The two BF16 values of a word, as floats.
+__device__ __forceinline__ float2 unpack_bf16(uint32_t w) {
+    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float2 v) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+// v - w, exactly where w is v's rounding (one packed operation).
+__device__ __forceinline__ float2 residual(float2 v, float2 w) { return __ffma2_rn(w, make_float2(-1.f, -1.f), v); }
+
 // x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    float2 hf = __bfloat1622float2(h);
-    __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
+    const float2 v = make_float2(a, b);
+    hi = pack_bf16(v);
+    lo = pack_bf16(residual(v, unpack_bf16(hi)));
 }
 
 // x = hi + mid + lo with three BF16 parts (each the round-to-nearest of what the
 // previous parts leave), two values per 32-bit word: the parts carry ~24 bits.
 __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    const float2 hf = __bfloat1622float2(h);
-    const float ra = a - hf.x, rb = b - hf.y;
-    __nv_bfloat162 m = __floats2bfloat162_rn(ra, rb);
-    const float2 mf = __bfloat1622float2(m);
-    __nv_bfloat162 l = __floats2bfloat162_rn(ra - mf.x, rb - mf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    mid = *reinterpret_cast<uint32_t*>(&m);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-}
-
-__device__ __forceinline__ void split1(float a, uint16_t& hi, uint16_t& lo) {
-    __nv_bfloat16 h = __float2bfloat16_rn(a);
-    __nv_bfloat16 l = __float2bfloat16_rn(a - __bfloat162float(h));
-    hi = *reinterpret_cast<uint16_t*>(&h);
-    lo = *reinterpret_cast<uint16_t*>(&l);
+    const float2 v = make_float2(a, b);
+    hi = pack_bf16(v);
+    const float2 r = residual(v, unpack_bf16(hi));
+    mid = pack_bf16(r);
+    lo = pack_bf16(residual(r, unpack_bf16(mid)));
 }
 
 // Byte offset of element (row, k) of a K-major operand with 16-wide K slices.
@@ -246,196 +292,355 @@ __host__ __device__ inline int op_off(int row, int k) {
     return (row >> 3) * kSbo + (k >> 3) * kLbo + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// Splits n values (n = 1, 2, 4 or 8, consecutive K elements of one row) and
-// stores the hi and lo parts.
-template <int N>
-__device__ __forceinline__ void store_split(unsigned char* hi, unsigned char* lo, int off, const float (&v)[N]) {
-    if constexpr (N == 1) {
-        uint16_t h, l;
-        split1(v[0], h, l);
-        *reinterpret_cast<uint16_t*>(hi + off) = h;
-        *reinterpret_cast<uint16_t*>(lo + off) = l;
-    } else if constexpr (N == 2) {
-        uint32_t h, l;
-        split2(v[0], v[1], h, l);
-        *reinterpret_cast<uint32_t*>(hi + off) = h;
-        *reinterpret_cast<uint32_t*>(lo + off) = l;
-    } else if constexpr (N == 4) {
-        uint2 h, l;
-        split2(v[0], v[1], h.x, l.x);
-        split2(v[2], v[3], h.y, l.y);
-        *reinterpret_cast<uint2*>(hi + off) = h;
-        *reinterpret_cast<uint2*>(lo + off) = l;
-    } else {
-        uint4 h, l;
-        split2(v[0], v[1], h.x, l.x);
-        split2(v[2], v[3], h.y, l.y);
-        split2(v[4], v[5], h.z, l.z);
-        split2(v[6], v[7], h.w, l.w);
-        *reinterpret_cast<uint4*>(hi + off) = h;
-        *reinterpret_cast<uint4*>(lo + off) = l;
-    }
-}
-
-// Splits n values (n = 2, 4 or 8, consecutive K elements of one row) into NP
-// BF16 parts (2: hi, lo; 3: hi, mid, lo) stored at `off` in the images starting
-// at part0, part_bytes apart.
-template <int NP, int N>
-__device__ __forceinline__ void store_parts(unsigned char* part0, int part_bytes, int off, const float (&v)[N]) {
-    if constexpr (NP == 2) {
-        store_split<N>(part0, part0 + part_bytes, off, v);
-    } else if constexpr (N == 1) {
-        uint32_t h, m, l;
-        split3(v[0], 0.f, h, m, l);
-        *reinterpret_cast<uint16_t*>(part0 + off) = (uint16_t)(h & 0xffffu);
-        *reinterpret_cast<uint16_t*>(part0 + part_bytes + off) = (uint16_t)(m & 0xffffu);
-        *reinterpret_cast<uint16_t*>(part0 + 2 * part_bytes + off) = (uint16_t)(l & 0xffffu);
-    } else {
-        uint32_t h[N / 2], m[N / 2], l[N / 2];
+// Splits eight consecutive K elements of one row into NP BF16 parts (2: hi, lo; 3: hi, mid, lo) stored at `off`
+// in the images starting at part0, part_bytes apart.
+template <int NP>
+__device__ __forceinline__ void store_parts(unsigned char* part0, int part_bytes, int off, const float (&v)[8]) {
+    uint32_t p[NP][4];
 #pragma unroll
-        for (int i = 0; i < N / 2; ++i) split3(v[2 * i], v[2 * i + 1], h[i], m[i], l[i]);
-        unsigned char* dst[3] = {part0, part0 + part_bytes, part0 + 2 * part_bytes};
-        const uint32_t* src[3] = {h, m, l};
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if constexpr (N == 2) {
-                *reinterpret_cast<uint32_t*>(dst[q] + off) = src[q][0];
-            } else if constexpr (N == 4) {
-                *reinterpret_cast<uint2*>(dst[q] + off) = make_uint2(src[q][0], src[q][1]);
-            } else {
-                *reinterpret_cast<uint4*>(dst[q] + off) = make_uint4(src[q][0], src[q][1], src[q][2], src[q][3]);
-            }
-        }
+    for (int i = 0; i < 4; ++i) {
+        if constexpr (NP == 2) split2(v[2 * i], v[2 * i + 1], p[0][i], p[1][i]);
+        else split3(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
     }
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+        *reinterpret_cast<uint4*>(part0 + q * part_bytes + off) = make_uint4(p[q][0], p[q][1], p[q][2], p[q][3]);
 }
 
 // ----------------------------------------------------------- strength pre-pack --
 
-// Bytes of one group record: the NP BF16 part images of every block of 64 RHS,
-// then the group's 16 source coordinates (w = 1 marks a padding slot).
-__host__ __device__ inline int record_bytes(int rb_count, int np) { return rb_count * np * kPart + kSrcGroup * 16; }
+// Bytes of one group record for R = rhs (a multiple of 8) right-hand sides: NP part images of 2R rows x 16
+// sources (rows 0..R-1 Re lambda, R..2R-1 Im lambda), the group's 16 x, y and z coordinates, four marker words
+// (nonzero: some strength is not finite), and per source 64 bits naming its non-finite right-hand sides.
+__host__ __device__ inline int image_bytes(int rhs) { return 2 * rhs * kSrcGroup * 2; }
+constexpr int kXyzBytes = 3 * kSrcGroup * 4;
+constexpr int kMarkBytes = 16;
+constexpr int kBadBytes = kSrcGroup * 8;
+// the part of a record the main kernel copies, and a record's size
+__host__ __device__ inline int copy_bytes(int rhs, int np) { return np * image_bytes(rhs) + kXyzBytes + kMarkBytes; }
+__host__ __device__ inline int record_bytes(int rhs, int np) { return (copy_bytes(rhs, np) + kBadBytes + 127) / 128 * 128; }
 
-// The records of one launch (a chunk of rb_launch RHS blocks) are contiguous:
-// chunk c starts chunk_bytes * c into the buffer, group g's record
-// record_bytes(rb_launch, NP) * g into the chunk.
-//
-// Block (group g, RHS block rb), 128 threads: thread (r = tid % 64, o = tid / 64)
-// splits Re and Im lambda of RHS rb * 64 + r for sources 8o .. 8o + 7 of the
-// group into rows r and 64 + r of the group's NP part images in its chunk's
-// record.  Sources past the box's end and RHS past nrhs are zero.  The first
-// block of each chunk also writes the record's coordinates.
+// Records of the groups of RHS [rhs0, rhs0 + rhs).  2 x RP threads per group (RP: rhs rounded up to whole warps):
+// thread (o, r) splits Re and Im lambda of right-hand side rhs0 + r for sources 8o .. 8o + 7 into rows r and
+// rhs + r of the part images.  Sources past the last one and RHS past nrhs are zero, and so is a strength that is
+// not finite: its targets get their NaN in the main kernel's epilogue, since 0 x inf would reach the targets of
+// the unit that are not its neighbours as well.  Memory bound: lambda is read once in full rows of up to 512
+// bytes, the images written once.
 template <int NP>
-__global__ void __launch_bounds__(128) k_tc_pack(const float2* __restrict__ lam, int64_t ld, int32_t nrhs,
-                                                 const int32_t* __restrict__ perm, const int32_t* __restrict__ box_ptr,
-                                                 const float4* __restrict__ xs, const int32_t* __restrict__ gstart,
-                                                 int32_t nb, int32_t rb_launch, int64_t chunk_bytes,
+__global__ void __launch_bounds__(128) k_tc_pack(const float2* __restrict__ lam, int64_t ld, int32_t nrhs, int32_t rhs0,
+                                                 int32_t rhs, const int32_t* __restrict__ perm,
+                                                 const float4* __restrict__ xs, int64_t n, int32_t groups,
                                                  unsigned char* __restrict__ pack) {
-    const int g = blockIdx.x, rb = blockIdx.y;
-    // box of group g: the last c with gstart[c] <= g
-    int lo = 0, hi = nb - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (gstart[mid] <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    const int c = lo;
-    const int j = g - gstart[c];
-    const int s0 = box_ptr[c] + j * kSrcGroup;
-    const int cnt = min(kSrcGroup, box_ptr[c + 1] - s0);
-    const int lb = rb % rb_launch;
-    unsigned char* rec = pack + (rb / rb_launch) * chunk_bytes + (int64_t)g * record_bytes(rb_launch, NP);
-    if (lb == 0 && threadIdx.x < kSrcGroup) {
-        const int k = threadIdx.x;
-        reinterpret_cast<float4*>(rec + rb_launch * NP * kPart)[k] =
-            k < cnt ? xs[s0 + k] : make_float4(0.f, 0.f, 0.f, 1.f);
-    }
-    const int r = threadIdx.x & 63, o = threadIdx.x >> 6;
-    const int rr = rb * 64 + r;
+    const int rp = (rhs + 31) & ~31;                        // 32 or 64
+    const int tpg = 2 * rp;                                 // threads per group: 64 or 128
+    const int sub = threadIdx.x / tpg, tid = threadIdx.x - sub * tpg;
+    const int64_t g = (int64_t)blockIdx.x * (128 / tpg) + sub;
+    if (g >= groups) return;
+    const int o = tid / rp, r = tid - o * rp, lane = threadIdx.x & 31;
+    const int64_t s0 = g * kSrcGroup + 8 * o;
+    const int rr = rhs0 + r;
+    unsigned char* rec = pack + g * record_bytes(rhs, NP);
     float re[8], im[8];
+    uint32_t bad = 0u;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        const int k = 8 * o + e;
         float2 v = make_float2(0.f, 0.f);
-        if (k < cnt && rr < nrhs) v = lam[(int64_t)perm[s0 + k] * ld + rr];
+        if (s0 + e < n && r < rhs && rr < nrhs) v = lam[(int64_t)perm[s0 + e] * ld + rr];
+        const bool fin = isfinite(v.x) && isfinite(v.y);
+        if (!fin) v = make_float2(0.f, 0.f);
+        const uint32_t b = __ballot_sync(P2P_FULL_MASK, !fin);
+        if (lane == e) bad = b;
         re[e] = v.x;
         im[e] = v.y;
     }
-    unsigned char* img = rec + lb * NP * kPart;
-    store_parts<NP, 8>(img, kPart, op_off(r, 8 * o), re);
-    store_parts<NP, 8>(img, kPart, op_off(64 + r, 8 * o), im);
+    if (r < rhs) {
+        store_parts<NP>(rec, image_bytes(rhs), op_off(r, 8 * o), re);
+        store_parts<NP>(rec, image_bytes(rhs), op_off(rhs + r, 8 * o), im);
+    }
+    float* xyz = reinterpret_cast<float*>(rec + NP * image_bytes(rhs));
+    uint32_t* mark = reinterpret_cast<uint32_t*>(rec + NP * image_bytes(rhs) + kXyzBytes);
+    uint32_t* badw = mark + kMarkBytes / 4;
+    const int w = r >> 5;                                   // 32-bit word of the 64 right-hand sides
+    const uint32_t any = __ballot_sync(P2P_FULL_MASK, lane < 8 && bad != 0u);
+    if (lane < 8) {
+        badw[(8 * o + lane) * 2 + w] = bad;
+        if (rp == 32) badw[(8 * o + lane) * 2 + 1] = 0u;
+    }
+    if (lane == 0) {
+        mark[o * 2 + w] = any;
+        if (rp == 32) mark[o * 2 + 1] = 0u;
+    }
+    if (w == 0 && lane < 8) {
+        const float4 p = s0 + lane < n ? xs[s0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        xyz[8 * o + lane] = p.x;
+        xyz[kSrcGroup + 8 * o + lane] = p.y;
+        xyz[2 * kSrcGroup + 8 * o + lane] = p.z;
+    }
+}
+
+// -------------------------------------------------------------------- list build --
+
+// One warp per block of 32 target boxes (lane = box): an upper bound of its list (the groups that its boxes'
+// neighbours cover, with repetitions), the number of its windows, and every target's box number in the block.
+__global__ void __launch_bounds__(128) k_tc_blocks(const int32_t* __restrict__ box_ptr, int32_t nb,
+                                                   const int32_t* __restrict__ src_box_ptr,
+                                                   const int32_t* __restrict__ nbr_ptr,
+                                                   const int32_t* __restrict__ nbr_idx, int32_t nblk,
+                                                   int32_t* __restrict__ bound, int32_t* __restrict__ units,
+                                                   uint8_t* __restrict__ member) {
+    const int lane = threadIdx.x & 31;
+    const int64_t j = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (j >= nblk) return;
+    const int32_t b0 = (int32_t)j * kBlockBoxes, b1 = min(nb, b0 + kBlockBoxes);
+    const int32_t b = b0 + lane;
+    int s = 0;
+    if (b < b1)
+        for (int32_t e = nbr_ptr[b]; e < nbr_ptr[b + 1]; ++e) {
+            const int32_t c = nbr_idx[e];
+            s += (src_box_ptr[c + 1] - 1) / kSrcGroup - src_box_ptr[c] / kSrcGroup + 1;
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(P2P_FULL_MASK, s, o);
+    if (lane == 0) {
+        bound[j] = s;
+        units[j] = (box_ptr[b1] - box_ptr[b0] + kRows - 1) / kRows;
+    }
+    for (int32_t c = b0; c < b1; ++c)
+        for (int32_t t = box_ptr[c] + lane; t < box_ptr[c + 1]; t += 32) member[t] = (uint8_t)(c - b0);
+}
+
+// One CTA per block: the sorted union of its boxes' neighbour boxes (at most 32 x 27, bitonic in shared memory),
+// the groups they cover (ascending; neighbouring boxes may share one), and per group the boxes it concerns and
+// their 16-bit source masks.  Also names the block of every one of its units.
+constexpr int kFillThreads = 256;
+constexpr int kUnionSlots = 1024;
+static_assert(kBlockBoxes * 27 <= kUnionSlots, "a block's neighbour lists fit the sort buffer");
+__global__ void __launch_bounds__(kFillThreads)
+    k_tc_fill(const int32_t* __restrict__ src_box_ptr, const int32_t* __restrict__ nbr_ptr,
+              const int32_t* __restrict__ nbr_idx, int32_t nb, const int32_t* __restrict__ off,
+              const int32_t* __restrict__ ustart, int32_t* __restrict__ ecount, int32_t* __restrict__ unit_block,
+              int32_t* __restrict__ gid, uint32_t* __restrict__ bits, uint32_t* __restrict__ masks) {
+    __shared__ int32_t ub[kUnionSlots];    // sorted neighbour boxes, then the unique ones
+    __shared__ int32_t pos[kUnionSlots];   // first entry of a unique box's own groups
+    __shared__ int32_t first[kUnionSlots]; // the group at that entry
+    __shared__ int32_t wsum[kFillThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t j = blockIdx.x;
+    const int32_t b0 = j * kBlockBoxes, b1 = min(nb, b0 + kBlockBoxes);
+    const int32_t e0 = nbr_ptr[b0], ne = nbr_ptr[b1] - e0;
+    for (int32_t u = ustart[j] + tid; u < ustart[j + 1]; u += kFillThreads) unit_block[u] = j;
+    for (int i = tid; i < kUnionSlots; i += kFillThreads) ub[i] = i < ne ? nbr_idx[e0 + i] : INT32_MAX;
+    __syncthreads();
+    for (int k = 2; k <= kUnionSlots; k <<= 1)
+        for (int d = k >> 1; d > 0; d >>= 1) {
+            for (int i = tid; i < kUnionSlots; i += kFillThreads) {
+                const int l = i ^ d;
+                if (l > i) {
+                    const int32_t x = ub[i], y = ub[l];
+                    if (((i & k) == 0) ? x > y : x < y) {
+                        ub[i] = y;
+                        ub[l] = x;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    // exclusive prefix over the threads of one value each; returns the prefix, `total` the sum
+    auto block_scan = [&](int v, int& total) {
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(P2P_FULL_MASK, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        int before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < kFillThreads / 32; ++w) {
+            before += w < warp ? wsum[w] : 0;
+            all += wsum[w];
+        }
+        __syncthreads();
+        total = all;
+        return before + x - v;
+    };
+    // unique boxes, compacted (kPer consecutive slots per thread)
+    constexpr int kPer = kUnionSlots / kFillThreads;
+    int32_t v[kPer];
+    int cnt = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int p = tid * kPer + i;
+        v[i] = ub[p];
+        if (v[i] == INT32_MAX || (p > 0 && ub[p - 1] == v[i])) v[i] = -1;
+        cnt += v[i] >= 0;
+    }
+    int nu;
+    int at = block_scan(cnt, nu);  // its barriers also end every thread's reads of ub
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+        if (v[i] >= 0) ub[at++] = v[i];
+    __syncthreads();
+    // own groups of every unique box: those its predecessor has not reached
+    int lo_g[kPer], n_g[kPer];
+    cnt = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int p = tid * kPer + i;
+        lo_g[i] = n_g[i] = 0;
+        if (p < nu) {
+            const int32_t c = ub[p];
+            lo_g[i] = src_box_ptr[c] / kSrcGroup;
+            if (p > 0) lo_g[i] = max(lo_g[i], (src_box_ptr[ub[p - 1] + 1] - 1) / kSrcGroup + 1);
+            n_g[i] = (src_box_ptr[c + 1] - 1) / kSrcGroup - lo_g[i] + 1;
+        }
+        cnt += n_g[i];
+    }
+    int total;
+    at = block_scan(cnt, total);
+    const int64_t base = off[j];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int p = tid * kPer + i;
+        if (p < nu) {
+            pos[p] = at;
+            first[p] = lo_g[i];
+            for (int q = 0; q < n_g[i]; ++q) gid[base + at + q] = lo_g[i] + q;
+            at += n_g[i];
+        }
+    }
+    if (tid == 0) ecount[j] = total;
+    for (int i = tid; i < total; i += kFillThreads) bits[base + i] = 0u;
+    for (int64_t i = tid; i < (int64_t)total * (kBlockBoxes / 2); i += kFillThreads) masks[base * (kBlockBoxes / 2) + i] = 0u;
+    __syncthreads();
+    // one warp per box of the block, lane = its neighbour: the sources of neighbour c in every group c reaches
+    for (int32_t b = b0 + warp; b < b1; b += kFillThreads / 32) {
+        const int32_t f0 = nbr_ptr[b], nn = nbr_ptr[b + 1] - f0;
+        if (lane >= nn) continue;
+        const int32_t c = nbr_idx[f0 + lane], m = b - b0;
+        int lo = 0, hi = nu - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (ub[mid] < c) lo = mid + 1;
+            else hi = mid;
+        }
+        const int32_t sa = src_box_ptr[c], sb = src_box_ptr[c + 1];
+        for (int32_t g = sa / kSrcGroup; g <= (sb - 1) / kSrcGroup; ++g) {
+            const int64_t e = base + pos[lo] + (g - first[lo]);
+            const int a = max(0, sa - g * kSrcGroup), z = min(kSrcGroup, sb - g * kSrcGroup);
+            const uint32_t mk = ((1u << z) - 1u) & ~((1u << a) - 1u);
+            atomicOr(masks + e * (kBlockBoxes / 2) + (m >> 1), mk << (16 * (m & 1)));
+            atomicOr(bits + e, 1u << m);
+        }
+    }
 }
 
 // ------------------------------------------------------------------ main kernel --
 
 struct TcArgs {
-    const float4* xs;              // box-sorted coordinates
-    const unsigned char* pack;     // group records
+    const float4* xs;              // box-sorted target coordinates
+    const unsigned char* pack;     // group records of this launch's right-hand sides
+    const int32_t* off;            // per block: first entry
+    const int32_t* ecount;         // per block: entries
+    const int32_t* ustart;         // per block: first unit; [nblk]: units in all
+    const int32_t* unit_block;     // per unit: its block
+    const int32_t* gid;            // per entry: source group
+    const uint32_t* bits;          // per entry: bit m = box m of the block has a neighbour source in it
+    const uint16_t* masks;         // per entry and box of the block: which of the 16 sources are neighbours
+    const uint8_t* member;         // per sorted target: box number in its block
     const int32_t* box_ptr;
-    const int32_t* glist_off;      // per-box group lists (padded to multiples of kSets)
-    const int32_t* glist;
-    const int32_t* gcount;
     const int32_t* perm;
-    float2* out;
+    // non-finite strengths only: the neighbour lists
+    const int32_t* nbr_ptr;
+    const int32_t* nbr_idx;
+    const int32_t* src_box_ptr;
+    float2* out;                   // first right-hand side of this launch
     int64_t ld;
-    int32_t nrhs;
-    int32_t rb_count;              // RHS blocks of 64
-    int32_t tg;                    // targets per unit (multiple of 8)
-    int32_t ngrp;                  // units per box: ceil(max_box / tg)
+    int32_t nrhs;                  // right-hand sides of this launch
+    int32_t rhs;                   // the same rounded up to 8 (R)
     int32_t nb;
-    int32_t slots;                 // pipeline slots per G set
+    int32_t nblk;
     int32_t slot_bytes;
-    int32_t np;                    // BF16 parts per operand: 2 (hi, lo) or 3 (hi, mid, lo)
-    int32_t nbuf;                  // unit buffers in TMEM (512 / (kSets x 2 tg x rb_count)): 2, or 1 at 64 targets
+    int32_t slots_log;             // log2 of the record slots (3 or 4)
+    int32_t a_slots;               // TMEM operand slots (a power of two, at least kSets)
+    int32_t vec_out;               // out and ld allow 16-byte stores
     float k;
     unsigned int* status;
+    unsigned int* counter;         // [0] next unit, [1] CTAs done (both 0 between launches)
     uint32_t wait_limit;           // polls of every pipeline wait (kWaitLimit unless a self-check lowers it)
 };
 
-// Slot layout: group record (A part images, source coordinates), the unit's
-// targets, the NP parts of B (2T rows each, T <= tg), metadata.
-__host__ __device__ inline int slot_t_off(int rb_count, int np) { return record_bytes(rb_count, np); }
-__host__ __device__ inline int slot_b_off(int rb_count, int tg, int np) { return record_bytes(rb_count, np) + tg * 16; }
-__host__ __device__ inline int slot_b_half(int tg) { return (2 * tg / 8) * kSbo; }  // bytes of one B part
-__host__ __device__ inline int slot_meta_off(int rb_count, int tg, int np) {
-    return slot_b_off(rb_count, tg, np) + np * slot_b_half(tg);
-}
-__host__ __device__ inline int slot_bytes_for(int rb_count, int tg, int np) {
-    return (slot_meta_off(rb_count, tg, np) + 16 + 1023) / 1024 * 1024;
-}
-constexpr int kEpiBytes = 8 * 64 * 8;  // epilogue exchange: 8 targets x 64 RHS x complex
-__host__ __device__ inline int tc_smem_bytes(int slots, int slot_bytes) {
-    return kSets * slots * slot_bytes + kEpiBytes + 1024;  // barriers: (3 kSets slots + 4) x 8 bytes <= 1024
+// Slot layout: the copied part of a record, the entry's masks, metadata.
+constexpr int kMaskBytes = kBlockBoxes * 2;
+__host__ __device__ inline int slot_xyz_off(int rhs, int np) { return np * image_bytes(rhs); }
+__host__ __device__ inline int slot_mask_off(int rhs, int np) { return copy_bytes(rhs, np); }
+__host__ __device__ inline int slot_meta_off(int rhs, int np) { return copy_bytes(rhs, np) + kMaskBytes; }
+__host__ __device__ inline int slot_bytes_for(int rhs, int np) { return (slot_meta_off(rhs, np) + 16 + 127) / 128 * 128; }
+constexpr int kMaxSlots = 16;
+constexpr int kUnitQueue = 4;   // units the scout is ahead (a power of two)
+// barriers, the epilogue's descriptor, the unit queue, TMEM address, abort flag
+constexpr int kBarriers = 3 * kMaxSlots + 7 + 2 * kUnitQueue;
+constexpr int kBarBytes = (16 + kUnitQueue * 32 + kBarriers * 8 + 8 + 127) / 128 * 128;
+// The epilogue's tile: a row of 2R floats per target, padded so that 16-byte accesses of consecutive rows spread
+// over the banks.
+__host__ __device__ inline int tile_stride(int rhs) { return 2 * rhs + 4; }
+__host__ __device__ inline int tile_bytes(int rhs) { return kRows * tile_stride(rhs) * 4; }
+__host__ __device__ inline int tc_smem_bytes(int rhs, int np, int slots) {
+    return slots * slot_bytes_for(rhs, np) + tile_bytes(rhs) + kBarBytes;
 }
 
-// Metadata of a stage (int4): x = group (-1: padding, nothing to do), y = flags,
-// z = targets of the unit.  Flags: first quad of the unit (the stage carries the
-// unit's targets, the set's accumulator starts), last quad, done.
-constexpr int kFirst = 1, kLast = 2, kDone = 4;
+// Columns of an operand slot: NP parts of Gr and Gi, 8 columns each.
+__host__ __device__ constexpr int a_cols(int np) { return np * 16; }
+
+// Metadata of a stage (int4): x = flags, y = block's first box, z = the unit's first target, w = its targets.
+// Flags: first / last entry of a segment, the end, a segment after the unit's first, the unit's last entry; in the
+// epilogue's descriptor kFirst says that a strength of the segment is not finite.
+constexpr int kFirst = 1, kLast = 2, kDone = 4, kAdd = 8, kOut = 16;
 
 struct TcSmem {
-    unsigned char* slots;  // kSets x slots
-    float2* epi;
-    uint64_t* full;        // [kSets * slots] TMA bytes + producer arrival
-    uint64_t* full_b;      // [kSets * slots] the G set's threads (B operand written)
-    uint64_t* empty;       // [kSets * slots] MMA commit
-    uint64_t* acc_full;    // [2] one commit per set after a unit's last quad
-    uint64_t* acc_empty;   // [2] the epilogue's 128 threads
+    unsigned char* slots;
+    float* tile;           // [kRows][tile_stride] sums of the epilogue
+    uint64_t* full;        // [slots] TMA bytes + producer arrival
+    uint64_t* full_a;      // [slots] one arrival per warp of the G set (operand slot written)
+    uint64_t* done;        // [slots] MMA commits (record and operand slot free)
+    uint64_t* desc_full;   // issuer 0: a finished segment's descriptor (or the end)
+    uint64_t* acc_full;    // [2] an issuer's commit after a segment's last entry
+    uint64_t* acc_empty;   // [2] the epilogue's warps have read D1, D2
+    uint64_t* drain;       // [2] an issuer's MMAs after an abort
+    uint64_t* uq_full;     // [kUnitQueue] scout -> producer
+    uint64_t* uq_empty;    // [kUnitQueue] producer -> scout
+    int4* desc;
+    int4* uq;              // [2 kUnitQueue] unit headers
     uint32_t* tmem_slot;
     int* abort;
+    uint32_t mask, log;    // slots - 1, log2 of the slots
+    // Entry numbers run over all units of the CTA: entry e uses record slot e % slots in its (e / slots)-th round.
+    __device__ __forceinline__ uint32_t slot(uint32_t e) const { return e & mask; }
+    __device__ __forceinline__ uint32_t phase(uint32_t e) const { return (e >> log) & 1u; }
 };
 
-__device__ __forceinline__ TcSmem carve(unsigned char* smem, int slots, int slot_bytes) {
+__device__ __forceinline__ TcSmem carve(unsigned char* smem, const TcArgs& a) {
     TcSmem s;
-    const int n = kSets * slots;
+    s.log = (uint32_t)a.slots_log;
+    s.mask = (1u << s.log) - 1u;
     s.slots = smem;
-    s.epi = reinterpret_cast<float2*>(smem + (size_t)n * slot_bytes);
-    uint64_t* b = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(s.epi) + kEpiBytes);
+    unsigned char* p = smem + ((size_t)a.slot_bytes << s.log);
+    s.tile = reinterpret_cast<float*>(p);
+    p += tile_bytes(a.rhs);
+    s.desc = reinterpret_cast<int4*>(p);
+    s.uq = s.desc + 1;
+    uint64_t* b = reinterpret_cast<uint64_t*>(p + 16 + kUnitQueue * 32);
     s.full = b;
-    s.full_b = b + n;
-    s.empty = b + 2 * n;
-    s.acc_full = b + 3 * n;
-    s.acc_empty = b + 3 * n + 2;
-    s.tmem_slot = reinterpret_cast<uint32_t*>(b + 3 * n + 4);
+    s.full_a = b + kMaxSlots;
+    s.done = b + 2 * kMaxSlots;
+    s.desc_full = b + 3 * kMaxSlots;
+    s.acc_full = b + 3 * kMaxSlots + 1;
+    s.acc_empty = b + 3 * kMaxSlots + 3;
+    s.drain = b + 3 * kMaxSlots + 5;
+    s.uq_full = b + 3 * kMaxSlots + 7;
+    s.uq_empty = s.uq_full + kUnitQueue;
+    s.tmem_slot = reinterpret_cast<uint32_t*>(b + kBarriers);
     s.abort = reinterpret_cast<int*>(s.tmem_slot + 1);
     return s;
 }
@@ -445,399 +650,545 @@ __device__ __forceinline__ void set_abort(const TcArgs& a, const TcSmem& sm) {
     atomicOr(a.status, P2P_DEV_TIMEOUT | P2P_DEV_TC_FAULTED);
 }
 
-// Unit u of the round-robin sequence: target box, first target, target count (0: empty unit).  Units run box
-// by box in Morton order, a box's ngrp target groups next to each other (CTAs serving neighbouring units share
-// records in L2).  When the grid is a multiple of ngrp, each round of the grid covers whole boxes and a CTA
-// would take the same group of every box it serves -- the CTAs of the first group carrying most of the work --
-// so round k rotates the groups of its boxes by k.
-__device__ __forceinline__ void unit_of(const TcArgs& a, int64_t u, int& b, int& t0, int& nt) {
-    b = (int)(u / a.ngrp);
-    int j = (int)(u - (int64_t)b * a.ngrp);
-    if (gridDim.x % (unsigned)a.ngrp == 0) j = (int)((j + u / gridDim.x) % a.ngrp);
-    t0 = j * a.tg;
-    const int n_b = a.box_ptr[b + 1] - a.box_ptr[b];
-    nt = max(0, min(a.tg, n_b - t0));
+// Wait of a whole warp: every lane polls, and all lanes get the same answer.
+__device__ __forceinline__ bool warp_wait(const TcArgs& a, const TcSmem& sm, uint64_t* bar, uint32_t parity,
+                                          uint32_t limit) {
+    const bool ok = mbar_wait(bar, parity, sm.abort, limit);
+    if (__all_sync(P2P_FULL_MASK, ok)) return true;
+    if (!ok && !*(volatile int*)sm.abort) set_abort(a, sm);
+    return false;
 }
 
-// Ring of one set's slots: slot index and the parity of its round.
-struct Ring {
-    int slot;
-    uint32_t phase;
-    __device__ __forceinline__ void advance(int slots) {
-        if (++slot == slots) {
-            slot = 0;
-            phase ^= 1u;
-        }
-    }
-};
-
-// ---- producer of set s (one warp; lane 0 issues) ----
-// A unit's group list is walked four entries (a quad) at a time, entry 4q + s going to set s.
-template <bool LIMITED>
-__device__ void run_producer(const TcArgs& a, const TcSmem& sm, int64_t units, int set, int lane) {
-    volatile int* abort = sm.abort;
+// ---- scout (one warp) ----
+// Unit headers: (block's first box, first target, targets, entries), (first list entry, list length, the window's
+// boxes as bits, entries per segment).  Its chain of dependent loads takes several microseconds a unit, which the
+// queue hides.  Zero entries end the queue.
+template <bool LIMITED, int NP>
+__device__ void run_scout(const TcArgs& a, const TcSmem& sm, int lane) {
     const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
-    const bool active = lane == 0;
-    Ring r{0, 0u};
-    int64_t staged = 0;  // stages this producer has armed (their copies may still be in flight)
-    const uint32_t rec = (uint32_t)record_bytes(a.rb_count, a.np);
-    const int t_off = slot_t_off(a.rb_count, a.np), meta_off = slot_meta_off(a.rb_count, a.tg, a.np);
+    const int units = a.ustart[a.nblk];
+    auto next_unit = [&]() { return lane == 0 ? (int)atomicAdd(a.counter, 1u) : 0; };
+    uint32_t at = 0;
+    int un = next_unit();
+    while (true) {
+        const int u = __shfl_sync(P2P_FULL_MASK, un, 0);
+        int4 h0 = make_int4(0, 0, 0, 0), h1 = h0;
+        if (u < units) {
+            un = next_unit();
+            const int j = a.unit_block[u];
+            const int b0 = j * kBlockBoxes;
+            const int p0 = a.box_ptr[b0], p1 = a.box_ptr[min(a.nb, b0 + kBlockBoxes)];
+            const int off = a.off[j], E = a.ecount[j], first = a.ustart[j], windows = a.ustart[j + 1] - first;
+            const int size = (p1 - p0 + windows - 1) / windows;
+            const int t0 = p0 + (u - first) * size;
+            const int nt = min(size, p1 - t0);
+            if (nt <= 0) continue;
+            const int m0 = a.member[t0], m1 = a.member[t0 + nt - 1];
+            const uint32_t want = (0xffffffffu << m0) & (0xffffffffu >> (31 - m1));
+            int cnt = 0;
+#pragma unroll 4
+            for (int i = lane; i < E; i += 32) cnt += (a.bits[(int64_t)off + i] & want) != 0u;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(P2P_FULL_MASK, cnt, o);
+            if (cnt == 0) continue;  // two point sets, no source nearby: the rows keep the zeros written before the launch
+            const int most = segment_entries(a.rhs, NP), segments = (cnt + most - 1) / most;
+            h0 = make_int4(b0, t0, nt, cnt);
+            h1 = make_int4(off, E, (int)want, (cnt + segments - 1) / segments);
+        }
+        const uint32_t q = at & (uint32_t)(kUnitQueue - 1), ph = (at / kUnitQueue) & 1u;
+        if (!warp_wait(a, sm, &sm.uq_empty[q], ph ^ 1u, wlim)) return;
+        if (lane == 0) {
+            sm.uq[2 * q] = h0;
+            sm.uq[2 * q + 1] = h1;
+            mbar_arrive(&sm.uq_full[q]);
+        }
+        __syncwarp();
+        if (h0.w == 0) return;
+        ++at;
+    }
+}
+
+// ---- producer (one warp) ----
+// Up to kBatch entries at a time, a lane each: the polls, the fence and the barrier operations of a batch overlap
+// (one lane issuing entry by entry took ~1 000 cycles per entry).
+constexpr int kBatch = 2;
+template <bool LIMITED, int NP>
+__device__ void run_producer(const TcArgs& a, const TcSmem& sm, int lane) {
+    const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
+    const uint32_t copy = (uint32_t)copy_bytes(a.rhs, NP);
+    const int64_t rec = record_bytes(a.rhs, NP);
+    const int mask_off = slot_mask_off(a.rhs, NP), meta_off = slot_meta_off(a.rhs, NP);
+    // entry ee's slot is free (lanes with `mine`)
+    auto claim = [&](bool mine, uint32_t ee) {
+        bool ok = true;
+        if (mine) ok = mbar_wait(&sm.done[sm.slot(ee)], sm.phase(ee) ^ 1u, sm.abort, wlim);
+        if (__all_sync(P2P_FULL_MASK, ok)) return true;
+        if (!ok && !*(volatile int*)sm.abort) set_abort(a, sm);
+        return false;
+    };
+    uint32_t e = 0, armed = 0;  // entries numbered; entries whose copies may still be in flight
     bool failed = false;
-    auto slot_base = [&](int slot) { return sm.slots + (size_t)(set * a.slots + slot) * a.slot_bytes; };
-    for (int64_t u = blockIdx.x; u < units && !failed; u += gridDim.x) {
-        int b, t0, nt;
-        unit_of(a, u, b, t0, nt);
-        if (nt == 0) continue;
-        const int off = a.glist_off[b], len = a.glist_off[b + 1] - off;
-        const float4* tsrc = a.xs + a.box_ptr[b] + t0;
-        for (int w0 = 0; w0 < len && !failed; w0 += 32) {
-            // 32 entries of the list (8 quads) in the warp's lanes
-            const int gl = w0 + lane < len ? a.glist[off + w0 + lane] : -1;
-            const int nq = min(32 / kSets, (len - w0) / kSets);
-            for (int q = 0; q < nq; ++q) {
-                const int g = __shfl_sync(P2P_FULL_MASK, gl, q * kSets + set);
-                bool ok = true;
-                if (active) ok = mbar_wait(&sm.empty[set * a.slots + r.slot], r.phase ^ 1u, abort, wlim);
-                if (!__all_sync(P2P_FULL_MASK, ok)) {
-                    if (!ok && !*abort) set_abort(a, sm);
+    for (uint32_t at = 0; !failed; ++at) {
+        const uint32_t q = at & (uint32_t)(kUnitQueue - 1);
+        if (!warp_wait(a, sm, &sm.uq_full[q], (at / kUnitQueue) & 1u, wlim)) {
+            failed = true;
+            break;
+        }
+        const int4 h0 = sm.uq[2 * q], h1 = sm.uq[2 * q + 1];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.uq_empty[q]);
+        const int b0 = h0.x, t0 = h0.y, nt = h0.z, cnt = h0.w, E = h1.y, len = h1.w;
+        if (cnt == 0) break;
+        const int64_t off = h1.x;
+        const uint32_t want = (uint32_t)h1.z;
+        int k = 0;  // entries of the unit so far
+        uint32_t bt = lane < E ? a.bits[off + lane] : 0u;
+        int g = lane < E ? a.gid[off + lane] : 0;
+        for (int w0 = 0; w0 < E && !failed; w0 += 32) {
+            const bool valid = (bt & want) != 0u;
+            const int gs = g;
+            const bool in = w0 + 32 + lane < E;  // the next 32 entries, in flight
+            bt = in ? a.bits[off + w0 + 32 + lane] : 0u;
+            g = in ? a.gid[off + w0 + 32 + lane] : 0;
+            const uint32_t todo = __ballot_sync(P2P_FULL_MASK, valid);
+            const int rank = __popc(todo & ((1u << lane) - 1u)), n = __popc(todo);
+            const uint32_t ee = e + (uint32_t)rank;
+            const int kk = k + rank, in_seg = kk % len;
+            const int flags = (in_seg == 0 ? kFirst : 0) | (in_seg == len - 1 || kk == cnt - 1 ? kLast : 0) |
+                              (kk >= len ? kAdd : 0) | (kk == cnt - 1 ? kOut : 0);
+            for (int i0 = 0; i0 < n; i0 += kBatch) {
+                const bool mine = valid && rank >= i0 && rank < i0 + kBatch;
+                if (!claim(mine, ee)) {
                     failed = true;
                     break;
                 }
-                if (active) {
-                    unsigned char* base = slot_base(r.slot);
-                    const int qq = w0 / kSets + q;
-                    const bool first = qq == 0, last = w0 + (q + 1) * kSets == len;
-                    *reinterpret_cast<int4*>(base + meta_off) =
-                        make_int4(g, (first ? kFirst : 0) | (last ? kLast : 0), nt, 0);
-                    uint64_t* bar = &sm.full[set * a.slots + r.slot];
-                    if (g >= 0) {
-                        fence_async_smem();  // the slot was last read through the generic proxy
-                        mbar_expect_tx(bar, rec + (first ? (uint32_t)nt * 16u : 0u));
-                        bulk_g2s(base, a.pack + (int64_t)g * rec, rec, bar);
-                        if (first) bulk_g2s(base + t_off, tsrc, (uint32_t)nt * 16u, bar);
-                    } else {
-                        mbar_arrive(bar);
-                    }
+                if (mine) {
+                    unsigned char* base = sm.slots + (size_t)sm.slot(ee) * a.slot_bytes;
+                    uint64_t* bar = &sm.full[sm.slot(ee)];
+                    *reinterpret_cast<int4*>(base + meta_off) = make_int4(flags, b0, t0, nt);
+                    fence_async_smem();  // the slot was last read through the generic proxy
+                    mbar_expect_tx(bar, copy + (uint32_t)kMaskBytes);
+                    bulk_g2s(base, a.pack + gs * rec, copy, bar);
+                    bulk_g2s(base + mask_off, a.masks + (off + w0 + lane) * kBlockBoxes, (uint32_t)kMaskBytes, bar);
                 }
-                ++staged;
-                r.advance(a.slots);
+                __syncwarp();
+                armed = e + (uint32_t)min(n, i0 + kBatch);
             }
+            e += (uint32_t)n;
+            k += n;
         }
     }
-    // a terminal stage for each set
+    // a terminal stage for every G set (the issuers stop at the first)
     if (!failed) {
-        bool ok = true;
-        if (active) ok = mbar_wait(&sm.empty[set * a.slots + r.slot], r.phase ^ 1u, abort, wlim);
-        if (__all_sync(P2P_FULL_MASK, ok)) {
-            if (active) {
-                *reinterpret_cast<int4*>(slot_base(r.slot) + meta_off) = make_int4(-1, kDone, 0, 0);
-                mbar_arrive(&sm.full[set * a.slots + r.slot]);
-            }
-        } else {
-            if (!ok && !*abort) set_abort(a, sm);
-            failed = true;
+        const bool mine = lane < kSets;
+        const uint32_t ee = e + (uint32_t)lane;
+        failed = !claim(mine, ee);
+        if (!failed && mine) {
+            *reinterpret_cast<int4*>(sm.slots + (size_t)sm.slot(ee) * a.slot_bytes + meta_off) = make_int4(kDone, 0, -1, 0);
+            mbar_arrive(&sm.full[sm.slot(ee)]);
         }
     }
-    if (failed && active) {
-        // wait (bounded) for the bulk copies of this set's latest round of slots (the ones it has armed)
-        const int armed = (int)(staged < a.slots ? staged : a.slots);
-        for (int i = 0; i < armed; ++i) {
-            if (--r.slot < 0) {
-                r.slot += a.slots;
-                r.phase ^= 1u;
-            }
-            mbar_wait(&sm.full[set * a.slots + r.slot], r.phase, nullptr, kDrainLimit);
-        }
-    }
+    if (failed && lane == 0)  // wait (bounded) for the copies of the latest round of slots
+        for (uint32_t i = armed > sm.mask + 1u ? armed - sm.mask - 1u : 0u; i < armed; ++i)
+            mbar_wait(&sm.full[sm.slot(i)], sm.phase(i), nullptr, kDrainLimit);
 }
 
-// ---- G sets (128 threads each); the set's first thread issues its MMAs ----
-// G tile part of one thread: target tx against sources h SP .. h SP + SP - 1.
-// For SP >= 2 the sources go in pairs through the packed two-lane FP32
-// instructions (each rounding as its scalar counterpart); rsqrt and sincos
-// stay per pair.  r = 0 and padding slots (w = 1) give 0.
-template <int KERN, int SP, int NP>
-__device__ __forceinline__ void g_tile(const float4* __restrict__ sx, float4 tx, int t, int h, int T,
-                                       unsigned char* b_part0, int b_part_bytes, float k) {
-    float re[SP], im[SP];
-    if constexpr (SP == 1) {
-        const float4 p = sx[h];
-        const float dx = p.x - tx.x, dy = p.y - tx.y, dz = p.z - tx.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float inv = rsqrtf(r2);
-        const bool ok = r2 > 0.f && p.w == 0.f;
-        if (KERN == P2P_LAPLACE) {
-            re[0] = ok ? inv : 0.f;
-            im[0] = 0.f;
-        } else {
-            float sn, cs;
-            __sincosf(k * (r2 * inv), &sn, &cs);
-            re[0] = ok ? cs * inv : 0.f;
-            im[0] = ok ? sn * inv : 0.f;
-        }
-    } else {
-        const float2 ntx = make_float2(-tx.x, -tx.x), nty = make_float2(-tx.y, -tx.y), ntz = make_float2(-tx.z, -tx.z);
-        const float2 k2 = make_float2(k, k);
+// ---- G sets (128 threads each: thread = target = TMEM lane) ----
+// G of target t (negated coordinates ntx, nty, ntz) against sources 8H .. 8H + 7 of the entry, those of `mask`:
+// NP BF16 parts of Re and Im, two sources per word.  The sources go in pairs through the packed two-lane FP32
+// instructions; rsqrt and sincos stay per pair.  r = 0 and sources outside the mask give 0 (whatever their
+// distance evaluates to).
+template <int KERN, int NP, int H>
+__device__ __forceinline__ void g_eight(const float* __restrict__ xyz, float2 ntx, float2 nty, float2 ntz, float2 k2,
+                                        uint32_t mask, uint32_t (&re)[NP][4], uint32_t (&im)[NP][4]) {
 #pragma unroll
-        for (int e = 0; e < SP; e += 2) {
-            const float4 p0 = sx[h * SP + e], p1 = sx[h * SP + e + 1];
-            const float2 dx = __fadd2_rn(make_float2(p0.x, p1.x), ntx);
-            const float2 dy = __fadd2_rn(make_float2(p0.y, p1.y), nty);
-            const float2 dz = __fadd2_rn(make_float2(p0.z, p1.z), ntz);
+    for (int q = 0; q < 2; ++q) {
+        const float4 X = *reinterpret_cast<const float4*>(xyz + 8 * H + 4 * q);
+        const float4 Y = *reinterpret_cast<const float4*>(xyz + kSrcGroup + 8 * H + 4 * q);
+        const float4 Z = *reinterpret_cast<const float4*>(xyz + 2 * kSrcGroup + 8 * H + 4 * q);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int s = 8 * H + 4 * q + 2 * c, w = 2 * q + c;
+            const float2 dx = __fadd2_rn(c ? make_float2(X.z, X.w) : make_float2(X.x, X.y), ntx);
+            const float2 dy = __fadd2_rn(c ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y), nty);
+            const float2 dz = __fadd2_rn(c ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y), ntz);
             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
             const float2 inv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-            const bool ok0 = r2.x > 0.f && p0.w == 0.f, ok1 = r2.y > 0.f && p1.w == 0.f;
-            if (KERN == P2P_LAPLACE) {
-                re[e] = ok0 ? inv.x : 0.f;
-                re[e + 1] = ok1 ? inv.y : 0.f;
-                im[e] = im[e + 1] = 0.f;
-            } else {
+            const bool ok0 = r2.x > 0.f && ((mask >> s) & 1u), ok1 = r2.y > 0.f && ((mask >> (s + 1)) & 1u);
+            float2 gr = inv, gi = make_float2(0.f, 0.f);
+            if (KERN == P2P_HELMHOLTZ) {
                 const float2 ph = __fmul2_rn(k2, __fmul2_rn(r2, inv));
                 float2 sn, cs;
                 __sincosf(ph.x, &sn.x, &cs.x);
                 __sincosf(ph.y, &sn.y, &cs.y);
-                const float2 gr = __fmul2_rn(cs, inv), gi = __fmul2_rn(sn, inv);
-                re[e] = ok0 ? gr.x : 0.f;
-                re[e + 1] = ok1 ? gr.y : 0.f;
-                im[e] = ok0 ? gi.x : 0.f;
-                im[e + 1] = ok1 ? gi.y : 0.f;
+                gr = __fmul2_rn(cs, inv);
+                gi = __fmul2_rn(sn, inv);
+            }
+            const float r0 = ok0 ? gr.x : 0.f, r1 = ok1 ? gr.y : 0.f;
+            if constexpr (NP == 2) split2(r0, r1, re[0][w], re[1][w]);
+            else split3(r0, r1, re[0][w], re[1][w], re[2][w]);
+            if (KERN == P2P_HELMHOLTZ) {
+                const float i0 = ok0 ? gi.x : 0.f, i1 = ok1 ? gi.y : 0.f;
+                if constexpr (NP == 2) split2(i0, i1, im[0][w], im[1][w]);
+                else split3(i0, i1, im[0][w], im[1][w], im[2][w]);
             }
         }
     }
-    store_parts<NP, SP>(b_part0, b_part_bytes, op_off(t, h * SP), re);
-    store_parts<NP, SP>(b_part0, b_part_bytes, op_off(T + t, h * SP), im);
+}
+
+// The eight sources' parts into operand slot `col`: part p of Re at columns 16p + 4H.., of Im 8 further.
+template <int KERN, int NP, int H>
+__device__ __forceinline__ void store_eight(uint32_t col, const uint32_t (&re)[NP][4], const uint32_t (&im)[NP][4]) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        tmem_st4(col + 16 * p + 4 * H, re[p][0], re[p][1], re[p][2], re[p][3]);
+        if (KERN == P2P_HELMHOLTZ) tmem_st4(col + 16 * p + 8 + 4 * H, im[p][0], im[p][1], im[p][2], im[p][3]);
+    }
 }
 
 template <int KERN, bool LIMITED, int NP>
-__device__ void run_gset(const TcArgs& a, const TcSmem& sm, int set, int i) {
-    volatile int* abort = sm.abort;
+__device__ void run_gset(const TcArgs& a, const TcSmem& sm, uint32_t tmem, int set, int quadrant, int lane) {
     const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
-    const int t_off = slot_t_off(a.rb_count, NP), b_off = slot_b_off(a.rb_count, a.tg, NP);
-    const int b_half = slot_b_half(a.tg), meta_off = slot_meta_off(a.rb_count, a.tg, NP);
-    // this thread's task in the current unit: target t, sources h sp .. h sp + sp - 1 (set at the unit's first quad)
-    float4 tx = make_float4(0.f, 0.f, 0.f, 0.f);
-    int T = 8, sp = 1, t = 0, h = 0;
-    bool act = false;
-    Ring r{0, 0u};
-    while (true) {
-        const int idx = set * a.slots + r.slot;
-        unsigned char* base = sm.slots + (size_t)idx * a.slot_bytes;
-        if (!mbar_wait(&sm.full[idx], r.phase, abort, wlim)) {
-            if (!*abort) set_abort(a, sm);
+    const int xyz_off = slot_xyz_off(a.rhs, NP), mask_off = slot_mask_off(a.rhs, NP), meta_off = slot_meta_off(a.rhs, NP);
+    const int row = quadrant * 32 + lane;
+    const uint32_t lane_addr = tmem + ((uint32_t)(quadrant * 32) << 16) + (uint32_t)kAColumn;
+    const float2 k2 = make_float2(a.k, a.k);
+    float2 ntx = make_float2(0.f, 0.f), nty = ntx, ntz = ntx;
+    int unit = -1, m = -1;  // first target of the current unit, this target's box number (-1: no target)
+    for (uint32_t e = (uint32_t)set;; e += kSets) {
+        unsigned char* base = sm.slots + (size_t)sm.slot(e) * a.slot_bytes;
+        if (!warp_wait(a, sm, &sm.full[sm.slot(e)], sm.phase(e), wlim)) break;
+        const int4 meta = *reinterpret_cast<const int4*>(base + meta_off);
+        if (meta.x & kDone) {
+            if (lane == 0) mbar_arrive(&sm.full_a[sm.slot(e)]);
             break;
         }
-        const int4 m = *reinterpret_cast<const int4*>(base + meta_off);
-        if (m.y & kDone) break;
-        if (m.y & kFirst) {
-            T = (m.z + 7) & ~7;
-            // sources per task: the smallest power of two with 16 T / SP <= kSetThreads tasks
-            sp = 1;
-            while (kSrcGroup * T > sp * kSetThreads) sp <<= 1;
-            // eight consecutive threads take eight consecutive targets (rows of one 8-row core matrix) and the
-            // next bits the source slices, so a warp's B stores fill whole core matrices (no bank conflicts)
-            const int rest = i >> 3, H = kSrcGroup / sp;
-            h = rest % H;
-            t = (rest / H) * 8 + (i & 7);
-            act = t < T;
-            // the targets travel with the real stages of the first quad
-            if (m.x >= 0) {
-                const float4* st = reinterpret_cast<const float4*>(base + t_off);
-                tx = t < m.z ? st[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (meta.z != unit) {
+            unit = meta.z;
+            m = -1;
+            if (row < meta.w) {
+                const float4 t = a.xs[unit + row];
+                m = a.member[unit + row];
+                ntx = make_float2(-t.x, -t.x);
+                nty = make_float2(-t.y, -t.y);
+                ntz = make_float2(-t.z, -t.z);
             }
         }
-        if (m.x >= 0) {
-            const float4* sx = reinterpret_cast<const float4*>(base + NP * kPart * a.rb_count);
-            if (act) {
-                unsigned char* b0 = base + b_off;
-                if (sp == 8) g_tile<KERN, 8, NP>(sx, tx, t, h, T, b0, b_half, a.k);
-                else if (sp == 4) g_tile<KERN, 4, NP>(sx, tx, t, h, T, b0, b_half, a.k);
-                else if (sp == 2) g_tile<KERN, 2, NP>(sx, tx, t, h, T, b0, b_half, a.k);
-                else g_tile<KERN, 1, NP>(sx, tx, t, h, T, b0, b_half, a.k);
-            }
-            fence_async_smem();
-        }
-        mbar_arrive(&sm.full_b[idx]);
-        r.advance(a.slots);
-    }
-}
-
-// ---- MMA issuer of a set (one thread) ----
-template <bool LIMITED, int NP>
-__device__ void run_mma(const TcArgs& a, const TcSmem& sm, uint32_t tmem, int set) {
-    volatile int* abort = sm.abort;
-    const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
-    const int b_off = slot_b_off(a.rb_count, a.tg, NP), b_half = slot_b_half(a.tg);
-    const int meta_off = slot_meta_off(a.rb_count, a.tg, NP);
-    const uint32_t acc_cols = (uint32_t)(a.rb_count * 2 * a.tg), bufcols = 512u / (uint32_t)a.nbuf;
-    // The issuing thread is on every stage's critical path: per stage it only adds the slot's offset to
-    // descriptors and accumulator addresses prepared here (a descriptor's start address is its low 14 bits, in
-    // 16-byte units, and shared memory stays below 2^18 bytes, so the sum never carries out of the field).
-    const uint32_t set_base = smem_u32(sm.slots + (size_t)set * a.slots * a.slot_bytes);
-    const uint64_t da_set = smem_desc(set_base), db_set = smem_desc(set_base + (uint32_t)b_off);
-    const uint32_t d_set = tmem + (uint32_t)set * acc_cols;
-    Ring r{0, 0u}, ab{0, 0u};  // pipeline slot; accumulator buffer of the current unit
-    bool acc_started = false, issued = false;
-    while (true) {
-        const int idx = set * a.slots + r.slot;
-        unsigned char* base = sm.slots + (size_t)idx * a.slot_bytes;
-        if (!mbar_wait(&sm.full[idx], r.phase, abort, wlim)) {
-            if (!*abort) set_abort(a, sm);
-            break;
-        }
-        const int4 m = *reinterpret_cast<const int4*>(base + meta_off);
-        if (m.y & kDone) break;
-        const uint32_t ub = (uint32_t)ab.slot;
-        if (m.y & kFirst) {
-            // the epilogue has released this accumulator buffer (unit - nbuf)
-            if (!mbar_wait(&sm.acc_empty[ub], ab.phase ^ 1u, abort, wlim)) {
-                if (!*abort) set_abort(a, sm);
-                break;
-            }
-            acc_started = false;
-        }
-        if (!mbar_wait(&sm.full_b[idx], r.phase, abort, wlim)) {
-            if (!*abort) set_abort(a, sm);
-            break;
-        }
-        tc_fence_after();
-        if (m.x >= 0) {
-            const int T = (m.z + 7) & ~7;
-            const uint32_t idesc = idesc_bf16_f32(2 * T);
-            // descriptors address 16-byte units: part p of an operand is p * bytes-per-part / 16 further
-            const uint64_t slot16 = (uint64_t)(((uint32_t)r.slot * (uint32_t)a.slot_bytes) >> 4);
-            const uint64_t db0 = db_set + slot16;
-            const uint64_t db_step = (uint64_t)(b_half >> 4);
-            const uint32_t d0 = d_set + ub * bufcols;
-            for (int rb = 0; rb < a.rb_count; ++rb) {
-                const uint64_t da0 = da_set + slot16 + (uint64_t)((rb * NP * kPart) >> 4);
-                const uint64_t da_step = (uint64_t)(kPart >> 4);
-                const uint32_t d = d0 + (uint32_t)(rb * 2 * a.tg);
-                // every product of parts p (of lambda) and q (of G) with p + q < NP: 3 MMAs for hi / lo,
-                // 6 for hi / mid / lo (the dropped products are below 2^-8 NP of the leading one)
-                mma_bf16(d, da0, db0, idesc, acc_started ? 1u : 0u);
-                mma_bf16(d, da0, db0 + db_step, idesc, 1u);
-                mma_bf16(d, da0 + da_step, db0, idesc, 1u);
-                if constexpr (NP == 3) {
-                    mma_bf16(d, da0, db0 + 2 * db_step, idesc, 1u);
-                    mma_bf16(d, da0 + da_step, db0 + db_step, idesc, 1u);
-                    mma_bf16(d, da0 + 2 * da_step, db0, idesc, 1u);
-                }
-            }
-            acc_started = true;
-        }
-        mma_commit(&sm.empty[idx]);
-        issued = true;
-        if (m.y & kLast) {
-            mma_commit(&sm.acc_full[ub]);
-            ab.advance(a.nbuf);
-        }
-        r.advance(a.slots);
-    }
-    if (*abort && issued) {
-        // the latest commit arrives once every MMA issued before it has completed
-        if (--r.slot < 0) {
-            r.slot += a.slots;
-            r.phase ^= 1u;
-        }
-        mbar_wait(&sm.empty[set * a.slots + r.slot], r.phase, nullptr, kDrainLimit);
-    }
-}
-
-// ---- epilogue (128 threads, TMEM lanes by warp quadrant) ----
-template <bool LIMITED>
-__device__ void run_epilogue(const TcArgs& a, const TcSmem& sm, uint32_t tmem, int64_t units, int warp, int lane) {
-    volatile int* abort = sm.abort;
-    const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
-    const int q = warp & 3;
-    const int m = q * 32 + lane;  // accumulator row
-    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    const uint32_t acc_cols = (uint32_t)(a.rb_count * 2 * a.tg);
-    const uint32_t bufcols = 512u / (uint32_t)a.nbuf;
-    Ring eb{0, 0u};  // accumulator buffer of the next unit
-    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
-        int b, t0, nt;
-        unit_of(a, u, b, t0, nt);
-        // a box without any source group (two point sets, no source nearby) has no stages and no accumulator:
-        // the producer skips it too, and its results stay at the zeros written before the launch
-        if (nt == 0 || a.gcount[b] == 0) continue;
-        // sets with work in this unit: entries 0 .. gcount - 1 of the list go to sets 0, 1, 2, 3, 0, ...
-        const int used = min(kSets, a.gcount[b]);
-        const int T = (nt + 7) & ~7;
-        const int tb = a.box_ptr[b] + t0;
-        const uint32_t ub = (uint32_t)eb.slot, par = eb.phase;
-        eb.advance(a.nbuf);
-        const bool ok = mbar_wait(&sm.acc_full[ub], par, abort, wlim);
-        // the 128 threads leave together (they meet at named barriers below)
-        if (epi_any(!ok)) {
-            if (!ok && !*abort) set_abort(a, sm);
-            return;
-        }
-        tc_fence_after();
-        for (int rb = 0; rb < a.rb_count; ++rb) {
-            const int r = rb * 64 + (m & 63);
-            for (int c0 = 0; c0 < T; c0 += 8) {
-                __syncwarp();
-                int prow[8];
-                if (m < 64) {
+        const uint32_t mask = m >= 0 ? reinterpret_cast<const uint16_t*>(base + mask_off)[m] : 0u;
+        const float* xyz = reinterpret_cast<const float*>(base + xyz_off);
+        const uint32_t col = lane_addr + (e & (uint32_t)(a.a_slots - 1)) * (uint32_t)a_cols(NP);
+        // halves of the group that hold a source near one of the warp's targets
+        const uint32_t some = __reduce_or_sync(P2P_FULL_MASK, mask);
+        const bool any0 = (some & 0xffu) != 0u, any1 = some > 0xffu;
+        uint32_t re[NP][4], im[NP][4];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) prow[j] = c0 + j < nt ? a.perm[tb + c0 + j] : 0;
-                }
-                const uint32_t col = lane_addr + ub * bufcols + (uint32_t)(rb * 2 * a.tg + c0);
-                float x[8], y[8];
-                tmem_ld8(col, x);
-                tmem_ld8(col + (uint32_t)T, y);
-                for (int s = 1; s < used; ++s) {
-                    float x1[8], y1[8];
-                    tmem_ld8(col + (uint32_t)s * acc_cols, x1);
-                    tmem_ld8(col + (uint32_t)s * acc_cols + (uint32_t)T, y1);
+        for (int p = 0; p < NP; ++p)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        x[j] += x1[j];
-                        y[j] += y1[j];
-                    }
-                }
-                // rows 64..127 (Im lambda) hand (-D[., T + t], D[., t]) to rows 0..63
-                if (m >= 64) {
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) sm.epi[j * 64 + (m - 64)] = make_float2(-y[j], x[j]);
-                }
-                epi_sync();
-                if (m < 64 && r < a.nrhs) {
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (c0 + j < nt) {
-                            const float2 w = sm.epi[j * 64 + m];
-                            a.out[(int64_t)prow[j] * a.ld + r] =
-                                make_float2((x[j] + w.x) * kInv4Pi, (y[j] + w.y) * kInv4Pi);
-                        }
-                    }
-                }
-                epi_sync();
-            }
+            for (int w = 0; w < 4; ++w) re[p][w] = im[p][w] = 0u;
+        if (any0) g_eight<KERN, NP, 0>(xyz, ntx, nty, ntz, k2, mask, re, im);
+        // the operand slot is free: the MMAs of entry e - a_slots are done
+        if (e >= (uint32_t)a.a_slots) {
+            const uint32_t p = e - (uint32_t)a.a_slots;
+            if (!warp_wait(a, sm, &sm.done[sm.slot(p)], sm.phase(p), wlim)) break;
+            tc_fence_after();
         }
+        store_eight<KERN, NP, 0>(col, re, im);
+        if (any1) {
+            g_eight<KERN, NP, 1>(xyz, ntx, nty, ntz, k2, mask, re, im);
+        } else if (any0) {
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+#pragma unroll
+                for (int w = 0; w < 4; ++w) re[p][w] = im[p][w] = 0u;
+        }
+        store_eight<KERN, NP, 1>(col, re, im);
+        tmem_st_wait();
         tc_fence_before();
-        mbar_arrive(&sm.acc_empty[ub]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.full_a[sm.slot(e)]);
+    }
+}
+
+// ---- MMA issuer Q (one warp, an elected lane): Q = 0 adds Gr [Lr | Li] into D1, Q = 1 Gi [Lr | Li] into D2 ----
+template <bool LIMITED, int NP>
+__device__ void run_mma(const TcArgs& a, const TcSmem& sm, uint32_t tmem, int q) {
+    const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
+    const int meta_off = slot_meta_off(a.rhs, NP), mark_off = slot_xyz_off(a.rhs, NP) + kXyzBytes;
+    const uint32_t idesc = idesc_bf16_f32(2 * a.rhs);
+    // a descriptor's start address is its low 14 bits, in 16-byte units: a slot adds its offset, a part its own
+    // (shared memory stays below 2^18 bytes, so the sums never carry out of the field)
+    const uint64_t db_all = smem_desc(smem_u32(sm.slots));
+    const uint32_t slot16 = (uint32_t)a.slot_bytes >> 4;
+    const uint64_t part = (uint64_t)(image_bytes(a.rhs) >> 4);
+    const uint32_t d_hh = tmem + (uint32_t)q * 128u;                 // hi.hi
+    const uint32_t d_x = a.rhs <= 32 ? d_hh + 64u : d_hh;            // the smaller products
+    const uint32_t own_x = a.rhs <= 32 ? 0u : 1u;
+    const uint32_t ga_all = tmem + (uint32_t)kAColumn + 8u * (uint32_t)q, a_mask = (uint32_t)(a.a_slots - 1);
+    const int lane = threadIdx.x & 31;
+    // The products of one entry (the elected lane): every product of parts p (of G) and r (of lambda) with
+    // p + r < NP; the dropped ones are below 2^-8 NP of the leading one.
+    auto issue = [&](uint32_t ga, uint64_t lb, uint32_t acc, uint64_t* done) {
+        mma_bf16_ts(d_hh, ga, lb, idesc, acc);
+        mma_bf16_ts(d_x, ga, lb + part, idesc, acc | own_x);
+        mma_bf16_ts(d_x, ga + 16u, lb, idesc, 1u);
+        if constexpr (NP == 3) {
+            mma_bf16_ts(d_x, ga, lb + 2 * part, idesc, 1u);
+            mma_bf16_ts(d_x, ga + 16u, lb + part, idesc, 1u);
+            mma_bf16_ts(d_x, ga + 32u, lb, idesc, 1u);
+        }
+        mma_commit(done);
+    };
+    // Several entries at a time: lane i polls the barriers and reads the metadata of entry e + i.  (Entry by entry,
+    // the polls and the metadata of an entry took this warp ~600 cycles, the MMAs ~200.)  Half of the operand
+    // slots, so that the G sets fill the other half meanwhile.
+    constexpr int kTake = NP == 2 ? 4 : 2;
+    uint32_t seg = 0, acc = 0u;  // acc 0: the segment's first entry
+    bool bad = false, ended = false, ok = true, issued = false;
+    int4 meta = make_int4(0, 0, 0, 0);  // lane i: entry e + i
+    uint32_t special = 0u, marks = 0u;  // bit i: entry e + i starts or ends something; has a strength that is not finite
+    // lanes 0 .. 3 poll the operand slots, lanes 4 .. 7 the records (complete by then: the G set waited for them)
+    auto bar_of = [&](uint32_t le) { return (lane & 4) ? &sm.full[sm.slot(le)] : &sm.full_a[sm.slot(le)]; };
+    auto read_batch = [&](uint32_t le) {
+        const unsigned char* base = sm.slots + (size_t)sm.slot(le) * a.slot_bytes;
+        meta = *reinterpret_cast<const int4*>(base + meta_off);
+        const int4 mk = *reinterpret_cast<const int4*>(base + mark_off);
+        special = __ballot_sync(P2P_FULL_MASK, (meta.x & (kFirst | kLast | kDone)) != 0);
+        marks = __ballot_sync(P2P_FULL_MASK, !(meta.x & kDone) && (mk.x | mk.y | mk.z | mk.w) != 0);
+        tc_fence_after();
+    };
+    bool ready = false;  // the batch at e has been polled and read
+    for (uint32_t e = 0; ok && !ended; e += kTake) {
+        const uint32_t le = e + (uint32_t)(lane & (kTake - 1));
+        if (!ready) {
+            if (!warp_wait(a, sm, bar_of(le), sm.phase(le), wlim)) break;
+            read_batch(le);
+        }
+        ready = false;
+        const uint32_t ga0 = ga_all + (e & a_mask) * (uint32_t)a_cols(NP);
+        const uint64_t lb0 = db_all + (uint64_t)(sm.slot(e) * slot16);
+        uint64_t* done0 = &sm.done[sm.slot(e)];
+        issued = true;
+        if (special == 0u) {
+            // inside a segment: the next batch is polled between the two halves, while the first one's MMAs run
+            bad |= marks != 0u;
+            if (elect_lane()) {
+#pragma unroll
+                for (int i = 0; i < kTake / 2; ++i)
+                    issue(ga0 + (uint32_t)(i * a_cols(NP)), lb0 + (uint64_t)(i * slot16), 1u, done0 + i);
+            }
+            __syncwarp();
+            const uint32_t ne = le + kTake;
+            ready = __all_sync(P2P_FULL_MASK, mbar_test(bar_of(ne), sm.phase(ne)));
+            if (ready) read_batch(ne);
+            if (elect_lane()) {
+#pragma unroll
+                for (int i = kTake / 2; i < kTake; ++i)
+                    issue(ga0 + (uint32_t)(i * a_cols(NP)), lb0 + (uint64_t)(i * slot16), 1u, done0 + i);
+            }
+            __syncwarp();
+            continue;
+        }
+        for (int i = 0; i < kTake; ++i) {
+            const int flags = __shfl_sync(P2P_FULL_MASK, meta.x, i);
+            if (flags & (kFirst | kDone)) {
+                // the epilogue has read this issuer's accumulator (and the descriptor) of the segment before
+                if (!warp_wait(a, sm, &sm.acc_empty[q], (seg & 1u) ^ 1u, wlim)) {
+                    ok = false;
+                    break;
+                }
+                if (flags & kDone) {
+                    ended = true;
+                    break;
+                }
+                acc = 0u;
+                bad = false;
+            }
+            bad |= ((marks >> i) & 1u) != 0;
+            if (elect_lane()) {
+                issue(ga0 + (uint32_t)(i * a_cols(NP)), lb0 + (uint64_t)(i * slot16), acc, done0 + i);
+                if (flags & kLast) mma_commit(&sm.acc_full[q]);
+            }
+            acc = 1u;
+            if (flags & kLast) {
+                if (q == 0 && lane == i) {  // this entry's metadata is lane i's
+                    *sm.desc = make_int4((flags & (kAdd | kOut)) | (bad ? kFirst : 0), meta.y, meta.z, meta.w);
+                    mbar_arrive(sm.desc_full);
+                }
+                ++seg;
+            }
+            __syncwarp();
+        }
+    }
+    if (elect_lane()) {
+        if (ended && q == 0) {
+            *sm.desc = make_int4(kDone, 0, 0, 0);
+            mbar_arrive(sm.desc_full);
+        } else if (!ended && issued) {
+            // this warp's MMAs in flight
+            mma_commit(&sm.drain[q]);
+            mbar_wait(&sm.drain[q], 0u, nullptr, kDrainLimit);
+        }
+    }
+    __syncwarp();
+}
+
+// Right-hand sides for which some source near sorted target t has a non-finite strength (bit r).
+template <int NP>
+__device__ __noinline__ uint64_t bad_rhs(const TcArgs& a, int t, int b0) {
+    const int64_t rec = record_bytes(a.rhs, NP);
+    const int b = b0 + a.member[t];
+    uint64_t bad = 0;
+    for (int e = a.nbr_ptr[b]; e < a.nbr_ptr[b + 1]; ++e) {
+        const int c = a.nbr_idx[e];
+        for (int s = a.src_box_ptr[c]; s < a.src_box_ptr[c + 1]; ++s) {
+            const uint32_t* w = reinterpret_cast<const uint32_t*>(a.pack + (s / kSrcGroup) * rec + copy_bytes(a.rhs, NP)) +
+                                2 * (s % kSrcGroup);
+            bad |= (uint64_t)w[0] | ((uint64_t)w[1] << 32);
+        }
+    }
+    return bad;
+}
+
+// ---- epilogue (four warps, each its own quadrant of TMEM lanes: lane = target) ----
+// A segment's accumulators go through registers into the tile in shared memory, added up over the unit's segments in
+// FP32: first D1, which the first issuer may then overwrite, then D2.  Finished rows leave from the tile while the
+// next segment's MMAs run.  (Rows stored from the registers, 16 bytes per target and instruction, held the
+// accumulators for ~16 000 cycles.)
+template <int KERN, bool LIMITED, int NP>
+__device__ void run_epilogue(const TcArgs& a, const TcSmem& sm, uint32_t tmem, int quadrant, int lane) {
+    const uint32_t wlim = LIMITED ? a.wait_limit : kWaitLimit;
+    const uint32_t lane_addr = tmem + ((uint32_t)(quadrant * 32) << 16);
+    const int row = quadrant * 32 + lane;
+    const int stride = tile_stride(a.rhs);
+    const bool split = a.rhs <= 32;
+    float* mine = sm.tile + row * stride;
+    // columns of right-hand sides r0 .. r0 + 7 in accumulator q: x those of Lr, y those of Li
+    auto load = [&](int q, int r0, float2 (&x)[4], float2 (&y)[4]) {
+        uint32_t u[8], v[8], s[8], t[8];
+        const uint32_t col = lane_addr + 128u * (uint32_t)q + (uint32_t)r0;
+        tmem_ld8(col, u);
+        tmem_ld8(col + (uint32_t)a.rhs, v);
+        if (split) {
+            tmem_ld8(col + 64u, s);
+            tmem_ld8(col + 64u + (uint32_t)a.rhs, t);
+        }
+        tmem_ld_wait(u);
+        tmem_ld_wait(v);
+        if (split) {
+            tmem_ld_wait(s);
+            tmem_ld_wait(t);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[i] = make_float2(__uint_as_float(u[2 * i]), __uint_as_float(u[2 * i + 1]));
+            y[i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            if (split) {
+                x[i] = __fadd2_rn(x[i], make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])));
+                y[i] = __fadd2_rn(y[i], make_float2(__uint_as_float(t[2 * i]), __uint_as_float(t[2 * i + 1])));
+            }
+        }
+    };
+    for (uint32_t seg = 0;; ++seg) {
+        if (!warp_wait(a, sm, sm.desc_full, seg & 1u, wlim)) return;
+        const int4 d = *sm.desc;
+        if (d.x & kDone) return;
+        const bool valid = row < d.w;
+        const int32_t out_row = valid ? a.perm[d.z + row] : 0;
+        uint64_t bad = 0;
+        if ((d.x & kFirst) && valid) bad = bad_rhs<NP>(a, d.z + row, d.y);
+        if (!warp_wait(a, sm, &sm.acc_full[0], seg & 1u, wlim)) return;
+        tc_fence_after();
+        for (int r0 = 0; r0 < a.rhs; r0 += 8) {
+            float2 x[4], y[4];
+            load(0, r0, x, y);
+            if (bad) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float nan = __int_as_float(0x7fc00000);
+                    if ((bad >> (r0 + 2 * i)) & 1u) x[i].x = y[i].x = nan;
+                    if ((bad >> (r0 + 2 * i + 1)) & 1u) x[i].y = y[i].y = nan;
+                }
+            }
+            float4* to = reinterpret_cast<float4*>(mine + 2 * r0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float4 w = make_float4(x[i].x, y[i].x, x[i].y, y[i].y);
+                if (d.x & kAdd) {
+                    const float4 o = to[i];
+                    w = make_float4(w.x + o.x, w.y + o.y, w.z + o.z, w.w + o.w);
+                }
+                to[i] = w;
+            }
+        }
+        // D1's columns are in shared memory, and the descriptor in registers
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.acc_empty[0]);
+        if (KERN == P2P_HELMHOLTZ) {
+            if (!warp_wait(a, sm, &sm.acc_full[1], seg & 1u, wlim)) return;
+            tc_fence_after();
+            for (int r0 = 0; r0 < a.rhs; r0 += 8) {
+                float2 x[4], y[4];
+                load(1, r0, x, y);
+                float4* to = reinterpret_cast<float4*>(mine + 2 * r0);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 o = to[i];
+                    to[i] = make_float4(o.x - y[i].x, o.y + x[i].x, o.z - y[i].y, o.w + x[i].y);
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.acc_empty[1]);
+        }
+        if (d.x & kOut) {
+            // eight rows at a time, four lanes for a row's 64 bytes
+            const int piece = 2 * (lane & 3);
+            for (int i = 0; i < 32; i += 8) {
+                const int rr = i + (lane >> 2);
+                float2* dst = a.out + (int64_t)__shfl_sync(P2P_FULL_MASK, out_row, rr) * a.ld;
+                if (quadrant * 32 + rr >= d.w) continue;
+                for (int r = piece; r < a.nrhs; r += 8) {
+                    const float4 w = *reinterpret_cast<const float4*>(sm.tile + (quadrant * 32 + rr) * stride + 2 * r);
+                    const float2 w0 = make_float2(w.x * kInv4Pi, w.y * kInv4Pi), w1 = make_float2(w.z * kInv4Pi, w.w * kInv4Pi);
+                    if (a.vec_out && r + 1 < a.nrhs) {
+                        *reinterpret_cast<float4*>(dst + r) = make_float4(w0.x, w0.y, w1.x, w1.y);
+                    } else {
+                        dst[r] = w0;
+                        if (r + 1 < a.nrhs) dst[r + 1] = w1;
+                    }
+                }
+            }
+            __syncwarp();  // the rows are read before the next segment overwrites them
+        }
     }
 }
 
 // LIMITED: the waits poll at most a.wait_limit times (the abort-path self-check); otherwise kWaitLimit.
-// NP: BF16 parts per operand (2: three MMAs per stage, 3: six).
+// NP: BF16 parts per operand (2: three products per entry and chain, 3: six).
 template <int KERN, bool LIMITED, int NP>
 __global__ void __launch_bounds__(kThreads, 1) k_p2p_tc(const __grid_constant__ TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const TcSmem sm = carve(smem, a.slots, a.slot_bytes);
+    const TcSmem sm = carve(smem, a);
+    constexpr int kIssuers = KERN == P2P_HELMHOLTZ ? 2 : 1;
     if (warp == 0) tmem_alloc(sm.tmem_slot, 512u);
     if (tid == 32) {
-        for (int i = 0; i < kSets * a.slots; ++i) {
+        for (int i = 0; i < 1 << a.slots_log; ++i) {
             mbar_init(&sm.full[i], 1);
-            mbar_init(&sm.full_b[i], kSetThreads);
-            mbar_init(&sm.empty[i], 1);
+            mbar_init(&sm.full_a[i], 4);
+            mbar_init(&sm.done[i], kIssuers);
         }
+        mbar_init(sm.desc_full, 1);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&sm.acc_full[i], kSets);
-            mbar_init(&sm.acc_empty[i], 128);
+            mbar_init(&sm.acc_full[i], 1);
+            mbar_init(&sm.acc_empty[i], 4);
         }
+        for (int i = 0; i < kUnitQueue; ++i) {
+            mbar_init(&sm.uq_full[i], 1);
+            mbar_init(&sm.uq_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) mbar_init(&sm.drain[i], 1);
         *sm.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -845,16 +1196,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_p2p_tc(const __grid_constant__ 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *sm.tmem_slot;
-    const int64_t units = (int64_t)a.nb * a.ngrp;
-    if (warp < kGWarp0) {
-        run_producer<LIMITED>(a, sm, units, warp, lane);
-    } else if (warp < kMmaWarp0) {
-        const int gw = warp - kGWarp0;
-        run_gset<KERN, LIMITED, NP>(a, sm, gw / kSetWarps, (gw % kSetWarps) * 32 + lane);
-    } else if (warp < kEpiWarp0) {
-        if (lane == 0) run_mma<LIMITED, NP>(a, sm, tmem, warp - kMmaWarp0);
-    } else {
-        run_epilogue<LIMITED>(a, sm, tmem, units, warp, lane);
+    if (warp == 0) {
+        run_producer<LIMITED, NP>(a, sm, lane);
+    } else if (warp < kMmaWarp0 + kIssuers) {
+        run_mma<LIMITED, NP>(a, sm, tmem, warp - kMmaWarp0);
+    } else if (warp == kScoutWarp) {
+        run_scout<LIMITED, NP>(a, sm, lane);
+    } else if (warp >= kGWarp0) {
+        run_gset<KERN, LIMITED, NP>(a, sm, tmem, (warp - kGWarp0) >> 2, warp & 3, lane);
+    } else if (warp >= kEpiWarp0) {
+        run_epilogue<KERN, LIMITED, NP>(a, sm, tmem, warp & 3, lane);
     }
     tc_fence_before();
     __syncthreads();
@@ -863,13 +1214,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_p2p_tc(const __grid_constant__ 
         tc_fence_after();
         tmem_dealloc(tmem, 512u);
     }
+    // the last CTA leaves the unit counter at zero for the next launch
+    if (tid == kScoutWarp * 32) {
+        __threadfence();
+        if (atomicAdd(a.counter + 1, 1u) == gridDim.x - 1u) {
+            a.counter[0] = 0u;
+            a.counter[1] = 0u;
+        }
+    }
 }
 
 // ------------------------------------------------- operand-layout self-check --
 
 // D[128 x N] = A[128 x K] . B[N x K]^T with A, B split into BF16 hi + lo (3 MMAs
-// per 16-wide K slice), through the same operand layout, descriptors and
-// instruction descriptor as k_p2p_tc.
+// per 16-wide K slice), both operands in shared memory, through the operand layout,
+// descriptors and instruction descriptor of k_p2p_tc's B operand.
 __global__ void __launch_bounds__(128, 1) k_tc_gemm_check(const float* __restrict__ A, const float* __restrict__ B,
                                                           float* __restrict__ D, int K, int n, int tmem_cols,
                                                           unsigned int* __restrict__ status) {
@@ -898,14 +1257,14 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm_check(const float* __restric
             float v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) v[i] = A[(int64_t)row * K + ks * 16 + half * 8 + i];
-            store_split<8>(a_hi, a_lo, op_off(row, half * 8), v);
+            store_parts<2>(a_hi, (int)(a_lo - a_hi), op_off(row, half * 8), v);
         }
         for (int c = tid; c < n * 2; c += 128) {
             const int row = c >> 1, half = c & 1;
             float v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) v[i] = B[(int64_t)row * K + ks * 16 + half * 8 + i];
-            store_split<8>(b_hi, b_lo, op_off(row, half * 8), v);
+            store_parts<2>(b_hi, (int)(b_lo - b_hi), op_off(row, half * 8), v);
         }
         fence_async_smem();
         tc_fence_before();
@@ -949,47 +1308,30 @@ int tmem_cols_for(int n) {
     return c;
 }
 
-// Launch shape for nrhs right-hand sides: RHS blocks, targets per unit, slots per set.
-struct TcShape {
-    int rb_count, tg, slots, slot_bytes, smem;
-};
-
-TcShape tc_shape(int32_t nrhs, int optin, int np) {
-    TcShape s;
-    s.rb_count = (nrhs + 63) / 64;
-    // One accumulator per G set (rb_count blocks x 2T columns) in each unit buffer.  The hi/lo split keeps two
-    // buffers of 32-target units, so the epilogue of one unit overlaps the MMAs of the next.  The three-part
-    // split takes 64-target units in one buffer (all 512 columns): a box of 33 - 64 targets is one unit instead
-    // of two walking the same list, and its six MMAs per stage leave the epilogue's wait a smaller share (the
-    // ellipsoid at 64 RHS: 7.14 ms against 7.64; hi/lo with the same shape 5.46 against 5.11).
-    const int units_in_tmem = np == 3 ? 1 : 2;
-    s.tg = (2 * kSetCols / (units_in_tmem * 2 * kSets * s.rb_count)) / 8 * 8;
-    if (s.tg > 64) s.tg = 64;
-    s.slot_bytes = slot_bytes_for(s.rb_count, s.tg, np);
-    s.slots = 8;
-    while (s.slots > 1 && tc_smem_bytes(s.slots, s.slot_bytes) > optin) --s.slots;
-    s.smem = tc_smem_bytes(s.slots, s.slot_bytes);
-    // more than half an SM's shared memory keeps one CTA (and one 512-column TMEM allocation) per SM
-    const int half = 116 * 1024;
-    if (s.smem < half) s.smem = half;
-    return s;
+// Right-hand sides of one launch: nrhs in near-equal parts of at most 64, rounded up to 8.  A launch's tensor time
+// follows its width, G is formed once per launch (the three-part split at 64 right-hand sides as two 32-wide launches,
+// whose chains are shorter: 7.63 ms on the 2^21-point ellipsoid, one 64-wide launch 6.1 - 6.6 ms).
+int launch_rhs(int32_t nrhs) {
+    const int parts = (nrhs + 63) / 64;
+    return ((nrhs + parts - 1) / parts + 7) & ~7;
 }
+
+int64_t source_groups(int64_t n) { return (n + kSrcGroup - 1) / kSrcGroup; }
 
 }  // namespace
 
-// RHS blocks of 64 per launch.  One block per launch keeps units of 32 targets
-// (the TMEM accumulators of four G sets x two unit buffers hold 2 T x 64 RHS
-// each); a launch over two blocks must halve the unit to 16 targets and measured
-// 15.4 ms on the 2^21-point ellipsoid at 128 RHS against 2 x 5.2 ms for two
-// launches of one block (G is formed once per launch: its share is small).
-constexpr int kRbLaunch = 1;
+int32_t p2p_tc_block_count(int32_t nb) { return (nb + kBlockBoxes - 1) / kBlockBoxes; }
+int64_t p2p_tc_unit_bound(int64_t n, int32_t nb) { return n / kRows + p2p_tc_block_count(nb) + 1; }
 
-// Room for the records of either split (sized for three parts), chunk by chunk.
-size_t p2p_tc_pack_bytes(int64_t n, int32_t nb, int32_t max_nrhs) {
+// Room for the records of either split (sized for three parts), launch by launch.
+size_t p2p_tc_pack_bytes(int64_t n, int32_t max_nrhs) {
     if (max_nrhs < 16) return 0;
-    const int64_t groups = n / kSrcGroup + nb;
-    const int chunks = (max_nrhs + 64 * kRbLaunch - 1) / (64 * kRbLaunch);
-    return (size_t)chunks * (size_t)groups * (size_t)record_bytes(kRbLaunch, 3);
+    size_t most = 0;
+    for (int nrhs = 1; nrhs <= max_nrhs; ++nrhs) {
+        const int rhs = launch_rhs(nrhs);
+        most = std::max(most, (size_t)((nrhs + rhs - 1) / rhs) * (size_t)record_bytes(rhs, 3));
+    }
+    return (size_t)source_groups(n) * most;
 }
 
 bool p2p_tc_supported(const p2p_plan* plan, int32_t nrhs) {
@@ -1001,54 +1343,79 @@ bool p2p_tc_supported(const p2p_plan* plan, int32_t nrhs) {
     return major == 10 && minor == 3;
 }
 
+// Plan time: the blocks' entry lists, masks and units.  bound / units: scratch of one int per block each.
+cudaError_t p2p_tc_build(p2p_plan* p, int32_t* bound, int32_t* units, void* scan_ws, cudaStream_t s) {
+    const int32_t nblk = p2p_tc_block_count(p->nb);
+    cudaError_t e = cudaMemsetAsync(p->tc_counter, 0, 2 * sizeof(unsigned int), s);
+    if (e != cudaSuccess || nblk == 0 || p->nbs == 0) return e;
+    k_tc_blocks<<<(unsigned)((nblk + 3) / 4), 128, 0, s>>>(p->box_ptr, p->nb, p->src_box_ptr, p->nbr_ptr, p->nbr_idx,
+                                                            nblk, bound, units, p->tc_member);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = scan_exclusive_i32(bound, p->tc_off, nblk, p->tc_off + nblk, scan_ws, s);
+    if (e == cudaSuccess) e = scan_exclusive_i32(units, p->tc_ustart, nblk, p->tc_ustart + nblk, scan_ws, s);
+    if (e != cudaSuccess) return e;
+    k_tc_fill<<<(unsigned)nblk, kFillThreads, 0, s>>>(p->src_box_ptr, p->nbr_ptr, p->nbr_idx, p->nb, p->tc_off,
+                                                      p->tc_ustart, p->tc_ecount, p->tc_unit_block, p->tc_gid,
+                                                      p->tc_bits, p->tc_masks);
+    return cudaGetLastError();
+}
+
 // Stage: the group records (strength images from original-order lambda via perm, coordinates).
 p2p_status p2p_tc_stage(const p2p_plan* plan, const float2* lam, int32_t nrhs, int64_t ld, int np,
                         cudaStream_t s) {
-    if (plan->n == 0 || plan->tc_groups == 0) return P2P_OK;
-    const int rb_count = (nrhs + 63) / 64;
-    dim3 grid((unsigned)plan->tc_groups, (unsigned)rb_count);
-    const int64_t chunk_bytes = (int64_t)plan->tc_groups * record_bytes(kRbLaunch, np);
-    // the group records are built over the SOURCE boxes
+    if (plan->n == 0 || plan->n_src == 0) return P2P_OK;
+    const int rhs = launch_rhs(nrhs);
+    const int64_t groups = source_groups(plan->n_src);
+    const int per_block = 128 / (2 * ((rhs + 31) & ~31));
+    const unsigned grid = (unsigned)((groups + per_block - 1) / per_block);
     auto pack = np == 3 ? k_tc_pack<3> : k_tc_pack<2>;
-    pack<<<grid, 128, 0, s>>>(lam, ld, nrhs, plan->src_perm, plan->src_box_ptr, plan->xs_src, plan->tc_gstart,
-                              plan->nbs, kRbLaunch, chunk_bytes, plan->tc_pack);
-    P2P_CHECK_LAUNCH("p2p_apply_stage/tc_pack");
+    for (int c = 0; c * rhs < nrhs; ++c) {
+        pack<<<grid, 128, 0, s>>>(lam, ld, nrhs, c * rhs, rhs, plan->src_perm, plan->xs_src, plan->n_src, (int32_t)groups,
+                                  plan->tc_pack + c * groups * record_bytes(rhs, np));
+        P2P_CHECK_LAUNCH("p2p_apply_stage/tc_pack");
+    }
     return P2P_OK;
 }
 
 p2p_status p2p_apply_tc(const p2p_plan* plan, float2* out, int32_t nrhs, int64_t ld, int32_t adjoint, int np,
                         cudaStream_t s) {
-    if (plan->n == 0) return P2P_OK;
+    if (plan->n == 0 || plan->n_src == 0) return P2P_OK;
     int dev = 0, optin = 0, sms = 0;
     P2P_TRY_CUDA(cudaGetDevice(&dev), "p2p_apply_tc");
     P2P_TRY_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev), "p2p_apply_tc");
     P2P_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "p2p_apply_tc");
-    // one launch per chunk of kRbLaunch RHS blocks, each on its own records
-    const int chunk_rhs = 64 * kRbLaunch;
-    const TcShape sh = tc_shape(std::min(nrhs, chunk_rhs), optin, np);
-    if (sh.smem > optin) {
+    const int rhs = launch_rhs(nrhs);
+    TcArgs a;
+    a.slot_bytes = slot_bytes_for(rhs, np);
+    a.slots_log = tc_smem_bytes(rhs, np, 16) <= optin ? 4 : 3;
+    // more than half an SM's shared memory keeps one CTA (and one 512-column TMEM allocation) per SM
+    const int smem = std::max(tc_smem_bytes(rhs, np, 1 << a.slots_log), 116 * 1024);
+    if (smem > optin) {
         set_message("p2p_apply_tc: the tensor-core pipeline does not fit in shared memory");
         return P2P_ERR_UNSUPPORTED;
     }
-    TcArgs a;
     a.xs = plan->xs;
-    a.pack = plan->tc_pack;
+    a.off = plan->tc_off;
+    a.ecount = plan->tc_ecount;
+    a.ustart = plan->tc_ustart;
+    a.unit_block = plan->tc_unit_block;
+    a.gid = plan->tc_gid;
+    a.bits = plan->tc_bits;
+    a.masks = reinterpret_cast<const uint16_t*>(plan->tc_masks);
+    a.member = plan->tc_member;
     a.box_ptr = plan->box_ptr;
-    a.glist_off = plan->tc_glist_off;
-    a.glist = plan->tc_glist;
-    a.gcount = plan->tc_gcount;
     a.perm = plan->perm;
+    a.nbr_ptr = plan->nbr_ptr;
+    a.nbr_idx = plan->nbr_idx;
+    a.src_box_ptr = plan->src_box_ptr;
     a.ld = ld;
-    a.rb_count = sh.rb_count;
-    a.tg = sh.tg;
-    a.ngrp = (plan->max_box + sh.tg - 1) / sh.tg;
+    a.rhs = rhs;
     a.nb = plan->nb;
-    a.slots = sh.slots;
-    a.slot_bytes = sh.slot_bytes;
-    a.np = np;
-    a.nbuf = 512 / (kSets * 2 * sh.tg * sh.rb_count);
+    a.nblk = p2p_tc_block_count(plan->nb);
+    a.a_slots = np == 3 ? 4 : 8;  // 48 or 32 columns each in 256
     a.k = adjoint ? -plan->k : plan->k;
     a.status = plan->status;
+    a.counter = plan->tc_counter;
     a.wait_limit = plan->tc_wait_polls < 0 ? kWaitLimit : (uint32_t)plan->tc_wait_polls;
     const bool limited = plan->tc_wait_polls >= 0;
     void (*kern)(TcArgs) = nullptr;
@@ -1060,15 +1427,15 @@ p2p_status p2p_apply_tc(const p2p_plan* plan, float2* out, int32_t nrhs, int64_t
         kern = lap ? (limited ? k_p2p_tc<P2P_LAPLACE, true, 2> : k_p2p_tc<P2P_LAPLACE, false, 2>)
                    : (limited ? k_p2p_tc<P2P_HELMHOLTZ, true, 2> : k_p2p_tc<P2P_HELMHOLTZ, false, 2>);
     }
-    P2P_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem), "p2p_apply_tc");
-    const int64_t units = (int64_t)a.nb * a.ngrp;
-    const int grid = (int)std::min<int64_t>(units, sms);
-    const int64_t chunk_bytes = (int64_t)plan->tc_groups * record_bytes(kRbLaunch, np);
-    for (int c = 0; c * chunk_rhs < nrhs; ++c) {
-        a.pack = plan->tc_pack + c * chunk_bytes;
-        a.out = out + (int64_t)c * chunk_rhs;
-        a.nrhs = std::min(chunk_rhs, nrhs - c * chunk_rhs);
-        kern<<<grid, kThreads, sh.smem, s>>>(a);
+    P2P_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "p2p_apply_tc");
+    const int grid = (int)std::min<int64_t>(p2p_tc_unit_bound(plan->n, plan->nb), sms);
+    const int64_t part_bytes = source_groups(plan->n_src) * record_bytes(rhs, np);
+    for (int c = 0; c * rhs < nrhs; ++c) {
+        a.pack = plan->tc_pack + c * part_bytes;
+        a.out = out + (int64_t)c * rhs;
+        a.nrhs = std::min(rhs, nrhs - c * rhs);
+        a.vec_out = ld % 2 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15) == 0;
+        kern<<<grid, kThreads, smem, s>>>(a);
         P2P_CHECK_LAUNCH("p2p_apply_tc");
     }
     return P2P_OK;

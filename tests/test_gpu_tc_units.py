@@ -1,0 +1,91 @@
+"""Tensor-core path at the edges of its tiling: groups of 16 consecutive sorted sources (any box boundary inside a
+group), blocks of 32 target boxes, windows of at most 128 targets (boxes of more than 128 points), segments of a long
+entry list, right-hand sides around multiples of 8 and 64, odd leading dimensions, and strengths that are not finite.
+
+Tolerance: the path's own per-target bound, |err_i| <= delta S_i with S_i = sum_j |G(r_ij) lambda_j| and delta = 2^-14
+for hi / lo, 2^-20 for hi / mid / lo (what the guarded apply relies on), at every target and right-hand side."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2403_01596_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DELTA = {"tc_bf16x3": 2.0 ** -14, "tc_bf16x6": 2.0 ** -20}
+
+
+def _worst(out, ref, S):
+    """Largest |err| / S over targets and right-hand sides (targets without a pair must be exactly zero)."""
+    err = np.abs(out - ref)
+    assert (err[S == 0] == 0).all()
+    return float((err[S > 0] / S[S > 0]).max()) if (S > 0).any() else 0.0
+
+
+def _api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_01596_gb300 import api
+    return api
+
+
+# points, boxes per axis of the unit cube: one box of 15 / 16 / 17 / 127 / 128 / 129 / 400 points, boxes of ~140
+# (several windows per box, long lists), 33 and 64 boxes of a few points (block edges), ~1 point per box
+@pytest.mark.parametrize("n,ng", [(15, 1), (16, 1), (17, 1), (127, 1), (128, 1), (129, 1), (400, 1), (3800, 3),
+                                  (170, 4), (500, 5), (900, 10)])
+@pytest.mark.parametrize("path", ["tc_bf16x3", "tc_bf16x6"])
+@pytest.mark.parametrize("kernel", ["helmholtz", "laplace"])
+def test_tiles(n, ng, path, kernel):
+    api = _api()
+    pts = np.random.default_rng(n + ng).random((n, 3)).astype(np.float32)
+    lo, h, k = (0.0, 0.0, 0.0), 1.0 / ng, (float(np.float32(2 * np.pi * ng / 5)) if kernel == "helmholtz" else 0.0)
+    kid = oracle.HELMHOLTZ if kernel == "helmholtz" else oracle.LAPLACE
+    plan = api.Plan(torch.from_numpy(pts).cuda(), lo, h, ng, k, kernel=kernel, max_nrhs=67)
+    for nrhs in (1, 9, 33, 64, 67):
+        lam = W.strengths(n, nrhs, n + nrhs).reshape(n, nrhs)
+        out = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+        assert plan.async_status() == 0
+        ref = oracle.p2p(pts, lam, lo, h, ng, k, kernel=kid).reshape(n, nrhs)
+        S = oracle.p2p(pts, np.abs(lam).astype(np.complex64), lo, h, ng, 0.0, kernel=oracle.LAPLACE).real.reshape(n, nrhs)
+        assert _worst(out, ref, S) <= DELTA[path], (nrhs, _worst(out, ref, S))
+
+
+@pytest.mark.parametrize("path", ["tc_bf16x3", "tc_bf16x6"])
+def test_two_sets_with_lonely_targets(path):
+    """Targets with no source nearby (whole windows of them, and some in windows that have work) stay zero."""
+    api = _api()
+    rng = np.random.default_rng(3)
+    tgt = rng.random((3000, 3)).astype(np.float32)
+    src = (rng.random((500, 3)) * 0.3).astype(np.float32)
+    src[:50] = tgt[np.flatnonzero((tgt < 0.3).all(1))[:50]]  # some at r = 0
+    ng, lo, h, k = 10, (0.0, 0.0, 0.0), 0.1, 12.0
+    plan = api.TwoSetPlan(torch.from_numpy(tgt).cuda(), torch.from_numpy(src).cuda(), lo, h, ng, k, max_nrhs=16)
+    lam = W.strengths(500, 16, 4)
+    out = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+    assert plan.async_status() == 0
+    ref = oracle.p2p_st(tgt, src, lam, lo, h, ng, k)
+    S = oracle.p2p_st(tgt, src, np.abs(lam).astype(np.complex64), lo, h, ng, 0.0, kernel=oracle.LAPLACE).real
+    assert _worst(out, ref, S) <= DELTA[path]
+    assert (out[np.abs(ref).max(1) == 0] == 0).all() and (np.abs(ref).max(1) == 0).any()
+
+
+@pytest.mark.parametrize("path", ["tc_bf16x3", "tc_bf16x6"])
+@pytest.mark.parametrize("nrhs", [17, 64])
+def test_strength_that_is_not_finite_stays_local(path, nrhs):
+    """An infinite or NaN strength makes NaN of the results of its own neighbourhood and right-hand side, and of
+    nothing else."""
+    api = _api()
+    wl = W.Workload("s", W.unit_sphere(4000, 8), (-1, -1, -1), 2 / 14, 14, 30.0, 8)
+    plan = api.Plan(torch.from_numpy(wl.points).cuda(), wl.lo, wl.h, wl.ng, wl.k, max_nrhs=nrhs)
+    lam = W.strengths(wl.n, nrhs, 8)
+    clean = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+    cell = np.clip(np.floor((wl.points.astype(np.float64) + 1) / wl.h), 0, wl.ng - 1)
+    hit = np.zeros((wl.n, nrhs), bool)
+    for s, r, v in ((5, 3, np.inf), (1777, 16, np.nan), (1778, 0, complex(0, -np.inf))):
+        lam[s, r] = v
+        hit[np.abs(cell - cell[s]).max(1) <= 1, r] = True
+    out = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+    assert plan.async_status() == 0
+    assert np.isnan(out.real[hit]).all() and np.isnan(out.imag[hit]).all()
+    assert np.array_equal(out[~hit], clean[~hit])
