@@ -433,10 +433,14 @@ p2p_status p2p_abs_sums(const p2p_plan* plan, const float2* lam, int64_t ld, int
 }
 
 cudaError_t p2p_group_configure(p2p_plan* p);
+cudaError_t p2p_multi_configure(p2p_plan* p);
+p2p_status p2p_multi_stage(const p2p_plan* p, const float2* lam, int32_t nrhs, int64_t ld, cudaStream_t s);
+p2p_status p2p_multi_launch(const p2p_plan* p, float2* out, int32_t nrhs, int64_t ld, float k, cudaStream_t s);
 p2p_status p2p_group_launch(const p2p_plan* p, float2* out, int64_t ld, float k, cudaStream_t s);
 
 cudaError_t p2p_pair_configure(p2p_plan* plan) {
     cudaError_t e = p2p_group_configure(plan);
+    if (e == cudaSuccess && plan->max_nrhs > 1) e = p2p_multi_configure(plan);
     if (e == cudaSuccess) e = configure_r<1>(plan);
     if (e == cudaSuccess) e = configure_r<2>(plan);
     if (e == cudaSuccess) e = configure_r<4>(plan);
@@ -468,6 +472,11 @@ static p2p_path resolve_path(const p2p_plan* plan, int32_t nrhs, p2p_path path) 
 }
 
 static bool is_tc(p2p_path path) { return path == P2P_PATH_TC_BF16X3 || path == P2P_PATH_TC_BF16X6; }
+// Several right-hand sides sharing G: every layout with full source lists, from the sorted strengths.
+static bool is_multi(const p2p_plan* plan, int32_t nrhs, p2p_path path) {
+    return path == P2P_PATH_FP32_SHARED && nrhs > 1 &&
+           (plan->layout == P2P_LAYOUT_INDEXED || plan->layout == P2P_LAYOUT_REDUNDANT);
+}
 static int tc_parts(p2p_path path) { return path == P2P_PATH_TC_BF16X6 ? 3 : 2; }
 
 P2P_API p2p_status p2p_apply_stage(const p2p_plan* plan, const void* lambda, int32_t nrhs, int64_t ld, p2p_path path,
@@ -481,6 +490,7 @@ P2P_API p2p_status p2p_apply_stage(const p2p_plan* plan, const void* lambda, int
     if (is_tc(path) && !p2p_tc_supported(plan, nrhs)) return P2P_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
     if (is_tc(path)) return p2p_tc_stage(plan, (const float2*)lambda, nrhs, ld, tc_parts(path), s);
+    if (is_multi(plan, nrhs, path)) return p2p_multi_stage(plan, (const float2*)lambda, nrhs, ld, s);
     if (plan->layout == P2P_LAYOUT_REPETITION) {
         // every target's record gets its own copy of its sources' strengths (the record head: 0)
         P2P_TRY_CUDA(stage_rows((const float2*)lambda, ld, plan->rec_src, plan->records, 1, plan->lam_buf, s),
@@ -554,6 +564,7 @@ P2P_API p2p_status p2p_apply_staged(const p2p_plan* plan, void* out, int32_t nrh
     if (a.atomic_out && !plan->two_sets)
         P2P_TRY_CUDA(cudaMemset2DAsync(out, (size_t)ld * 8, 0, (size_t)nrhs * 8, (size_t)plan->n, s), "p2p_apply/zero");
     if (plan->n_items == 0) return P2P_OK;
+    if (is_multi(plan, nrhs, path)) return p2p_multi_launch(plan, (float2*)out, nrhs, ld, a.k, s);
     const int R = path == P2P_PATH_FP32_PER_RHS ? 1 : (nrhs >= 4 ? 4 : (nrhs >= 2 ? 2 : 1));
     return R == 1 ? launch_pair<1>(plan, a, s) : (R == 2 ? launch_pair<2>(plan, a, s) : launch_pair<4>(plan, a, s));
 }

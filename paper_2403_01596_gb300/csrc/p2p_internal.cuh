@@ -109,6 +109,7 @@ struct p2p_plan {
     int32_t direct_grid;    // persistent grid of the direct kernel (blocks of kDirectWarps warps)
     int32_t grid[3];        // persistent grid of the pair kernel for R = 1, 2, 4 right-hand sides per pass
     int32_t grid_warps[3];  // warps per block of that grid (the tuning's, halved until a block fits)
+    int32_t multi_grid[3];  // persistent grid of the several-right-hand-sides kernel for 2, 4, 8 per launch
     float2* lam_buf;        // [max(n, packed) * max_nrhs] sorted / packed strengths
     float2* g_buf;          // [n * max_nrhs] sorted upstream gradient (coordinate gradient)
     unsigned int* status;   // device status word
@@ -150,6 +151,9 @@ size_t p2p_tc_pack_bytes(int64_t n, int32_t max_nrhs);
 int32_t p2p_tc_block_count(int32_t nb);
 int64_t p2p_tc_unit_bound(int64_t n, int32_t nb);
 inline size_t p2p_tc_entry_bound(int64_t sources, int64_t nnz) { return (size_t)(sources / 16 + 2 * nnz + 4); }
+
+// Several right-hand sides in FP32 (p2p_multi.cu): staged columns of nrhs right-hand sides.
+int32_t p2p_multi_columns(int32_t nrhs);
 
 namespace p2p_detail {
 

@@ -1,0 +1,417 @@
+// Several right-hand sides in FP32: the near-field sum of 2 .. 8 right-hand sides
+// per launch with G evaluated once for all of them.
+//
+// What bounds it.  A pair costs 3 MUFU operations and ~14 FP32 ones for G, and 4
+// FP32 operations per right-hand side, so from four right-hand sides on the FMA
+// pipe is the limit (46 lane operations per pair at eight: 0.16 ms for the
+// 1.4e8 pairs of a 500 000-point assembly on 152 SMs).  The staged pipeline
+// (p2p_pair.cuh) spends more than that around it: at four right-hand sides its two
+// stages of a whole 192-source chunk take 25 KB per warp, so 8 warps fill an SM, eight
+// right-hand sides are two sweeps that form G twice, and their strengths are
+// loaded synchronously.
+//
+// Here an item (target box, source chunk) streams through the warp in sub-chunks
+// of at most 32 sources, three steps deep -- source indices in a register,
+// coordinates and strengths in flight into one half of the warp's buffer
+// (cp.async), the sweep on the other half -- and the accumulators stay in registers
+// across the sub-chunks: 7 KB per warp at eight right-hand sides, 16 warps per SM at
+// 128 registers.  The stream runs on over target groups and items, so the next item's
+// first sources are on their way while this one's slices are summed.
+//
+// Strengths are staged by blocks of right-hand sides, a row per source with the real
+// parts before the imaginary parts, so that the complex multiply-add runs on the
+// packed two-lane FP32 instructions over pairs of right-hand sides without moves; the
+// distances run packed over pairs of targets.  Every packed operation rounds as its
+// scalar counterpart in pair_core, in the same order.
+//
+// Measured on one GB300, applies including the staging, against the staged pipeline at 4 right-hand sides per sweep:
+// the 500 000-point assembly with 8 right-hand sides 0.423 ms (0.896), 300 001 points on a sphere at 47 per box with 5
+// 0.447 ms (0.786), with 12 (Laplace) 0.513 ms (0.867), at 7 per box with 3 in the redundant layout 0.106 ms (0.317: no
+// per-box repack of the strengths), 10 371 points with 2 28 us (30).
+#include <algorithm>
+
+#include "p2p_pair.cuh"
+
+using namespace p2p_detail;
+using namespace p2p_pair;
+
+namespace {
+
+constexpr int kMultiWarps = 8;   // warps per block
+constexpr int kSub = 32;         // sources of a sub-chunk at most
+
+struct MultiArgs {
+    const ItemRec* items;
+    int32_t n_items;
+    const float4* xs;       // box-sorted source coordinates
+    const float4* xt;       // box-sorted target coordinates
+    const int32_t* nb_src;  // per-box source lists (box-sorted indices)
+    const float* lam;       // staged strengths of this block: 2R floats per source
+    const int32_t* perm;
+    float2* out;            // first right-hand side of this block
+    int64_t ld;
+    int32_t nrhs;           // right-hand sides of this block (<= R)
+    float k;
+    int32_t tg;
+    int32_t atomic_out;
+};
+
+__host__ __device__ constexpr int stage_floats(int R) { return kSub * (4 + 2 * R); }
+__host__ __device__ constexpr int warp_floats(int R) { return 2 * stage_floats(R) + 32 * 2 * R; }
+
+// A place in the warp's stream of sub-chunks: the item, its target group and the group's sub-chunk.
+struct Place {
+    int32_t src_off, ns, tb, nt, m_end, map_full, map_last;  // of the item (ItemRec)
+    int32_t item;   // index in the item list (>= n_items: the stream has ended)
+    int t0, s0;
+    int32_t map;
+    int len;        // sources of the sub-chunk: whole rounds of the map's Q slices
+};
+
+__device__ __forceinline__ void set_item(Place& p, int32_t rec) {
+    p.src_off = __shfl_sync(P2P_FULL_MASK, rec, 0);
+    p.ns = __shfl_sync(P2P_FULL_MASK, rec, 1);
+    p.tb = __shfl_sync(P2P_FULL_MASK, rec, 2);
+    p.nt = __shfl_sync(P2P_FULL_MASK, rec, 3);
+    p.m_end = __shfl_sync(P2P_FULL_MASK, rec, 4) & 0xFFFF;
+    p.map_full = __shfl_sync(P2P_FULL_MASK, rec, 5);
+    p.map_last = __shfl_sync(P2P_FULL_MASK, rec, 6);
+}
+__device__ __forceinline__ void set_group(Place& p, int tg) {
+    p.map = p.t0 + tg >= p.nt ? p.map_last : p.map_full;
+}
+__device__ __forceinline__ void set_len(Place& p) {
+    const int Q = map_q(p.map);
+    p.len = min(p.ns - p.s0, (kSub / Q) * Q);
+}
+
+template <int R>
+struct Stream {
+    const MultiArgs& a;
+    int lane;
+    int32_t stride;
+    int32_t rec;      // record of the item after the latest place's, field f in lane f
+    int32_t rec_item;
+    float* base;
+
+    __device__ __forceinline__ float* buf(int h) const { return base + h * stage_floats(R); }
+    __device__ __forceinline__ Place first(int32_t item) {
+        Place p;
+        p.item = item;
+        set_item(p, load_rec_lane(a.items, item, a.n_items, lane));
+        rec_item = item + stride;
+        rec = load_rec_lane(a.items, rec_item, a.n_items, lane);
+        p.t0 = p.s0 = 0;
+        set_group(p, a.tg);
+        set_len(p);
+        return p;
+    }
+    __device__ __forceinline__ Place next(const Place& c) {
+        Place p = c;
+        p.s0 += p.len;
+        if (p.s0 >= p.ns) {
+            p.s0 = 0;
+            p.t0 += a.tg;
+            if (p.t0 >= p.nt) {
+                p.t0 = 0;
+                p.item = rec_item;
+                if (p.item < a.n_items) {
+                    set_item(p, rec);
+                    rec_item += stride;
+                    rec = load_rec_lane(a.items, rec_item, a.n_items, lane);
+                }
+            }
+            set_group(p, a.tg);
+        }
+        set_len(p);
+        return p;
+    }
+    __device__ __forceinline__ int index(const Place& p) const {
+        return p.item < a.n_items && lane < p.len ? __ldg(a.nb_src + p.src_off + p.s0 + lane) : 0;
+    }
+    // copies of the sub-chunk at p (lane's source j) into half h; one group per call, possibly empty
+    __device__ __forceinline__ void copy(const Place& p, int j, int h) const {
+        if (p.item < a.n_items && lane < p.len) {
+            cp_async16(buf(h) + 4 * lane, a.xs + j);
+            float* dst = buf(h) + 4 * kSub + 2 * R * lane;
+            const float* src = a.lam + (int64_t)j * (2 * R);
+#pragma unroll
+            for (int i = 0; i < 2 * R; i += 4) cp_async16(dst + i, src + i);
+        }
+        cp_async_commit();
+    }
+};
+
+// One source against the lane's TT targets (negated coordinates), R right-hand sides.  own: a source of the targets'
+// own cell, where r = 0 gives nothing; other sources start r^2 at the smallest normal float (pair_core).
+template <int KERN, int R, int TT>
+__device__ __forceinline__ void multi_core(const float4 p, const float* __restrict__ l, bool own, const float (&nx)[TT],
+                                           const float (&ny)[TT], const float (&nz)[TT], float2 (&re)[TT][R / 2],
+                                           float2 (&im)[TT][R / 2], float k) {
+    float2 lr[R / 2], li[R / 2];
+    if constexpr (R == 2) {
+        const float4 v = *reinterpret_cast<const float4*>(l);
+        lr[0] = make_float2(v.x, v.y);
+        li[0] = make_float2(v.z, v.w);
+    } else {
+#pragma unroll
+        for (int i = 0; i < R / 4; ++i) {
+            const float4 v = reinterpret_cast<const float4*>(l)[i], w = reinterpret_cast<const float4*>(l + R)[i];
+            lr[2 * i] = make_float2(v.x, v.y);
+            lr[2 * i + 1] = make_float2(v.z, v.w);
+            li[2 * i] = make_float2(w.x, w.y);
+            li[2 * i + 1] = make_float2(w.z, w.w);
+        }
+    }
+    const float base = own ? 0.f : 1.17549435e-38f;
+    float gr[TT], gi[TT];
+    if constexpr (TT % 2 == 0) {
+        const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y), pz = make_float2(p.z, p.z);
+#pragma unroll
+        for (int u = 0; u < TT; u += 2) {
+            const float2 dx = __fadd2_rn(px, make_float2(nx[u], nx[u + 1]));
+            const float2 dy = __fadd2_rn(py, make_float2(ny[u], ny[u + 1]));
+            const float2 dz = __fadd2_rn(pz, make_float2(nz[u], nz[u + 1]));
+            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, make_float2(base, base))));
+            float2 inv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+            inv.x = r2.x > 0.f ? inv.x : 0.f;
+            inv.y = r2.y > 0.f ? inv.y : 0.f;
+            if (KERN == P2P_HELMHOLTZ) {
+                const float2 ph = __fmul2_rn(make_float2(k, k), __fmul2_rn(r2, inv));
+                float2 sn, cs;
+                __sincosf(ph.x, &sn.x, &cs.x);
+                __sincosf(ph.y, &sn.y, &cs.y);
+                const float2 r = __fmul2_rn(cs, inv), i = __fmul2_rn(sn, inv);
+                gr[u] = r.x;
+                gr[u + 1] = r.y;
+                gi[u] = i.x;
+                gi[u + 1] = i.y;
+            } else {
+                gr[u] = inv.x;
+                gr[u + 1] = inv.y;
+            }
+        }
+    } else {
+        const float dx = p.x + nx[0], dy = p.y + ny[0], dz = p.z + nz[0];
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, base)));
+        float inv = rsqrtf(r2);
+        inv = r2 > 0.f ? inv : 0.f;
+        if (KERN == P2P_HELMHOLTZ) {
+            float sn, cs;
+            __sincosf(k * (r2 * inv), &sn, &cs);
+            gr[0] = cs * inv;
+            gi[0] = sn * inv;
+        } else {
+            gr[0] = inv;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < TT; ++u) {
+        const float2 g = make_float2(gr[u], gr[u]);
+        if (KERN == P2P_HELMHOLTZ) {
+            const float2 h = make_float2(gi[u], gi[u]), nh = make_float2(-gi[u], -gi[u]);
+#pragma unroll
+            for (int i = 0; i < R / 2; ++i) {
+                re[u][i] = __ffma2_rn(g, lr[i], __ffma2_rn(nh, li[i], re[u][i]));
+                im[u][i] = __ffma2_rn(g, li[i], __ffma2_rn(h, lr[i], im[u][i]));
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < R / 2; ++i) {
+                re[u][i] = __ffma2_rn(g, lr[i], re[u][i]);
+                im[u][i] = __ffma2_rn(g, li[i], im[u][i]);
+            }
+        }
+    }
+}
+
+// The target group at `cur` (whose sub-chunk is on its way into half h) through all of its sub-chunks, and its
+// results.  nxt: the place after cur, its indices in j.  Leaves cur, nxt, j and h at the next group's first sub-chunk.
+template <int KERN, int R, int TT>
+__device__ __forceinline__ void run_group(Stream<R>& st, Place& cur, Place& nxt, int& j, int& h, float* red) {
+    const MultiArgs& a = st.a;
+    const int lane = st.lane;
+    const int32_t map = cur.map;
+    const int G = map_g(map), Q = map_q(map), q = map_div(map, lane), g = lane - q * G;
+    const int tb = cur.tb + cur.t0, nt = min(a.tg, cur.nt - cur.t0), m_end = cur.m_end;
+    const int32_t perm0 = lane < nt ? __ldg(a.perm + tb + lane) : 0;
+    float nx[TT], ny[TT], nz[TT];
+    float2 re[TT][R / 2], im[TT][R / 2];
+#pragma unroll
+    for (int u = 0; u < TT; ++u) {
+        const int t = g + u * G;
+        const float4 x = t < nt && q < Q ? __ldg(a.xt + tb + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        nx[u] = -x.x;
+        ny[u] = -x.y;
+        nz[u] = -x.z;
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) re[u][i] = im[u][i] = make_float2(0.f, 0.f);
+    }
+    while (true) {
+        st.copy(nxt, j, h ^ 1);
+        const Place after = nxt.item < a.n_items ? st.next(nxt) : nxt;
+        const int ja = st.index(after);
+        cp_async_wait<1>();
+        __syncwarp();
+        if (q < Q) {
+            const float* buf = st.buf(h);
+            const int own = m_end - cur.s0;
+            for (int s = q; s < cur.len; s += Q)
+                multi_core<KERN, R, TT>(*reinterpret_cast<const float4*>(buf + 4 * s), buf + 4 * kSub + 2 * R * s, s < own, nx,
+                                        ny, nz, re, im, a.k);
+        }
+        __syncwarp();  // the half is read before the copies of the place after next overwrite it
+        const bool last = cur.s0 + cur.len >= cur.ns;
+        cur = nxt;
+        nxt = after;
+        j = ja;
+        h ^= 1;
+        if (last) break;
+    }
+    // slice partials -> results, one target of every lane at a time: (Re, Re, Im, Im) of two right-hand sides per
+    // 16 bytes, lane after lane
+    float4* red4 = reinterpret_cast<float4*>(red);
+#pragma unroll
+    for (int u = 0; u < TT; ++u) {
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) red4[i * 32 + lane] = make_float4(re[u][i].x, re[u][i].y, im[u][i].x, im[u][i].y);
+        __syncwarp();
+        const int here = min(G, nt - u * G);  // targets u G .. u G + here - 1
+        for (int e0 = 0; e0 < G * (R / 2); e0 += 32) {
+            const int e = e0 + lane;
+            const int i = min(map_div(map, min(e, 127)), R / 2 - 1), gg = e - i * G;
+            const bool on = e < G * (R / 2) && gg < here;
+            const int t = u * G + gg;
+            int32_t row = __shfl_sync(P2P_FULL_MASK, perm0, t & 31);
+            if (!on) continue;
+            if (t >= 32) row = __ldg(a.perm + tb + t);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int qq = 0; qq < Q; ++qq) {
+                const float4 w = red4[i * 32 + qq * G + gg];
+                v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+            }
+            float2* dst = a.out + (int64_t)row * a.ld + 2 * i;
+            const float2 o0 = make_float2(v.x * kInv4Pi, v.z * kInv4Pi), o1 = make_float2(v.y * kInv4Pi, v.w * kInv4Pi);
+            if (2 * i < a.nrhs) {
+                if (a.atomic_out) atomicAdd(dst, o0);
+                else dst[0] = o0;
+            }
+            if (2 * i + 1 < a.nrhs) {
+                if (a.atomic_out) atomicAdd(dst + 1, o1);
+                else dst[1] = o1;
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <int KERN, int R>
+__global__ void __launch_bounds__(kMultiWarps * 32, 2) k_pair_multi(const __grid_constant__ MultiArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ws = reinterpret_cast<float*>(smem_raw) + warp * warp_floats(R);
+    Stream<R> st{a, lane, (int32_t)gridDim.x * kMultiWarps, 0, 0, ws};
+    float* red = ws + 2 * stage_floats(R);
+    const int32_t item = (int32_t)blockIdx.x * kMultiWarps + warp;
+    if (item >= a.n_items) return;
+    Place cur = st.first(item);
+    st.copy(cur, st.index(cur), 0);
+    Place nxt = st.next(cur);
+    int j = st.index(nxt), h = 0;
+    while (cur.item < a.n_items) {
+        const int tt = map_tt(cur.map);
+        if (tt == 1) run_group<KERN, R, 1>(st, cur, nxt, j, h, red);
+        else if (tt == 2) run_group<KERN, R, 2>(st, cur, nxt, j, h, red);
+        else run_group<KERN, R, 4>(st, cur, nxt, j, h, red);
+    }
+    cp_async_wait<0>();
+}
+
+// dst: 2R floats per source, Re of right-hand sides 0 .. R - 1, then Im (zero past nrhs).
+template <int R>
+__global__ void k_multi_stage(const float2* __restrict__ src, int64_t ld, const int32_t* __restrict__ rows, int64_t n,
+                              int32_t nrhs, float* __restrict__ dst) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n * R) return;
+    const int64_t s = i / R;
+    const int r = (int)(i - s * R);
+    const float2 v = r < nrhs ? src[(int64_t)rows[s] * ld + r] : make_float2(0.f, 0.f);
+    dst[s * 2 * R + r] = v.x;
+    dst[s * 2 * R + R + r] = v.y;
+}
+
+// Right-hand sides of a launch (2, 4 or 8 accumulators) for the `left` ones still to do.
+int block_width(int left) { return left > 4 ? 8 : (left > 2 ? 4 : 2); }
+
+using MultiKernel = void (*)(MultiArgs);
+MultiKernel multi_kernel(const p2p_plan* p, int R) {
+    if (p->kernel == P2P_HELMHOLTZ)
+        return R == 8 ? k_pair_multi<P2P_HELMHOLTZ, 8> : (R == 4 ? k_pair_multi<P2P_HELMHOLTZ, 4> : k_pair_multi<P2P_HELMHOLTZ, 2>);
+    return R == 8 ? k_pair_multi<P2P_LAPLACE, 8> : (R == 4 ? k_pair_multi<P2P_LAPLACE, 4> : k_pair_multi<P2P_LAPLACE, 2>);
+}
+
+}  // namespace
+
+// Staged columns (complex) of nrhs right-hand sides: every block rounded up to its width.
+int32_t p2p_multi_columns(int32_t nrhs) {
+    if (nrhs <= 1) return nrhs;
+    int c = 0;
+    for (int b = 0; b < nrhs; b += 8) c += block_width(std::min(8, nrhs - b));
+    return c;
+}
+
+// Persistent grids for 2, 4 and 8 right-hand sides per launch.
+cudaError_t p2p_multi_configure(p2p_plan* p) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
+        const int R = 2 << i, smem = kMultiWarps * warp_floats(R) * (int)sizeof(float);
+        int per_sm = 0;
+        MultiKernel kern = multi_kernel(p, R);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMultiWarps * 32, smem);
+        p->multi_grid[i] = e == cudaSuccess ? per_sm * sms : 0;
+    }
+    return e;
+}
+
+p2p_status p2p_multi_stage(const p2p_plan* p, const float2* lam, int32_t nrhs, int64_t ld, cudaStream_t s) {
+    float* dst = reinterpret_cast<float*>(p->lam_buf);
+    for (int b = 0; b < nrhs; b += 8) {
+        const int n = std::min(8, nrhs - b), R = block_width(n);
+        const unsigned blocks = (unsigned)((p->n_src * R + 255) / 256);
+        auto stage = R == 8 ? k_multi_stage<8> : (R == 4 ? k_multi_stage<4> : k_multi_stage<2>);
+        stage<<<blocks, 256, 0, s>>>(lam + b, ld, p->src_perm, p->n_src, n, dst);
+        P2P_CHECK_LAUNCH("p2p_apply_stage/multi");
+        dst += p->n_src * 2 * R;
+    }
+    return P2P_OK;
+}
+
+// Results are stored where a box's list is one chunk, else added (the caller has zeroed them).
+p2p_status p2p_multi_launch(const p2p_plan* p, float2* out, int32_t nrhs, int64_t ld, float k, cudaStream_t s) {
+    MultiArgs a;
+    a.items = p->items;
+    a.n_items = (int32_t)p->n_items;
+    a.xs = p->xs_src;
+    a.xt = p->xs;
+    a.nb_src = p->nb_src;
+    a.lam = reinterpret_cast<const float*>(p->lam_buf);
+    a.perm = p->perm;
+    a.ld = ld;
+    a.k = k;
+    a.tg = p->tune.target_group;
+    a.atomic_out = p->max_chunks > 1;
+    for (int b = 0; b < nrhs; b += 8) {
+        a.nrhs = std::min(8, nrhs - b);
+        const int R = block_width(a.nrhs), smem = kMultiWarps * warp_floats(R) * (int)sizeof(float);
+        const int grid = (int)std::min<int64_t>(p->multi_grid[R == 8 ? 2 : R / 4], ((int64_t)a.n_items + kMultiWarps - 1) / kMultiWarps);
+        if (grid <= 0) return P2P_ERR_UNSUPPORTED;
+        a.out = out + b;
+        multi_kernel(p, R)<<<grid, kMultiWarps * 32, smem, s>>>(a);
+        P2P_CHECK_LAUNCH("p2p_apply/multi");
+        a.lam += p->n_src * 2 * R;
+    }
+    return P2P_OK;
+}
