@@ -442,8 +442,8 @@ cudaError_t p2p_pair_configure(p2p_plan* plan) {
     cudaError_t e = p2p_group_configure(plan);
     if (e == cudaSuccess && plan->max_nrhs > 1) e = p2p_multi_configure(plan);
     if (e == cudaSuccess) e = configure_r<1>(plan);
-    if (e == cudaSuccess) e = configure_r<2>(plan);
-    if (e == cudaSuccess) e = configure_r<4>(plan);
+    if (e == cudaSuccess && plan->max_nrhs >= 2) e = configure_r<2>(plan);
+    if (e == cudaSuccess && plan->max_nrhs >= 4) e = configure_r<4>(plan);
     plan->direct_grid = 0;
     if (e == cudaSuccess && plan->direct_k > 0) {
         int dev = 0, sms = 0, per_sm = 0;

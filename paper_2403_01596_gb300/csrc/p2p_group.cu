@@ -12,7 +12,7 @@
 // each member then sweeps its list from shared memory only.  Each result is
 // stored once (no atomics, no zeroing).
 //
-// Plan time (k_group_build, one warp per group): the members' neighbour lists
+// Plan time (k_group_build, four warps per group): the members' neighbour lists
 // (contiguous in the CSR) are sorted and made unique into the union, a prefix of
 // the union boxes' sizes places them in the buffer, the members' lists become
 // buffer positions, and the members are ranked by cost.  Groups are ordered by
@@ -53,40 +53,38 @@ namespace {
 #endif
 
 constexpr int kGroupWarps = P2P_GROUP_WARPS;  // warps of the apply kernel's blocks
-constexpr int kBuildWarps = 4;
+constexpr int kBuildThreads = 128;
 constexpr int kUnionMax = kGroupBoxes * 27;  // union entries of a group at most
 constexpr int pow2_at_least(int x) { return x <= 1 ? 1 : 2 * pow2_at_least((x + 1) / 2); }
 constexpr int kSortSlots = pow2_at_least(kUnionMax);
 constexpr int kPass = 4 * 32;    // targets of one pass of a member
 static_assert(kGroupBoxes >= 1 && kGroupBoxes <= 32, "members are ranked by one warp");
 
-// One warp per group g: union of the members' neighbour boxes, its buffer
-// offsets, the members' position lists, lane maps and cost ranks.  maxes[0]:
-// largest union (sources), maxes[1]: largest sum of the members' padded list
-// lengths.
-__global__ void __launch_bounds__(kBuildWarps * 32)
+// One block of kBuildThreads per group g: union of the members' neighbour boxes, its buffer offsets, the members'
+// position lists, lane maps and cost ranks.  maxes[0]: largest union (sources), maxes[1]: largest sum of the members'
+// padded list lengths.  Latency bound (a group is ~200 entries): with one warp per group the 244 groups of an
+// 80 000-point plan took 85 us, with four 33 us.
+__global__ void __launch_bounds__(kBuildThreads)
     k_group_build(const int32_t* __restrict__ nbr_ptr, const int32_t* __restrict__ nbr_idx,
                   const int32_t* __restrict__ nbr_self, const int32_t* __restrict__ box_ptr,
                   const int32_t* __restrict__ src_box_ptr, const int32_t* __restrict__ box_src,
-                  const int32_t* __restrict__ pk_off, int32_t nb, int32_t n_groups, int32_t* __restrict__ g_union,
+                  const int32_t* __restrict__ pk_off, int32_t nb, int32_t* __restrict__ g_union,
                   int32_t* __restrict__ g_nunion, int16_t* __restrict__ g_pos, int32_t* __restrict__ g_mend,
                   int32_t* __restrict__ g_map, int32_t* __restrict__ g_morder, int4* __restrict__ g_copy,
-                  uint64_t* __restrict__ keys, int32_t* __restrict__ vals, int32_t* __restrict__ maxes) {
-    __shared__ int32_t buf_all[kBuildWarps][kSortSlots];
-    __shared__ int32_t off_all[kBuildWarps][kUnionMax + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t g = (int64_t)blockIdx.x * kBuildWarps + warp;
-    if (g >= n_groups) return;
-    int32_t* buf = buf_all[warp];
-    int32_t* uoff = off_all[warp];
+                  uint32_t* __restrict__ keys, int32_t* __restrict__ vals, int32_t* __restrict__ maxes) {
+    __shared__ int32_t buf[kSortSlots];
+    __shared__ int32_t uoff[kUnionMax + 1];
+    __shared__ int warp_sum[kBuildThreads / 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t g = blockIdx.x;
     const int32_t b0 = (int32_t)g * kGroupBoxes, b1 = min(nb, b0 + kGroupBoxes);
     const int32_t e0 = nbr_ptr[b0], ne = nbr_ptr[b1] - e0;  // <= kUnionMax (lists hold <= 27 entries)
-    for (int i = lane; i < kSortSlots; i += 32) buf[i] = i < ne ? nbr_idx[e0 + i] : INT32_MAX;
-    __syncwarp();
+    for (int i = tid; i < kSortSlots; i += kBuildThreads) buf[i] = i < ne ? nbr_idx[e0 + i] : INT32_MAX;
+    __syncthreads();
     // bitonic sort of the slots, ascending
     for (int k = 2; k <= kSortSlots; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < kSortSlots; i += 32) {
+            for (int i = tid; i < kSortSlots; i += kBuildThreads) {
                 const int l = i ^ j;
                 if (l > i) {
                     const int32_t x = buf[i], y = buf[l];
@@ -97,76 +95,81 @@ __global__ void __launch_bounds__(kBuildWarps * 32)
                     }
                 }
             }
-            __syncwarp();
+            __syncthreads();
         }
     }
-    // unique entries, compacted into the union (kSortSlots / 32 consecutive slots per lane)
-    constexpr int kPer = kSortSlots / 32;
+    // exclusive prefix of one value per thread, and the sum
+    auto block_scan = [&](int v, int& total) {
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(P2P_FULL_MASK, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        int before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < kBuildThreads / 32; ++w) {
+            before += w < warp ? warp_sum[w] : 0;
+            all += warp_sum[w];
+        }
+        __syncthreads();
+        total = all;
+        return before + x - v;
+    };
+    // unique entries, compacted into the union (kPer consecutive slots per thread)
+    constexpr int kPer = kSortSlots / kBuildThreads > 0 ? kSortSlots / kBuildThreads : 1;
     int32_t v[kPer];
     int cnt = 0;
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
-        const int i = lane * kPer + u;
-        v[u] = buf[i];
-        const bool keep = v[u] != INT32_MAX && (i == 0 || buf[i - 1] != v[u]);
-        if (!keep) v[u] = -1;
-        cnt += keep;
+        const int i = tid * kPer + u;
+        v[u] = i < kSortSlots ? buf[i] : INT32_MAX;
+        if (v[u] == INT32_MAX || (i > 0 && buf[i - 1] == v[u])) v[u] = -1;
+        cnt += v[u] >= 0;
     }
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(P2P_FULL_MASK, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int nu = __shfl_sync(P2P_FULL_MASK, incl, 31);
-    __syncwarp();
-    int pos = incl - cnt;
+    int nu;
+    int pos = block_scan(cnt, nu);  // its barriers also end every thread's reads of buf
     int32_t* U = g_union + g * kUnionMax;
 #pragma unroll
     for (int u = 0; u < kPer; ++u)
         if (v[u] >= 0) {
             U[pos] = v[u];
-            buf[pos] = v[u];  // the union stays in shared memory for the lookups below (pos <= slot index)
+            buf[pos] = v[u];  // the union stays in shared memory for the lookups below
             ++pos;
         }
-    __syncwarp();
+    __syncthreads();
     // buffer offsets of the union boxes: exclusive prefix of their sizes
     int sz[kPer];
     int tot = 0;
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
-        const int i = lane * kPer + u;
+        const int i = tid * kPer + u;
         sz[u] = i < nu ? src_box_ptr[buf[i] + 1] - src_box_ptr[buf[i]] : 0;
         tot += sz[u];
     }
-    int run = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(P2P_FULL_MASK, run, o);
-        if (lane >= o) run += y;
-    }
-    int acc = run - tot;
+    int total;
+    int acc = block_scan(tot, total);
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
-        const int i = lane * kPer + u;
-        if (i <= nu && i < kUnionMax + 1) uoff[i] = acc;
+        const int i = tid * kPer + u;
+        if (i < nu) uoff[i] = acc;
         acc += sz[u];
     }
-    const int total = __shfl_sync(P2P_FULL_MASK, run, 31);
-    if (lane == 0) {
+    if (tid == 0) {
         g_nunion[g] = nu;
         uoff[nu] = total;
         atomicMax(&maxes[0], total);
         atomicMax(&maxes[1], pk_off[b1] - pk_off[b0]);
     }
-    __syncwarp();
+    __syncthreads();
     // the copies that stage the union: source start, buffer offset and length of every union box
-    for (int i = lane; i < nu; i += 32)
+    for (int i = tid; i < nu; i += kBuildThreads)
         g_copy[g * kUnionMax + i] = make_int4(src_box_ptr[buf[i]], uoff[i], uoff[i + 1] - uoff[i], 0);
     // members: their lists (own box first, then the others ascending, as the plan's source lists) as buffer
     // positions; lane = entry of the member's neighbour list, moved to its place in that order
-    int64_t cost = 0;
-    for (int32_t b = b0; b < b1; ++b) {
+    for (int32_t b = b0 + warp; b < b1; b += kBuildThreads / 32) {
         const int32_t f0 = nbr_ptr[b], ne_b = nbr_ptr[b + 1] - f0;  // <= 27
         const int32_t c = lane < ne_b ? nbr_idx[f0 + lane] : -1;
         int sp;
@@ -195,32 +198,39 @@ __global__ void __launch_bounds__(kBuildWarps * 32)
             const int y = __shfl_up_sync(P2P_FULL_MASK, li, o);
             if (lane >= o) li += y;
         }
-        int16_t* list = g_pos + pk_off[b] + (li - len);
-        for (int e = 0; e < len; ++e) list[e] = (int16_t)(start + e);
+        // neighbour after neighbour, each a run of consecutive positions
+        for (int e = 0; e < ne_b; ++e) {
+            const int s0 = __shfl_sync(P2P_FULL_MASK, start, e), m = __shfl_sync(P2P_FULL_MASK, len, e);
+            int16_t* list = g_pos + pk_off[b] + __shfl_sync(P2P_FULL_MASK, li - len, e);
+            for (int p = lane; p < m; p += 32) list[p] = (int16_t)(s0 + p);
+        }
         const int own_len = __shfl_sync(P2P_FULL_MASK, len, 0);
         if (lane == 0) {
             const int32_t nt = box_ptr[b + 1] - box_ptr[b], S = box_src[b];
             g_mend[b] = sp < 0 ? 0 : own_len;
-            cost += (int64_t)nt * S;
             // lane maps of a full pass and of the last pass
             g_map[2 * (int64_t)b] = p2p_lane_map(min(nt, kPass), S, 32, P2P_GROUP_PER_ITER);
             g_map[2 * (int64_t)b + 1] = p2p_lane_map(nt - ((nt - 1) / kPass) * kPass, S, 32, P2P_GROUP_PER_ITER);
         }
     }
-    if (lane == 0) {
-        keys[g] = 0xFFFFFFFFull - (uint64_t)min(cost, (int64_t)0xFFFFFFFF);
-        vals[g] = (int32_t)g;
-    }
     // members by decreasing cost (ties by position)
-    const int nm = b1 - b0;
-    int64_t mc = -1;
-    if (lane < nm) mc = (int64_t)(box_ptr[b0 + lane + 1] - box_ptr[b0 + lane]) * box_src[b0 + lane];
-    int rank = 0;
-    for (int j = 0; j < nm; ++j) {
-        const int64_t cj = __shfl_sync(P2P_FULL_MASK, mc, j);
-        rank += (cj > mc) || (cj == mc && j < lane);
+    if (warp == 0) {
+        const int nm = b1 - b0;
+        int64_t mc = -1;
+        if (lane < nm) mc = (int64_t)(box_ptr[b0 + lane + 1] - box_ptr[b0 + lane]) * box_src[b0 + lane];
+        int rank = 0;
+        int64_t cost = 0;
+        for (int j = 0; j < nm; ++j) {
+            const int64_t cj = __shfl_sync(P2P_FULL_MASK, mc, j);
+            rank += (cj > mc) || (cj == mc && j < lane);
+            cost += cj;
+        }
+        if (lane < nm) g_morder[g * kGroupBoxes + rank] = lane;
+        if (lane == 0) {
+            keys[g] = cost_key<kCostBits>(cost);
+            vals[g] = (int32_t)g;
+        }
     }
-    if (lane < nm) g_morder[g * kGroupBoxes + rank] = lane;
 }
 
 struct GroupArgs {
@@ -494,31 +504,29 @@ __global__ void __launch_bounds__(kGroupWarps * 32, P2P_GROUP_MIN_BLOCKS) k_pair
 }  // namespace
 
 // Plan time: builds the groups of a plan (g_* arrays carved by the plan) and orders them heaviest first.
-// keys / vals / keys_alt / vals_alt / radix_ws: sort scratch of at least n_groups entries.  Returns the
-// largest union and the largest group list total in cap[0], cap[1].
-cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* nbr_idx, uint64_t* keys,
-                            int32_t* vals, uint64_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
+// keys / vals / keys_alt / vals_alt / radix_ws: sort scratch of at least n_groups entries.  The largest union and the
+// largest group list total are in cap[0], cap[1] once the stream has come this far.
+cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* nbr_idx, uint32_t* keys,
+                            int32_t* vals, uint32_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
                             cudaStream_t s, int32_t* cap) {
     cap[0] = cap[1] = 0;
     const int32_t ng = p->n_groups;
     if (ng == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(maxes, 0, 2 * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
-    k_group_build<<<(unsigned)((ng + kBuildWarps - 1) / kBuildWarps), kBuildWarps * 32, 0, s>>>(
+    k_group_build<<<(unsigned)ng, kBuildThreads, 0, s>>>(
         nbr_ptr, nbr_idx, p->two_sets ? p->nbr_self : nullptr, p->box_ptr, p->src_box_ptr, p->box_src, p->pk_off,
-        p->nb, ng, p->g_union, p->g_nunion, p->g_pos, p->g_mend, p->g_map, p->g_morder, p->g_copy, keys, vals,
+        p->nb, p->g_union, p->g_nunion, p->g_pos, p->g_mend, p->g_map, p->g_morder, p->g_copy, keys, vals,
         maxes);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     bool in_alt = false;
-    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, ng, 32, radix_ws, s, &in_alt);
+    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, ng, kCostBits, radix_ws, s, &in_alt);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(p->g_order, in_alt ? vals_alt : vals, (size_t)ng * sizeof(int32_t), cudaMemcpyDeviceToDevice,
                         s);
     if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(cap, maxes, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return e;
-    return cudaStreamSynchronize(s);
+    return cudaMemcpyAsync(cap, maxes, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
 }
 
 // Persistent grid of the group kernel for the plan's buffer sizes (0: no block fits).

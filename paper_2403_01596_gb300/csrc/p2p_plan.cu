@@ -23,8 +23,8 @@ void set_message(const char* msg) { snprintf(g_last_error, sizeof(g_last_error),
 using namespace p2p_detail;
 
 // Box-group kernel tables (p2p_group.cu).
-cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* nbr_idx, uint64_t* keys,
-                            int32_t* vals, uint64_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
+cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* nbr_idx, uint32_t* keys,
+                            int32_t* vals, uint32_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
                             cudaStream_t s, int32_t* cap);
 
 // Tensor-core lists (p2p_tc.cu).
@@ -48,8 +48,25 @@ __device__ __forceinline__ uint32_t cell_of(float x, double lo, double h, int ng
     return (uint32_t)f;
 }
 
-__global__ void k_keys(const float* __restrict__ pts, int64_t n, double lo0, double lo1, double lo2, double h, int ng,
-                       uint64_t* __restrict__ keys, int32_t* __restrict__ vals, int32_t* __restrict__ bad) {
+// The same cell from FP32 arithmetic where that is safe: q = (x - lo) / h evaluated in floats is off by less than
+// (4 |q| + |lo| / h + 1) 2^-23 (rounding of lo, the difference, 1 / h and the product), so a q further than that from
+// every integer has the right floor; the others take the double division.  FP64 runs at 1/64 of the FP32 rate here:
+// 2^20 points took 83 us in doubles.
+struct AxisGrid {
+    double lo, h;
+    float lo_f, inv_h, slack;  // slack: (|lo| / h + 1) 2^-23
+};
+__device__ __forceinline__ uint32_t cell_fast(float x, const AxisGrid& g, int ng) {
+    const float q = (x - g.lo_f) * g.inv_h;
+    const float f = floorf(q);
+    const float off = fminf(q - f, f + 1.f - q);
+    if (!(off > fmaf(fabsf(q), 4.8e-7f, g.slack))) return cell_of(x, g.lo, g.h, ng);  // also where q is not finite
+    return (uint32_t)fminf(fmaxf(f, 0.f), (float)(ng - 1));
+}
+
+template <typename K>
+__global__ void k_keys(const float* __restrict__ pts, int64_t n, AxisGrid g0, AxisGrid g1, AxisGrid g2, int ng,
+                       K* __restrict__ keys, int32_t* __restrict__ vals, int32_t* __restrict__ bad) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
@@ -57,31 +74,76 @@ __global__ void k_keys(const float* __restrict__ pts, int64_t n, double lo0, dou
         *bad = 1;
         x = y = z = 0.f;
     }
-    keys[i] = p2p_morton(cell_of(x, lo0, h, ng), cell_of(y, lo1, h, ng), cell_of(z, lo2, h, ng));
+    keys[i] = (K)p2p_morton(cell_fast(x, g0, ng), cell_fast(y, g1, ng), cell_fast(z, g2, ng));
     vals[i] = (int32_t)i;
 }
 
-__global__ void k_heads(const uint64_t* __restrict__ keys, int64_t n, int32_t* __restrict__ head) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    head[s] = (s == 0 || keys[s] != keys[s - 1]) ? 1 : 0;
+// Boxes are the runs of equal sorted keys.  A block of kThreads threads takes kHeads consecutive keys per thread:
+// k_heads counts the run heads of every block, k_rle numbers them from the scanned counts and writes the boxes.
+constexpr int kHeads = 4;
+template <typename K>
+__device__ __forceinline__ int heads_of(const K* __restrict__ keys, int64_t n, int64_t s0, bool (&head)[kHeads]) {
+    K prev = s0 > 0 && s0 < n ? keys[s0 - 1] : (K)0;
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < kHeads; ++i) {
+        const bool in = s0 + i < n;
+        const K k = in ? keys[s0 + i] : (K)0;
+        head[i] = in && (s0 + i == 0 || k != prev);
+        prev = k;
+        c += head[i];
+    }
+    return c;
 }
 
-__global__ void k_rle(const uint64_t* __restrict__ keys, const int32_t* __restrict__ vals,
-                      const int32_t* __restrict__ head, const int32_t* __restrict__ ex, int64_t n,
-                      int32_t* __restrict__ perm, int32_t* __restrict__ point_box, int64_t* __restrict__ box_keys,
-                      int32_t* __restrict__ box_ptr) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const int32_t id = ex[s] + head[s] - 1;
-    if (head[s]) {
-        box_keys[id] = (int64_t)keys[s];
-        box_ptr[id] = (int32_t)s;
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_heads(const K* __restrict__ keys, int64_t n, int32_t* __restrict__ count) {
+    const int64_t s0 = ((int64_t)blockIdx.x * kThreads + threadIdx.x) * kHeads;
+    bool head[kHeads];
+    int c = heads_of(keys, n, s0, head);
+    __shared__ int sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    c = __reduce_add_sync(P2P_FULL_MASK, c);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&sum, c);
+    __syncthreads();
+    if (threadIdx.x == 0) count[blockIdx.x] = sum;
+}
+
+template <typename K>
+__global__ void __launch_bounds__(kThreads)
+    k_rle(const K* __restrict__ keys, const int32_t* __restrict__ vals, const int32_t* __restrict__ first, int64_t n,
+          int32_t* __restrict__ perm, int32_t* __restrict__ point_box, int64_t* __restrict__ box_keys,
+          int32_t* __restrict__ box_ptr) {
+    __shared__ int warp_sum[kThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t s0 = ((int64_t)blockIdx.x * kThreads + threadIdx.x) * kHeads;
+    bool head[kHeads];
+    const int c = heads_of(keys, n, s0, head);
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(P2P_FULL_MASK, x, o);
+        if (lane >= o) x += y;
     }
-    const int32_t orig = vals[s];
-    perm[s] = orig;
-    point_box[orig] = id;
-    if (s == n - 1) box_ptr[id + 1] = (int32_t)n;
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    int id = first[blockIdx.x] + x - c - 1;  // the run that position s0 - 1 belongs to
+    for (int w = 0; w < warp; ++w) id += warp_sum[w];
+#pragma unroll
+    for (int i = 0; i < kHeads; ++i) {
+        const int64_t s = s0 + i;
+        if (s >= n) break;
+        if (head[i]) {
+            ++id;
+            box_keys[id] = (int64_t)keys[s];
+            box_ptr[id] = (int32_t)s;
+        }
+        const int32_t orig = vals[s];
+        perm[s] = orig;
+        point_box[orig] = id;
+        if (s == n - 1) box_ptr[id + 1] = (int32_t)n;
+    }
 }
 
 // --------------------------------------------------------------- neighbours --
@@ -113,58 +175,66 @@ __device__ __forceinline__ int32_t warp_sort_asc(int32_t v, int lane) {
     return v;
 }
 
-// One warp per target box; lane l < 27 probes the offset (l%3-1, (l/3)%3-1, l/9-1)
-// among the source boxes' keys (the same keys for a one-set structure, TWO = false).
-template <bool FILL, bool TWO>
-__global__ void k_neighbors(const int64_t* __restrict__ box_keys, int32_t nb, const int64_t* __restrict__ src_keys,
-                            int32_t nbs, const int32_t* __restrict__ src_box_ptr, int ng, int32_t* __restrict__ cnt,
-                            int32_t* __restrict__ src_cnt, const int32_t* __restrict__ nbr_ptr,
-                            int32_t* __restrict__ nbr_idx, int32_t* __restrict__ nbr_self, int32_t* __restrict__ bad) {
+// One warp per target box; lane l < 27 probes the offset (l%3-1, (l/3)%3-1, l/9-1) among the source boxes' keys (the
+// same keys for a one-set structure, TWO = false) and keeps what it found; sum: the sources of all neighbourhoods.
+template <bool TWO>
+__global__ void __launch_bounds__(kThreads)
+    k_nbr_find(const int64_t* __restrict__ box_keys, int32_t nb, const int64_t* __restrict__ src_keys, int32_t nbs,
+               const int32_t* __restrict__ src_box_ptr, int ng, int32_t* __restrict__ cnt, int32_t* __restrict__ found,
+               unsigned long long* __restrict__ sum, int32_t* __restrict__ bad) {
+    __shared__ unsigned long long block_sum;
+    if (threadIdx.x == 0) block_sum = 0ull;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (b >= nb) return;
-    const uint64_t key = (uint64_t)box_keys[b];
-    const int cx = (int)p2p_compact3(key), cy = (int)p2p_compact3(key >> 1), cz = (int)p2p_compact3(key >> 2);
-    int32_t id = -1;
-    if (lane < 27) {
-        int x = cx + lane % 3 - 1, y = cy + (lane / 3) % 3 - 1, z = cz + lane / 9 - 1;
-        if (x >= 0 && y >= 0 && z >= 0 && x < ng && y < ng && z < ng)
-            id = find_key(src_keys, nbs, (int64_t)p2p_morton(x, y, z));
-    }
-    const unsigned found = __ballot_sync(P2P_FULL_MASK, id >= 0);
-    if (!FILL) {
+    if (b < nb) {
+        const uint64_t key = (uint64_t)box_keys[b];
+        const int cx = (int)p2p_compact3(key), cy = (int)p2p_compact3(key >> 1), cz = (int)p2p_compact3(key >> 2);
+        int32_t id = -1;
+        if (lane < 27) {
+            int x = cx + lane % 3 - 1, y = cy + (lane / 3) % 3 - 1, z = cz + lane / 9 - 1;
+            if (x >= 0 && y >= 0 && z >= 0 && x < ng && y < ng && z < ng)
+                id = find_key(src_keys, nbs, (int64_t)p2p_morton(x, y, z));
+            found[b * 27 + lane] = id;
+        }
+        const unsigned any = __ballot_sync(P2P_FULL_MASK, id >= 0);
         int s = id >= 0 ? src_box_ptr[id + 1] - src_box_ptr[id] : 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(P2P_FULL_MASK, s, o);
         if (lane == 0) {
-            cnt[b] = __popc(found);
-            src_cnt[b] = s;
+            cnt[b] = __popc(any);
+            if (s) atomicAdd(&block_sum, (unsigned long long)s);
             if (b > 0 && box_keys[b - 1] >= box_keys[b]) *bad = 1;  // keys must strictly ascend
-            if (!TWO && !((found >> 13) & 1u)) *bad = 1;             // a box must find itself
+            if (!TWO && !((any >> 13) & 1u)) *bad = 1;               // a box must find itself
         }
-    } else {
-        int32_t v = warp_sort_asc(id >= 0 ? id : INT32_MAX, lane);
-        if (lane < __popc(found)) nbr_idx[nbr_ptr[b] + lane] = v;
-        if (TWO) {
-            // position of the source box of the target box's own cell (probe 13) in the sorted list
-            const int32_t self = __shfl_sync(P2P_FULL_MASK, id, 13);
-            const unsigned at = __ballot_sync(P2P_FULL_MASK, self >= 0 && v == self);
-            if (lane == 0) nbr_self[b] = at ? __ffs(at) - 1 : -1;
-        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && block_sum) atomicAdd(sum, block_sum);
+}
+
+// The found neighbours of every box in ascending order.
+template <bool TWO>
+__global__ void __launch_bounds__(kThreads)
+    k_nbr_fill(const int32_t* __restrict__ found, int32_t nb, const int32_t* __restrict__ nbr_ptr,
+               int32_t* __restrict__ nbr_idx, int32_t* __restrict__ nbr_self) {
+    const int lane = threadIdx.x & 31;
+    const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (b >= nb) return;
+    const int32_t id = lane < 27 ? found[b * 27 + lane] : -1;
+    const int n = __popc(__ballot_sync(P2P_FULL_MASK, id >= 0));
+    const int32_t v = warp_sort_asc(id >= 0 ? id : INT32_MAX, lane);
+    if (lane < n) nbr_idx[nbr_ptr[b] + lane] = v;
+    if (TWO) {
+        // position of the source box of the target box's own cell (probe 13) in the sorted list
+        const int32_t self = __shfl_sync(P2P_FULL_MASK, id, 13);
+        const unsigned at = __ballot_sync(P2P_FULL_MASK, self >= 0 && v == self);
+        if (lane == 0) nbr_self[b] = at ? __ffs(at) - 1 : -1;
     }
 }
 
 __global__ void k_keys_ascending(const int64_t* __restrict__ keys, int32_t n, int32_t* __restrict__ bad) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > 0 && i < n && keys[i - 1] >= keys[i]) *bad = 1;
-}
-
-__global__ void k_sum_i32(const int32_t* __restrict__ v, int64_t n, unsigned long long* __restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    long long s = i < n ? (long long)v[i] : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(P2P_FULL_MASK, s, o);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, (unsigned long long)s);
 }
 
 // -------------------------------------------------------------------- plans --
@@ -177,60 +247,93 @@ __global__ void k_gather_xyz(const float* __restrict__ pts, const int32_t* __res
     xs[s] = make_float4(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], 0.f);
 }
 
-// Per target box: S_b, work-item count ceil(S_b / chunk) and the padded length
-// of its source list, and the size of the source box of its own cell (the
-// sources that can sit at r = 0 from one of its targets).  Validates the CSR
-// (ascending ids in range; a one-set structure lists each box itself, a two-set
-// structure's nbr_self must point into the list or be -1).
-__global__ void k_box_info(const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ src_box_ptr,
-                           int32_t nbs, const int32_t* __restrict__ nbr_ptr, const int32_t* __restrict__ nbr_idx,
-                           const int32_t* __restrict__ nbr_self, int32_t nb, int64_t nnz, int chunk, int upper,
-                           int32_t* __restrict__ box_src, int32_t* __restrict__ list_len,
-                           int32_t* __restrict__ n_chunks, int32_t* __restrict__ padded, int32_t* __restrict__ self_len,
-                           int32_t* __restrict__ maxes, unsigned int* __restrict__ status) {
-    int32_t b = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (b >= nb) return;
-    int32_t e0 = nbr_ptr[b], e1 = nbr_ptr[b + 1];
+// What plan creation has to know of the lists before it builds them (device, then host).
+struct ListInfo {
+    int32_t max_len, max_box;  // longest source list, largest box
+    int32_t tails;             // lists just over one default chunk: a full item plus a short tail item
+    int32_t packed;            // entries of all lists, each padded to 4
+    int32_t items[3];          // work items with the chunk of each candidate tuning
+    unsigned int status;       // nonzero: invalid CSR
+};
+
+// Per target box: S_b, the length of its source list, and the size of the source box of its own cell (the sources
+// that can sit at r = 0 from one of its targets).  Validates the CSR (ascending ids in range; a one-set structure
+// lists each box itself, a two-set structure's nbr_self must point into the list or be -1).
+__global__ void __launch_bounds__(kThreads)
+    k_box_info(const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ src_box_ptr, int32_t nbs,
+               const int32_t* __restrict__ nbr_ptr, const int32_t* __restrict__ nbr_idx,
+               const int32_t* __restrict__ nbr_self, int32_t nb, int64_t nnz, int chunk0, int chunk1, int chunk2,
+               int upper, int32_t* __restrict__ box_src, int32_t* __restrict__ list_len, int32_t* __restrict__ self_len,
+               ListInfo* __restrict__ info) {
+    const int32_t b = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
     int64_t s = 0, s_up = 0;
-    int32_t self = -1, self_n = 0;
-    bool ok = e0 >= 0 && e1 >= e0 && e1 <= nnz && e1 - e0 <= 27;
-    if (ok) {
-        const int32_t want = nbr_self ? nbr_self[b] : -2;
-        if (nbr_self && (want < -1 || want >= e1 - e0)) ok = false;
-        for (int32_t e = e0; ok && e < e1; ++e) {
-            int32_t c = nbr_idx[e];
-            if (c < 0 || c >= nbs || (e > e0 && c <= nbr_idx[e - 1])) {
-                ok = false;
-                break;
+    int32_t self_n = 0, own = 0;
+    bool bad = false;
+    if (b < nb) {
+        const int32_t e0 = nbr_ptr[b], e1 = nbr_ptr[b + 1];
+        int32_t self = -1;
+        bool ok = e0 >= 0 && e1 >= e0 && e1 <= nnz && e1 - e0 <= 27;
+        if (ok) {
+            const int32_t want = nbr_self ? nbr_self[b] : -2;
+            if (nbr_self && (want < -1 || want >= e1 - e0)) ok = false;
+            int32_t prev = -1;
+            for (int32_t e = e0; ok && e < e1; ++e) {
+                const int32_t c = nbr_idx[e];
+                if (c < 0 || c >= nbs || c <= prev) {
+                    ok = false;
+                    break;
+                }
+                prev = c;
+                const int32_t sz = src_box_ptr[c + 1] - src_box_ptr[c];
+                if (nbr_self ? (e - e0 == want) : (c == b)) {
+                    self = e - e0;
+                    self_n = sz;
+                }
+                s += sz;
+                if (c >= b) s_up += sz;
             }
-            const int32_t sz = src_box_ptr[c + 1] - src_box_ptr[c];
-            if (nbr_self ? (e - e0 == want) : (c == b)) {
-                self = e - e0;
-                self_n = sz;
-            }
-            s += sz;
-            if (c >= b) s_up += sz;
         }
+        own = box_ptr[b + 1] - box_ptr[b];
+        bad = !ok || (!nbr_self && self < 0) || own <= 0 || s > INT32_MAX - 4;
+        if (bad) {
+            s = 0;
+            s_up = 0;
+            self_n = 0;
+        }
+        box_src[b] = (int32_t)s;
+        self_len[b] = self_n;
+        list_len[b] = (int32_t)(upper ? s_up : s);
     }
-    int32_t own = box_ptr[b + 1] - box_ptr[b];
-    if (!ok || (!nbr_self && self < 0) || own <= 0 || s > INT32_MAX - 4) {
-        atomicOr(status, P2P_DEV_BAD_INPUT);
-        s = 0;
-        s_up = 0;
-        self_n = 0;
+    // one set of atomics per warp
+    const int32_t len = (int32_t)(upper ? s_up : s);
+    const bool tail = len > chunk0 && 3ll * len <= 4ll * chunk0;
+    const int32_t max_len = __reduce_max_sync(P2P_FULL_MASK, len), max_own = __reduce_max_sync(P2P_FULL_MASK, own);
+    const int32_t padded = __reduce_add_sync(P2P_FULL_MASK, (len + 3) & ~3);
+    const int32_t i0 = __reduce_add_sync(P2P_FULL_MASK, (int32_t)(((int64_t)len + chunk0 - 1) / chunk0));
+    const int32_t i1 = __reduce_add_sync(P2P_FULL_MASK, (int32_t)(((int64_t)len + chunk1 - 1) / chunk1));
+    const int32_t i2 = __reduce_add_sync(P2P_FULL_MASK, (int32_t)(((int64_t)len + chunk2 - 1) / chunk2));
+    const int tails = __popc(__ballot_sync(P2P_FULL_MASK, tail));
+    const bool any_bad = __any_sync(P2P_FULL_MASK, bad);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&info->max_len, max_len);
+        atomicMax(&info->max_box, max_own);
+        if (tails) atomicAdd(&info->tails, tails);
+        atomicAdd(&info->packed, padded);
+        atomicAdd(&info->items[0], i0);
+        atomicAdd(&info->items[1], i1);
+        atomicAdd(&info->items[2], i2);
+        if (any_bad) atomicOr(&info->status, P2P_DEV_BAD_INPUT);
     }
-    box_src[b] = (int32_t)s;
-    self_len[b] = self_n;
-    const int64_t len = upper ? s_up : s;  // length of the box's source list
-    list_len[b] = (int32_t)len;
-    int32_t c = (int32_t)((len + chunk - 1) / chunk);
-    n_chunks[b] = c;
-    padded[b] = (int32_t)((len + 3) & ~3ll);
-    atomicMax(&maxes[0], c);
-    atomicMax(&maxes[1], own);
-    // lists just over one chunk: a full item plus a short tail item (counted for the default-tuning choice)
-    if (len > chunk && 3 * len <= 4ll * chunk) atomicAdd(&maxes[2], 1);
-    atomicAdd(&maxes[3], c);  // work items in all
+}
+
+// Items and padded length of every box's list for the chosen chunk.
+__global__ void k_list_sizes(const int32_t* __restrict__ list_len, int32_t nb, int chunk, int32_t* __restrict__ n_chunks,
+                             int32_t* __restrict__ padded) {
+    const int32_t b = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (b >= nb) return;
+    const int32_t len = list_len[b];
+    n_chunks[b] = (int32_t)(((int64_t)len + chunk - 1) / chunk);
+    padded[b] = (len + 3) & ~3;
 }
 
 // Work-item records (unsorted) and their sort keys: larger cost (targets x
@@ -239,7 +342,7 @@ __global__ void k_item_records(const int32_t* __restrict__ n_chunks, const int32
                                const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ list_len,
                                const int32_t* __restrict__ self_len, const int32_t* __restrict__ pk_off, int32_t nb,
                                int chunk, int tg, int two_sets, ItemRec* __restrict__ recs,
-                               uint64_t* __restrict__ keys, int32_t* __restrict__ vals) {
+                               uint32_t* __restrict__ keys, int32_t* __restrict__ vals) {
     int32_t b = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
     if (b >= nb) return;
     const int32_t c = n_chunks[b], o = item_off[b];
@@ -262,7 +365,7 @@ __global__ void k_item_records(const int32_t* __restrict__ n_chunks, const int32
         r.map_last = p2p_lane_map(last, r.ns);
         r.b = b;
         recs[o + i] = r;
-        keys[o + i] = 0xFFFFFFFFull - (uint64_t)min((int64_t)nt * r.ns, (int64_t)0xFFFFFFFF);
+        keys[o + i] = cost_key<kCostBits>((int64_t)nt * r.ns);
         vals[o + i] = o + i;
     }
 }
@@ -277,7 +380,7 @@ __global__ void k_item_gather(const ItemRec* __restrict__ recs, const int32_t* _
 // `lanes` lanes (passes of up to 4 * lanes targets), sort keys by decreasing cost.
 __global__ void k_direct_items(const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ list_len,
                                const int32_t* __restrict__ self_len, const int32_t* __restrict__ pk_off, int32_t nb,
-                               int lanes, ItemRec* __restrict__ recs, uint64_t* __restrict__ keys,
+                               int lanes, ItemRec* __restrict__ recs, uint32_t* __restrict__ keys,
                                int32_t* __restrict__ vals) {
     const int32_t b = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
     if (b >= nb) return;
@@ -294,7 +397,7 @@ __global__ void k_direct_items(const int32_t* __restrict__ box_ptr, const int32_
     r.map_last = p2p_lane_map(last, S, lanes, 8);
     r.b = b;
     recs[b] = r;
-    keys[b] = 0xFFFFFFFFull - (uint64_t)min((int64_t)nt * S, (int64_t)0xFFFFFFFF);
+    keys[b] = cost_key<kFineCostBits>((int64_t)nt * S);
     vals[b] = b;
 }
 
@@ -346,28 +449,25 @@ __global__ void k_pack(const float4* __restrict__ xs, const int32_t* __restrict_
     const int32_t total = __shfl_sync(P2P_FULL_MASK, incl, 31);
     const int64_t base = pk_off[b];
     const int32_t padded = pk_off[b + 1] - pk_off[b];
-    for (int32_t p0 = 0; p0 < padded; p0 += 32) {
-        const int32_t p = p0 + lane;
-        int32_t seg = 0;
-        for (int e = 0; e < ne; ++e) {
-            int32_t ex = __shfl_sync(P2P_FULL_MASK, excl, e);
-            if (p >= ex) seg = e;
+    // neighbour after neighbour, each a run of consecutive indices (looking up the neighbour of every entry instead
+    // took 55 us for the 15 M entries of the 2^20-point sphere at 32 points per box)
+    for (int e = 0; e < ne; ++e) {
+        const int32_t s0 = __shfl_sync(P2P_FULL_MASK, start, e), m = __shfl_sync(P2P_FULL_MASK, len, e);
+        const int64_t to = base + __shfl_sync(P2P_FULL_MASK, excl, e);
+        for (int32_t p = lane; p < m; p += 32) {
+            const int32_t j = s0 + p;
+            nb_src[to + p] = j;
+            if (pk_xyz) {
+                pk_xyz[to + p] = xs[j];
+                pk_src[to + p] = perm[j];
+            }
         }
-        const int32_t s0 = __shfl_sync(P2P_FULL_MASK, start, seg);
-        const int32_t x0 = __shfl_sync(P2P_FULL_MASK, excl, seg);
-        if (p < total) {
-            const int32_t j = s0 + (p - x0);
-            nb_src[base + p] = j;
-            if (pk_xyz) {
-                pk_xyz[base + p] = xs[j];
-                pk_src[base + p] = perm[j];
-            }
-        } else if (p < padded) {
-            nb_src[base + p] = -1;
-            if (pk_xyz) {
-                pk_xyz[base + p] = make_float4(0.f, 0.f, 0.f, 0.f);
-                pk_src[base + p] = -1;
-            }
+    }
+    if (lane < padded - total) {
+        nb_src[base + total + lane] = -1;
+        if (pk_xyz) {
+            pk_xyz[base + total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            pk_src[base + total + lane] = -1;
         }
     }
 }
@@ -476,9 +576,11 @@ int ceil_log2(int v) {
     return b;
 }
 
+inline int64_t head_blocks(int64_t n) { return (n + kThreads * kHeads - 1) / (kThreads * kHeads); }
+
 struct BinLayout {
     uint64_t *keys, *keys_alt;
-    int32_t *vals, *vals_alt, *head, *ex, *small;
+    int32_t *vals, *vals_alt, *heads, *first, *small;
     void *radix_ws, *scan_ws;
     size_t bytes;
 };
@@ -491,17 +593,50 @@ BinLayout bin_layout(int64_t n, void* work) {
     L.keys_alt = c.take<uint64_t>(m);
     L.vals = c.take<int32_t>(m);
     L.vals_alt = c.take<int32_t>(m);
-    L.head = c.take<int32_t>(m);
-    L.ex = c.take<int32_t>(m);
+    L.heads = c.take<int32_t>((size_t)head_blocks((int64_t)m));
+    L.first = c.take<int32_t>((size_t)head_blocks((int64_t)m));
     L.small = c.take<int32_t>(4);
     L.radix_ws = c.take<char>(radix_workspace_bytes(n));
-    L.scan_ws = c.take<char>(scan_workspace_bytes(n));
+    L.scan_ws = c.take<char>(scan_workspace_bytes(head_blocks((int64_t)m)));
     L.bytes = align_up(c.off, 256);
     return L;
 }
 
+// Morton keys of width K (32 bits hold grids of up to 1024 boxes per axis), their stable sort and the boxes.
+// L.small: [0] non-finite flag, [1] number of boxes.
+template <typename K>
+cudaError_t bin_sorted(const BinLayout& L, const float* pts, int64_t n, const double lo[3], double h, int32_t ng, int bits,
+                       int32_t* perm, int32_t* point_box, int64_t* box_keys, int32_t* box_ptr, cudaStream_t s) {
+    AxisGrid g[3];
+    for (int i = 0; i < 3; ++i) {
+        g[i].lo = lo[i];
+        g[i].h = h;
+        g[i].lo_f = (float)lo[i];
+        g[i].inv_h = (float)(1.0 / h);
+        // grids so small or large that FP32 would flush or overflow keep the double division
+        const bool plain = h > 1e-30 && h < 1e30 && fabs(lo[i]) < 1e30;
+        g[i].slack = plain ? (float)((fabs(lo[i]) / h + 1.0) * 1.2e-7) : INFINITY;
+    }
+    K* keys = reinterpret_cast<K*>(L.keys);
+    K* keys_alt = reinterpret_cast<K*>(L.keys_alt);
+    k_keys<K><<<blocks_for(n, kThreads), kThreads, 0, s>>>(pts, n, g[0], g[1], g[2], ng, keys, L.vals, L.small);
+    cudaError_t e = cudaGetLastError();
+    bool in_alt = false;
+    if (e == cudaSuccess) e = radix_sort_pairs(keys, L.vals, keys_alt, L.vals_alt, n, bits, L.radix_ws, s, &in_alt);
+    if (e != cudaSuccess) return e;
+    const K* ks = in_alt ? keys_alt : keys;
+    const int32_t* vs = in_alt ? L.vals_alt : L.vals;
+    const int64_t blocks = head_blocks(n);
+    k_heads<K><<<(unsigned)blocks, kThreads, 0, s>>>(ks, n, L.heads);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = scan_exclusive_i32(L.heads, L.first, blocks, L.small + 1, L.scan_ws, s);
+    if (e != cudaSuccess) return e;
+    k_rle<K><<<(unsigned)blocks, kThreads, 0, s>>>(ks, vs, L.first, n, perm, point_box, box_keys, box_ptr);
+    return cudaGetLastError();
+}
+
 struct NbrLayout {
-    int32_t *cnt, *src_cnt, *bad;
+    int32_t *cnt, *found, *bad;
     unsigned long long* sum;
     void* scan_ws;
     size_t bytes;
@@ -510,11 +645,11 @@ struct NbrLayout {
 NbrLayout nbr_layout(int32_t nb, void* work) {
     Carver c{static_cast<char*>(work), 0, (size_t)-1};
     NbrLayout L;
-    size_t m = (size_t)(nb > 0 ? nb : 1);
+    const size_t m = (size_t)(nb > 0 ? nb : 1);
     L.cnt = c.take<int32_t>(m);
-    L.src_cnt = c.take<int32_t>(m);
-    L.bad = c.take<int32_t>(2);
-    L.sum = c.take<unsigned long long>(1);
+    L.found = c.take<int32_t>(27 * m);
+    L.sum = c.take<unsigned long long>(4);
+    L.bad = reinterpret_cast<int32_t*>(L.sum + 1);
     L.scan_ws = c.take<char>(scan_workspace_bytes(nb));
     L.bytes = align_up(c.off, 256);
     return L;
@@ -573,11 +708,12 @@ int32_t auto_warp_boxes(int64_t n, int32_t nb) {
 
 struct PlanLayout {
     p2p_plan p;  // pointers only
-    int32_t *n_chunks, *item_off, *padded, *maxes, *small, *list_len, *self_len;
+    int32_t *n_chunks, *item_off, *padded, *maxes, *list_len, *self_len;
+    ListInfo* info;
     void* scan_ws;
     // item-sort scratch (aliases the strength staging buffer when it is large enough)
     ItemRec* recs;
-    uint64_t *keys, *keys_alt;
+    uint32_t *keys, *keys_alt;
     int32_t *vals, *vals_alt;
     void* radix_ws;
     size_t bytes;
@@ -654,21 +790,21 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     L.item_off = c.take<int32_t>(mb + 1);
     L.padded = c.take<int32_t>(mb);
     L.maxes = c.take<int32_t>(4);
-    L.small = c.take<int32_t>(4);
+    L.info = c.take<ListInfo>(1);
     L.scan_ws = c.take<char>(scan_workspace_bytes((int64_t)mx));
     // sort scratch: inside lam_buf if it fits, else after everything else
     Carver sc{reinterpret_cast<char*>(L.p.lam_buf), 0, lam_bytes};
     sc.take<ItemRec>(max_items);
-    sc.take<uint64_t>(max_items);
-    sc.take<uint64_t>(max_items);
+    sc.take<uint32_t>(max_items);
+    sc.take<uint32_t>(max_items);
     sc.take<int32_t>(max_items);
     sc.take<int32_t>(max_items);
     sc.take<char>(radix_workspace_bytes((int64_t)max_items));
     Carver& cs = (sc.off <= lam_bytes) ? sc : c;
     if (&cs == &sc) sc.off = 0;
     L.recs = cs.take<ItemRec>(max_items);
-    L.keys = cs.take<uint64_t>(max_items);
-    L.keys_alt = cs.take<uint64_t>(max_items);
+    L.keys = cs.take<uint32_t>(max_items);
+    L.keys_alt = cs.take<uint32_t>(max_items);
     L.vals = cs.take<int32_t>(max_items);
     L.vals_alt = cs.take<int32_t>(max_items);
     L.radix_ws = cs.take<char>(radix_workspace_bytes((int64_t)max_items));
@@ -765,18 +901,10 @@ P2P_API p2p_status p2p_bin_points(const float* pts, int64_t n, const double lo[3
     if (work_bytes < L.bytes) return P2P_ERR_WORKSPACE;
 
     P2P_TRY_CUDA(cudaMemsetAsync(L.small, 0, 4 * sizeof(int32_t), s), "p2p_bin_points");
-    k_keys<<<blocks_for(n, kThreads), kThreads, 0, s>>>(pts, n, lo[0], lo[1], lo[2], h, ng, L.keys, L.vals, L.small);
-    P2P_CHECK_LAUNCH("p2p_bin_points/keys");
-    bool in_alt = false;
-    P2P_TRY_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, n, 3 * ceil_log2(ng), L.radix_ws, s, &in_alt),
-                 "p2p_bin_points/sort");
-    const uint64_t* ks = in_alt ? L.keys_alt : L.keys;
-    const int32_t* vs = in_alt ? L.vals_alt : L.vals;
-    k_heads<<<blocks_for(n, kThreads), kThreads, 0, s>>>(ks, n, L.head);
-    P2P_CHECK_LAUNCH("p2p_bin_points/heads");
-    P2P_TRY_CUDA(scan_exclusive_i32(L.head, L.ex, n, L.small + 1, L.scan_ws, s), "p2p_bin_points/scan");
-    k_rle<<<blocks_for(n, kThreads), kThreads, 0, s>>>(ks, vs, L.head, L.ex, n, perm, point_box, box_keys, box_ptr);
-    P2P_CHECK_LAUNCH("p2p_bin_points/rle");
+    const int bits = 3 * ceil_log2(ng);
+    const cudaError_t e = bits <= 32 ? bin_sorted<uint32_t>(L, pts, n, lo, h, ng, bits, perm, point_box, box_keys, box_ptr, s)
+                                     : bin_sorted<uint64_t>(L, pts, n, lo, h, ng, bits, perm, point_box, box_keys, box_ptr, s);
+    P2P_TRY_CUDA(e, "p2p_bin_points");
     int32_t host[2] = {0, 0};
     P2P_TRY_CUDA(cudaMemcpyAsync(host, L.small, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s), "p2p_bin_points");
     P2P_TRY_CUDA(cudaStreamSynchronize(s), "p2p_bin_points");
@@ -814,39 +942,34 @@ p2p_status build_neighbors(const int64_t* box_keys, int32_t num_boxes, const int
     if ((int64_t)num_boxes * 27 >= INT32_MAX) return P2P_ERR_UNSUPPORTED;
     NbrLayout L = nbr_layout(num_boxes, work);
     if (work_bytes < L.bytes) return P2P_ERR_WORKSPACE;
-    P2P_TRY_CUDA(cudaMemsetAsync(L.bad, 0, 2 * sizeof(int32_t), s), "p2p_build_neighbors");
-    P2P_TRY_CUDA(cudaMemsetAsync(L.sum, 0, sizeof(unsigned long long), s), "p2p_build_neighbors");
+    // [0] sources, [1] flag of invalid keys, [2] (filled below) list entries
+    P2P_TRY_CUDA(cudaMemsetAsync(L.sum, 0, 4 * sizeof(unsigned long long), s), "p2p_build_neighbors");
     const unsigned wblocks = blocks_for((int64_t)num_boxes * 32, kThreads);
     if (two) {
         if (num_src > 1) {
             k_keys_ascending<<<blocks_for(num_src, kThreads), kThreads, 0, s>>>(src_keys, num_src, L.bad);
             P2P_CHECK_LAUNCH("p2p_build_neighbors_st/keys");
         }
-        k_neighbors<false, true><<<wblocks, kThreads, 0, s>>>(box_keys, num_boxes, src_keys, num_src, src_box_ptr, ng,
-                                                              L.cnt, L.src_cnt, nullptr, nullptr, nullptr, L.bad);
+        k_nbr_find<true><<<wblocks, kThreads, 0, s>>>(box_keys, num_boxes, src_keys, num_src, src_box_ptr, ng, L.cnt,
+                                                      L.found, L.sum, L.bad);
     } else {
-        k_neighbors<false, false><<<wblocks, kThreads, 0, s>>>(box_keys, num_boxes, src_keys, num_src, src_box_ptr, ng,
-                                                               L.cnt, L.src_cnt, nullptr, nullptr, nullptr, L.bad);
+        k_nbr_find<false><<<wblocks, kThreads, 0, s>>>(box_keys, num_boxes, src_keys, num_src, src_box_ptr, ng, L.cnt,
+                                                       L.found, L.sum, L.bad);
     }
-    P2P_CHECK_LAUNCH("p2p_build_neighbors/count");
+    P2P_CHECK_LAUNCH("p2p_build_neighbors/find");
     P2P_TRY_CUDA(scan_exclusive_i32(L.cnt, nbr_ptr, num_boxes, nbr_ptr + num_boxes, L.scan_ws, s),
                  "p2p_build_neighbors/scan");
-    if (two)
-        k_neighbors<true, true><<<wblocks, kThreads, 0, s>>>(box_keys, num_boxes, src_keys, num_src, src_box_ptr, ng,
-                                                             nullptr, nullptr, nbr_ptr, nbr_idx, nbr_self, L.bad);
-    else
-        k_neighbors<true, false><<<wblocks, kThreads, 0, s>>>(box_keys, num_boxes, src_keys, num_src, src_box_ptr, ng,
-                                                              nullptr, nullptr, nbr_ptr, nbr_idx, nullptr, L.bad);
+    if (two) k_nbr_fill<true><<<wblocks, kThreads, 0, s>>>(L.found, num_boxes, nbr_ptr, nbr_idx, nbr_self);
+    else k_nbr_fill<false><<<wblocks, kThreads, 0, s>>>(L.found, num_boxes, nbr_ptr, nbr_idx, nullptr);
     P2P_CHECK_LAUNCH("p2p_build_neighbors/fill");
-    k_sum_i32<<<blocks_for(num_boxes, kThreads), kThreads, 0, s>>>(L.src_cnt, num_boxes, L.sum);
-    P2P_CHECK_LAUNCH("p2p_build_neighbors/sum");
-    int32_t bad = 0, total = 0;
-    unsigned long long src = 0;
-    P2P_TRY_CUDA(cudaMemcpyAsync(&bad, L.bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "p2p_build_neighbors");
-    P2P_TRY_CUDA(cudaMemcpyAsync(&total, nbr_ptr + num_boxes, sizeof(int32_t), cudaMemcpyDeviceToHost, s),
+    P2P_TRY_CUDA(cudaMemcpyAsync(L.sum + 2, nbr_ptr + num_boxes, sizeof(int32_t), cudaMemcpyDeviceToDevice, s),
                  "p2p_build_neighbors");
-    P2P_TRY_CUDA(cudaMemcpyAsync(&src, L.sum, sizeof(src), cudaMemcpyDeviceToHost, s), "p2p_build_neighbors");
+    unsigned long long host[3] = {0, 0, 0};
+    P2P_TRY_CUDA(cudaMemcpyAsync(host, L.sum, sizeof(host), cudaMemcpyDeviceToHost, s), "p2p_build_neighbors");
     P2P_TRY_CUDA(cudaStreamSynchronize(s), "p2p_build_neighbors");
+    const bool bad = (uint32_t)host[1] != 0;
+    const int32_t total = (int32_t)host[2];
+    const unsigned long long src = host[0];
     if (bad) return P2P_ERR_INVALID;
     *nnz = total;
     *sources = (int64_t)src;
@@ -985,23 +1108,33 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
         *plan = p;
         return P2P_OK;
     }
-    FAIL_CUDA(cudaMemsetAsync(L.maxes, 0, 4 * sizeof(int32_t), s), "p2p_plan_create");
     k_gather_xyz<<<blocks_for(n, kThreads), kThreads, 0, s>>>(in.pts, in.perm, n, p->xs);
     FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/gather");
     if (in.two_sets && in.n_src > 0) {
         k_gather_xyz<<<blocks_for(in.n_src, kThreads), kThreads, 0, s>>>(in.src_pts, in.src_perm, in.n_src, p->xs_src);
         FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/gather_sources");
     }
+    // The lists' sizes for every tuning the plan may take, read back once; nothing is built from an invalid CSR.
     const int upper = layout == P2P_LAYOUT_SYMMETRIC;
-    auto box_info = [&]() {
-        k_box_info<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(in.box_ptr, p->src_box_ptr, p->nbs, in.nbr_ptr,
-                                                                 in.nbr_idx, p->nbr_self, nb, in.nnz, t.chunk, upper,
-                                                                 p->box_src, L.list_len, L.n_chunks, L.padded,
-                                                                 L.self_len, L.maxes, p->status);
-        return cudaGetLastError();
-    };
-    FAIL_CUDA(box_info(), "p2p_plan_create/box_info");
-    if (tuning_is_auto(tuning)) {
+    const bool choose = tuning_is_auto(tuning);
+    const p2p_tuning* candidates[3] = {&t, choose ? &kWideTuning : &t, choose ? &kNarrowTuning : &t};
+    FAIL_CUDA(cudaMemsetAsync(L.info, 0, sizeof(ListInfo), s), "p2p_plan_create");
+    k_box_info<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(
+        in.box_ptr, p->src_box_ptr, p->nbs, in.nbr_ptr, in.nbr_idx, p->nbr_self, nb, in.nnz, candidates[0]->chunk,
+        candidates[1]->chunk, candidates[2]->chunk, upper, p->box_src, L.list_len, L.self_len, L.info);
+    FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/box_info");
+    ListInfo info;
+    int sms = 0, dev = 0;
+    FAIL_CUDA(cudaGetDevice(&dev), "p2p_plan_create");
+    FAIL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "p2p_plan_create");
+    FAIL_CUDA(cudaMemcpyAsync(&info, L.info, sizeof(info), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
+    FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
+    if (info.status) {
+        free(p);
+        return P2P_ERR_INVALID;
+    }
+    int which = 0;
+    if (choose) {
         // When most source lists hold just over one default chunk (193 .. 256 sources), every box would get a
         // full item and a short tail item with the same fixed cost; 256-source items (6 warps per block, so two
         // blocks still fit an SM) give those boxes one item each.  When the whole plan has fewer than 2.5 items
@@ -1009,24 +1142,16 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
         // 128-source items spread it (measured on the 32 768-point cube, 8^3 boxes: 3 584 items of 192
         // sources 60.4 us, 5 400 of 128 51.2 us, of 96 52.2 us, of 64 59.4 us).  The workspace is sized for
         // the narrow chunk.
-        int32_t counts[2] = {0, 0};  // tails, items
-        int sms = 0, dev = 0;
-        FAIL_CUDA(cudaGetDevice(&dev), "p2p_plan_create");
-        FAIL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "p2p_plan_create");
-        FAIL_CUDA(cudaMemcpyAsync(counts, L.maxes + 2, sizeof(counts), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
-        FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
-        const p2p_tuning* sw = nullptr;
-        if (2ll * counts[0] > nb) sw = &kWideTuning;
-        else if (2ll * counts[1] < 5ll * 16 * sms) sw = &kNarrowTuning;
-        if (sw) {
-            t.chunk = sw->chunk;
-            t.warps_per_cta = sw->warps_per_cta;
-            p->tune = t;
-            FAIL_CUDA(cudaMemsetAsync(L.maxes, 0, 4 * sizeof(int32_t), s), "p2p_plan_create");
-            FAIL_CUDA(box_info(), "p2p_plan_create/box_info");
-        }
+        if (2ll * info.tails > nb) which = 1;
+        else if (2ll * info.items[0] < 5ll * 16 * sms) which = 2;
+        t.chunk = candidates[which]->chunk;
+        t.warps_per_cta = candidates[which]->warps_per_cta;
+        p->tune = t;
     }
-    FAIL_CUDA(scan_exclusive_i32(L.n_chunks, L.item_off, nb, L.small, L.scan_ws, s), "p2p_plan_create/scan");
+    const int64_t items = info.items[which];
+    k_list_sizes<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(L.list_len, nb, t.chunk, L.n_chunks, L.padded);
+    FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/sizes");
+    FAIL_CUDA(scan_exclusive_i32(L.n_chunks, L.item_off, nb, nullptr, L.scan_ws, s), "p2p_plan_create/scan");
     FAIL_CUDA(scan_exclusive_i32(L.padded, p->pk_off, nb, p->pk_off + nb, L.scan_ws, s),
               "p2p_plan_create/scan_lists");
     k_pack<<<blocks_for((int64_t)nb * 32, kThreads), kThreads, 0, s>>>(p->xs_src, p->src_perm, p->src_box_ptr,
@@ -1048,30 +1173,13 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
                                                                  L.self_len, p->pk_off, nb, t.chunk, t.target_group,
                                                                  p->two_sets, L.recs, L.keys, L.vals);
     FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/items");
-    int32_t host[4] = {0, 0, 0, 0};
-    unsigned int status = 0;
-    int32_t packed = 0;
-    FAIL_CUDA(cudaMemcpyAsync(host, L.maxes, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
-    FAIL_CUDA(cudaMemcpyAsync(host + 2, L.small, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
-    FAIL_CUDA(cudaMemcpyAsync(&status, p->status, sizeof(status), cudaMemcpyDeviceToHost, s), "p2p_plan_create");
-    FAIL_CUDA(cudaMemcpyAsync(&packed, p->pk_off + nb, sizeof(int32_t), cudaMemcpyDeviceToHost, s),
-              "p2p_plan_create");
-    FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
-    if (!status) {
-        const int64_t items = host[2];
+    if (items > 0) {
         bool in_alt = false;
-        FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, items, 32, L.radix_ws, s, &in_alt),
+        FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, items, kCostBits, L.radix_ws, s, &in_alt),
                   "p2p_plan_create/sort");
-        if (items > 0) {
-            k_item_gather<<<blocks_for(items, kThreads), kThreads, 0, s>>>(L.recs, in_alt ? L.vals_alt : L.vals,
-                                                                           items, p->items);
-            FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/order");
-        }
-        FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
-    }
-    if (status) {
-        free(p);
-        return P2P_ERR_INVALID;
+        k_item_gather<<<blocks_for(items, kThreads), kThreads, 0, s>>>(L.recs, in_alt ? L.vals_alt : L.vals, items,
+                                                                       p->items);
+        FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/order");
     }
     if (p->tc_pack)  // n_chunks and padded are free once the items are built
         FAIL_CUDA(p2p_tc_build(p, L.n_chunks, L.padded, L.scan_ws, s), "p2p_plan_create/tc_lists");
@@ -1086,12 +1194,11 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
                                                                          nb, 32 / wb, L.recs, L.keys, L.vals);
             FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/direct_items");
             bool in_alt = false;
-            FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, nb, 32, L.radix_ws, s, &in_alt),
+            FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, nb, kFineCostBits, L.radix_ws, s, &in_alt),
                       "p2p_plan_create/direct_sort");
             k_item_gather<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(L.recs, in_alt ? L.vals_alt : L.vals, nb,
                                                                         p->ditems);
             FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/direct_order");
-            FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
         }
     } else {
         p->tune.warp_boxes = -1;
@@ -1103,12 +1210,16 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     p->group_cap = 0;
     p->group_pos_cap = 0;
     if (p->tune.warp_boxes == -2 && (layout != P2P_LAYOUT_INDEXED || nb == 0)) p->tune.warp_boxes = -1;
+    int32_t cap[2] = {0, 0};
     if (p->tune.warp_boxes == -2) {
         p->n_groups = (nb + kGroupBoxes - 1) / kGroupBoxes;
-        int32_t cap[2] = {0, 0};
         FAIL_CUDA(p2p_group_build(p, in.nbr_ptr, in.nbr_idx, L.keys, L.vals, L.keys_alt, L.vals_alt, L.radix_ws,
                                   L.maxes, s, cap),
                   "p2p_plan_create/groups");
+    }
+    // the plan is complete when this returns: later calls may use it on any stream
+    FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
+    if (p->tune.warp_boxes == -2) {
         if (cap[0] > 0 && cap[0] <= kGroupCapMax) {
             p->group_k = 1;
             p->group_cap = (cap[0] + 3) & ~3;
@@ -1117,10 +1228,10 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
             p->tune.warp_boxes = -1;
         }
     }
-    p->max_chunks = host[0];
-    p->max_box = host[1];
-    p->n_items = host[2];
-    p->packed = packed;
+    p->max_chunks = (int32_t)(((int64_t)info.max_len + t.chunk - 1) / t.chunk);
+    p->max_box = info.max_box;
+    p->n_items = items;
+    p->packed = info.packed;
     FAIL_CUDA(p2p_pair_configure(p), "p2p_plan_create/occupancy");
 #undef FAIL_CUDA
     *plan = p;

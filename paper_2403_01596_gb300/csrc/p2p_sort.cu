@@ -74,73 +74,130 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const int32_t* __res
     if (total_dev && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total_dev = off + total;
 }
 
+// Radix sort: per pass a histogram of every tile (k_radix_hist), an exclusive scan along each digit's row of tiles
+// (k_radix_rows) and the scatter, which adds the digits' totals itself.  Tiles shrink with n so that a few hundred
+// blocks work on small inputs as well (at 96 000 keys 24 tiles of 4 096 left most SMs idle).  Latency bound on plans of
+// ordinary size; measured on one GB300 at 70 637 points: a pass 9.5 us (18 us with a three-launch scan of all
+// counts and tiles of 4 096 keys ranked 256 at a time).
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortSub = 16;                           // sub-chunks of 256 keys per tile
-constexpr int kSortTile = kSortThreads * kSortSub;     // 4096 keys per block
+constexpr int kMaxSub = 16;  // keys per thread at most
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                             uint32_t mask, int32_t* __restrict__ hist, int tiles) {
+__host__ __device__ inline int sort_sub(int64_t n) { return n <= (1 << 18) ? 4 : (n <= (1 << 22) ? 8 : kMaxSub); }
+__host__ __device__ inline int64_t sort_tiles(int64_t n) {
+    const int64_t tile = (int64_t)kSortThreads * sort_sub(n);
+    return n > 0 ? (n + tile - 1) / tile : 1;
+}
+
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const K* __restrict__ keys, int64_t n, int sub, int shift,
+                                                             uint32_t mask, int32_t* __restrict__ hist, int64_t tiles) {
     __shared__ int cnt[kRadix];
     for (int d = threadIdx.x; d < kRadix; d += kSortThreads) cnt[d] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    for (int i = threadIdx.x; i < kSortTile; i += kSortThreads) {
-        int64_t idx = base + i;
+    const int64_t base = (int64_t)blockIdx.x * kSortThreads * sub;
+    for (int c = 0; c < sub; ++c) {
+        const int64_t idx = base + (int64_t)c * kSortThreads + threadIdx.x;
         if (idx < n) atomicAdd(&cnt[(uint32_t)(keys[idx] >> shift) & mask], 1);
     }
     __syncthreads();
     for (int d = threadIdx.x; d < kRadix; d += kSortThreads) hist[(int64_t)d * tiles + blockIdx.x] = cnt[d];
 }
 
-// Stable scatter: within a tile, keys are ranked in index order sub-chunk by
-// sub-chunk; inside a sub-chunk the rank among equal digits comes from the
-// warp match mask (lanes) and a per-digit prefix over warps.
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const uint64_t* __restrict__ keys_in,
-                                                                const int32_t* __restrict__ vals_in,
-                                                                uint64_t* __restrict__ keys_out,
-                                                                int32_t* __restrict__ vals_out, int64_t n, int shift,
-                                                                uint32_t mask, const int32_t* __restrict__ hist_off,
-                                                                int tiles) {
-    __shared__ int base[kRadix];
-    __shared__ int warp_cnt[kSortWarps][kRadix];
-    __shared__ int warp_base[kSortWarps][kRadix];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int d = tid; d < kRadix; d += kSortThreads) {
-        base[d] = hist_off[(int64_t)d * tiles + blockIdx.x];
-        for (int w = 0; w < kSortWarps; ++w) warp_cnt[w][d] = 0;
+// Exclusive scan of one value per thread over a block of kSortThreads; total: the block's sum.
+__device__ __forceinline__ int sort_block_scan(int v, int* warp_sum, int& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(P2P_FULL_MASK, x, o);
+        if (lane >= o) x += y;
     }
+    __syncthreads();  // an earlier scan's sums have been read
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+        before += w < warp ? warp_sum[w] : 0;
+        all += warp_sum[w];
+    }
+    total = all;
+    return before + x - v;
+}
+
+// Block d: digit d's counts over the tiles become exclusive prefixes, their sum totals[d].
+__global__ void __launch_bounds__(kSortThreads) k_radix_rows(int32_t* __restrict__ hist, int64_t tiles,
+                                                             int32_t* __restrict__ totals) {
+    __shared__ int warp_sum[kSortWarps];
+    int32_t* row = hist + (int64_t)blockIdx.x * tiles;
+    int run = 0;
+    for (int64_t t0 = 0; t0 < tiles; t0 += kSortThreads) {
+        const int64_t t = t0 + threadIdx.x;
+        const int v = t < tiles ? row[t] : 0;
+        int total;
+        const int pre = sort_block_scan(v, warp_sum, total);
+        if (t < tiles) row[t] = run + pre;
+        run += total;
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = run;
+}
+
+// Stable scatter.  Warp w of a tile owns 32 sub consecutive keys and ranks them in order: the lanes of a round by
+// their match mask, the rounds by the warp's running count of every digit; the warps' counts are scanned once.
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K* __restrict__ keys_in,
+                                                                const int32_t* __restrict__ vals_in,
+                                                                K* __restrict__ keys_out, int32_t* __restrict__ vals_out,
+                                                                int64_t n, int sub, int shift, uint32_t mask,
+                                                                const int32_t* __restrict__ hist,
+                                                                const int32_t* __restrict__ totals, int64_t tiles) {
+    __shared__ int cnt[kSortWarps][kRadix];
+    __shared__ int warp_sum[kSortWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int w = 0; w < kSortWarps; ++w) cnt[w][tid] = 0;
+    int unused;
+    const int base = sort_block_scan(totals[tid], warp_sum, unused) + hist[(int64_t)tid * tiles + blockIdx.x];
     __syncthreads();
     const unsigned lt_mask = (1u << lane) - 1u;
-    const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
-    for (int c = 0; c < kSortSub; ++c) {
-        const int64_t idx = tile0 + (int64_t)c * kSortThreads + tid;
-        const bool valid = idx < n;
-        uint64_t key = valid ? keys_in[idx] : 0ull;
-        int32_t val = valid ? vals_in[idx] : 0;
-        const int d = valid ? (int)((uint32_t)(key >> shift) & mask) : kRadix;  // kRadix = sentinel
-        const unsigned peers = __match_any_sync(P2P_FULL_MASK, d);
-        const int rank = __popc(peers & lt_mask);
-        const bool leader = (__ffs(peers) - 1) == lane;
-        if (valid && leader) warp_cnt[warp][d] = __popc(peers);
-        __syncthreads();
-        for (int dd = tid; dd < kRadix; dd += kSortThreads) {
-            int run = base[dd];
-            for (int w = 0; w < kSortWarps; ++w) {
-                int cnt = warp_cnt[w][dd];
-                warp_base[w][dd] = run;
-                warp_cnt[w][dd] = 0;
-                run += cnt;
-            }
-            base[dd] = run;
+    const int64_t first = (int64_t)blockIdx.x * kSortThreads * sub + (int64_t)warp * 32 * sub + lane;
+    K key[kMaxSub];
+    int rank[kMaxSub];
+#pragma unroll
+    for (int c = 0; c < kMaxSub; ++c) {
+        if (c < sub) {
+            const int64_t idx = first + (int64_t)c * 32;
+            const bool valid = idx < n;
+            key[c] = valid ? keys_in[idx] : (K)0;
+            const int d = valid ? (int)((uint32_t)(key[c] >> shift) & mask) : kRadix;  // kRadix: no key
+            const unsigned peers = __match_any_sync(P2P_FULL_MASK, d);
+            const int before = valid ? cnt[warp][d] : 0;
+            rank[c] = before + __popc(peers & lt_mask);
+            __syncwarp();
+            if (valid && (__ffs(peers) - 1) == lane) cnt[warp][d] = before + __popc(peers);
+            __syncwarp();
         }
-        __syncthreads();
-        if (valid) {
-            const int dst = warp_base[warp][d] + rank;
-            keys_out[dst] = key;
-            vals_out[dst] = val;
+    }
+    __syncthreads();
+    int run = base;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+        const int c = cnt[w][tid];
+        cnt[w][tid] = run;
+        run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kMaxSub; ++c) {
+        if (c < sub) {
+            const int64_t idx = first + (int64_t)c * 32;
+            if (idx < n) {
+                const int dst = cnt[warp][(uint32_t)(key[c] >> shift) & mask] + rank[c];
+                keys_out[dst] = key[c];
+                vals_out[dst] = vals_in[idx];
+            }
         }
     }
 }
@@ -178,36 +235,30 @@ cudaError_t scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32
 }
 
 size_t radix_workspace_bytes(int64_t n) {
-    int64_t tiles = (n + kSortTile - 1) / kSortTile;
-    if (tiles < 1) tiles = 1;
-    size_t h = align_up((size_t)tiles * kRadix * 4, 256);
-    return 2 * h + scan_workspace_bytes(tiles * kRadix);
+    return align_up((size_t)sort_tiles(n) * kRadix * 4, 256) + kRadix * 4;
 }
 
-cudaError_t radix_sort_pairs(uint64_t* keys, int32_t* vals, uint64_t* keys_alt, int32_t* vals_alt, int64_t n,
-                             int bits, void* work, cudaStream_t s, bool* result_in_alt) {
+template <typename K>
+cudaError_t radix_sort_pairs(K* keys, int32_t* vals, K* keys_alt, int32_t* vals_alt, int64_t n, int bits, void* work,
+                             cudaStream_t s, bool* result_in_alt) {
     *result_in_alt = false;
     if (n <= 1 || bits <= 0) return cudaSuccess;
-    const int tiles = (int)((n + kSortTile - 1) / kSortTile);
-    char* w = static_cast<char*>(work);
-    const size_t h = align_up((size_t)tiles * kRadix * 4, 256);
-    int32_t* hist = reinterpret_cast<int32_t*>(w);
-    int32_t* hist_off = reinterpret_cast<int32_t*>(w + h);
-    void* scan_work = w + 2 * h;
-    uint64_t *kin = keys, *kout = keys_alt;
+    const int64_t tiles = sort_tiles(n);
+    const int sub = sort_sub(n);
+    int32_t* hist = static_cast<int32_t*>(work);
+    int32_t* totals = reinterpret_cast<int32_t*>(static_cast<char*>(work) + align_up((size_t)tiles * kRadix * 4, 256));
+    K *kin = keys, *kout = keys_alt;
     int32_t *vin = vals, *vout = vals_alt;
-    for (int shift = 0; shift < bits; shift += kRadixBits) {
-        const int pass_bits = bits - shift < kRadixBits ? bits - shift : kRadixBits;
-        const uint32_t mask = (1u << pass_bits) - 1u;
-        k_radix_hist<<<tiles, kSortThreads, 0, s>>>(kin, n, shift, mask, hist, tiles);
-        cudaError_t e = cudaGetLastError();
+    const int passes = (bits + kRadixBits - 1) / kRadixBits, pass_bits = (bits + passes - 1) / passes;
+    for (int shift = 0; shift < bits; shift += pass_bits) {
+        const uint32_t mask = (1u << (bits - shift < pass_bits ? bits - shift : pass_bits)) - 1u;
+        k_radix_hist<K><<<(unsigned)tiles, kSortThreads, 0, s>>>(kin, n, sub, shift, mask, hist, tiles);
+        k_radix_rows<<<kRadix, kSortThreads, 0, s>>>(hist, tiles, totals);
+        k_radix_scatter<K><<<(unsigned)tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, sub, shift, mask, hist, totals,
+                                                                    tiles);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = scan_exclusive_i32(hist, hist_off, (int64_t)tiles * kRadix, nullptr, scan_work, s);
-        if (e != cudaSuccess) return e;
-        k_radix_scatter<<<tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, mask, hist_off, tiles);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        uint64_t* tk = kin;
+        K* tk = kin;
         kin = kout;
         kout = tk;
         int32_t* tv = vin;
@@ -217,5 +268,10 @@ cudaError_t radix_sort_pairs(uint64_t* keys, int32_t* vals, uint64_t* keys_alt, 
     }
     return cudaSuccess;
 }
+
+template cudaError_t radix_sort_pairs<uint64_t>(uint64_t*, int32_t*, uint64_t*, int32_t*, int64_t, int, void*,
+                                                cudaStream_t, bool*);
+template cudaError_t radix_sort_pairs<uint32_t>(uint32_t*, int32_t*, uint32_t*, int32_t*, int64_t, int, void*,
+                                                cudaStream_t, bool*);
 
 }  // namespace p2p_detail
