@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(kBuildThreads)
 }
 
 struct GroupArgs {
+    p2p_detail::GroupOut o; // results (first: a batch's staging kernel writes them per apply)
     const int32_t* order;   // groups, heaviest first
     int32_t n_groups;
     int32_t nb;
@@ -254,8 +255,6 @@ struct GroupArgs {
     const float4* xt;       // box-sorted target coordinates
     const float2* lam;      // staged strengths, box-sorted source order
     const int32_t* perm;
-    float2* out;
-    int64_t ld;
     float k;
 };
 
@@ -362,8 +361,8 @@ __device__ __forceinline__ void member_pass(const GroupArgs& a, const float4* __
             v.x += w.x;
             v.y += w.y;
         }
-        const int64_t row = (int64_t)(t == lane ? perm0 : __ldg(a.perm + tb + t)) * a.ld;
-        a.out[row] = make_float2(v.x * kInv4Pi, v.y * kInv4Pi);
+        const int64_t row = (int64_t)(t == lane ? perm0 : __ldg(a.perm + tb + t)) * a.o.ld;
+        a.o.out[row] = make_float2(v.x * kInv4Pi, v.y * kInv4Pi);
     }
     __syncwarp();
 }
@@ -446,59 +445,136 @@ __device__ __forceinline__ void prefetch_copies(const GroupArgs& a, int32_t g, i
     cp_async_commit();
 }
 
-// Block = one group at a time: warp w takes the group's w-th costliest member, then further members from a
-// shared counter as it finishes.
+// One group of a block: warp w takes the group's w-th costliest member, then further members from a shared counter.
+// `top` and `a` are the same arguments; a may be read only after the first barrier (a batch fills it meanwhile).
+// prefetch(): starts the copies of the next group's copy list.
+template <int KERN, typename Prefetch>
+__device__ __forceinline__ void sweep_group(const GroupArgs& top, const GroupArgs& a, int32_t g, const GroupSmem& sm,
+                                            Prefetch prefetch) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2* red = sm.red + warp * kMaxTT * 32;
+    const int nu = __ldg(top.g_nunion + g);
+    const int32_t b0 = g * kGroupBoxes;
+    const int nm = min(top.nb - b0, kGroupBoxes);
+    const int32_t* order = top.g_morder + (int64_t)g * kGroupBoxes;
+    const int32_t pos0 = __ldg(top.pk_off + b0), npos = __ldg(top.pk_off + b0 + nm) - pos0;
+    // this group's copy list has arrived, and every warp has finished the previous group
+    cp_async_wait<0>();
+    __syncthreads();
+    // the union: one warp per union box, its sources contiguous in the buffer; the members' position lists
+    // contiguous from the group's first list (every list padded to 4 entries, so 8-byte copies)
+    for (int u = warp; u < nu; u += kGroupWarps) {
+        const int4 c = sm.ents[u];
+        for (int e = lane; e < c.z; e += 32) {
+            cp_async16(sm.sx + c.y + e, a.xs + c.x + e);
+            cp_async8(sm.sl + c.y + e, a.lam + c.x + e);
+        }
+    }
+    for (int e = threadIdx.x; e < npos / 4; e += kGroupWarps * 32)
+        cp_async8(sm.pos + 4 * e, a.g_pos + pos0 + 4 * e);
+    cp_async_commit();
+    // this warp's first member, loaded while the union is staged
+    Member m;
+    const bool has = warp < nm;
+    if (has) load_member(a, b0 + __ldg(order + warp), lane, m);
+    if (threadIdx.x == 0) *sm.next = kGroupWarps;
+    cp_async_wait<0>();
+    __syncthreads();
+    // the next group's copy list, in flight while this group is swept
+    prefetch();
+    if (has) {
+        sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
+        while (true) {
+            int idx = 0;
+            if (lane == 0) idx = atomicAdd(sm.next, 1);
+            idx = __shfl_sync(P2P_FULL_MASK, idx, 0);
+            if (idx >= nm) break;
+            load_member(a, b0 + __ldg(order + idx), lane, m);
+            sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
+        }
+    }
+}
+
 template <int KERN>
 __global__ void __launch_bounds__(kGroupWarps * 32, P2P_GROUP_MIN_BLOCKS) k_pair_group(const __grid_constant__ GroupArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const GroupSmem sm = group_smem(smem, a.cap, a.pos_cap);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* red = sm.red + warp * kMaxTT * 32;
     // the first group's union copies, read ahead into shared memory like every later group's
     if (blockIdx.x < a.n_groups) prefetch_copies(a, __ldg(a.order + blockIdx.x), sm.ents);
     for (int64_t gi = blockIdx.x; gi < a.n_groups; gi += gridDim.x) {
-        const int32_t g = __ldg(a.order + gi);
-        const int nu = __ldg(a.g_nunion + g);
-        const int32_t b0 = g * kGroupBoxes;
-        const int nm = min(a.nb - b0, kGroupBoxes);
-        const int32_t* order = a.g_morder + (int64_t)g * kGroupBoxes;
-        const int32_t pos0 = __ldg(a.pk_off + b0), npos = __ldg(a.pk_off + b0 + nm) - pos0;
-        // this group's copy list has arrived, and every warp has finished the previous group
-        cp_async_wait<0>();
-        __syncthreads();
-        // the union: one warp per union box, its sources contiguous in the buffer; the members' position lists
-        // contiguous from the group's first list (every list padded to 4 entries, so 8-byte copies)
-        for (int u = warp; u < nu; u += kGroupWarps) {
-            const int4 c = sm.ents[u];
-            for (int e = lane; e < c.z; e += 32) {
-                cp_async16(sm.sx + c.y + e, a.xs + c.x + e);
-                cp_async8(sm.sl + c.y + e, a.lam + c.x + e);
-            }
-        }
-        for (int e = threadIdx.x; e < npos / 4; e += kGroupWarps * 32)
-            cp_async8(sm.pos + 4 * e, a.g_pos + pos0 + 4 * e);
-        cp_async_commit();
-        // this warp's first member, loaded while the union is staged
-        Member m;
-        const bool has = warp < nm;
-        if (has) load_member(a, b0 + __ldg(order + warp), lane, m);
-        if (threadIdx.x == 0) *sm.next = kGroupWarps;
-        cp_async_wait<0>();
-        __syncthreads();
-        // the next group's copy list, in flight while this group is swept
-        if (gi + gridDim.x < a.n_groups) prefetch_copies(a, __ldg(a.order + gi + gridDim.x), sm.ents);
-        if (has) {
-            sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
-            while (true) {
-                int idx = 0;
-                if (lane == 0) idx = atomicAdd(sm.next, 1);
-                idx = __shfl_sync(P2P_FULL_MASK, idx, 0);
-                if (idx >= nm) break;
-                load_member(a, b0 + __ldg(order + idx), lane, m);
-                sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
-            }
-        }
+        sweep_group<KERN>(a, a, __ldg(a.order + gi), sm, [&]() {
+            if (gi + gridDim.x < a.n_groups) prefetch_copies(a, __ldg(a.order + gi + gridDim.x), sm.ents);
+        });
     }
+}
+
+// The groups of several plans in one persistent launch: order holds (plan, group), plan after plan, each plan's
+// heaviest first.  A group's arguments are copied into shared memory while the group before is swept.
+template <int KERN>
+__global__ void __launch_bounds__(kGroupWarps * 32, P2P_GROUP_MIN_BLOCKS)
+    k_pair_group_batched(const GroupArgs* __restrict__ geoms, const int2* __restrict__ order, int32_t total, int32_t cap,
+                         int32_t pos_cap) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ GroupArgs args[2];
+    const GroupSmem sm = group_smem(smem, cap, pos_cap);
+    static_assert(sizeof(GroupArgs) % 8 == 0 && sizeof(GroupArgs) / 8 <= kGroupWarps * 32, "one copy step");
+    auto fetch = [&](const int2 e, int to) {
+        if (threadIdx.x < sizeof(GroupArgs) / 8)
+            reinterpret_cast<uint64_t*>(&args[to])[threadIdx.x] = reinterpret_cast<const uint64_t*>(geoms + e.x)[threadIdx.x];
+        prefetch_copies(geoms[e.x], e.y, sm.ents);
+    };
+    if (blockIdx.x >= total) return;
+    int2 e = __ldg(order + blockIdx.x);
+    fetch(e, 0);
+    int cur = 0;
+    for (int64_t gi = blockIdx.x; gi < total; gi += gridDim.x) {
+        const bool more = gi + gridDim.x < total;
+        const int2 en = more ? __ldg(order + gi + gridDim.x) : e;
+        sweep_group<KERN>(geoms[e.x], args[cur], e.y, sm, [&]() {
+            if (more) fetch(en, cur ^ 1);
+        });
+        e = en;
+        cur ^= 1;
+    }
+}
+
+// (plan, group) of every position: off[g] is plan g's first.
+struct GroupOffsets {
+    int32_t off[kMaxBatchPlans + 1];
+    int32_t count;
+};
+__global__ void k_group_order(const GroupArgs* __restrict__ geoms, const GroupOffsets o, int2* __restrict__ order) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= o.off[o.count]) return;
+    int g = 0;
+    while (g + 1 < o.count && o.off[g + 1] <= i) ++g;
+    order[i] = make_int2(g, geoms[g].order[i - o.off[g]]);
+}
+
+GroupArgs group_args(const p2p_plan* p) {
+    GroupArgs a{};
+    a.order = p->g_order;
+    a.n_groups = p->n_groups;
+    a.nb = p->nb;
+    a.cap = p->group_cap;
+    a.pos_cap = p->group_pos_cap;
+    a.g_union = p->g_union;
+    a.g_nunion = p->g_nunion;
+    a.g_pos = p->g_pos;
+    a.g_mend = p->g_mend;
+    a.g_map = p->g_map;
+    a.g_morder = p->g_morder;
+    a.g_copy = p->g_copy;
+    a.pk_off = p->pk_off;
+    a.box_ptr = p->box_ptr;
+    a.box_src = p->box_src;
+    a.src_box_ptr = p->src_box_ptr;
+    a.xs = p->xs_src;
+    a.xt = p->xs;
+    a.lam = p->lam_buf;
+    a.perm = p->perm;
+    a.k = p->k;
+    return a;
 }
 
 }  // namespace
@@ -549,29 +625,9 @@ cudaError_t p2p_group_configure(p2p_plan* p) {
 
 // Apply: one right-hand side from the staged strengths (box-sorted source order) into out.
 p2p_status p2p_group_launch(const p2p_plan* p, float2* out, int64_t ld, float k, cudaStream_t s) {
-    GroupArgs a;
-    a.order = p->g_order;
-    a.n_groups = p->n_groups;
-    a.nb = p->nb;
-    a.cap = p->group_cap;
-    a.pos_cap = p->group_pos_cap;
-    a.g_union = p->g_union;
-    a.g_nunion = p->g_nunion;
-    a.g_pos = p->g_pos;
-    a.g_mend = p->g_mend;
-    a.g_map = p->g_map;
-    a.g_morder = p->g_morder;
-    a.g_copy = p->g_copy;
-    a.pk_off = p->pk_off;
-    a.box_ptr = p->box_ptr;
-    a.box_src = p->box_src;
-    a.src_box_ptr = p->src_box_ptr;
-    a.xs = p->xs_src;
-    a.xt = p->xs;
-    a.lam = p->lam_buf;
-    a.perm = p->perm;
-    a.out = out;
-    a.ld = ld;
+    GroupArgs a = group_args(p);
+    a.o.out = out;
+    a.o.ld = ld;
     a.k = k;
     const size_t smem = group_smem_bytes(p->group_cap, p->group_pos_cap);
     auto kern = p->kernel == P2P_LAPLACE ? k_pair_group<P2P_LAPLACE> : k_pair_group<P2P_HELMHOLTZ>;
@@ -579,5 +635,78 @@ p2p_status p2p_group_launch(const p2p_plan* p, float2* out, int64_t ld, float k,
     const int grid = (int)std::min<int64_t>(p->group_grid, p->n_groups);
     kern<<<grid, kGroupWarps * 32, smem, s>>>(a);
     P2P_CHECK_LAUNCH("p2p_apply/group");
+    return P2P_OK;
+}
+
+// ---------------------------------------------------------------- batches --
+
+// Whether a batch of these plans runs its one right-hand side through the box-group kernel: every plan does so by
+// itself, with one kernel function, and the largest of their buffers still fits three blocks per SM's shared memory
+// as the plans' own do (the launch takes one size for all).
+bool p2p_group_batch_possible(const p2p_plan* const* plans, int32_t count, int32_t nrhs) {
+    if (nrhs != 1 || count > kMaxBatchPlans) return false;
+    for (int g = 0; g < count; ++g)
+        if (!plans[g]->group_k || plans[g]->group_grid <= 0 || plans[g]->kernel != plans[0]->kernel) return false;
+    return true;
+}
+
+size_t p2p_group_batch_bytes(const p2p_plan* const* plans, int32_t count) {
+    int64_t total = 0;
+    for (int g = 0; g < count; ++g) total += plans[g]->n_groups;
+    return align_up(sizeof(GroupArgs) * kMaxBatchPlans, 256) + align_up((size_t)total * sizeof(int2), 256);
+}
+
+// Fills b from workspace ws (p2p_group_batch_bytes, 256-byte aligned); b->grid is 0 where no block fits.  The copy
+// from `host` is complete when the stream has come this far: the caller synchronises before the arguments leave scope.
+cudaError_t p2p_group_batch_create(p2p_group_batch* b, const p2p_plan* const* plans, int32_t count, void* ws,
+                                   cudaStream_t s) {
+    GroupArgs host[kMaxBatchPlans];
+    GroupOffsets o{};
+    o.count = count;
+    int32_t cap = 0, pos_cap = 0;
+    for (int g = 0; g < count; ++g) {
+        host[g] = group_args(plans[g]);
+        o.off[g + 1] = o.off[g] + plans[g]->n_groups;
+        cap = std::max(cap, plans[g]->group_cap);
+        pos_cap = std::max(pos_cap, plans[g]->group_pos_cap);
+    }
+    GroupArgs* geoms = static_cast<GroupArgs*>(ws);
+    int2* order = reinterpret_cast<int2*>(static_cast<char*>(ws) + align_up(sizeof(GroupArgs) * kMaxBatchPlans, 256));
+    b->geoms = reinterpret_cast<unsigned char*>(geoms);
+    b->geom_bytes = sizeof(GroupArgs);
+    b->order = order;
+    b->total = o.off[count];
+    b->cap = cap;
+    b->pos_cap = pos_cap;
+    b->kernel = plans[0]->kernel;
+    b->smem = group_smem_bytes(cap, pos_cap);
+    b->grid = 0;
+    int dev = 0, sms = 0, optin = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    auto kern = b->kernel == P2P_LAPLACE ? k_pair_group_batched<P2P_LAPLACE> : k_pair_group_batched<P2P_HELMHOLTZ>;
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return e;
+    if (b->smem + fa.sharedSizeBytes > (size_t)optin) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGroupWarps * 32, b->smem);
+    if (e != cudaSuccess || per_sm == 0) return e;
+    e = cudaMemcpyAsync(geoms, host, sizeof(GroupArgs) * count, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+    k_group_order<<<(unsigned)((b->total + 255) / 256), 256, 0, s>>>(geoms, o, order);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) b->grid = std::min(per_sm * sms, b->total);
+    return e;
+}
+
+p2p_status p2p_group_batch_launch(const p2p_group_batch* b, cudaStream_t s) {
+    auto kern = b->kernel == P2P_LAPLACE ? k_pair_group_batched<P2P_LAPLACE> : k_pair_group_batched<P2P_HELMHOLTZ>;
+    kern<<<b->grid, kGroupWarps * 32, b->smem, s>>>(reinterpret_cast<const GroupArgs*>(b->geoms),
+                                                    static_cast<const int2*>(b->order), b->total, b->cap, b->pos_cap);
+    P2P_CHECK_LAUNCH("p2p_batch_apply/group");
     return P2P_OK;
 }

@@ -163,6 +163,14 @@ namespace p2p_detail {
 #endif
 constexpr int kGroupBoxes = P2P_GROUP_BOXES;
 
+// Results of a box-group launch: leading dimension ld.
+struct GroupOut {
+    float2* out;
+    int64_t ld;
+};
+
+constexpr int kMaxBatchPlans = 16;
+
 // thread-local message of the last CUDA failure
 void set_cuda_error(cudaError_t e, const char* where);
 void set_message(const char* msg);
@@ -210,6 +218,20 @@ __device__ __forceinline__ uint32_t cost_key(int64_t cost) {
 }
 
 }  // namespace p2p_detail
+
+// Box groups of several plans in one launch (p2p_group.cu); geoms holds one argument block per plan, geom_bytes
+// apart, each starting with its GroupOut.
+struct p2p_group_batch {
+    unsigned char* geoms;
+    size_t geom_bytes, smem;
+    void* order;
+    int32_t total, cap, pos_cap, kernel, grid;  // grid 0: not used
+};
+bool p2p_group_batch_possible(const p2p_plan* const* plans, int32_t count, int32_t nrhs);
+size_t p2p_group_batch_bytes(const p2p_plan* const* plans, int32_t count);
+cudaError_t p2p_group_batch_create(p2p_group_batch* b, const p2p_plan* const* plans, int32_t count, void* ws,
+                                   cudaStream_t s);
+p2p_status p2p_group_batch_launch(const p2p_group_batch* b, cudaStream_t s);
 
 // Persistent grid sizes of the pair kernel for the plan's kernel, layout and
 // tuning (resident blocks per SM x SMs), one per right-hand-side block width.

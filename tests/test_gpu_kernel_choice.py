@@ -1,0 +1,72 @@
+"""The kernel a plan chooses for one right-hand side, at box counts on both sides of every line of the choice, and the
+batched box-group launch: results against the staged pipeline on the same plan data.
+
+Tolerance: both evaluate the same FP32 terms in another order; each is within 2^-20 S_i of the exact sum, so they
+differ by at most 2^-19 S_i, S_i = sum_j |G(r_ij) lambda_j| (the Laplace apply of |lambda|)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2403_01596_gb300 import workloads as W  # noqa: E402
+
+
+def _api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_01596_gb300 import api
+    return api
+
+
+def _close(api, plan, pts, lo, h, ng, lam, out):
+    ref = api.Plan(pts, lo, h, ng, plan.k, kernel=plan.kernel, tuning={"warp_boxes": -1}).apply(lam)
+    S = api.Plan(pts, lo, h, ng, kernel="laplace", tuning={"warp_boxes": -1}).apply(lam.abs().to(torch.complex64)).real
+    return bool(((out - ref).abs() <= 2.0 ** -19 * S + 1e-30).all())
+
+
+# points in the unit cube, boxes per axis (all of them occupied or nearly): box counts around 2 500, 6 000, 15 000 and
+# 45 000 at 1 to 30 points per box
+@pytest.mark.parametrize("n,ng", [(1500, 12), (2900, 14), (6000, 13), (6500, 14), (13000, 14), (22000, 13), (24000, 14),
+                                  (31000, 14), (50000, 14), (110000, 18), (125000, 19), (40000, 24), (43000, 25),
+                                  (100000, 24), (106000, 25), (270000, 35), (290000, 36), (200000, 14)])
+@pytest.mark.parametrize("kernel", ["helmholtz", "laplace"])
+@pytest.mark.parametrize("layout", ["indexed", "redundant"])
+def test_choice(n, ng, kernel, layout):
+    api = _api()
+    pts = torch.rand(n, 3, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")
+    lo, h = (0.0, 0.0, 0.0), 1.0 / ng
+    lam = torch.from_numpy(W.strengths(n, 1, n)).cuda()
+    plan = api.Plan(pts, lo, h, ng, 2 * np.pi * ng / 4, kernel=kernel, layout=layout)
+    out = plan.apply(lam)
+    assert plan.async_status() == 0
+    assert _close(api, plan, pts, lo, h, ng, lam, out), plan.info
+
+
+@pytest.mark.parametrize("kernel", ["helmholtz", "laplace"])
+def test_batched_groups(kernel):
+    """Plans on the box-group kernel in one launch: every plan's rows equal its own apply bit for bit (the same
+    members swept the same way), eagerly, replayed, and after the strengths change."""
+    api = _api()
+    plans, lams = [], []
+    for i, (n, ng, request) in enumerate([(3000, 6, -2), (1, 2, -2), (17, 1, -2), (40001, 14, 0), (5000, 7, -2)]):
+        pts = torch.rand(n, 3, generator=torch.Generator(device="cuda").manual_seed(i), device="cuda")
+        plans.append(api.Plan(pts, (0.0, 0.0, 0.0), 1.0 / ng, ng, 2 * np.pi * ng / 4, kernel=kernel,
+                              tuning={"warp_boxes": request}))
+        assert plans[-1].info["tuning"]["warp_boxes"] == -2
+        lams.append(torch.from_numpy(W.strengths(n, 1, i)).cuda())
+    src = torch.rand(900, 3, generator=torch.Generator(device="cuda").manual_seed(9), device="cuda") * 0.4
+    two = api.TwoSetPlan(plans[0].structure.points, src, (0.0, 0.0, 0.0), 1.0 / 6, 6, 9.0, kernel=kernel,
+                         tuning={"warp_boxes": -2})
+    plans.append(two)
+    lams.append(torch.from_numpy(W.strengths(900, 1, 9)).cuda())
+    batch = api.Batch(plans)
+    for o, p, l in zip(batch.apply(lams), plans, lams):
+        assert torch.equal(o[:, 0], p.apply(l))
+    outs = batch.capture(lams)
+    for scale in (1.0, 2.0):
+        for l in lams:
+            l.mul_(scale)
+        batch.replay()
+        for o, p, l in zip(outs, plans, lams):
+            assert torch.equal(o[:, 0], p.apply(l)) and p.async_status() == 0
