@@ -681,29 +681,47 @@ p2p_tuning resolve_tuning(const p2p_tuning* t) {
     return r;
 }
 
-// Boxes per warp of the direct kernel for a plan left to choose (warp_boxes = 0), from the mean number of
-// targets per box D.  Measured on GB300: the 2^20-point sphere at D = 8 (185 us with four boxes per warp
-// against 217 us staged) and D = 16 (staged 290 us, direct 293 - 340 us), and square plates of 2^10 - 2^20
-// points at D = 1.0 - 4 (at 2^20 points: D = 4.1, eight boxes per warp 74 us, four 82 us, staged 258 us;
-// D = 1.6, sixteen 64 us; D = 1.0 - 1.1, thirty-two 39 - 47 us).
 // Largest union the box-group kernel stages (sources; 24 bytes each in shared memory; its positions are 16-bit).
 constexpr int32_t kGroupCapMax = 8192;
 
+// The one-right-hand-side kernel of a plan left to choose (warp_boxes = 0), from the mean number of targets per box D
+// and the number of boxes: > 0 boxes per warp of the direct kernel, -2 the box-group kernel (indexed layout only,
+// other layouts take the staged pipeline), -1 the staged pipeline.
 //
-// Above that, up to D = 24, the box-group kernel (-2; indexed layout only, other layouts keep the staged
-// pipeline): the sphere at D = 16, 259 us against 292 us staged (groups of 16 boxes, 24 warps per SM); at D = 32
-// it measured 571 us against 474 staged, at D = 8 222 us against the direct kernel's 185.  A uniform cube gives
-// the same ranking (D = 16: 0.228 ms against 0.274 staged, D = 24: 0.470 against 0.512, D = 32: 0.137 against
-// 0.122).
+// The direct kernel with several boxes per warp does the least work per pair on sparse boxes, but a box there is a
+// long serial chain on a few lanes: its heaviest boxes alone take 20 - 50 us at D = 3 - 9, so it pays once the rest
+// of the chip needs that long too.  Few boxes are best cut into the staged pipeline's items, which spread one box over
+// several warps.  Measured on GB300 (applies in us, Helmholtz on a sphere / in a cube, staged | group | direct with 1
+// / 4 / 8 boxes per warp):
+//   D = 1.6 (plate): 635 boxes 6.1 | 7.3 | 4.9 / 8.5 / 9.5; 10 319: 15 | 13 | 11 / 10 / 11.5, sixteen 11.7;
+//             165 629: 148 | 124 | 93 / 34 / 26.5, sixteen 25.6
+//   D = 2.3 (plate): 28 275: 31 | 26 | 21 / 16 / 16.5, sixteen 20; 453 351: 421 | 379 | 289 / 125 / 91, sixteen 102
+//   D = 3.5:   1 140: 6.4 | 8.3 | 6.6 / 13.6 / 22.4       4 605: 9.3 | 9.4 | 8.8 / 14.3 / 23.2
+//             18 924: 24 | 23 | 18.7 / 17.0 / 25          75 224: 82 | 71 | 56 / 37 / 43
+//            285 361: 307 | 284 | 237 / 129 / 119
+//   D = 6.2:   2 636: 10.3 | 10.7 | 10.7 / 32 / 51        10 263: 20 | 18.6 | 19.7 / 39 / 61
+//             42 015: 60 | 54 | 53 / 58 / 79              165 248: 231 | 209 | 218 / 160 / 176
+//   D = 8-9:   1 792: 11.7 | 11.5 | 15 / 50 / 92           7 197: 20 | 16.5 | 23 / 54 / 96
+//             28 916: 58 | 51 | 56 / 77 / 110             62 577: 107 | 97 | 102 / 102 / 133 (Laplace 91 | 81 | 81 / 70)
+//            131 431: 218 | 197 | 219 / 188 / 225
+//   D = 10.8: 97 091: 224 | 201 | 241 / 262 / 309
+//   D = 14:    1 201: 12.9 | 16 | 25 / 77 / 152             4 829: 25 | 21 | 39    18 863: 72 | 66 | 78
+//   D = 20:      784: 13.8 | 25 | 48                        3 296: 31 | 35 | 54    13 599: 88 | 85 | 102
+//   cube, D = 9: 6 859: 30 | 25 | 31 / 86 / 156; D = 16: 1 000: 17 | 27, 17 576: 118 | 98; D = 21: 3 375: 40 | 45,
+//   12 167: 147 | 151; D = 32 (4 096 boxes): 122 | 137
+// Laplace gives the same ranking at about two thirds of the times, with several boxes per warp a little earlier.
 int32_t auto_warp_boxes(int64_t n, int32_t nb) {
     if (nb <= 0) return -1;
     const double d = (double)n / nb;
-    if (d <= 1.3) return 32;
-    if (d <= 2.5) return 16;
-    if (d <= 6.0) return 8;
-    if (d <= 12.0) return 4;
-    if (d <= 24.0) return -2;
-    return -1;
+    if (d > 24.0) return -1;
+    if (d > 12.0) return nb >= 6000 || (nb >= 1000 && d <= 19.5) ? -2 : -1;
+    if (nb < 2500) return d <= 2.5 ? 1 : -1;
+    if (d <= 1.3) return nb < 15000 ? 4 : 32;
+    if (d <= 1.9) return nb < 15000 ? 4 : 16;
+    if (d <= 2.5) return nb < 15000 ? 4 : 8;
+    if (d <= 5.0) return nb < 15000 ? 1 : (nb < 150000 ? 4 : 8);
+    if (d <= 7.0) return nb < 45000 ? 1 : 4;
+    return d <= 9.0 && nb >= 55000 ? 4 : -2;
 }
 
 struct PlanLayout {
