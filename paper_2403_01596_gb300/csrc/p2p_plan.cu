@@ -341,7 +341,7 @@ __global__ void k_list_sizes(const int32_t* __restrict__ list_len, int32_t nb, i
 __global__ void k_item_records(const int32_t* __restrict__ n_chunks, const int32_t* __restrict__ item_off,
                                const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ list_len,
                                const int32_t* __restrict__ self_len, const int32_t* __restrict__ pk_off, int32_t nb,
-                               int chunk, int tg, int two_sets, ItemRec* __restrict__ recs,
+                               int chunk, int tg, int two_sets, bool fine, ItemRec* __restrict__ recs,
                                uint32_t* __restrict__ keys, int32_t* __restrict__ vals) {
     int32_t b = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
     if (b >= nb) return;
@@ -365,7 +365,7 @@ __global__ void k_item_records(const int32_t* __restrict__ n_chunks, const int32
         r.map_last = p2p_lane_map(last, r.ns);
         r.b = b;
         recs[o + i] = r;
-        keys[o + i] = cost_key<kCostBits>((int64_t)nt * r.ns);
+        keys[o + i] = fine ? cost_key<kFineCostBits>((int64_t)nt * r.ns) : cost_key<kCostBits>((int64_t)nt * r.ns);
         vals[o + i] = o + i;
     }
 }
@@ -1187,13 +1187,16 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
             p->rec_src);
         FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/rep_fill");
     }
+    // few items: an exact order keeps the last ones short (32 768-point cube, 5 574 items: 53.3 us, by 8 bits 53.9)
+    const bool fine = items <= 16384;
     k_item_records<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(L.n_chunks, L.item_off, in.box_ptr, L.list_len,
                                                                  L.self_len, p->pk_off, nb, t.chunk, t.target_group,
-                                                                 p->two_sets, L.recs, L.keys, L.vals);
+                                                                 p->two_sets, fine, L.recs, L.keys, L.vals);
     FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/items");
     if (items > 0) {
         bool in_alt = false;
-        FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, items, kCostBits, L.radix_ws, s, &in_alt),
+        FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, items, fine ? kFineCostBits : kCostBits,
+                                   L.radix_ws, s, &in_alt),
                   "p2p_plan_create/sort");
         k_item_gather<<<blocks_for(items, kThreads), kThreads, 0, s>>>(L.recs, in_alt ? L.vals_alt : L.vals, items,
                                                                        p->items);
