@@ -59,6 +59,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Loads libp2p.so (building it in-tree first if it is missing)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -130,12 +132,15 @@ def check(status: int, where: str):
         raise P2PError(status, where)
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+def _ptr(t) -> int:
+    return 0 if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if stream is None else int(stream.cuda_stream))
+def _stream(stream):
+    """A cudaStream_t: a torch stream's handle, or the handle itself."""
+    if stream is None:
+        return 0
+    return stream if type(stream) is int else int(stream.cuda_stream)
 
 
 def _lo(lo):

@@ -25,8 +25,9 @@ PATHS = {"auto": C.P2P_PATH_AUTO, "fp32_per_rhs": C.P2P_PATH_FP32_PER_RHS, "fp32
          "tc_bf16x3": C.P2P_PATH_TC_BF16X3, "tc_bf16x6": C.P2P_PATH_TC_BF16X6}
 
 
-def _stream():
-    return torch.cuda.current_stream()
+def _stream() -> int:
+    """Handle of the current CUDA stream (without a torch stream object: 0.3 us against 3)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _bytes(n: int, device) -> torch.Tensor:
@@ -175,6 +176,14 @@ class Plan:
 
     def apply(self, lam: torch.Tensor, out: torch.Tensor | None = None, adjoint: bool = False,
               path: str = "auto") -> torch.Tensor:
+        shape = lam.shape
+        if (out is None and lam.dtype is torch.complex64 and lam.is_cuda and lam.is_contiguous()
+                and 1 <= len(shape) <= 2 and shape[0] == self.structure.n):
+            # the common call: the same checks, no intermediate views (small applies are bound by this code)
+            nrhs = shape[1] if len(shape) == 2 else 1
+            out = torch.empty_like(lam)
+            C.p2p_apply_path(self._plan, lam, out, nrhs, nrhs, adjoint, PATHS[path], _stream())
+            return out
         lam2 = self._check_lam(lam)
         nrhs = lam2.shape[1]
         if lam2.stride(0) != nrhs:

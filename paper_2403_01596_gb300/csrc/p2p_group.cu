@@ -617,7 +617,8 @@ cudaError_t p2p_group_configure(p2p_plan* p) {
     const size_t smem = group_smem_bytes(p->group_cap, p->group_pos_cap);
     if (smem > (size_t)optin) return cudaSuccess;
     auto kern = p->kernel == P2P_LAPLACE ? k_pair_group<P2P_LAPLACE> : k_pair_group<P2P_HELMHOLTZ>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is the function's, shared by every plan: raised to the most a block may have, once and for all launches
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGroupWarps * 32, smem);
     if (e == cudaSuccess) p->group_grid = per_sm * sms;
     return e;
@@ -631,7 +632,6 @@ p2p_status p2p_group_launch(const p2p_plan* p, float2* out, int64_t ld, float k,
     a.k = k;
     const size_t smem = group_smem_bytes(p->group_cap, p->group_pos_cap);
     auto kern = p->kernel == P2P_LAPLACE ? k_pair_group<P2P_LAPLACE> : k_pair_group<P2P_HELMHOLTZ>;
-    P2P_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "p2p_apply/group");
     const int grid = (int)std::min<int64_t>(p->group_grid, p->n_groups);
     kern<<<grid, kGroupWarps * 32, smem, s>>>(a);
     P2P_CHECK_LAUNCH("p2p_apply/group");
