@@ -404,9 +404,9 @@ P2P_API p2p_status p2p_apply_path(const p2p_plan* plan, const void* lambda, void
 /*
  * The two phases of p2p_apply_path, for callers that overlap or time them
  * separately.  p2p_apply_stage gathers lambda into the plan's staging buffer
- * in the order the chosen path reads it (box-sorted rows, or the per-box
- * packed rows of the redundant layout, Sec. 3.3; for the tensor-core path, the
- * BF16 hi/lo record of every 16-source group); p2p_apply_staged then runs the
+ * in the order the chosen path reads it (box-sorted rows, the records of the
+ * repetition layout, Sec. 3.3; for the tensor-core path, the BF16 record of
+ * every group of 16 sorted sources); p2p_apply_staged then runs the
  * pair kernel (or the tensor-core kernel) on the staged strengths and writes
  * out.  Both must be given the same nrhs and path; no other call on the plan
  * may come between them.  The arguments mean what they mean for

@@ -1,6 +1,5 @@
-// Apply path of the P2P operator: strength staging (sorted gather for the
-// indexed layout of Sec. 3.2, repack into the per-box redundant tiles of Sec.
-// 3.3), the FP32 pair kernel, its adjoint and the coordinate gradient.
+// Apply path of the P2P operator: strength staging (the gather into box-sorted
+// order, the repack into the repetition layout's records), the FP32 pair kernel, its adjoint and the coordinate gradient.
 //
 // The pair kernel's device code (work items, staging, lane mapping) lives in
 // p2p_pair.cuh, shared with the persistent batched launch.
@@ -411,9 +410,8 @@ p2p_status check_apply_args(const p2p_plan* plan, const void* lam, const void* o
 // i.e. sum_s |G(r) lambda_sq| for both kernels (|exp(ikr)| = 1), through the staged pipeline with the Laplace
 // kernel on the strengths' magnitudes (lambda: leading dimension ld; S: nrhs).  Uses the plan's staging buffer.
 p2p_status p2p_abs_sums(const p2p_plan* plan, const float2* lam, int64_t ld, int32_t nrhs, float2* S, cudaStream_t s) {
-    const bool red = plan->layout == P2P_LAYOUT_REDUNDANT;
-    const int32_t* rows = red ? plan->pk_src : plan->src_perm;
-    const int64_t nrows = red ? plan->packed : plan->n_src;
+    const int32_t* rows = plan->src_perm;
+    const int64_t nrows = plan->n_src;
     if (nrows > 0) {
         const int64_t total = nrows * nrhs;
         k_gather_abs<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(lam, ld, rows, nrows, nrhs, plan->lam_buf);
@@ -497,10 +495,8 @@ P2P_API p2p_status p2p_apply_stage(const p2p_plan* plan, const void* lambda, int
                      "p2p_apply_stage");
         return P2P_OK;
     }
-    const bool red = plan->layout == P2P_LAYOUT_REDUNDANT;
-    const int32_t* rows = red ? plan->pk_src : plan->src_perm;  // strengths live on the sources
-    const int64_t nrows = red ? plan->packed : plan->n_src;
-    P2P_TRY_CUDA(stage_rows((const float2*)lambda, ld, rows, nrows, nrhs, plan->lam_buf, s), "p2p_apply_stage");
+    P2P_TRY_CUDA(stage_rows((const float2*)lambda, ld, plan->src_perm, plan->n_src, nrhs, plan->lam_buf, s),
+                 "p2p_apply_stage");  // strengths live on the sources
     return P2P_OK;
 }
 

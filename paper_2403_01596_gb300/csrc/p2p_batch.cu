@@ -38,8 +38,8 @@ constexpr int kMaxBatch = kMaxBatchPlans;
 struct BatchGeom {
     PairArgs a;
     int64_t n;
-    int64_t nrows;         // staged rows (points or packed entries)
-    const int32_t* rows;   // original index of every staged row (-1: padding)
+    int64_t nrows;         // staged rows
+    const int32_t* rows;   // original index of every staged row
 };
 
 struct BatchIO {
@@ -278,8 +278,8 @@ P2P_API p2p_status p2p_batch_create(p2p_batch** batch, const p2p_plan* const* pl
         host[g].a = base_args(p);
         host[g].a.nrhs = nrhs;
         host[g].n = p->n;
-        host[g].nrows = host[g].a.red ? p->packed : p->n_src;   // staged strengths live on the sources
-        host[g].rows = host[g].a.red ? p->pk_src : p->src_perm;
+        host[g].nrows = p->n_src;  // staged strengths live on the sources
+        host[g].rows = p->src_perm;
         max_chunk = std::max(max_chunk, p->tune.chunk);
         if (host[g].a.sym) b->sym_any = 1;
         off.off[g + 1] = off.off[g] + p->n_items;

@@ -10,9 +10,9 @@
 // complete source list, so every result is written once, without atomics), and
 // the sources are read straight from global memory through the L1, with the
 // next sources prefetched into registers, instead of being staged in shared
-// memory.  The redundant layout (Sec. 3.3) reads the box's contiguous tile of
-// coordinates and repacked strengths; the indexed layout (Sec. 3.2) reads the
-// box's source list and gathers through it.  The sources are swept in blocks of
+// memory.  Both layouts read the box's source list and gather the strengths
+// through it; the coordinates come the same way (indexed, Sec. 3.2) or from the
+// box's contiguous tile (redundant, Sec. 3.3).  The sources are swept in blocks of
 // two per lane with the next block's loads in flight; 64 registers per thread
 // keep 32 warps per SM resident, which is what hides the L2 latency (deeper
 // blocks cost occupancy and measured slower).
@@ -41,8 +41,8 @@ struct DirectArgs {
     const float4* xs;       // box-sorted source coordinates (indexed layout)
     const float4* xt;       // box-sorted target coordinates
     const float4* pk_xyz;   // redundant layout: per-box source tiles
-    const int32_t* nb_src;  // indexed layout: per-box source lists (box-sorted source indices)
-    const float2* lam;      // staged strengths of one right-hand side: sorted rows or packed rows
+    const int32_t* nb_src;  // per-box source lists (box-sorted source indices)
+    const float2* lam;      // staged strengths of one right-hand side in box-sorted source order
     const int32_t* perm;    // target permutation (sorted position -> original index)
     float2* out;
     int64_t ld;
@@ -57,7 +57,7 @@ constexpr int kBlock = P2P_DIRECT_BLOCK;  // sources per lane per block of the s
 // The lane's sources s0, s0 + Q, ... < ns in blocks of kBlock: while a block is
 // evaluated (pair(p, l, own) per source, own = s < m_end: a source of the box's
 // own cell, where r = 0 is possible) the next block's coordinates and strengths
-// are already being loaded, and for the indexed layout the list entries of the
+// are already being loaded, and the list entries of the
 // block after that as well.  The own cell's sources (the list's prefix) go
 // through the same pipeline as the rest.
 template <bool RED, typename Pair>
@@ -67,12 +67,12 @@ __device__ __forceinline__ void sweep_blocks(const DirectArgs& a, int32_t off, i
     const int stride = kBlock * Q;
     float4 p[kBlock];
     float2 l[kBlock];
-    int j[kBlock];  // indexed layout: list entries of the next block to load
+    int j[kBlock];  // list entries of the next block to load
     auto load_idx = [&](int base) {
 #pragma unroll
         for (int u = 0; u < kBlock; ++u) {
             const int s = base + u * Q;
-            j[u] = (!RED && s < ns) ? __ldg(a.nb_src + off + s) : 0;
+            j[u] = s < ns ? __ldg(a.nb_src + off + s) : 0;
         }
     };
     auto load_data = [&](int base, float4 (&pp)[kBlock], float2 (&ll)[kBlock]) {
@@ -82,13 +82,8 @@ __device__ __forceinline__ void sweep_blocks(const DirectArgs& a, int32_t off, i
             pp[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             ll[u] = make_float2(0.f, 0.f);
             if (s < ns) {
-                if (RED) {
-                    pp[u] = __ldg(a.pk_xyz + off + s);
-                    ll[u] = __ldg(a.lam + off + s);
-                } else {
-                    pp[u] = __ldg(a.xs + j[u]);
-                    ll[u] = __ldg(a.lam + j[u]);
-                }
+                pp[u] = RED ? __ldg(a.pk_xyz + off + s) : __ldg(a.xs + j[u]);
+                ll[u] = __ldg(a.lam + j[u]);
             }
         }
     };

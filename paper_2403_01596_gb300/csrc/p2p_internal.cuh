@@ -96,7 +96,6 @@ struct p2p_plan {
     int32_t* pk_off;        // [nb + 1] offsets of the per-box source lists (each padded to 4 entries)
     int32_t* nb_src;        // [packed] box-sorted index of every listed source, -1 for padding
     float4* pk_xyz;         // [packed] redundant layout: per-box copy of the listed coordinates
-    int32_t* pk_src;        // [packed] redundant layout: original index of every listed source, -1 for padding
     // repetition layout (Sec. 3.3): one record per target -- its coordinates, then its neighbourhood's sources
     int64_t records;        // entries of all records (sum over boxes of n_b (1 + S_b)), 0 for other layouts
     int32_t* rec_off;       // [n + 1] first entry of the record of every target (box-sorted order)
@@ -110,7 +109,7 @@ struct p2p_plan {
     int32_t grid[3];        // persistent grid of the pair kernel for R = 1, 2, 4 right-hand sides per pass
     int32_t grid_warps[3];  // warps per block of that grid (the tuning's, halved until a block fits)
     int32_t multi_grid[3];  // persistent grid of the several-right-hand-sides kernel for 2, 4, 8 per launch
-    float2* lam_buf;        // [max(n, packed) * max_nrhs] sorted / packed strengths
+    float2* lam_buf;        // [n_src * max_nrhs] sorted strengths (repetition layout: [records])
     float2* g_buf;          // [n * max_nrhs] sorted upstream gradient (coordinate gradient)
     unsigned int* status;   // device status word
     long long* scratch64;   // small device scratch (pair count)

@@ -6,16 +6,18 @@
 // source list: the box's own sources first, then those of its other neighbour
 // boxes in ascending id.  The indexed layout (Sec. 3.2) lists box-sorted
 // indices and gathers coordinates and strengths through them; the redundant
-// layout (Sec. 3.3) holds a per-box copy of the coordinates and a per-apply
-// repack of the strengths, so a chunk is one contiguous tile.
+// layout (Sec. 3.3) holds a per-box copy of the coordinates, so a chunk's are one
+// contiguous tile, and gathers the strengths.  (Repacking the strengths into tiles
+// as well took a pass over the whole lists per apply: 73 us of 522 on the 2^20-point
+// sphere at 32 points per box; gathered, the apply takes 490 us instead of 530.)
 //
 // Pipeline.  The kernel is persistent: warp w of W takes items w, w + W, ... of
 // the heaviest-first list (a fixed stride, so the records of the next items can be
 // loaded ahead) and keeps two shared-memory stages.  While it sweeps
 // the targets of item i against stage i % 2, the sources of item i + 1 are
 // already on their way into the other stage -- with cp.async (per-lane 16/8 B
-// asynchronous copies) for the indexed gather, or with one or two TMA bulk
-// copies (cp.async.bulk, completion on an mbarrier) for the redundant tile.
+// asynchronous copies) for the gathers, with a TMA bulk copy (cp.async.bulk,
+// completion on an mbarrier) for the redundant layout's coordinates.
 // Waits on an mbarrier are bounded; on expiry the warp sets the status word,
 // drains its copies (bounded) and stops.
 //
@@ -58,7 +60,7 @@ struct PairArgs {
     const float4* xt;       // box-sorted target coordinates (= xs when sources are the targets)
     const float4* pk_xyz;   // redundant layout: per-box source tiles
     const int32_t* nb_src;  // per-box source lists (box-sorted indices)
-    const float2* lam;      // staged strengths, row stride nrhs: sorted (indexed) or packed (redundant)
+    const float2* lam;      // staged strengths in box-sorted source order, row stride nrhs
     const float2* gsrc;     // staged upstream gradient (coordinate gradient only), row stride nrhs
     const int32_t* perm;
     float2* out;
@@ -166,7 +168,7 @@ __device__ __forceinline__ WarpSmem warp_smem(unsigned char* ws, int chunk, int 
     return w;
 }
 
-// Indexed layout, two items ahead: one TMA bulk copy of the chunk's source
+// Two items ahead: one TMA bulk copy of the chunk's source
 // list (box-sorted indices) into index stage `i` (lane 0 only).
 __device__ __forceinline__ void issue_index_copy(const PairArgs& a, const ItemRec& r, const WarpSmem& w, int i) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -176,9 +178,9 @@ __device__ __forceinline__ void issue_index_copy(const PairArgs& a, const ItemRe
 }
 
 // One item ahead: the chunk's coordinates and (when one pass covers every
-// right-hand side, nrhs == R) strengths into data stage `i`.  Redundant: two
-// TMA bulk copies of the contiguous tile (lane 0).  Indexed: per-lane cp.async
-// gathers through index stage `ii`, which the caller has waited for.
+// right-hand side, nrhs == R) strengths into data stage `i`: per-lane cp.async
+// gathers through index stage `ii`, which the caller has waited for; the redundant
+// layout's coordinates by one TMA bulk copy of the contiguous tile (lane 0).
 template <int R>
 __device__ __forceinline__ void issue_data(const PairArgs& a, const ItemRec& r, const WarpSmem& w, int i, int ii,
                                            int lane) {
@@ -189,16 +191,15 @@ __device__ __forceinline__ void issue_data(const PairArgs& a, const ItemRec& r, 
             // the stage was last read through the generic proxy; order those reads before the bulk write
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             const uint32_t n4 = (uint32_t)((r.ns + 3) & ~3);
-            const uint32_t bytes = n4 * 16u + (lam_async ? n4 * (uint32_t)R * 8u : 0u);
-            mbar_expect_tx(&w.bar[i], bytes);
+            mbar_expect_tx(&w.bar[i], n4 * 16u);
             bulk_g2s(st.sx, a.pk_xyz + r.src_off, n4 * 16u, &w.bar[i]);
-            if (lam_async) bulk_g2s(st.sl, a.lam + (int64_t)r.src_off * R, n4 * (uint32_t)R * 8u, &w.bar[i]);
         }
-    } else {
-        const int* idx = w.index(ii);
+    }
+    const int* idx = w.index(ii);
+    if (!a.red || lam_async) {
         for (int p = lane; p < r.ns; p += 32) {
             const int j = idx[p];
-            cp_async16(st.sx + p, a.xs + j);
+            if (!a.red) cp_async16(st.sx + p, a.xs + j);
             if (lam_async) {
                 if (R == 1) cp_async8(st.sl + p, a.lam + j);
                 else {
@@ -216,7 +217,7 @@ __device__ __forceinline__ void issue_data(const PairArgs& a, const ItemRec& r, 
 template <int R>
 __device__ __forceinline__ void load_lam_block(const PairArgs& a, const ItemRec& r, float2* sl, int rb, int lane) {
     for (int p = lane; p < r.ns; p += 32) {
-        const int64_t row = (int64_t)(a.red ? r.src_off + p : a.nb_src[r.src_off + p]) * a.nrhs + rb;
+        const int64_t row = (int64_t)a.nb_src[r.src_off + p] * a.nrhs + rb;
 #pragma unroll
         for (int q = 0; q < R; ++q) sl[p * R + q] = (rb + q < a.nrhs) ? a.lam[row + q] : make_float2(0.f, 0.f);
     }
@@ -645,7 +646,7 @@ __device__ __forceinline__ ItemRec gather_rec(int32_t v) {
 // (n of them).  `args_of(rec)` points to the PairArgs an item belongs to.  At the
 // top of iteration k the warp holds records k .. k+2 (lane-distributed) and
 // starts loading record k+3; it issues the index copy of item k+2 (index stage
-// (k+2) % 3, indexed layouts) and the data copies of item k+1 (data stage
+// (k+2) % 3) and the data copies of item k+1 (data stage
 // (k+1) % 2), then waits for item k's data and sweeps it.  Every mbarrier wait
 // is bounded.
 template <int R, typename ArgsOf>
@@ -670,13 +671,11 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
     const PairArgs* a0 = args_of(r0);
     const PairArgs* a1 = has1 ? args_of(r1) : nullptr;
     if (lane == 0) {
-        if (!a0->red) issue_index_copy(*a0, r0, w, 0);
-        if (a1 && !a1->red) issue_index_copy(*a1, r1, w, 1);
+        issue_index_copy(*a0, r0, w, 0);
+        if (a1) issue_index_copy(*a1, r1, w, 1);
     }
-    if (!a0->red) {
-        failed |= !mbar_wait(&w.bar[2], parity[2]);
-        parity[2] ^= 1u;
-    }
+    failed |= !mbar_wait(&w.bar[2], parity[2]);
+    parity[2] ^= 1u;
     failed = !__all_sync(P2P_FULL_MASK, !failed);
     if (!failed) issue_data<R>(*a0, r0, w, 0, 0, lane);
     int64_t k = 0;
@@ -688,15 +687,13 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
         const ItemRec r2 = gather_rec(v2);
         const PairArgs* a2 = i2 < n ? args_of(r2) : nullptr;
         // index copy of item k+2 (item k's list stays in its own stage until it is scattered)
-        if (a2 && !a2->red && lane == 0) issue_index_copy(*a2, r2, w, i2s);
+        if (a2 && lane == 0) issue_index_copy(*a2, r2, w, i2s);
         // data of item k+1
         if (a1) {
-            if (!a1->red) {
-                failed |= !mbar_wait(&w.bar[2 + i1s], parity[2 + i1s]);
-                parity[2 + i1s] ^= 1u;
-                failed = !__all_sync(P2P_FULL_MASK, !failed);
-                if (failed) break;
-            }
+            failed |= !mbar_wait(&w.bar[2 + i1s], parity[2 + i1s]);
+            parity[2 + i1s] ^= 1u;
+            failed = !__all_sync(P2P_FULL_MASK, !failed);
+            if (failed) break;
             issue_data<R>(*a1, r1, w, nxt, i1s, lane);
         }
         // wait for item k's data

@@ -406,13 +406,12 @@ __global__ void k_direct_items(const int32_t* __restrict__ box_ptr, const int32_
 // cell in a two-set plan), then the other neighbour boxes in ascending id (the
 // order the pair kernel's r = 0 mask relies on) -- as box-sorted source indices
 // (nb_src, the index arrays of the indexing method, Sec. 3.2) and, for the
-// redundant layout, as a copy of the coordinates plus original indices (the
-// repetition of Sec. 3.3).  xs, perm and box_ptr are the SOURCE side.
-__global__ void k_pack(const float4* __restrict__ xs, const int32_t* __restrict__ perm,
-                       const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ nbr_ptr,
+// redundant layout, as a copy of the coordinates (the repetition of Sec. 3.3).  xs
+// and box_ptr are the SOURCE side.
+__global__ void k_pack(const float4* __restrict__ xs, const int32_t* __restrict__ box_ptr, const int32_t* __restrict__ nbr_ptr,
                        const int32_t* __restrict__ nbr_idx, const int32_t* __restrict__ nbr_self,
                        const int32_t* __restrict__ pk_off, int32_t nb, int upper, int32_t* __restrict__ nb_src,
-                       float4* __restrict__ pk_xyz, int32_t* __restrict__ pk_src) {
+                       float4* __restrict__ pk_xyz) {
     const int lane = threadIdx.x & 31;
     const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (b >= nb) return;
@@ -457,18 +456,12 @@ __global__ void k_pack(const float4* __restrict__ xs, const int32_t* __restrict_
         for (int32_t p = lane; p < m; p += 32) {
             const int32_t j = s0 + p;
             nb_src[to + p] = j;
-            if (pk_xyz) {
-                pk_xyz[to + p] = xs[j];
-                pk_src[to + p] = perm[j];
-            }
+            if (pk_xyz) pk_xyz[to + p] = xs[j];
         }
     }
     if (lane < padded - total) {
         nb_src[base + total + lane] = -1;
-        if (pk_xyz) {
-            pk_xyz[base + total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-            pk_src[base + total + lane] = -1;
-        }
+        if (pk_xyz) pk_xyz[base + total + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -772,14 +765,13 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     L.p.pk_off = c.take<int32_t>(mb + 1);
     L.p.nb_src = c.take<int32_t>(list_bound);
     L.p.pk_xyz = red ? c.take<float4>(list_bound) : nullptr;
-    L.p.pk_src = red ? c.take<int32_t>(list_bound) : nullptr;
     const bool rep = layout == P2P_LAYOUT_REPETITION;
     const size_t mr = (size_t)(records > 0 ? records : 1);
     L.p.rec_off = rep ? c.take<int32_t>(m + 1) : nullptr;
     L.p.rec_boff = rep ? c.take<int32_t>(mb + 1) : nullptr;
     L.p.rec_xyz = rep ? c.take<float4>(mr) : nullptr;
     L.p.rec_src = rep ? c.take<int32_t>(mr) : nullptr;
-    size_t lam_rows = red ? (ms > list_bound ? ms : list_bound) : ms;
+    size_t lam_rows = ms;
     if (rep && mr > lam_rows) lam_rows = mr;
     // rows of max_nrhs strengths (as they come, or packed), or sorted rows of the padded blocks of p2p_multi.cu
     size_t lam_count = lam_rows * (size_t)max_nrhs;
@@ -1172,9 +1164,8 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     FAIL_CUDA(scan_exclusive_i32(L.n_chunks, L.item_off, nb, nullptr, L.scan_ws, s), "p2p_plan_create/scan");
     FAIL_CUDA(scan_exclusive_i32(L.padded, p->pk_off, nb, p->pk_off + nb, L.scan_ws, s),
               "p2p_plan_create/scan_lists");
-    k_pack<<<blocks_for((int64_t)nb * 32, kThreads), kThreads, 0, s>>>(p->xs_src, p->src_perm, p->src_box_ptr,
-                                                                      in.nbr_ptr, in.nbr_idx, p->nbr_self, p->pk_off,
-                                                                      nb, upper, p->nb_src, p->pk_xyz, p->pk_src);
+    k_pack<<<blocks_for((int64_t)nb * 32, kThreads), kThreads, 0, s>>>(
+        p->xs_src, p->src_box_ptr, in.nbr_ptr, in.nbr_idx, p->nbr_self, p->pk_off, nb, upper, p->nb_src, p->pk_xyz);
     FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/pack");
     if (layout == P2P_LAYOUT_REPETITION) {
         // per-target records (L.padded is free once the list offsets are scanned)
