@@ -17,8 +17,7 @@ using p2p_direct::kDirectWarps;
 
 namespace {
 
-// Persistent pair kernel: warp w of the grid takes items w, w + W, w + 2W, ...
-// of the plan's heaviest-first item list (W = warps in the grid).
+// Persistent pair kernel: the warps of the grid take turns in the plan's heaviest-first item list.
 template <int R>
 __global__ void __launch_bounds__(P2P_PAIR_MAX_THREADS, R == 1 ? P2P_PAIR_MIN_BLOCKS : 1)
     k_pair(const __grid_constant__ PairArgs a) {

@@ -10,7 +10,7 @@
 //                   atomics;
 //   k_pair_batched  a persistent grid (resident blocks x SMs) whose warps take
 //                   work items (geometry, box, source chunk) from one combined
-//                   list, warp w taking items w, w + W, ... (W warps).  The list
+//                   list in turns (p2p_turn).  The list
 //                   is the plans' own item lists (each heaviest first) one after
 //                   the other in the order the plans were given, so the warps work
 //                   on one geometry's data at a time and the last geometry's light

@@ -232,6 +232,15 @@ cudaError_t p2p_group_batch_create(p2p_group_batch* b, const p2p_plan* const* pl
                                    cudaStream_t s);
 p2p_status p2p_group_batch_launch(const p2p_group_batch* b, cudaStream_t s);
 
+// Position in a heaviest-first list of a worker's k-th item, w of W workers: w, and back and forth from there
+// (w, 2W - 1 - w, 2W + w, ...), so that the worker with a round's heaviest item gets the next round's lightest; with
+// a fixed stride the differences of all rounds add up.  Increases with k.  Used where the sources are staged in
+// shared memory (start of a kernel's item costs little, the sums of the costs decide): 8 right-hand sides on a
+// 40 000-point shell assembly 423 -> 405 us, 262 144 sphere points at 64 per box 816 -> 811 us.  Not used by the
+// direct and box-group kernels, which were slower with it (65 536-point plate 79.8 -> 85.8 us, sixteen pieces
+// 270 -> 286 us): there neighbours in the list share their sources in the L1 or L2.
+__host__ __device__ inline int64_t p2p_turn(int64_t k, int64_t w, int64_t W) { return k * W + ((k & 1) ? W - 1 - w : w); }
+
 // Persistent grid sizes of the pair kernel for the plan's kernel, layout and
 // tuning (resident blocks per SM x SMs), one per right-hand-side block width.
 cudaError_t p2p_pair_configure(p2p_plan* plan);

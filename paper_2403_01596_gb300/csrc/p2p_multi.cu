@@ -89,7 +89,7 @@ template <int R>
 struct Stream {
     const MultiArgs& a;
     int lane;
-    int32_t stride;
+    int32_t worker, workers, turn;
     int32_t rec;      // record of the item after the latest place's, field f in lane f
     int32_t rec_item;
     float* base;
@@ -99,7 +99,7 @@ struct Stream {
         Place p;
         p.item = item;
         set_item(p, load_rec_lane(a.items, item, a.n_items, lane));
-        rec_item = item + stride;
+        rec_item = (int32_t)min((int64_t)a.n_items, p2p_turn(++turn, worker, workers));
         rec = load_rec_lane(a.items, rec_item, a.n_items, lane);
         p.t0 = p.s0 = 0;
         set_group(p, a.tg);
@@ -117,7 +117,7 @@ struct Stream {
                 p.item = rec_item;
                 if (p.item < a.n_items) {
                     set_item(p, rec);
-                    rec_item += stride;
+                    rec_item = (int32_t)min((int64_t)a.n_items, p2p_turn(++turn, worker, workers));
                     rec = load_rec_lane(a.items, rec_item, a.n_items, lane);
                 }
             }
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kMultiWarps * 32, 2) k_pair_multi(const __grid
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* ws = reinterpret_cast<float*>(smem_raw) + warp * warp_floats(R);
-    Stream<R> st{a, lane, (int32_t)gridDim.x * kMultiWarps, 0, 0, ws};
+    Stream<R> st{a, lane, (int32_t)(blockIdx.x * kMultiWarps + warp), (int32_t)gridDim.x * kMultiWarps, 0, 0, 0, ws};
     float* red = ws + 2 * stage_floats(R);
     const int32_t item = (int32_t)blockIdx.x * kMultiWarps + warp;
     if (item >= a.n_items) return;

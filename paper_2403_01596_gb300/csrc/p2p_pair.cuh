@@ -11,9 +11,9 @@
 // as well took a pass over the whole lists per apply: 73 us of 522 on the 2^20-point
 // sphere at 32 points per box; gathered, the apply takes 490 us instead of 530.)
 //
-// Pipeline.  The kernel is persistent: warp w of W takes items w, w + W, ... of
-// the heaviest-first list (a fixed stride, so the records of the next items can be
-// loaded ahead) and keeps two shared-memory stages.  While it sweeps
+// Pipeline.  The kernel is persistent: warp w of W takes the items of its turns in
+// the heaviest-first list (p2p_turn: known beforehand, so the records of the next items
+// can be loaded ahead) and keeps two shared-memory stages.  While it sweeps
 // the targets of item i against stage i % 2, the sources of item i + 1 are
 // already on their way into the other stage -- with cp.async (per-lane 16/8 B
 // asynchronous copies) for the gathers, with a TMA bulk copy (cp.async.bulk,
@@ -642,7 +642,7 @@ __device__ __forceinline__ ItemRec gather_rec(int32_t v) {
     return r;
 }
 
-// The per-warp pipeline over the items first, first + stride, ... of `items`
+// The per-warp pipeline over the items p2p_turn(0, 1, ..., first, stride) of `items`
 // (n of them).  `args_of(rec)` points to the PairArgs an item belongs to.  At the
 // top of iteration k the warp holds records k .. k+2 (lane-distributed) and
 // starts loading record k+3; it issues the index copy of item k+2 (index stage
@@ -664,10 +664,10 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
     bool failed = false;
     // prologue: records 0..2, index copies of items 0 and 1, data of item 0
     int32_t v0 = load_rec_lane(items, first, n, lane);
-    int32_t v1 = load_rec_lane(items, first + stride, n, lane);
-    int32_t v2 = load_rec_lane(items, first + 2 * stride, n, lane);
+    int32_t v1 = load_rec_lane(items, p2p_turn(1, first, stride), n, lane);
+    int32_t v2 = load_rec_lane(items, p2p_turn(2, first, stride), n, lane);
     ItemRec r0 = gather_rec(v0), r1 = gather_rec(v1);
-    const bool has1 = first + stride < n;
+    const bool has1 = p2p_turn(1, first, stride) < n;
     const PairArgs* a0 = args_of(r0);
     const PairArgs* a1 = has1 ? args_of(r1) : nullptr;
     if (lane == 0) {
@@ -682,7 +682,7 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
     while (!failed) {
         const int cur = (int)(k & 1), nxt = cur ^ 1;
         const int i0 = (int)(k % 3), i1s = (int)((k + 1) % 3), i2s = (int)((k + 2) % 3);  // index stages
-        const int64_t i1 = first + (k + 1) * stride, i2 = first + (k + 2) * stride, i3 = first + (k + 3) * stride;
+        const int64_t i2 = p2p_turn(k + 2, first, stride), i3 = p2p_turn(k + 3, first, stride);
         const int32_t v3 = load_rec_lane(items, i3, n, lane);  // consumed two iterations later
         const ItemRec r2 = gather_rec(v2);
         const PairArgs* a2 = i2 < n ? args_of(r2) : nullptr;
@@ -715,7 +715,6 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
         a1 = a2;
         v2 = v3;
         ++k;
-        (void)i1;
     }
     if (failed) {
         if (lane == 0) atomicOr(status, P2P_DEV_TIMEOUT);
