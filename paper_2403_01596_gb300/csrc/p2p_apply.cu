@@ -85,181 +85,6 @@ DirectKernel direct_kernel(const p2p_plan* p) {
     return red ? direct_kernel_k<P2P_LAPLACE, true>(p->direct_k) : direct_kernel_k<P2P_LAPLACE, false>(p->direct_k);
 }
 
-// ------------------------------------------------------ coordinate gradient --
-
-__host__ __device__ inline int grad_smem_bytes(int chunk) { return chunk * 16 + chunk * 16 + 32 * kMaxTT * 16; }
-
-template <int KERN, int TT>
-__device__ __forceinline__ void grad_targets(const PairArgs& a, const float4* __restrict__ sx,
-                                             const float4* __restrict__ slg, float4* red, int ns, int tbase, int nt,
-                                             int32_t map, int rhs, int lane) {
-    const int G = map_g(map), Q = map_q(map);
-    const int q = map_div(map, lane);
-    const int g = lane - q * G;
-    float4 tx[TT];
-    float2 tl[TT], tgv[TT];
-    float acc[TT][3];
-#pragma unroll
-    for (int u = 0; u < TT; ++u) {
-        const int t = g + u * G;
-        const bool ok = t < nt;
-        tx[u] = ok ? a.xt[tbase + t] : make_float4(0.f, 0.f, 0.f, 0.f);
-        tl[u] = ok ? a.lam[(int64_t)(tbase + t) * a.nrhs + rhs] : make_float2(0.f, 0.f);
-        tgv[u] = ok ? a.gsrc[(int64_t)(tbase + t) * a.nrhs + rhs] : make_float2(0.f, 0.f);
-        acc[u][0] = acc[u][1] = acc[u][2] = 0.f;
-    }
-    if (q < Q && TT % 2 == 0) {
-        // targets in pairs on the packed two-lane FP32 instructions (rsqrt, sincos per pair)
-        constexpr int V = TT / 2 > 0 ? TT / 2 : 1;
-        float2 px2[V], py2[V], pz2[V], lx2[V], ly2[V], gx2[V], gy2[V], ax[V], ay[V], az[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const int u0 = 2 * v, u1 = (2 * v + 1) % TT;
-            px2[v] = make_float2(tx[u0].x, tx[u1].x);
-            py2[v] = make_float2(tx[u0].y, tx[u1].y);
-            pz2[v] = make_float2(tx[u0].z, tx[u1].z);
-            lx2[v] = make_float2(tl[u0].x, tl[u1].x);
-            ly2[v] = make_float2(tl[u0].y, tl[u1].y);
-            gx2[v] = make_float2(tgv[u0].x, tgv[u1].x);
-            gy2[v] = make_float2(tgv[u0].y, tgv[u1].y);
-            ax[v] = ay[v] = az[v] = make_float2(0.f, 0.f);
-        }
-        const float2 k2 = make_float2(a.k, a.k);
-        for (int s = q; s < ns; s += Q) {
-            const float4 p = sx[s];
-            const float4 lg = slg[s];  // (lambda_s.re, lambda_s.im, g_s.re, g_s.im)
-            const float2 npx = make_float2(-p.x, -p.x), npy = make_float2(-p.y, -p.y), npz = make_float2(-p.z, -p.z);
-            const float2 sl_x = make_float2(lg.x, lg.x), sl_y = make_float2(lg.y, lg.y);
-            const float2 sg_x = make_float2(lg.z, lg.z), sg_y = make_float2(lg.w, lg.w);
-            const float2 nsl_x = make_float2(-lg.x, -lg.x), nsg_y = make_float2(-lg.w, -lg.w);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const float2 dx = __fadd2_rn(px2[v], npx), dy = __fadd2_rn(py2[v], npy), dz = __fadd2_rn(pz2[v], npz);
-                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-                float2 inv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-                inv.x = r2.x > 0.f ? inv.x : 0.f;
-                inv.y = r2.y > 0.f ? inv.y : 0.f;
-                const float2 inv2 = __fmul2_rn(inv, inv);
-                // C = conj(g_t) lambda_s + conj(g_s) lambda_t
-                const float2 cr = __ffma2_rn(gx2[v], sl_x, __ffma2_rn(gy2[v], sl_y,
-                                  __ffma2_rn(sg_x, lx2[v], __fmul2_rn(sg_y, ly2[v]))));
-                const float2 ci = __ffma2_rn(gx2[v], sl_y, __ffma2_rn(gy2[v], nsl_x,
-                                  __ffma2_rn(sg_x, ly2[v], __fmul2_rn(nsg_y, lx2[v]))));
-                float2 w;
-                if (KERN == P2P_HELMHOLTZ) {
-                    const float2 kr = __fmul2_rn(k2, __fmul2_rn(r2, inv));
-                    float2 sn, cs;
-                    __sincosf(kr.x, &sn.x, &cs.x);
-                    __sincosf(kr.y, &sn.y, &cs.y);
-                    const float2 ncs = make_float2(-cs.x, -cs.y), nsn = make_float2(-sn.x, -sn.y);
-                    const float2 dgr = __fmul2_rn(__ffma2_rn(nsn, kr, ncs), inv2);
-                    const float2 dgi = __fmul2_rn(__ffma2_rn(cs, kr, nsn), inv2);
-                    w = __ffma2_rn(dgr, cr, __fmul2_rn(make_float2(-dgi.x, -dgi.y), ci));
-                } else {
-                    w = __fmul2_rn(make_float2(-inv2.x, -inv2.y), cr);
-                }
-                w = __fmul2_rn(w, inv);
-                ax[v] = __ffma2_rn(w, dx, ax[v]);
-                ay[v] = __ffma2_rn(w, dy, ay[v]);
-                az[v] = __ffma2_rn(w, dz, az[v]);
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            acc[2 * v][0] = ax[v].x;
-            acc[2 * v][1] = ay[v].x;
-            acc[2 * v][2] = az[v].x;
-            acc[(2 * v + 1) % TT][0] = ax[v].y;
-            acc[(2 * v + 1) % TT][1] = ay[v].y;
-            acc[(2 * v + 1) % TT][2] = az[v].y;
-        }
-    } else if (q < Q) {
-        const float k = a.k;
-        for (int s = q; s < ns; s += Q) {
-            const float4 p = sx[s];
-            const float4 lg = slg[s];  // (lambda_s.re, lambda_s.im, g_s.re, g_s.im)
-#pragma unroll
-            for (int u = 0; u < TT; ++u) {
-                const float dx = tx[u].x - p.x, dy = tx[u].y - p.y, dz = tx[u].z - p.z;
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                float inv = rsqrtf(r2);
-                inv = r2 > 0.f ? inv : 0.f;
-                const float inv2 = inv * inv;
-                // C = conj(g_t) lambda_s + conj(g_s) lambda_t
-                const float cr = tgv[u].x * lg.x + tgv[u].y * lg.y + lg.z * tl[u].x + lg.w * tl[u].y;
-                const float ci = tgv[u].x * lg.y - tgv[u].y * lg.x + lg.z * tl[u].y - lg.w * tl[u].x;
-                float w;
-                if (KERN == P2P_HELMHOLTZ) {
-                    const float kr = k * (r2 * inv);
-                    float sn, cs;
-                    __sincosf(kr, &sn, &cs);
-                    const float dgr = (-cs - sn * kr) * inv2;
-                    const float dgi = (cs * kr - sn) * inv2;
-                    w = dgr * cr - dgi * ci;
-                } else {
-                    w = -inv2 * cr;
-                }
-                w *= inv;
-                acc[u][0] = fmaf(w, dx, acc[u][0]);
-                acc[u][1] = fmaf(w, dy, acc[u][1]);
-                acc[u][2] = fmaf(w, dz, acc[u][2]);
-            }
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < TT; ++u) red[lane * TT + u] = make_float4(acc[u][0], acc[u][1], acc[u][2], 0.f);
-    __syncwarp();
-    for (int t = lane; t < nt; t += 32) {
-        const int u = map_div(map, t);
-        const int gg = t - u * G;
-        float v0 = 0.f, v1 = 0.f, v2 = 0.f;
-        for (int qq = 0; qq < Q; ++qq) {
-            const float4 w = red[(qq * G + gg) * TT + u];
-            v0 += w.x;
-            v1 += w.y;
-            v2 += w.z;
-        }
-        float* dst = a.grad + (int64_t)a.perm[tbase + t] * 3;
-        atomicAdd(dst, v0 * kInv4Pi);
-        atomicAdd(dst + 1, v1 * kInv4Pi);
-        atomicAdd(dst + 2, v2 * kInv4Pi);
-    }
-    __syncwarp();
-}
-
-// One warp per work item; sources gathered through the box's source list.
-template <int KERN>
-__global__ void __launch_bounds__(512) k_grad(const __grid_constant__ PairArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t item = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (item >= a.n_items) return;
-    const int chunk = a.chunk;
-    unsigned char* ws = smem_raw + (size_t)warp * grad_smem_bytes(chunk);
-    float4* sx = reinterpret_cast<float4*>(ws);
-    float4* slg = reinterpret_cast<float4*>(ws + chunk * 16);
-    float4* red = reinterpret_cast<float4*>(ws + chunk * 32);
-    const ItemRec r = a.items[item];
-    for (int p = lane; p < r.ns; p += 32) sx[p] = a.xs[a.nb_src[r.src_off + p]];
-    for (int rhs = 0; rhs < a.nrhs; ++rhs) {
-        __syncwarp();
-        for (int p = lane; p < r.ns; p += 32) {
-            const int64_t row = (int64_t)a.nb_src[r.src_off + p] * a.nrhs + rhs;
-            const float2 l = a.lam[row], gg = a.gsrc[row];
-            slg[p] = make_float4(l.x, l.y, gg.x, gg.y);
-        }
-        __syncwarp();
-        for (int t0 = 0; t0 < r.nt; t0 += a.tg) {
-            const int nt = min(a.tg, r.nt - t0);
-            const int32_t map = (t0 + a.tg >= r.nt) ? r.map_last : r.map_full;
-            const int tt = map_tt(map);
-            if (tt == 1) grad_targets<KERN, 1>(a, sx, slg, red, r.ns, r.tb + t0, nt, map, rhs, lane);
-            else if (tt == 2) grad_targets<KERN, 2>(a, sx, slg, red, r.ns, r.tb + t0, nt, map, rhs, lane);
-            else grad_targets<KERN, 4>(a, sx, slg, red, r.ns, r.tb + t0, nt, map, rhs, lane);
-        }
-    }
-}
-
 // ----------------------------------------------------------------- staging --
 
 // dst[s * nrhs + q] = src[rows[s] * ld + q]  (rows[s] < 0: zero)
@@ -433,6 +258,8 @@ cudaError_t p2p_group_configure(p2p_plan* p);
 cudaError_t p2p_multi_configure(p2p_plan* p);
 p2p_status p2p_multi_stage(const p2p_plan* p, const float2* lam, int32_t nrhs, int64_t ld, cudaStream_t s);
 p2p_status p2p_multi_launch(const p2p_plan* p, float2* out, int32_t nrhs, int64_t ld, float k, cudaStream_t s);
+p2p_status p2p_grad_launch(const p2p_plan* p, const float2* lam, const float2* g, float* grad, int32_t nrhs, int64_t ld,
+                           cudaStream_t s);
 p2p_status p2p_group_launch(const p2p_plan* p, float2* out, int64_t ld, float k, cudaStream_t s);
 
 cudaError_t p2p_pair_configure(p2p_plan* plan) {
@@ -594,21 +421,7 @@ P2P_API p2p_status p2p_grad_points(const p2p_plan* plan, const void* lambda, con
     if (!grad || ((uintptr_t)grad & 3)) return P2P_ERR_INVALID;
     if (plan->layout == P2P_LAYOUT_SYMMETRIC) return P2P_ERR_UNSUPPORTED;  // needs the full source lists
     if (plan->two_sets) return P2P_ERR_UNSUPPORTED;                         // one point set only
-    cudaStream_t s = (cudaStream_t)stream;
-    P2P_TRY_CUDA(stage_rows((const float2*)lambda, ld, plan->perm, plan->n, nrhs, plan->lam_buf, s),
-                 "p2p_grad_points/stage");
-    P2P_TRY_CUDA(stage_rows((const float2*)g, ld, plan->perm, plan->n, nrhs, plan->g_buf, s), "p2p_grad_points/stage");
-    P2P_TRY_CUDA(cudaMemsetAsync(grad, 0, (size_t)plan->n * 3 * sizeof(float), s), "p2p_grad_points/zero");
-    PairArgs a = base_args(plan);
-    a.grad = grad;
-    a.nrhs = nrhs;
-    const int warps = plan->tune.warps_per_cta;
-    const int smem = warps * grad_smem_bytes(a.chunk);
-    auto kern = plan->kernel == P2P_HELMHOLTZ ? k_grad<P2P_HELMHOLTZ> : k_grad<P2P_LAPLACE>;
-    P2P_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "p2p_grad_points");
-    kern<<<(unsigned)((a.n_items + warps - 1) / warps), warps * 32, smem, s>>>(a);
-    P2P_CHECK_LAUNCH("p2p_grad_points/kernel");
-    return P2P_OK;
+    return p2p_grad_launch(plan, (const float2*)lambda, (const float2*)g, grad, nrhs, ld, (cudaStream_t)stream);
 }
 
 }  // extern "C"

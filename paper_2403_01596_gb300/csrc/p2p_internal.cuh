@@ -109,8 +109,8 @@ struct p2p_plan {
     int32_t grid[3];        // persistent grid of the pair kernel for R = 1, 2, 4 right-hand sides per pass
     int32_t grid_warps[3];  // warps per block of that grid (the tuning's, halved until a block fits)
     int32_t multi_grid[3];  // persistent grid of the several-right-hand-sides kernel for 2, 4, 8 per launch
-    float2* lam_buf;        // [n_src * max_nrhs] sorted strengths (repetition layout: [records])
-    float2* g_buf;          // [n * max_nrhs] sorted upstream gradient (coordinate gradient)
+    float2* lam_buf;        // [n_src * max_nrhs] sorted strengths (repetition layout: [records]), or the coordinate
+                            // gradient's rows of (strength, upstream gradient)
     unsigned int* status;   // device status word
     long long* scratch64;   // small device scratch (pair count)
     // tensor-core path (plans with max_nrhs >= 16)
@@ -236,8 +236,8 @@ p2p_status p2p_group_batch_launch(const p2p_group_batch* b, cudaStream_t s);
 // (w, 2W - 1 - w, 2W + w, ...), so that the worker with a round's heaviest item gets the next round's lightest; with
 // a fixed stride the differences of all rounds add up.  Increases with k.  Used where the sources are staged in
 // shared memory (start of a kernel's item costs little, the sums of the costs decide): 8 right-hand sides on a
-// 40 000-point shell assembly 423 -> 405 us, 262 144 sphere points at 64 per box 816 -> 811 us.  Not used by the
-// direct and box-group kernels, which were slower with it (65 536-point plate 79.8 -> 85.8 us, sixteen pieces
+// 500 000-point shell assembly 423 -> 405 us, 2^20 sphere points at 64 per box 816 -> 811 us.  Not used by the
+// direct and box-group kernels, which were slower with it (2^20-point Laplace plate 79.8 -> 85.8 us, sixteen pieces of 65 536 points
 // 270 -> 286 us): there neighbours in the list share their sources in the L1 or L2.
 __host__ __device__ inline int64_t p2p_turn(int64_t k, int64_t w, int64_t W) { return k * W + ((k & 1) ? W - 1 - w : w); }
 

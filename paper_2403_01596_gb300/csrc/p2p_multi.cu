@@ -39,6 +39,7 @@ namespace {
 
 constexpr int kMultiWarps = 8;   // warps per block
 constexpr int kSub = 32;         // sources of a sub-chunk at most
+constexpr int kGradBlocks = 2;   // resident blocks per SM of the gradient
 
 struct MultiArgs {
     const ItemRec* items;
@@ -225,15 +226,42 @@ __device__ __forceinline__ void multi_core(const float4 p, const float* __restri
     }
 }
 
-// The target group at `cur` (whose sub-chunk is on its way into half h) through all of its sub-chunks, and its
-// results.  nxt: the place after cur, its indices in j.  Leaves cur, nxt, j and h at the next group's first sub-chunk.
+// The target group at `cur` (whose sub-chunk is on its way into half h) through all of its sub-chunks: pair(p, l, own)
+// for the sources of the lane's slice q of Q, own: a source of the targets' own cell.  nxt: the place after cur, its
+// indices in j.  Leaves cur, nxt, j and h at the next group's first sub-chunk.
+template <int R, typename Pair>
+__device__ __forceinline__ void sweep_stream(Stream<R>& st, Place& cur, Place& nxt, int& j, int& h, int q, int Q, Pair pair) {
+    const int m_end = cur.m_end;
+    while (true) {
+        st.copy(nxt, j, h ^ 1);
+        const Place after = nxt.item < st.a.n_items ? st.next(nxt) : nxt;
+        const int ja = st.index(after);
+        cp_async_wait<1>();
+        __syncwarp();
+        if (q < Q) {
+            const float* buf = st.buf(h);
+            const int own = m_end - cur.s0;
+            for (int s = q; s < cur.len; s += Q)
+                pair(*reinterpret_cast<const float4*>(buf + 4 * s), buf + 4 * kSub + 2 * R * s, s < own);
+        }
+        __syncwarp();  // the half is read before the copies of the place after next overwrite it
+        const bool last = cur.s0 + cur.len >= cur.ns;
+        cur = nxt;
+        nxt = after;
+        j = ja;
+        h ^= 1;
+        if (last) break;
+    }
+}
+
+// One target group (sweep_stream) and its results.
 template <int KERN, int R, int TT>
 __device__ __forceinline__ void run_group(Stream<R>& st, Place& cur, Place& nxt, int& j, int& h, float* red) {
     const MultiArgs& a = st.a;
     const int lane = st.lane;
     const int32_t map = cur.map;
     const int G = map_g(map), Q = map_q(map), q = map_div(map, lane), g = lane - q * G;
-    const int tb = cur.tb + cur.t0, nt = min(a.tg, cur.nt - cur.t0), m_end = cur.m_end;
+    const int tb = cur.tb + cur.t0, nt = min(a.tg, cur.nt - cur.t0);
     const int32_t perm0 = lane < nt ? __ldg(a.perm + tb + lane) : 0;
     float nx[TT], ny[TT], nz[TT];
     float2 re[TT][R / 2], im[TT][R / 2];
@@ -247,27 +275,9 @@ __device__ __forceinline__ void run_group(Stream<R>& st, Place& cur, Place& nxt,
 #pragma unroll
         for (int i = 0; i < R / 2; ++i) re[u][i] = im[u][i] = make_float2(0.f, 0.f);
     }
-    while (true) {
-        st.copy(nxt, j, h ^ 1);
-        const Place after = nxt.item < a.n_items ? st.next(nxt) : nxt;
-        const int ja = st.index(after);
-        cp_async_wait<1>();
-        __syncwarp();
-        if (q < Q) {
-            const float* buf = st.buf(h);
-            const int own = m_end - cur.s0;
-            for (int s = q; s < cur.len; s += Q)
-                multi_core<KERN, R, TT>(*reinterpret_cast<const float4*>(buf + 4 * s), buf + 4 * kSub + 2 * R * s, s < own, nx,
-                                        ny, nz, re, im, a.k);
-        }
-        __syncwarp();  // the half is read before the copies of the place after next overwrite it
-        const bool last = cur.s0 + cur.len >= cur.ns;
-        cur = nxt;
-        nxt = after;
-        j = ja;
-        h ^= 1;
-        if (last) break;
-    }
+    sweep_stream<R>(st, cur, nxt, j, h, q, Q, [&](const float4& p, const float* l, bool own) {
+        multi_core<KERN, R, TT>(p, l, own, nx, ny, nz, re, im, a.k);
+    });
     // slice partials -> results, one target of every lane at a time: (Re, Re, Im, Im) of two right-hand sides per
     // 16 bytes, lane after lane
     float4* red4 = reinterpret_cast<float4*>(red);
@@ -325,6 +335,174 @@ __global__ void __launch_bounds__(kMultiWarps * 32, 2) k_pair_multi(const __grid
         else run_group<KERN, R, 4>(st, cur, nxt, j, h, red);
     }
     cp_async_wait<0>();
+}
+
+// ------------------------------------------------------ coordinate gradient --
+
+// The derivative with respect to the target's coordinates, one right-hand side per launch.  A pair is 3 MUFU and ~30
+// FP32 operations (19 of them on the packed instructions), so both pipes and the issue slots are about equally busy;
+// what the kernel must avoid is standing still.  One item per warp, staged whole and synchronously before its sweep,
+// left 18 warps per SM waiting for two dependent gathers at every item.  Here the rows (lambda, g) come through the
+// same stream as the strengths of two right-hand sides, 16 warps per SM at 128 registers (at 80 registers, 24 warps,
+// the sweep spills: 143 us instead of 126); one launch stages both inputs and zeroes the result.  Staging
+// included: 262 144 points on a sphere at 16 per box 147 -> 126 us, Laplace on 500 001 points of an ellipsoid at 8
+// 160 -> 120 us, 12 001 points at 10 31 -> 22 us, 500 001 points at 50 554 -> 552 us (issue-bound before and after).
+constexpr int kGradWarpFloats = 2 * stage_floats(2) + 32 * kMaxTT * 4;
+
+// One source against the lane's TT targets (negated coordinates; strengths and upstream values tl, tg).
+template <int KERN, int TT>
+__device__ __forceinline__ void grad_core(const float4 p, const float4 lg, const float (&nx)[TT], const float (&ny)[TT],
+                                          const float (&nz)[TT], const float2 (&tl)[TT], const float2 (&tg)[TT],
+                                          float (&acc)[TT][3], float k) {
+    // with d = source - target: grad = w d, w = (G'(r) / r) C, C = conj(g_t) lambda_s + conj(g_s) lambda_t
+    if constexpr (TT % 2 == 0) {
+        const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y), pz = make_float2(p.z, p.z);
+        const float2 lx = make_float2(lg.x, lg.x), ly = make_float2(lg.y, lg.y), gx = make_float2(lg.z, lg.z),
+                     gy = make_float2(lg.w, lg.w);
+        const float2 nlx = make_float2(-lg.x, -lg.x), ngy = make_float2(-lg.w, -lg.w);
+#pragma unroll
+        for (int u = 0; u < TT; u += 2) {
+            const float2 dx = __fadd2_rn(px, make_float2(nx[u], nx[u + 1]));
+            const float2 dy = __fadd2_rn(py, make_float2(ny[u], ny[u + 1]));
+            const float2 dz = __fadd2_rn(pz, make_float2(nz[u], nz[u + 1]));
+            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+            float2 inv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+            inv.x = r2.x > 0.f ? inv.x : 0.f;
+            inv.y = r2.y > 0.f ? inv.y : 0.f;
+            const float2 inv2 = __fmul2_rn(inv, inv);
+            const float2 tlx = make_float2(tl[u].x, tl[u + 1].x), tly = make_float2(tl[u].y, tl[u + 1].y);
+            const float2 tgx = make_float2(tg[u].x, tg[u + 1].x), tgy = make_float2(tg[u].y, tg[u + 1].y);
+            const float2 cr = __ffma2_rn(tgx, lx, __ffma2_rn(tgy, ly, __ffma2_rn(gx, tlx, __fmul2_rn(gy, tly))));
+            float2 w;
+            if (KERN == P2P_HELMHOLTZ) {
+                const float2 ci = __ffma2_rn(tgx, ly, __ffma2_rn(tgy, nlx, __ffma2_rn(gx, tly, __fmul2_rn(ngy, tlx))));
+                const float2 kr = __fmul2_rn(make_float2(k, k), __fmul2_rn(r2, inv));
+                float2 sn, cs;
+                __sincosf(kr.x, &sn.x, &cs.x);
+                __sincosf(kr.y, &sn.y, &cs.y);
+                // -G' r^2 = (cos + kr sin) + i (sin - kr cos), the sign goes into d
+                const float2 a = __ffma2_rn(sn, kr, cs);
+                const float2 b = __ffma2_rn(make_float2(-cs.x, -cs.y), kr, sn);
+                w = __ffma2_rn(a, cr, __fmul2_rn(make_float2(-b.x, -b.y), ci));
+                w = __fmul2_rn(w, inv2);
+            } else {
+                w = __fmul2_rn(inv2, cr);
+            }
+            w = __fmul2_rn(w, inv);
+            float2 ax = make_float2(acc[u][0], acc[u + 1][0]), ay = make_float2(acc[u][1], acc[u + 1][1]),
+                   az = make_float2(acc[u][2], acc[u + 1][2]);
+            ax = __ffma2_rn(w, dx, ax);
+            ay = __ffma2_rn(w, dy, ay);
+            az = __ffma2_rn(w, dz, az);
+            acc[u][0] = ax.x;
+            acc[u + 1][0] = ax.y;
+            acc[u][1] = ay.x;
+            acc[u + 1][1] = ay.y;
+            acc[u][2] = az.x;
+            acc[u + 1][2] = az.y;
+        }
+    } else {
+        const float dx = p.x + nx[0], dy = p.y + ny[0], dz = p.z + nz[0];
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        float inv = rsqrtf(r2);
+        inv = r2 > 0.f ? inv : 0.f;
+        const float cr = fmaf(tg[0].x, lg.x, fmaf(tg[0].y, lg.y, fmaf(lg.z, tl[0].x, lg.w * tl[0].y)));
+        float w = cr;
+        if (KERN == P2P_HELMHOLTZ) {
+            const float ci = fmaf(tg[0].x, lg.y, fmaf(tg[0].y, -lg.x, fmaf(lg.z, tl[0].y, -lg.w * tl[0].x)));
+            const float kr = k * (r2 * inv);
+            float sn, cs;
+            __sincosf(kr, &sn, &cs);
+            w = fmaf(fmaf(sn, kr, cs), cr, -fmaf(-cs, kr, sn) * ci);
+        }
+        w = w * (inv * inv) * inv;
+        acc[0][0] = fmaf(w, dx, acc[0][0]);
+        acc[0][1] = fmaf(w, dy, acc[0][1]);
+        acc[0][2] = fmaf(w, dz, acc[0][2]);
+    }
+}
+
+// One target group of the gradient: its sums are added to the (zeroed) result.
+template <int KERN, int TT>
+__device__ __forceinline__ void run_grad(Stream<2>& st, Place& cur, Place& nxt, int& j, int& h, float* red, float* out) {
+    const MultiArgs& a = st.a;
+    const int lane = st.lane;
+    const int32_t map = cur.map;
+    const int G = map_g(map), Q = map_q(map), q = map_div(map, lane), g = lane - q * G;
+    const int tb = cur.tb + cur.t0, nt = min(a.tg, cur.nt - cur.t0);
+    const int32_t perm0 = lane < nt ? __ldg(a.perm + tb + lane) : 0;
+    float nx[TT], ny[TT], nz[TT], acc[TT][3];
+    float2 tl[TT], tg[TT];
+#pragma unroll
+    for (int u = 0; u < TT; ++u) {
+        const int t = g + u * G;
+        const bool on = t < nt && q < Q;
+        const float4 x = on ? __ldg(a.xt + tb + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 v = on ? __ldg(reinterpret_cast<const float4*>(a.lam) + tb + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        nx[u] = -x.x;
+        ny[u] = -x.y;
+        nz[u] = -x.z;
+        tl[u] = make_float2(v.x, v.y);
+        tg[u] = make_float2(v.z, v.w);
+        acc[u][0] = acc[u][1] = acc[u][2] = 0.f;
+    }
+    sweep_stream<2>(st, cur, nxt, j, h, q, Q, [&](const float4& p, const float* l, bool) {
+        grad_core<KERN, TT>(p, *reinterpret_cast<const float4*>(l), nx, ny, nz, tl, tg, acc, a.k);
+    });
+    float4* red4 = reinterpret_cast<float4*>(red);
+#pragma unroll
+    for (int u = 0; u < TT; ++u) red4[u * 32 + lane] = make_float4(acc[u][0], acc[u][1], acc[u][2], 0.f);
+    __syncwarp();
+    for (int t = lane; t < nt; t += 32) {
+        const int u = map_div(map, t), gg = t - u * G;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int qq = 0; qq < Q; ++qq) {
+            const float4 w = red4[u * 32 + qq * G + gg];
+            v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, 0.f);
+        }
+        float* dst = out + (int64_t)(t == lane ? perm0 : __ldg(a.perm + tb + t)) * 3;
+        atomicAdd(dst, v.x * kInv4Pi);
+        atomicAdd(dst + 1, v.y * kInv4Pi);
+        atomicAdd(dst + 2, v.z * kInv4Pi);
+    }
+    __syncwarp();
+}
+
+template <int KERN>
+__global__ void __launch_bounds__(kMultiWarps * 32, kGradBlocks) k_grad(const __grid_constant__ MultiArgs a, float* out) {
+    __shared__ __align__(16) float smem[kMultiWarps * kGradWarpFloats];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ws = smem + warp * kGradWarpFloats;
+    Stream<2> st{a, lane, (int32_t)(blockIdx.x * kMultiWarps + warp), (int32_t)gridDim.x * kMultiWarps, 0, 0, 0, ws};
+    float* red = ws + 2 * stage_floats(2);
+    const int32_t item = (int32_t)blockIdx.x * kMultiWarps + warp;
+    if (item >= a.n_items) return;
+    Place cur = st.first(item);
+    st.copy(cur, st.index(cur), 0);
+    Place nxt = st.next(cur);
+    int j = st.index(nxt), h = 0;
+    while (cur.item < a.n_items) {
+        const int tt = map_tt(cur.map);
+        if (tt == 1) run_grad<KERN, 1>(st, cur, nxt, j, h, red, out);
+        else if (tt == 2) run_grad<KERN, 2>(st, cur, nxt, j, h, red, out);
+        else run_grad<KERN, 4>(st, cur, nxt, j, h, red, out);
+    }
+    cp_async_wait<0>();
+}
+
+// dst[q * n + s] = (lambda, g)[rows[s] * ld + q], and the result's 3 n floats zeroed.
+__global__ void k_grad_stage(const float2* __restrict__ lam, const float2* __restrict__ g, int64_t ld,
+                             const int32_t* __restrict__ rows, int64_t n, int32_t nrhs, float4* __restrict__ dst,
+                             float* __restrict__ grad) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n) return;
+    const int64_t row = (int64_t)rows[s] * ld;
+    for (int q = 0; q < nrhs; ++q) {
+        const float2 a = lam[row + q], b = g[row + q];
+        dst[q * n + s] = make_float4(a.x, a.y, b.x, b.y);
+    }
+    if (grad)
+        for (int i = 0; i < 3; ++i) grad[i * n + s] = 0.f;
 }
 
 // dst: 2R floats per source, Re of right-hand sides 0 .. R - 1, then Im (zero past nrhs).
@@ -412,6 +590,43 @@ p2p_status p2p_multi_launch(const p2p_plan* p, float2* out, int32_t nrhs, int64_
         multi_kernel(p, R)<<<grid, kMultiWarps * 32, smem, s>>>(a);
         P2P_CHECK_LAUNCH("p2p_apply/multi");
         a.lam += p->n_src * 2 * R;
+    }
+    return P2P_OK;
+}
+
+// The coordinate gradient (one point set), added up over the right-hand sides.
+p2p_status p2p_grad_launch(const p2p_plan* p, const float2* lam, const float2* g, float* grad, int32_t nrhs, int64_t ld,
+                           cudaStream_t s) {
+    int dev = 0, sms = 0;
+    P2P_TRY_CUDA(cudaGetDevice(&dev), "p2p_grad_points/device");
+    P2P_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "p2p_grad_points/device");
+    float4* rows = reinterpret_cast<float4*>(p->lam_buf);
+    // a result that overlaps an input is zeroed once all of it has been staged
+    const char *lo = reinterpret_cast<const char*>(grad), *hi = lo + (size_t)p->n * 3 * sizeof(float);
+    const size_t in_bytes = ((size_t)(p->n - 1) * ld + nrhs) * sizeof(float2);
+    bool overlap = false;
+    for (const char* v : {reinterpret_cast<const char*>(lam), reinterpret_cast<const char*>(g)})
+        overlap |= v < hi && lo < v + in_bytes;
+    k_grad_stage<<<(unsigned)((p->n + 255) / 256), 256, 0, s>>>(lam, g, ld, p->perm, p->n, nrhs, rows,
+                                                               overlap ? nullptr : grad);
+    P2P_CHECK_LAUNCH("p2p_grad_points/stage");
+    if (overlap) P2P_TRY_CUDA(cudaMemsetAsync(grad, 0, (size_t)p->n * 3 * sizeof(float), s), "p2p_grad_points/zero");
+    MultiArgs a{};
+    a.items = p->items;
+    a.n_items = (int32_t)p->n_items;
+    a.xs = p->xs_src;
+    a.xt = p->xs;
+    a.nb_src = p->nb_src;
+    a.perm = p->perm;
+    a.k = p->k;
+    a.tg = p->tune.target_group;
+    const int64_t blocks = ((int64_t)a.n_items + kMultiWarps - 1) / kMultiWarps;
+    if (blocks == 0) return P2P_OK;
+    for (int q = 0; q < nrhs; ++q) {
+        a.lam = reinterpret_cast<const float*>(rows + (int64_t)q * p->n);
+        auto kern = p->kernel == P2P_HELMHOLTZ ? k_grad<P2P_HELMHOLTZ> : k_grad<P2P_LAPLACE>;
+        kern<<<(unsigned)std::min<int64_t>(blocks, (int64_t)sms * kGradBlocks), kMultiWarps * 32, 0, s>>>(a, grad);
+        P2P_CHECK_LAUNCH("p2p_grad_points/kernel");
     }
     return P2P_OK;
 }

@@ -61,10 +61,8 @@ struct PairArgs {
     const float4* pk_xyz;   // redundant layout: per-box source tiles
     const int32_t* nb_src;  // per-box source lists (box-sorted indices)
     const float2* lam;      // staged strengths in box-sorted source order, row stride nrhs
-    const float2* gsrc;     // staged upstream gradient (coordinate gradient only), row stride nrhs
     const int32_t* perm;
     float2* out;
-    float* grad;
     unsigned int* status;
     int64_t ld;
     int32_t nrhs;
@@ -734,10 +732,8 @@ inline PairArgs base_args(const p2p_plan* p) {
     a.pk_xyz = p->pk_xyz;
     a.nb_src = p->nb_src;
     a.lam = p->lam_buf;
-    a.gsrc = p->g_buf;
     a.perm = p->perm;
     a.out = nullptr;
-    a.grad = nullptr;
     a.status = p->status;
     a.ld = 0;
     a.nrhs = 1;

@@ -776,9 +776,10 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     // rows of max_nrhs strengths (as they come, or packed), or sorted rows of the padded blocks of p2p_multi.cu
     size_t lam_count = lam_rows * (size_t)max_nrhs;
     if (lam_count < ms * (size_t)p2p_multi_columns(max_nrhs)) lam_count = ms * (size_t)p2p_multi_columns(max_nrhs);
+    // ... or the coordinate gradient's rows (lambda, g)
+    if (!two_sets && lam_count < 2 * m * (size_t)max_nrhs) lam_count = 2 * m * (size_t)max_nrhs;
     const size_t lam_bytes = lam_count * sizeof(float2);
     L.p.lam_buf = c.take<float2>(lam_count);
-    L.p.g_buf = two_sets ? nullptr : c.take<float2>(m * (size_t)max_nrhs);
     const size_t tc_bytes = p2p_tc_pack_bytes((int64_t)ms, max_nrhs);
     if (tc_bytes) {
         const size_t blocks = (size_t)p2p_tc_block_count((int32_t)mb), entries = p2p_tc_entry_bound(sources, nnz);
