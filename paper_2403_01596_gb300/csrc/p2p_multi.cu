@@ -11,11 +11,11 @@
 // loaded synchronously.
 //
 // Here an item (target box, source chunk) streams through the warp in sub-chunks
-// of at most 32 sources, three steps deep -- source indices in a register,
+// of at most 64 sources, three steps deep -- source indices in registers,
 // coordinates and strengths in flight into one half of the warp's buffer
 // (cp.async), the sweep on the other half -- and the accumulators stay in registers
-// across the sub-chunks: 7 KB per warp at eight right-hand sides, 16 warps per SM at
-// 128 registers.  The stream runs on over target groups and items, so the next item's
+// across the sub-chunks: 5 KB of shared memory per warp at two right-hand sides, 12 KB at
+// eight, 16 or 12 warps per SM.  The stream runs on over target groups and items, so the next item's
 // first sources are on their way while this one's slices are summed.
 //
 // Strengths are staged by blocks of right-hand sides, a row per source with the real
@@ -25,9 +25,9 @@
 // scalar counterpart in pair_core, in the same order.
 //
 // Measured on one GB300, applies including the staging, against the staged pipeline at 4 right-hand sides per sweep:
-// the 500 000-point assembly with 8 right-hand sides 0.423 ms (0.896), 300 001 points on a sphere at 47 per box with 5
-// 0.447 ms (0.786), with 12 (Laplace) 0.513 ms (0.867), at 7 per box with 3 in the redundant layout 0.106 ms (0.317: no
-// per-box repack of the strengths), 10 371 points with 2 28 us (30).
+// the 500 000-point assembly with 8 right-hand sides 0.41 ms (0.90), 300 001 points on a sphere at 47 per box with 5
+// 0.44 ms (0.79), with 12 (Laplace) 0.51 ms (0.87), at 7 per box with 3 in the redundant layout 0.10 ms (0.32: no
+// per-box repack of the strengths), 10 371 points with 2 23 us (30).
 #include <algorithm>
 
 #include "p2p_pair.cuh"
@@ -37,9 +37,21 @@ using namespace p2p_pair;
 
 namespace {
 
-constexpr int kMultiWarps = 8;   // warps per block
-constexpr int kSub = 32;         // sources of a sub-chunk at most
-constexpr int kGradBlocks = 2;   // resident blocks per SM of the gradient
+// Sources of a sub-chunk at most.  A sub-chunk costs ~150 instructions around its sweep, which weigh most where a pair
+// costs little: 64 instead of 32 took 3 right-hand sides on 200 001 points from 75 to 71 us and the Laplace gradient on
+// 500 001 points from 120 to 107 us, and changed 8 right-hand sides by 1 % at most.
+constexpr int kSub = 64;
+constexpr int kLaneSrc = kSub / 32;     // of which a lane copies
+
+// Warps of an SM: two blocks of 8 at 128 registers, or one of 12 at 168 where that is faster although fewer warps are
+// resident: 8 right-hand sides (which spill at 128) 424 -> 417 us on the 500 000-point assembly and 225 -> 218 us on
+// 300 001 sphere points, the Helmholtz gradient 550 -> 516 us on 500 001 points at 50 per box; the Laplace gradient
+// (107 -> 116 us on 500 001 points at 8) and 3 right-hand sides (71 -> 80 us) are slower with 12.
+struct Shape {
+    int warps, blocks;
+};
+__host__ __device__ constexpr Shape multi_shape(int R) { return R == 8 ? Shape{12, 1} : Shape{8, 2}; }
+__host__ __device__ constexpr Shape grad_shape(int kernel) { return kernel == P2P_HELMHOLTZ ? Shape{12, 1} : Shape{8, 2}; }
 
 struct MultiArgs {
     const ItemRec* items;
@@ -86,6 +98,11 @@ __device__ __forceinline__ void set_len(Place& p) {
     p.len = min(p.ns - p.s0, (kSub / Q) * Q);
 }
 
+// Sorted source indices of a sub-chunk, a lane's own.
+struct Sources {
+    int32_t v[kLaneSrc];
+};
+
 template <int R>
 struct Stream {
     const MultiArgs& a;
@@ -127,17 +144,25 @@ struct Stream {
         set_len(p);
         return p;
     }
-    __device__ __forceinline__ int index(const Place& p) const {
-        return p.item < a.n_items && lane < p.len ? __ldg(a.nb_src + p.src_off + p.s0 + lane) : 0;
-    }
-    // copies of the sub-chunk at p (lane's source j) into half h; one group per call, possibly empty
-    __device__ __forceinline__ void copy(const Place& p, int j, int h) const {
-        if (p.item < a.n_items && lane < p.len) {
-            cp_async16(buf(h) + 4 * lane, a.xs + j);
-            float* dst = buf(h) + 4 * kSub + 2 * R * lane;
-            const float* src = a.lam + (int64_t)j * (2 * R);
+    __device__ __forceinline__ Sources index(const Place& p) const {
+        Sources j;
 #pragma unroll
-            for (int i = 0; i < 2 * R; i += 4) cp_async16(dst + i, src + i);
+        for (int i = 0; i < kLaneSrc; ++i)
+            j.v[i] = p.item < a.n_items && 32 * i + lane < p.len ? __ldg(a.nb_src + p.src_off + p.s0 + 32 * i + lane) : 0;
+        return j;
+    }
+    // copies of the sub-chunk at p (lane's sources j) into half h; one group per call, possibly empty
+    __device__ __forceinline__ void copy(const Place& p, const Sources& j, int h) const {
+#pragma unroll
+        for (int c = 0; c < kLaneSrc; ++c) {
+            const int l = 32 * c + lane;
+            if (p.item < a.n_items && l < p.len) {
+                cp_async16(buf(h) + 4 * l, a.xs + j.v[c]);
+                float* dst = buf(h) + 4 * kSub + 2 * R * l;
+                const float* src = a.lam + (int64_t)j.v[c] * (2 * R);
+#pragma unroll
+                for (int i = 0; i < 2 * R; i += 4) cp_async16(dst + i, src + i);
+            }
         }
         cp_async_commit();
     }
@@ -230,12 +255,12 @@ __device__ __forceinline__ void multi_core(const float4 p, const float* __restri
 // for the sources of the lane's slice q of Q, own: a source of the targets' own cell.  nxt: the place after cur, its
 // indices in j.  Leaves cur, nxt, j and h at the next group's first sub-chunk.
 template <int R, typename Pair>
-__device__ __forceinline__ void sweep_stream(Stream<R>& st, Place& cur, Place& nxt, int& j, int& h, int q, int Q, Pair pair) {
+__device__ __forceinline__ void sweep_stream(Stream<R>& st, Place& cur, Place& nxt, Sources& j, int& h, int q, int Q, Pair pair) {
     const int m_end = cur.m_end;
     while (true) {
         st.copy(nxt, j, h ^ 1);
         const Place after = nxt.item < st.a.n_items ? st.next(nxt) : nxt;
-        const int ja = st.index(after);
+        const Sources ja = st.index(after);
         cp_async_wait<1>();
         __syncwarp();
         if (q < Q) {
@@ -256,7 +281,7 @@ __device__ __forceinline__ void sweep_stream(Stream<R>& st, Place& cur, Place& n
 
 // One target group (sweep_stream) and its results.
 template <int KERN, int R, int TT>
-__device__ __forceinline__ void run_group(Stream<R>& st, Place& cur, Place& nxt, int& j, int& h, float* red) {
+__device__ __forceinline__ void run_group(Stream<R>& st, Place& cur, Place& nxt, Sources& j, int& h, float* red) {
     const MultiArgs& a = st.a;
     const int lane = st.lane;
     const int32_t map = cur.map;
@@ -316,18 +341,21 @@ __device__ __forceinline__ void run_group(Stream<R>& st, Place& cur, Place& nxt,
 }
 
 template <int KERN, int R>
-__global__ void __launch_bounds__(kMultiWarps * 32, 2) k_pair_multi(const __grid_constant__ MultiArgs a) {
+__global__ void __launch_bounds__(multi_shape(R).warps * 32, multi_shape(R).blocks)
+    k_pair_multi(const __grid_constant__ MultiArgs a) {
+    constexpr int kWarps = multi_shape(R).warps;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* ws = reinterpret_cast<float*>(smem_raw) + warp * warp_floats(R);
-    Stream<R> st{a, lane, (int32_t)(blockIdx.x * kMultiWarps + warp), (int32_t)gridDim.x * kMultiWarps, 0, 0, 0, ws};
+    Stream<R> st{a, lane, (int32_t)(blockIdx.x * kWarps + warp), (int32_t)gridDim.x * kWarps, 0, 0, 0, ws};
     float* red = ws + 2 * stage_floats(R);
-    const int32_t item = (int32_t)blockIdx.x * kMultiWarps + warp;
+    const int32_t item = (int32_t)blockIdx.x * kWarps + warp;
     if (item >= a.n_items) return;
     Place cur = st.first(item);
     st.copy(cur, st.index(cur), 0);
     Place nxt = st.next(cur);
-    int j = st.index(nxt), h = 0;
+    Sources j = st.index(nxt);
+    int h = 0;
     while (cur.item < a.n_items) {
         const int tt = map_tt(cur.map);
         if (tt == 1) run_group<KERN, R, 1>(st, cur, nxt, j, h, red);
@@ -343,10 +371,10 @@ __global__ void __launch_bounds__(kMultiWarps * 32, 2) k_pair_multi(const __grid
 // FP32 operations (19 of them on the packed instructions), so both pipes and the issue slots are about equally busy;
 // what the kernel must avoid is standing still.  One item per warp, staged whole and synchronously before its sweep,
 // left 18 warps per SM waiting for two dependent gathers at every item.  Here the rows (lambda, g) come through the
-// same stream as the strengths of two right-hand sides, 16 warps per SM at 128 registers (at 80 registers, 24 warps,
-// the sweep spills: 143 us instead of 126); one launch stages both inputs and zeroes the result.  Staging
-// included: 262 144 points on a sphere at 16 per box 147 -> 126 us, Laplace on 500 001 points of an ellipsoid at 8
-// 160 -> 120 us, 12 001 points at 10 31 -> 22 us, 500 001 points at 50 554 -> 552 us (issue-bound before and after).
+// same stream as the strengths of two right-hand sides (at 80 registers, 24 warps, the sweep spills and takes 13 %
+// longer than with 16 warps); one launch stages both inputs and zeroes the result.  Staging included: 262 144 points on
+// a sphere at 16 per box 147 -> 118 us, Laplace on 500 001 points of an ellipsoid at 8 160 -> 107 us, 12 001 points at
+// 10 31 -> 22 us, 500 001 points at 50 554 -> 516 us.
 constexpr int kGradWarpFloats = 2 * stage_floats(2) + 32 * kMaxTT * 4;
 
 // One source against the lane's TT targets (negated coordinates; strengths and upstream values tl, tg).
@@ -424,7 +452,7 @@ __device__ __forceinline__ void grad_core(const float4 p, const float4 lg, const
 
 // One target group of the gradient: its sums are added to the (zeroed) result.
 template <int KERN, int TT>
-__device__ __forceinline__ void run_grad(Stream<2>& st, Place& cur, Place& nxt, int& j, int& h, float* red, float* out) {
+__device__ __forceinline__ void run_grad(Stream<2>& st, Place& cur, Place& nxt, Sources& j, int& h, float* red, float* out) {
     const MultiArgs& a = st.a;
     const int lane = st.lane;
     const int32_t map = cur.map;
@@ -469,18 +497,21 @@ __device__ __forceinline__ void run_grad(Stream<2>& st, Place& cur, Place& nxt, 
 }
 
 template <int KERN>
-__global__ void __launch_bounds__(kMultiWarps * 32, kGradBlocks) k_grad(const __grid_constant__ MultiArgs a, float* out) {
-    __shared__ __align__(16) float smem[kMultiWarps * kGradWarpFloats];
+__global__ void __launch_bounds__(grad_shape(KERN).warps * 32, grad_shape(KERN).blocks)
+    k_grad(const __grid_constant__ MultiArgs a, float* out) {
+    constexpr int kWarps = grad_shape(KERN).warps;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* ws = smem + warp * kGradWarpFloats;
-    Stream<2> st{a, lane, (int32_t)(blockIdx.x * kMultiWarps + warp), (int32_t)gridDim.x * kMultiWarps, 0, 0, 0, ws};
+    float* ws = reinterpret_cast<float*>(smem_raw) + warp * kGradWarpFloats;
+    Stream<2> st{a, lane, (int32_t)(blockIdx.x * kWarps + warp), (int32_t)gridDim.x * kWarps, 0, 0, 0, ws};
     float* red = ws + 2 * stage_floats(2);
-    const int32_t item = (int32_t)blockIdx.x * kMultiWarps + warp;
+    const int32_t item = (int32_t)blockIdx.x * kWarps + warp;
     if (item >= a.n_items) return;
     Place cur = st.first(item);
     st.copy(cur, st.index(cur), 0);
     Place nxt = st.next(cur);
-    int j = st.index(nxt), h = 0;
+    Sources j = st.index(nxt);
+    int h = 0;
     while (cur.item < a.n_items) {
         const int tt = map_tt(cur.map);
         if (tt == 1) run_grad<KERN, 1>(st, cur, nxt, j, h, red, out);
@@ -544,11 +575,11 @@ cudaError_t p2p_multi_configure(p2p_plan* p) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
-        const int R = 2 << i, smem = kMultiWarps * warp_floats(R) * (int)sizeof(float);
+        const int R = 2 << i, warps = multi_shape(R).warps, smem = warps * warp_floats(R) * (int)sizeof(float);
         int per_sm = 0;
         MultiKernel kern = multi_kernel(p, R);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMultiWarps * 32, smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem);
         p->multi_grid[i] = e == cudaSuccess ? per_sm * sms : 0;
     }
     return e;
@@ -583,11 +614,11 @@ p2p_status p2p_multi_launch(const p2p_plan* p, float2* out, int32_t nrhs, int64_
     a.atomic_out = p->max_chunks > 1;
     for (int b = 0; b < nrhs; b += 8) {
         a.nrhs = std::min(8, nrhs - b);
-        const int R = block_width(a.nrhs), smem = kMultiWarps * warp_floats(R) * (int)sizeof(float);
-        const int grid = (int)std::min<int64_t>(p->multi_grid[R == 8 ? 2 : R / 4], ((int64_t)a.n_items + kMultiWarps - 1) / kMultiWarps);
+        const int R = block_width(a.nrhs), warps = multi_shape(R).warps, smem = warps * warp_floats(R) * (int)sizeof(float);
+        const int grid = (int)std::min<int64_t>(p->multi_grid[R == 8 ? 2 : R / 4], ((int64_t)a.n_items + warps - 1) / warps);
         if (grid <= 0) return P2P_ERR_UNSUPPORTED;
         a.out = out + b;
-        multi_kernel(p, R)<<<grid, kMultiWarps * 32, smem, s>>>(a);
+        multi_kernel(p, R)<<<grid, warps * 32, smem, s>>>(a);
         P2P_CHECK_LAUNCH("p2p_apply/multi");
         a.lam += p->n_src * 2 * R;
     }
@@ -620,12 +651,16 @@ p2p_status p2p_grad_launch(const p2p_plan* p, const float2* lam, const float2* g
     a.perm = p->perm;
     a.k = p->k;
     a.tg = p->tune.target_group;
-    const int64_t blocks = ((int64_t)a.n_items + kMultiWarps - 1) / kMultiWarps;
+    const Shape shape = grad_shape(p->kernel);
+    const int64_t blocks = ((int64_t)a.n_items + shape.warps - 1) / shape.warps;
     if (blocks == 0) return P2P_OK;
+    const int smem = shape.warps * kGradWarpFloats * (int)sizeof(float);
+    auto kern = p->kernel == P2P_HELMHOLTZ ? k_grad<P2P_HELMHOLTZ> : k_grad<P2P_LAPLACE>;
+    if (smem > 48 * 1024)
+        P2P_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "p2p_grad_points");
     for (int q = 0; q < nrhs; ++q) {
         a.lam = reinterpret_cast<const float*>(rows + (int64_t)q * p->n);
-        auto kern = p->kernel == P2P_HELMHOLTZ ? k_grad<P2P_HELMHOLTZ> : k_grad<P2P_LAPLACE>;
-        kern<<<(unsigned)std::min<int64_t>(blocks, (int64_t)sms * kGradBlocks), kMultiWarps * 32, 0, s>>>(a, grad);
+        kern<<<(unsigned)std::min<int64_t>(blocks, (int64_t)sms * shape.blocks), shape.warps * 32, smem, s>>>(a, grad);
         P2P_CHECK_LAUNCH("p2p_grad_points/kernel");
     }
     return P2P_OK;
