@@ -42,6 +42,7 @@ namespace {
 // 500 001 points from 120 to 107 us, and changed 8 right-hand sides by 1 % at most.
 constexpr int kSub = 64;
 constexpr int kLaneSrc = kSub / 32;     // of which a lane copies
+constexpr int kBlockRhs = 8;            // right-hand sides per launch at most
 
 // Warps of an SM: two blocks of 8 at 128 registers, or one of 12 at 168 where that is faster although fewer warps are
 // resident: 8 right-hand sides (which spill at 128) 424 -> 417 us on the 500 000-point assembly and 225 -> 218 us on
@@ -536,21 +537,23 @@ __global__ void k_grad_stage(const float2* __restrict__ lam, const float2* __res
         for (int i = 0; i < 3; ++i) grad[i * n + s] = 0.f;
 }
 
-// dst: 2R floats per source, Re of right-hand sides 0 .. R - 1, then Im (zero past nrhs).
-template <int R>
-__global__ void k_multi_stage(const float2* __restrict__ src, int64_t ld, const int32_t* __restrict__ rows, int64_t n,
-                              int32_t nrhs, float* __restrict__ dst) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * R) return;
-    const int64_t s = i / R;
-    const int r = (int)(i - s * R);
-    const float2 v = r < nrhs ? src[(int64_t)rows[s] * ld + r] : make_float2(0.f, 0.f);
-    dst[s * 2 * R + r] = v.x;
-    dst[s * 2 * R + R + r] = v.y;
-}
-
 // Right-hand sides of a launch (2, 4 or 8 accumulators) for the `left` ones still to do.
-int block_width(int left) { return left > 4 ? 8 : (left > 2 ? 4 : 2); }
+__host__ __device__ inline int block_width(int left) { return left > 4 ? 8 : (left > 2 ? 4 : 2); }
+
+// All blocks of the right-hand sides, one after the other (kBlockRhs wide, the last one as wide as its launch): 2R floats
+// per source, Re of the block's right-hand sides, then Im (zero past nrhs).  One thread per source and column.
+__global__ void k_multi_stage(const float2* __restrict__ src, int64_t ld, const int32_t* __restrict__ rows, int64_t n,
+                              int32_t nrhs, int32_t columns, float* __restrict__ dst) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n * columns) return;
+    const int64_t s = i / columns;
+    const int c = (int)(i - s * columns), b = c & ~(kBlockRhs - 1), r = c - b;
+    const int R = block_width(min(kBlockRhs, nrhs - b));
+    const float2 v = c < nrhs ? src[(int64_t)rows[s] * ld + c] : make_float2(0.f, 0.f);
+    float* d = dst + n * 2 * b + s * 2 * R + r;
+    d[0] = v.x;
+    d[R] = v.y;
+}
 
 using MultiKernel = void (*)(MultiArgs);
 MultiKernel multi_kernel(const p2p_plan* p, int R) {
@@ -565,7 +568,7 @@ MultiKernel multi_kernel(const p2p_plan* p, int R) {
 int32_t p2p_multi_columns(int32_t nrhs) {
     if (nrhs <= 1) return nrhs;
     int c = 0;
-    for (int b = 0; b < nrhs; b += 8) c += block_width(std::min(8, nrhs - b));
+    for (int b = 0; b < nrhs; b += kBlockRhs) c += block_width(std::min(kBlockRhs, nrhs - b));
     return c;
 }
 
@@ -586,15 +589,10 @@ cudaError_t p2p_multi_configure(p2p_plan* p) {
 }
 
 p2p_status p2p_multi_stage(const p2p_plan* p, const float2* lam, int32_t nrhs, int64_t ld, cudaStream_t s) {
-    float* dst = reinterpret_cast<float*>(p->lam_buf);
-    for (int b = 0; b < nrhs; b += 8) {
-        const int n = std::min(8, nrhs - b), R = block_width(n);
-        const unsigned blocks = (unsigned)((p->n_src * R + 255) / 256);
-        auto stage = R == 8 ? k_multi_stage<8> : (R == 4 ? k_multi_stage<4> : k_multi_stage<2>);
-        stage<<<blocks, 256, 0, s>>>(lam + b, ld, p->src_perm, p->n_src, n, dst);
-        P2P_CHECK_LAUNCH("p2p_apply_stage/multi");
-        dst += p->n_src * 2 * R;
-    }
+    const int32_t columns = p2p_multi_columns(nrhs);
+    k_multi_stage<<<(unsigned)((p->n_src * columns + 255) / 256), 256, 0, s>>>(lam, ld, p->src_perm, p->n_src, nrhs, columns,
+                                                                              reinterpret_cast<float*>(p->lam_buf));
+    P2P_CHECK_LAUNCH("p2p_apply_stage/multi");
     return P2P_OK;
 }
 
@@ -612,8 +610,8 @@ p2p_status p2p_multi_launch(const p2p_plan* p, float2* out, int32_t nrhs, int64_
     a.k = k;
     a.tg = p->tune.target_group;
     a.atomic_out = p->max_chunks > 1;
-    for (int b = 0; b < nrhs; b += 8) {
-        a.nrhs = std::min(8, nrhs - b);
+    for (int b = 0; b < nrhs; b += kBlockRhs) {
+        a.nrhs = std::min(kBlockRhs, nrhs - b);
         const int R = block_width(a.nrhs), warps = multi_shape(R).warps, smem = warps * warp_floats(R) * (int)sizeof(float);
         const int grid = (int)std::min<int64_t>(p->multi_grid[R == 8 ? 2 : R / 4], ((int64_t)a.n_items + warps - 1) / warps);
         if (grid <= 0) return P2P_ERR_UNSUPPORTED;

@@ -42,3 +42,30 @@ def test_widths(n, ng, tuning, kernel, layout):
             assert plan.async_status() == 0
             assert (np.abs(got[:, :nrhs] - ref[:, :nrhs]) <= 2.0 ** -20 * S[:, :nrhs]).all(), nrhs
             assert (got[:, nrhs:] == complex(7, 7)).all()
+
+
+@pytest.mark.parametrize("n,ng,flat", [(2000, 12, False), (5000, 16, False), (55000, 46, True), (57000, 46, True)])
+@pytest.mark.parametrize("kernel,layout", [("helmholtz", "indexed"), ("laplace", "redundant")])
+def test_two_on_both_sides_of_the_kernel_choice(n, ng, flat, kernel, layout):
+    """Two right-hand sides with few boxes, with boxes of few points, and with boxes of just under and just over the
+    points at which the streamed kernel is left, against the oracle and against each alone; same bound (twice it
+    between two computed results)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_01596_gb300 import api
+    pts = np.random.default_rng(n).random((n, 3)).astype(np.float32)
+    if flat:
+        pts[:, 2] = 0.5
+    lo, h = (0.0, 0.0, 0.0), 1.0 / ng
+    k = float(np.float32(2 * np.pi * ng / 4)) if kernel == "helmholtz" else 0.0
+    kid = oracle.HELMHOLTZ if kernel == "helmholtz" else oracle.LAPLACE
+    plan = api.Plan(torch.from_numpy(pts).cuda(), lo, h, ng, k, kernel=kernel, layout=layout, max_nrhs=2)
+    lam = W.strengths(n, 2, n).reshape(n, 2)
+    S = oracle.p2p(pts, np.abs(lam).astype(np.complex64), lo, h, ng, 0.0, kernel=oracle.LAPLACE).real.reshape(n, 2)
+    ref = oracle.p2p(pts, lam, lo, h, ng, k, kernel=kid, adjoint=True).reshape(n, 2)
+    lam_d = torch.from_numpy(lam).cuda()
+    got = plan.apply(lam_d, adjoint=True).cpu().numpy()
+    alone = np.stack([plan.apply(lam_d[:, q].contiguous(), adjoint=True).cpu().numpy() for q in range(2)], 1)
+    assert plan.async_status() == 0
+    assert (np.abs(got - ref) <= 2.0 ** -20 * S).all()
+    assert (np.abs(got - alone) <= 2.0 ** -19 * S).all()
