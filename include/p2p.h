@@ -101,7 +101,7 @@ typedef enum {
 typedef enum {
     P2P_PATH_AUTO = 0,        /* FP32 shared-G for nrhs < 16, tensor-core path otherwise (when available) */
     P2P_PATH_FP32_PER_RHS = 1,/* FP32; G re-evaluated for every right-hand side */
-    P2P_PATH_FP32_SHARED = 2, /* FP32; each G evaluated once and applied to up to 4 RHS at a time */
+    P2P_PATH_FP32_SHARED = 2, /* FP32; each G evaluated once and applied to up to 8 RHS at a time */
     P2P_PATH_TC_BF16X3 = 3,   /* G tile and strengths split into BF16 hi + lo, 3 tcgen05 MMAs per 16
                                  sources, FP32 accumulation in tensor memory; plans with max_nrhs >= 16
                                  on an sm_103 device, else P2P_ERR_UNSUPPORTED */
@@ -123,10 +123,11 @@ typedef enum {
  * of many targets; the direct kernel gives each warp 1, 2, 4, 8, 16 or 32 whole
  * boxes (32 / warp_boxes lanes each) and reads the sources through the L1, which
  * suits sparse boxes (a few targets each), where a staged item carries too little
- * work for its fixed cost.  0: the plan decides from its mean box occupancy D (the
- * direct kernel with 32, 16, 8 or 4 boxes per warp up to D = 1.3, 2.5, 6 and 12,
- * the box-group kernel for 12 < D <= 24 on the indexed layout, the staged pipeline
- * above); -1: the staged pipeline; 1 .. 32: the direct kernel with that many boxes
+ * work for its fixed cost.  0: the plan decides from its mean box occupancy D and
+ * its number of boxes (with many boxes the direct kernel with 32 .. 4 boxes per warp
+ * up to D = 9, the box-group kernel up to D = 24 on the indexed layout, the staged
+ * pipeline above; with few boxes fewer boxes per warp, or the staged pipeline);
+ * -1: the staged pipeline; 1 .. 32: the direct kernel with that many boxes
  * per warp; -2 (indexed layout only): the box-group
  * kernel, in which groups of 16 consecutive target boxes stage the union of their
  * neighbourhoods in shared memory once and every box sweeps its own neighbour
@@ -285,9 +286,9 @@ P2P_API p2p_status p2p_build_neighbors_st(const int64_t* tgt_keys, int32_t num_t
  *   kernel, k                    Green's function and wavenumber (k finite; ignored for Laplace)
  *   layout                       source layout
  *   max_nrhs                     largest nrhs any apply on this plan will use, 1..256; from 16 up
- *                                the workspace also holds the tensor-core path's per-box group lists
- *                                and its strength records, (n / 16 + num_boxes) x
- *                                (ceil(max_nrhs / 64) x 8192 + 256) bytes
+ *                                the workspace also holds the tensor-core path's entry lists
+ *                                and its strength records, one per 16 sorted sources and
+ *                                block of up to 64 right-hand sides
  *   tuning                 [host] NULL for defaults
  *   workspace              [dev] at least p2p_plan_workspace_size bytes, 256-byte aligned;
  *                                owned by the caller, must outlive the plan
@@ -329,7 +330,7 @@ P2P_API p2p_status p2p_plan_create(p2p_plan** plan, const float* pts, int64_t n,
  * A^H g (n_src rows) is the plan with the two sets exchanged applied with
  * adjoint = 1 in p2p_apply_path, since G(x, y) = G(y, x) (p2p_apply_path with
  * adjoint = 1 on a two-set plan computes conj(A) lambda).  The tensor-core
- * workspace term counts n_src / 16 + num_src_boxes groups.  Other arguments as
+ * workspace term counts the sources' records.  Other arguments as
  * for p2p_plan_create.
  */
 P2P_API p2p_status p2p_plan_workspace_size_st(int64_t n_tgt, int32_t num_tgt_boxes, int64_t n_src,
@@ -467,7 +468,7 @@ P2P_API p2p_status p2p_apply_guarded(const p2p_plan* plan, const void* lambda, v
  * repetition kernel near its optimum (Sec. 4.3); a batch runs such pieces, or
  * unrelated geometries of uneven box occupancy, together: the plans' work items
  * (each plan's own list, heaviest first) form one queue, plan after plan in the
- * order given, and warp w of a persistent grid of W warps takes items w, w + W, ...
+ * order given, and the warps of a persistent grid take turns in it.
  * Giving the plans from smallest to largest leaves the tail to the largest
  * geometry's lightest items.
  *

@@ -299,8 +299,9 @@ static bool is_tc(p2p_path path) { return path == P2P_PATH_TC_BF16X3 || path == 
 // Several right-hand sides on the streamed kernel (p2p_multi.cu): every layout with full source lists, from the sorted
 // strengths.  Two of them stay with the staged pipeline where the plan has few boxes, fewer the more points each holds:
 // one box's chain then decides, and the streamed kernel stages a box's list once per 32 targets.  Measured with two
-// right-hand sides on spheres, streamed / staged, us: 1132 boxes of 7 points 19.5 / 19.5, 2326 of 7 21 / 21, 3850 of 7 23 / 25; 499 of 16 30 / 27, 1854 of 16 35 / 37, 2672 of 16 35 / 40; 620 of 26 30 / 28, 2279 of 29 (Laplace) 43 / 42, 4191 of 29 80 / 92 (Laplace 62 / 69);
-// 1389 of 47 71 / 68 (Laplace 54 / 50), 7156 of 42 233 / 249.  From three right-hand sides on the streamed kernel won
+// right-hand sides on spheres, streamed / staged, us: 1132 boxes of 7 points 19.5 / 19.5, 2326 of 7 21 / 21, 3850
+// of 7 23 / 25; 499 of 16 30 / 27, 2672 of 16 35 / 40; 620 of 26 30 / 28, 2279 of 29 (Laplace) 43 / 38, 4191 of 29
+// 80 / 92 (Laplace 62 / 69); 1389 of 47 71 / 64 (Laplace 54 / 46), 7156 of 42 233 / 249.  From three right-hand sides on the streamed kernel won
 // everywhere from 8 000 points up (499 boxes of 16 with three: 34 / 42).
 static bool is_multi(const p2p_plan* plan, int32_t nrhs, p2p_path path) {
     if (path != P2P_PATH_FP32_SHARED || nrhs < 2) return false;

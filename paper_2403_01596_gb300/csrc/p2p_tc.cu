@@ -24,7 +24,8 @@
 // target box of the unit.  (An earlier kernel had one target box per unit, T <= 32
 // or 64 targets on the MMA's N side and both operands in shared memory: 3.7 M
 // stages on the 2^21-point ellipsoid against 1.27 M entries here, every stage
-// bound by its hand-offs; DESIGN has both sides measured.)
+// bound by its hand-offs; 64 right-hand sides there 5.15 ms per apply against 3.55,
+// 24 in three parts on a 200 003-point sphere 676 us against 320.)
 //
 // Group records.  The B operand of a source group does not depend on the targets,
 // so a pass per apply (k_tc_pack) writes every group's part images, already in the
