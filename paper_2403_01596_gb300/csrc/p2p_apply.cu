@@ -286,6 +286,9 @@ p2p_status p2p_tc_stage(const p2p_plan* plan, const float2* lam, int32_t nrhs, i
 p2p_status p2p_apply_tc(const p2p_plan* plan, float2* out, int32_t nrhs, int64_t ld, int32_t adjoint, int np,
                         cudaStream_t s);
 bool p2p_tc_supported(const p2p_plan* plan, int32_t nrhs);
+p2p_status p2p_tcb_stage(const p2p_plan* plan, const float2* lam, int32_t nrhs, int64_t ld, int np, cudaStream_t s);
+p2p_status p2p_tcb_apply(const p2p_plan* plan, float2* out, int32_t nrhs, int64_t ld, int32_t adjoint, int np,
+                         cudaStream_t s);
 
 extern "C" {
 
@@ -309,6 +312,17 @@ static bool is_multi(const p2p_plan* plan, int32_t nrhs, p2p_path path) {
     return nrhs > 2 || (plan->nb >= 2048 && (int64_t)plan->nb * plan->nb >= 80 * plan->n);
 }
 static int tc_parts(p2p_path path) { return path == P2P_PATH_TC_BF16X6 ? 3 : 2; }
+// One box per unit (p2p_tc_box.cu) instead of 128 targets: where units of 128 targets are too few for the SMs, and for
+// three parts with more than 32 right-hand sides per launch, whose chains would have to be too short (kSegment).
+// Measured on spheres at 20 points per box, us, 128 targets / one box: hi / lo, 16 right-hand sides, 8 193 points 48 / 39,
+// 16 385 62 / 55, 30 001 73 / 93; 64: 16 385 69 / 56, 30 001 89 / 93 (at 45 per box 117 / 111), 60 001 141 / 157; three
+// parts, 32: 8 193 66 / 52, 16 385 76 / 77, 30 001 99 / 124; 64: 60 001 260 / 227.
+static bool tc_by_box(const p2p_plan* plan, int32_t nrhs, int parts) {
+    if (!plan->tcb_gstart) return false;
+    const bool wide = p2p_tc_launch_rhs(nrhs) > 32;
+    if (parts == 3) return wide || plan->n < 12000;
+    return plan->n < (wide ? kTcBoxTargets : 20000);
+}
 
 P2P_API p2p_status p2p_apply_stage(const p2p_plan* plan, const void* lambda, int32_t nrhs, int64_t ld, p2p_path path,
                                    p2p_stream_t stream) {
@@ -320,7 +334,9 @@ P2P_API p2p_status p2p_apply_stage(const p2p_plan* plan, const void* lambda, int
     path = resolve_path(plan, nrhs, path);
     if (is_tc(path) && !p2p_tc_supported(plan, nrhs)) return P2P_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
-    if (is_tc(path)) return p2p_tc_stage(plan, (const float2*)lambda, nrhs, ld, tc_parts(path), s);
+    if (is_tc(path))
+        return (tc_by_box(plan, nrhs, tc_parts(path)) ? p2p_tcb_stage : p2p_tc_stage)(plan, (const float2*)lambda, nrhs, ld,
+                                                                                       tc_parts(path), s);
     if (is_multi(plan, nrhs, path)) return p2p_multi_stage(plan, (const float2*)lambda, nrhs, ld, s);
     if (plan->layout == P2P_LAYOUT_REPETITION) {
         // every target's record gets its own copy of its sources' strengths (the record head: 0)
@@ -347,7 +363,9 @@ P2P_API p2p_status p2p_apply_staged(const p2p_plan* plan, void* out, int32_t nrh
     if (plan->two_sets)
         P2P_TRY_CUDA(cudaMemset2DAsync(out, (size_t)ld * 8, 0, (size_t)nrhs * 8, (size_t)plan->n, s), "p2p_apply/zero");
     if (plan->n_src == 0) return P2P_OK;
-    if (is_tc(path)) return p2p_apply_tc(plan, (float2*)out, nrhs, ld, adjoint, tc_parts(path), s);
+    if (is_tc(path))
+        return (tc_by_box(plan, nrhs, tc_parts(path)) ? p2p_tcb_apply : p2p_apply_tc)(plan, (float2*)out, nrhs, ld, adjoint,
+                                                                                      tc_parts(path), s);
     if (plan->layout == P2P_LAYOUT_REPETITION) {
         const float k = adjoint ? -plan->k : plan->k;
         const unsigned blocks = (unsigned)((plan->n + 255) / 256);

@@ -124,6 +124,12 @@ struct p2p_plan {
     uint8_t* tc_member;     // [n] box number in its block of every sorted target
     unsigned int* tc_counter;  // [2] unit counter and CTA count of a running launch, zero between launches
     unsigned char* tc_pack; // per-apply group records: BF16 part images of the strengths, source coordinates
+    // tensor-core path by single boxes (p2p_tc_box.cu), where p2p_tcb_planned: null otherwise
+    int32_t* tcb_gstart;    // [nbs + 1] first 16-source group of every source box
+    int32_t tcb_groups;     // bound of the groups: records of one launch in tc_pack
+    int32_t* tcb_glist_off; // [nb + 1] offsets of the per-box group lists
+    int32_t* tcb_glist;     // per box: the groups of its neighbour boxes (ascending box id), padded to four with -1
+    int32_t* tcb_gcount;    // [nb] groups in the list of every box (without padding)
     int32_t tc_wait_polls;  // poll bound of the tensor-core pipeline's waits, -1: the default (a self-check
                             // lowers it to make the abort path run)
     // box-group kernel (p2p_group.cu; indexed layout, one right-hand side): kGroupBoxes consecutive target boxes
@@ -150,6 +156,17 @@ size_t p2p_tc_pack_bytes(int64_t n, int32_t max_nrhs);
 int32_t p2p_tc_block_count(int32_t nb);
 int64_t p2p_tc_unit_bound(int64_t n, int32_t nb);
 inline size_t p2p_tc_entry_bound(int64_t sources, int64_t nnz) { return (size_t)(sources / 16 + 2 * nnz + 4); }
+
+int p2p_tc_launch_rhs(int32_t nrhs);
+
+// The tensor-core kernel with one target box per unit (p2p_tc_box.cu) serves the calls that p2p_tc_by_box names: plans of
+// up to kTcBoxTargets targets, and three parts with more than 32 right-hand sides per launch.
+constexpr int64_t kTcBoxTargets = 40000;
+inline bool p2p_tcb_planned(int64_t n, int32_t max_nrhs) { return max_nrhs >= 16 && (n < kTcBoxTargets || max_nrhs > 32); }
+size_t p2p_tcb_pack_bytes(int64_t n, int32_t nb, int32_t max_nrhs);
+inline size_t p2p_tcb_list_bound(int64_t sources, int64_t nnz, int32_t nb) {
+    return (size_t)(sources / 16 + nnz + 3 * (int64_t)nb + 4);
+}
 
 // Several right-hand sides in FP32 (p2p_multi.cu): staged columns of nrhs right-hand sides.
 int32_t p2p_multi_columns(int32_t nrhs);

@@ -29,6 +29,7 @@ cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* 
 
 // Tensor-core lists (p2p_tc.cu).
 cudaError_t p2p_tc_build(p2p_plan* p, int32_t* bound, int32_t* units, void* scan_ws, cudaStream_t s);
+cudaError_t p2p_tcb_build(p2p_plan* p, int32_t* scratch, void* scan_ws, cudaStream_t s);
 
 namespace {
 
@@ -792,7 +793,13 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
         L.p.tc_masks = c.take<uint32_t>(entries * 16);
         L.p.tc_member = c.take<uint8_t>(m);
         L.p.tc_counter = c.take<unsigned int>(2);
-        L.p.tc_pack = c.take<unsigned char>(tc_bytes);
+        const bool by_box = p2p_tcb_planned((int64_t)m, max_nrhs);
+        const size_t box_bytes = by_box ? p2p_tcb_pack_bytes((int64_t)ms, (int32_t)mbs, max_nrhs) : 0;
+        L.p.tc_pack = c.take<unsigned char>(tc_bytes > box_bytes ? tc_bytes : box_bytes);
+        L.p.tcb_gstart = by_box ? c.take<int32_t>(mbs + 1) : nullptr;
+        L.p.tcb_glist_off = by_box ? c.take<int32_t>(mb + 1) : nullptr;
+        L.p.tcb_gcount = by_box ? c.take<int32_t>(mb) : nullptr;
+        L.p.tcb_glist = by_box ? c.take<int32_t>(p2p_tcb_list_bound(sources, nnz, (int32_t)mb)) : nullptr;
     }
     const size_t mx = mb > mbs ? mb : mbs;
     L.n_chunks = c.take<int32_t>(mx);
@@ -1196,6 +1203,10 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     }
     if (p->tc_pack)  // n_chunks and padded are free once the items are built
         FAIL_CUDA(p2p_tc_build(p, L.n_chunks, L.padded, L.scan_ws, s), "p2p_plan_create/tc_lists");
+    if (p->tcb_gstart) {
+        p->tcb_groups = (int32_t)(p->n_src / 16 + p->nbs);
+        FAIL_CUDA(p2p_tcb_build(p, L.n_chunks, L.scan_ws, s), "p2p_plan_create/tc_box_lists");
+    }
     // direct kernel: one item per target box (the item-sort scratch is free again)
     p->direct_k = 0;
     if (layout != P2P_LAYOUT_SYMMETRIC && layout != P2P_LAYOUT_REPETITION) {

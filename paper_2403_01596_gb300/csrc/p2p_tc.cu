@@ -54,7 +54,7 @@
 // right-hand sides the small products (all but hi.hi) have accumulators of their
 // own.  The tensor core's FP32 accumulation truncates, ~2^-26 of the accumulator
 // per MMA in the same direction, so chains are kept short: a unit's list is cut
-// into near-equal segments (segment_entries), and the epilogue adds the segments in
+// into near-equal segments (kSegment), and the epilogue adds the segments in
 // FP32.
 //
 // Every wait is bounded: a wait that runs out sets the plan's status word and an
@@ -86,11 +86,11 @@ constexpr int kRows = 128;             // targets per unit (MMA M)
 constexpr int kBlockBoxes = 32;        // target boxes per list block (a bit each)
 constexpr int kSets = 4;               // G sets; set s takes entries s, s + kSets, ...
 // Entries added up in one accumulator chain at most.  With accumulators of their own for the small products (at most
-// 32 right-hand sides) a chain takes one truncated addition per entry, otherwise every product of the split: 3 for
-// hi / lo, whose products are far less exact than that, and 6 for the three-part split, which at 48 entries measured
-// 1.3e-6 of S_i on boxes of ~140 points (the split promises 2^-20) and at 16 still 1.4 times the relative error of
-// chains of ~55 additions (1.1e-6 against 7.8e-7).
-__host__ __device__ inline int segment_entries(int rhs, int np) { return np == 3 && rhs > 32 ? 10 : 48; }
+// 32 right-hand sides) a chain takes one truncated addition per entry, otherwise the 3 products of hi / lo, which are far
+// less exact than that.  (Six products per entry would need segments of 6 to 8 entries to be as exact as chains of ~55
+// additions, and the epilogue's share makes that slower than one box per unit: 2^21-point ellipsoid, 64 right-hand sides
+// 7.4 ms against 6.9.  p2p_tc_box.cu takes those calls.)
+constexpr int kSegment = 48;
 constexpr int kAColumn = 256;          // first TMEM column of the operand slots
 constexpr int kMmaWarp0 = 1, kScoutWarp = 3, kEpiWarp0 = 4, kGWarp0 = 8;
 constexpr int kWarps = kGWarp0 + 4 * kSets;
@@ -692,7 +692,7 @@ __device__ void run_scout(const TcArgs& a, const TcSmem& sm, int lane) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(P2P_FULL_MASK, cnt, o);
             if (cnt == 0) continue;  // two point sets, no source nearby: the rows keep the zeros written before the launch
-            const int most = segment_entries(a.rhs, NP), segments = (cnt + most - 1) / most;
+            const int segments = (cnt + kSegment - 1) / kSegment;
             h0 = make_int4(b0, t0, nt, cnt);
             h1 = make_int4(off, E, (int)want, (cnt + segments - 1) / segments);
         }
@@ -1322,6 +1322,8 @@ int64_t source_groups(int64_t n) { return (n + kSrcGroup - 1) / kSrcGroup; }
 }  // namespace
 
 int32_t p2p_tc_block_count(int32_t nb) { return (nb + kBlockBoxes - 1) / kBlockBoxes; }
+int p2p_tc_launch_rhs(int32_t nrhs) { return launch_rhs(nrhs); }
+
 int64_t p2p_tc_unit_bound(int64_t n, int32_t nb) { return n / kRows + p2p_tc_block_count(nb) + 1; }
 
 // Room for the records of either split (sized for three parts), launch by launch.
