@@ -89,3 +89,26 @@ def test_strength_that_is_not_finite_stays_local(path, nrhs):
     assert plan.async_status() == 0
     assert np.isnan(out.real[hit]).all() and np.isnan(out.imag[hit]).all()
     assert np.array_equal(out[~hit], clean[~hit])
+
+
+@pytest.mark.parametrize("n,ng", [(15, 1), (17, 1), (128, 1), (129, 1), (400, 1), (3800, 3), (170, 4), (900, 10)])
+@pytest.mark.parametrize("kernel,path,widths", [("helmholtz", "tc_bf16x3", (1, 33, 67)), ("laplace", "tc_bf16x3", (9, 64)),
+                                                ("helmholtz", "tc_bf16x6", (1, 9, 32)), ("laplace", "tc_bf16x6", (24,))])
+def test_tiles_in_a_large_plan(n, ng, kernel, path, widths):
+    """The same boxes in the corner of a plan of 42 000 more points, about one per box, so that it is large enough for
+    units of 128 targets."""
+    api = _api()
+    rng = np.random.default_rng(n + ng)
+    ng2, h = ng + 42, 1.0 / ng
+    far = rng.random((42000, 3)) * [ng2, ng2, 40] + [0, 0, ng + 2]  # in cells, at least two cells from the corner's boxes
+    pts = np.concatenate([rng.random((n, 3)), far * h]).astype(np.float32)
+    lo, k, m = (0.0, 0.0, 0.0), (float(np.float32(2 * np.pi * ng / 5)) if kernel == "helmholtz" else 0.0), len(pts)
+    kid = oracle.HELMHOLTZ if kernel == "helmholtz" else oracle.LAPLACE
+    plan = api.Plan(torch.from_numpy(pts).cuda(), lo, h, ng2, k, kernel=kernel, max_nrhs=67)
+    for nrhs in widths:
+        lam = W.strengths(m, nrhs, n + nrhs).reshape(m, nrhs)
+        out = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+        assert plan.async_status() == 0
+        ref = oracle.p2p(pts, lam, lo, h, ng2, k, kernel=kid).reshape(m, nrhs)
+        S = oracle.p2p(pts, np.abs(lam).astype(np.complex64), lo, h, ng2, 0.0, kernel=oracle.LAPLACE).real.reshape(m, nrhs)
+        assert _worst(out, ref, S) <= DELTA[path], (nrhs, _worst(out, ref, S))
