@@ -18,7 +18,7 @@ between timed steps, outside the timed events.
 
 After the timed steps (outside them) the default run adds two sub-records to
 its line: `redundant` -- the same sweep through the redundant layout of Sec.
-3.3 (per-occupancy repack and pair-kernel times, the pair kernel against the
+3.3 (per-occupancy staging and pair-kernel times, the pair kernel against the
 MUFU roofline, and the apply against its binding term, HBM or MUFU) -- and
 `multirhs` -- the 2:1:1 ellipsoid (2^21 points, 64 right-hand sides): the
 tensor-core path against the per-RHS and shared-G FP32 paths, rel-L2 per RHS
@@ -725,11 +725,11 @@ def measure_multirhs(scale, steps, samples, free_first=()):
 
 
 def measure_redundant(wls, pts, structures, pairs, steps, flush, peaks, sms):
-    """The redundant layout (Sec. 3.3: per-box copies of each neighbourhood's coordinates, strengths repacked
-    every apply) on the occupancy sweep: per occupancy the repack and pair-kernel times (CUDA events, L2
-    flushed before each apply), the apply rate, the pair kernel against R_MUFU, and the binding term of the
-    whole apply: max(P / R_MUFU, bytes / HBM) with bytes = packed (16 + 8) + n (8 + 8) for the pair kernel and
-    packed (4 + 8 + 8) for the repack."""
+    """The redundant layout (Sec. 3.3: per-box copies of each neighbourhood's coordinates, strengths gathered
+    through the lists) on the occupancy sweep: per occupancy the staging (repack_ms) and pair-kernel times (CUDA
+    events, L2 flushed before each apply), the apply rate, the pair kernel against R_MUFU, and the binding term of
+    the whole apply: max(P / R_MUFU, bytes / HBM) with bytes = packed (16 + 4) + n (8 + 8) for the pair kernel and
+    n (4 + 8 + 8) for the staging."""
     import torch
     from paper_2403_01596_gb300 import _capi as C
     from paper_2403_01596_gb300 import api, workloads as W
@@ -759,8 +759,8 @@ def measure_redundant(wls, pts, structures, pairs, steps, flush, peaks, sms):
         stage_ms = statistics.mean(e[0].elapsed_time(e[1]) for e in evs)
         pair_ms = statistics.mean(e[1].elapsed_time(e[2]) for e in evs)
         packed = int(st.sources)  # sum over boxes of the sources in each neighbourhood (the per-box copies)
-        kbytes = packed * (16 + 8) + wl.n * (8 + 8)
-        rbytes = packed * (4 + 8 + 8)
+        kbytes = packed * (16 + 4) + wl.n * (8 + 8)
+        rbytes = wl.n * (4 + 8 + 8)
         t_mufu, t_hbm = P / r_mufu, (kbytes + rbytes) / hbm
         t_apply = (stage_ms + pair_ms) * 1e-3
         rows.append({"occupancy": wl.meta["target_occupancy"], "pairs": P, "packed": packed,
