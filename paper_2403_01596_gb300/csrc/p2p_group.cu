@@ -583,8 +583,8 @@ GroupArgs group_args(const p2p_plan* p) {
 // keys / vals / keys_alt / vals_alt / radix_ws: sort scratch of at least n_groups entries.  The largest union and the
 // largest group list total are in cap[0], cap[1] once the stream has come this far.
 cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* nbr_idx, uint32_t* keys,
-                            int32_t* vals, uint32_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
-                            cudaStream_t s, int32_t* cap) {
+                            int32_t* vals, uint32_t* keys_alt, int32_t* vals_alt, void* radix_ws, size_t radix_bytes,
+                            int32_t* maxes, cudaStream_t s, int32_t* cap) {
     cap[0] = cap[1] = 0;
     const int32_t ng = p->n_groups;
     if (ng == 0) return cudaSuccess;
@@ -597,7 +597,7 @@ cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     bool in_alt = false;
-    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, ng, kCostBits, radix_ws, s, &in_alt);
+    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, ng, kCostBits, radix_ws, radix_bytes, s, &in_alt);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(p->g_order, in_alt ? vals_alt : vals, (size_t)ng * sizeof(int32_t), cudaMemcpyDeviceToDevice,
                         s);

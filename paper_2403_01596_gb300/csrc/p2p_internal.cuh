@@ -214,10 +214,11 @@ cudaError_t scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32
                                cudaStream_t s);
 
 // Stable LSD radix sort of (key, int32 value) pairs on the low `bits` bits of 32- or 64-bit keys.
+// radix_workspace_bytes(n) is enough for every count up to n; less than a sort needs is cudaErrorInvalidValue.
 size_t radix_workspace_bytes(int64_t n);
 template <typename K>
 cudaError_t radix_sort_pairs(K* keys, int32_t* vals, K* keys_alt, int32_t* vals_alt, int64_t n, int bits, void* work,
-                             cudaStream_t s, bool* result_in_alt);
+                             size_t work_bytes, cudaStream_t s, bool* result_in_alt);
 
 // Sort key that puts the expensive (targets x sources) first, Bits wide: 8 bits are an eighth of a power of two wide,
 // so one radix pass orders work items and groups, those of one bucket in the order of their boxes; 16 bits order the

@@ -24,8 +24,8 @@ using namespace p2p_detail;
 
 // Box-group kernel tables (p2p_group.cu).
 cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* nbr_idx, uint32_t* keys,
-                            int32_t* vals, uint32_t* keys_alt, int32_t* vals_alt, void* radix_ws, int32_t* maxes,
-                            cudaStream_t s, int32_t* cap);
+                            int32_t* vals, uint32_t* keys_alt, int32_t* vals_alt, void* radix_ws, size_t radix_bytes,
+                            int32_t* maxes, cudaStream_t s, int32_t* cap);
 
 // Tensor-core lists (p2p_tc.cu).
 cudaError_t p2p_tc_build(p2p_plan* p, int32_t* bound, int32_t* units, void* scan_ws, cudaStream_t s);
@@ -576,7 +576,7 @@ struct BinLayout {
     uint64_t *keys, *keys_alt;
     int32_t *vals, *vals_alt, *heads, *first, *small;
     void *radix_ws, *scan_ws;
-    size_t bytes;
+    size_t radix_bytes, bytes;
 };
 
 BinLayout bin_layout(int64_t n, void* work) {
@@ -590,7 +590,8 @@ BinLayout bin_layout(int64_t n, void* work) {
     L.heads = c.take<int32_t>((size_t)head_blocks((int64_t)m));
     L.first = c.take<int32_t>((size_t)head_blocks((int64_t)m));
     L.small = c.take<int32_t>(4);
-    L.radix_ws = c.take<char>(radix_workspace_bytes(n));
+    L.radix_bytes = radix_workspace_bytes(n);
+    L.radix_ws = c.take<char>(L.radix_bytes);
     L.scan_ws = c.take<char>(scan_workspace_bytes(head_blocks((int64_t)m)));
     L.bytes = align_up(c.off, 256);
     return L;
@@ -616,7 +617,7 @@ cudaError_t bin_sorted(const BinLayout& L, const float* pts, int64_t n, const do
     k_keys<K><<<blocks_for(n, kThreads), kThreads, 0, s>>>(pts, n, g[0], g[1], g[2], ng, keys, L.vals, L.small);
     cudaError_t e = cudaGetLastError();
     bool in_alt = false;
-    if (e == cudaSuccess) e = radix_sort_pairs(keys, L.vals, keys_alt, L.vals_alt, n, bits, L.radix_ws, s, &in_alt);
+    if (e == cudaSuccess) e = radix_sort_pairs(keys, L.vals, keys_alt, L.vals_alt, n, bits, L.radix_ws, L.radix_bytes, s, &in_alt);
     if (e != cudaSuccess) return e;
     const K* ks = in_alt ? keys_alt : keys;
     const int32_t* vs = in_alt ? L.vals_alt : L.vals;
@@ -728,7 +729,7 @@ struct PlanLayout {
     uint32_t *keys, *keys_alt;
     int32_t *vals, *vals_alt;
     void* radix_ws;
-    size_t bytes;
+    size_t radix_bytes, bytes;
 };
 
 // Sizes of a plan: n targets in nb boxes, n_src sources in nbs boxes (two_sets), sources = sum of S_b.
@@ -817,7 +818,8 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     sc.take<uint32_t>(max_items);
     sc.take<int32_t>(max_items);
     sc.take<int32_t>(max_items);
-    sc.take<char>(radix_workspace_bytes((int64_t)max_items));
+    L.radix_bytes = radix_workspace_bytes((int64_t)max_items);
+    sc.take<char>(L.radix_bytes);
     Carver& cs = (sc.off <= lam_bytes) ? sc : c;
     if (&cs == &sc) sc.off = 0;
     L.recs = cs.take<ItemRec>(max_items);
@@ -825,7 +827,7 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     L.keys_alt = cs.take<uint32_t>(max_items);
     L.vals = cs.take<int32_t>(max_items);
     L.vals_alt = cs.take<int32_t>(max_items);
-    L.radix_ws = cs.take<char>(radix_workspace_bytes((int64_t)max_items));
+    L.radix_ws = cs.take<char>(L.radix_bytes);
     L.bytes = align_up(c.off, 256);
     return L;
 }
@@ -1195,7 +1197,7 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     if (items > 0) {
         bool in_alt = false;
         FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, items, fine ? kFineCostBits : kCostBits,
-                                   L.radix_ws, s, &in_alt),
+                                   L.radix_ws, L.radix_bytes, s, &in_alt),
                   "p2p_plan_create/sort");
         k_item_gather<<<blocks_for(items, kThreads), kThreads, 0, s>>>(L.recs, in_alt ? L.vals_alt : L.vals, items,
                                                                        p->items);
@@ -1218,7 +1220,7 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
                                                                          nb, 32 / wb, L.recs, L.keys, L.vals);
             FAIL_CUDA(cudaGetLastError(), "p2p_plan_create/direct_items");
             bool in_alt = false;
-            FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, nb, kFineCostBits, L.radix_ws, s, &in_alt),
+            FAIL_CUDA(radix_sort_pairs(L.keys, L.vals, L.keys_alt, L.vals_alt, nb, kFineCostBits, L.radix_ws, L.radix_bytes, s, &in_alt),
                       "p2p_plan_create/direct_sort");
             k_item_gather<<<blocks_for(nb, kThreads), kThreads, 0, s>>>(L.recs, in_alt ? L.vals_alt : L.vals, nb,
                                                                         p->ditems);
@@ -1238,7 +1240,7 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     if (p->tune.warp_boxes == -2) {
         p->n_groups = (nb + kGroupBoxes - 1) / kGroupBoxes;
         FAIL_CUDA(p2p_group_build(p, in.nbr_ptr, in.nbr_idx, L.keys, L.vals, L.keys_alt, L.vals_alt, L.radix_ws,
-                                  L.maxes, s, cap),
+                                  L.radix_bytes, L.maxes, s, cap),
                   "p2p_plan_create/groups");
     }
     // the plan is complete when this returns: later calls may use it on any stream

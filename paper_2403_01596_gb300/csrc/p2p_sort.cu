@@ -85,8 +85,10 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kMaxSub = 16;  // keys per thread at most
 
-__host__ __device__ inline int sort_sub(int64_t n) { return n <= (1 << 18) ? 4 : (n <= (1 << 22) ? 8 : kMaxSub); }
-__host__ __device__ inline int64_t sort_tiles(int64_t n) {
+constexpr int64_t kSortSteps[2] = {1 << 18, 1 << 22};  // largest counts with 4 and with 8 keys per thread
+
+inline int sort_sub(int64_t n) { return n <= kSortSteps[0] ? 4 : (n <= kSortSteps[1] ? 8 : kMaxSub); }
+inline int64_t sort_tiles(int64_t n) {
     const int64_t tile = (int64_t)kSortThreads * sort_sub(n);
     return n > 0 ? (n + tile - 1) / tile : 1;
 }
@@ -234,15 +236,24 @@ cudaError_t scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32
     return cudaGetLastError();
 }
 
+// Scratch of one sort of n pairs: counts of every tile, totals of every digit.
+static size_t radix_need_bytes(int64_t n) { return align_up((size_t)sort_tiles(n) * kRadix * 4, 256) + kRadix * 4; }
+
+// A plan sizes its scratch for a bound and sorts the pairs there are, and the larger tiles past a step need less than
+// the smaller ones before it (262 144 keys 256 tiles, 262 145 keys 129): the most of all counts up to n.
 size_t radix_workspace_bytes(int64_t n) {
-    return align_up((size_t)sort_tiles(n) * kRadix * 4, 256) + kRadix * 4;
+    size_t most = radix_need_bytes(n);
+    for (const int64_t step : kSortSteps)
+        if (n > step && radix_need_bytes(step) > most) most = radix_need_bytes(step);
+    return most;
 }
 
 template <typename K>
 cudaError_t radix_sort_pairs(K* keys, int32_t* vals, K* keys_alt, int32_t* vals_alt, int64_t n, int bits, void* work,
-                             cudaStream_t s, bool* result_in_alt) {
+                             size_t work_bytes, cudaStream_t s, bool* result_in_alt) {
     *result_in_alt = false;
     if (n <= 1 || bits <= 0) return cudaSuccess;
+    if (work_bytes < radix_need_bytes(n)) return cudaErrorInvalidValue;
     const int64_t tiles = sort_tiles(n);
     const int sub = sort_sub(n);
     int32_t* hist = static_cast<int32_t*>(work);
@@ -269,9 +280,9 @@ cudaError_t radix_sort_pairs(K* keys, int32_t* vals, K* keys_alt, int32_t* vals_
     return cudaSuccess;
 }
 
-template cudaError_t radix_sort_pairs<uint64_t>(uint64_t*, int32_t*, uint64_t*, int32_t*, int64_t, int, void*,
+template cudaError_t radix_sort_pairs<uint64_t>(uint64_t*, int32_t*, uint64_t*, int32_t*, int64_t, int, void*, size_t,
                                                 cudaStream_t, bool*);
-template cudaError_t radix_sort_pairs<uint32_t>(uint32_t*, int32_t*, uint32_t*, int32_t*, int64_t, int, void*,
+template cudaError_t radix_sort_pairs<uint32_t>(uint32_t*, int32_t*, uint32_t*, int32_t*, int64_t, int, void*, size_t,
                                                 cudaStream_t, bool*);
 
 }  // namespace p2p_detail
