@@ -102,8 +102,8 @@ typedef enum {
     P2P_PATH_AUTO = 0,        /* FP32 shared-G for nrhs < 16, tensor-core path otherwise (when available) */
     P2P_PATH_FP32_PER_RHS = 1,/* FP32; G re-evaluated for every right-hand side */
     P2P_PATH_FP32_SHARED = 2, /* FP32; each G evaluated once and applied to up to 8 RHS at a time */
-    P2P_PATH_TC_BF16X3 = 3,   /* G tile and strengths split into BF16 hi + lo, 3 tcgen05 MMAs per 16
-                                 sources, FP32 accumulation in tensor memory; plans with max_nrhs >= 16
+    P2P_PATH_TC_BF16X3 = 3,   /* G tile and strengths split into BF16 hi + lo, 3 or 4 tcgen05 MMAs per
+                                 16 sources, FP32 accumulation in tensor memory; plans with max_nrhs >= 16
                                  on an sm_103 device, else P2P_ERR_UNSUPPORTED */
     P2P_PATH_TC_BF16X6 = 4    /* as P2P_PATH_TC_BF16X3 with three BF16 parts (hi + mid + lo, ~24 bits)
                                  and the 6 MMAs whose part products are not below 2^-24 of the term:

@@ -12,9 +12,10 @@
 // and Im out[t, r] = D1[t, R + r] + D2[t, r].  The Laplace kernel needs D1 alone.
 // G is formed on the CUDA cores in FP32 (rsqrt, sincos), both operands are split
 // x = hi + lo into BF16, and three products (hi.hi + hi.lo + lo.hi, kind::f16,
-// FP32 accumulation in TMEM) keep the product error near 2^-16.  With NP = 3 parts
-// (hi + mid + lo, ~24 bits) six products take every p.q with p + q < 3, and the
-// product error is near 2^-24.
+// FP32 accumulation in TMEM) keep the product error near 2^-16; with more than 32
+// right-hand sides lo.lo is added as well, which pays for the longer chains there
+// (kSegment).  With NP = 3 parts (hi + mid + lo, ~24 bits) six products take every
+// p.q with p + q < 3, and the product error is near 2^-24.
 //
 // Why this shape.  G is the MMA's A operand and goes from registers straight into
 // tensor memory: a thread owns one target (one TMEM lane), reads the entry's
@@ -54,8 +55,8 @@
 // right-hand sides the small products (all but hi.hi) have accumulators of their
 // own.  The tensor core's FP32 accumulation truncates, ~2^-26 of the accumulator
 // per MMA in the same direction, so chains are kept short: a unit's list is cut
-// into near-equal segments (kSegment), and the epilogue adds the segments in
-// FP32.
+// into near-equal segments (kSegment, kSegmentWide), and the epilogue adds the
+// segments in FP32.
 //
 // Every wait is bounded: a wait that runs out sets the plan's status word and an
 // abort flag; every role then stops, the producer waits (bounded) for the bulk
@@ -86,11 +87,19 @@ constexpr int kRows = 128;             // targets per unit (MMA M)
 constexpr int kBlockBoxes = 32;        // target boxes per list block (a bit each)
 constexpr int kSets = 4;               // G sets; set s takes entries s, s + kSets, ...
 // Entries added up in one accumulator chain at most.  With accumulators of their own for the small products (at most
-// 32 right-hand sides) a chain takes one truncated addition per entry, otherwise the 3 products of hi / lo, which are far
-// less exact than that.  (Six products per entry would need segments of 6 to 8 entries to be as exact as chains of ~55
-// additions, and the epilogue's share makes that slower than one box per unit: 2^21-point ellipsoid, 64 right-hand sides
-// 7.4 ms against 6.9.  p2p_tc_box.cu takes those calls.)
-constexpr int kSegment = 48;
+// 32 right-hand sides) a chain takes one truncated addition per entry.  Wider launches have no TMEM left for that: every
+// product of an entry is a truncated addition to the one accumulator, and with the three of hi / lo the error came out
+// above that of the split alone even with short segments.  The fourth product, lo.lo, takes the split's own error from 4.4e-6
+// to 3.5e-6, more than those additions cost, and the issuers have time for it (a G set takes ~750 cycles for an entry, its
+// MMAs 384, 512 with the fourth).  Relative L2 error / time, 64 right-hand sides on 200 003 sphere points at 20
+// per box and on the 2^21-point ellipsoid, entries per segment x products:
+//   48 x 3  4.53e-6 331 us, 5.00e-6 3556 us      16 x 3  4.47e-6 401 us, 5.06e-6 4340 us   (split alone 4.4e-6)
+//   48 x 4  3.65e-6 346 us, 3.70e-6 3673 us      64 x 4  3.74e-6 332 us, 3.80e-6 3546 us
+//   96 x 4  3.77e-6 319 us, 3.94e-6 3372 us; at 47 points per box, 40 right-hand sides 4.39e-6 (64 x 4: 3.93e-6)
+// (Six products per entry would need segments of 6 to 8 entries to be as exact as chains of ~55 additions, and the
+// epilogue's share makes that slower than one box per unit: 2^21-point ellipsoid, 64 right-hand sides 7.4 ms against 6.9.
+// p2p_tc_box.cu takes those calls.)
+constexpr int kSegment = 48, kSegmentWide = 64;
 constexpr int kAColumn = 256;          // first TMEM column of the operand slots
 constexpr int kMmaWarp0 = 1, kScoutWarp = 3, kEpiWarp0 = 4, kGWarp0 = 8;
 constexpr int kWarps = kGWarp0 + 4 * kSets;
@@ -692,7 +701,8 @@ __device__ void run_scout(const TcArgs& a, const TcSmem& sm, int lane) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(P2P_FULL_MASK, cnt, o);
             if (cnt == 0) continue;  // two point sets, no source nearby: the rows keep the zeros written before the launch
-            const int segments = (cnt + kSegment - 1) / kSegment;
+            const int most = a.rhs <= 32 ? kSegment : kSegmentWide;
+            const int segments = (cnt + most - 1) / most;
             h0 = make_int4(b0, t0, nt, cnt);
             h1 = make_int4(off, E, (int)want, (cnt + segments - 1) / segments);
         }
@@ -923,16 +933,18 @@ __device__ void run_mma(const TcArgs& a, const TcSmem& sm, uint32_t tmem, int q)
     const uint64_t part = (uint64_t)(image_bytes(a.rhs) >> 4);
     const uint32_t d_hh = tmem + (uint32_t)q * 128u;                 // hi.hi
     const uint32_t d_x = a.rhs <= 32 ? d_hh + 64u : d_hh;            // the smaller products
-    const uint32_t own_x = a.rhs <= 32 ? 0u : 1u;
+    const uint32_t one_x = a.rhs <= 32 ? 0u : 1u;                    // 1: they share the accumulator of hi.hi
     const uint32_t ga_all = tmem + (uint32_t)kAColumn + 8u * (uint32_t)q, a_mask = (uint32_t)(a.a_slots - 1);
     const int lane = threadIdx.x & 31;
     // The products of one entry (the elected lane): every product of parts p (of G) and r (of lambda) with
-    // p + r < NP; the dropped ones are below 2^-8 NP of the leading one.
+    // p + r < NP, and lo.lo of a wide hi / lo launch; the dropped ones are below 2^-8 NP of the leading one.
     auto issue = [&](uint32_t ga, uint64_t lb, uint32_t acc, uint64_t* done) {
         mma_bf16_ts(d_hh, ga, lb, idesc, acc);
-        mma_bf16_ts(d_x, ga, lb + part, idesc, acc | own_x);
+        mma_bf16_ts(d_x, ga, lb + part, idesc, acc | one_x);
         mma_bf16_ts(d_x, ga + 16u, lb, idesc, 1u);
-        if constexpr (NP == 3) {
+        if constexpr (NP == 2) {
+            if (one_x) mma_bf16_ts(d_x, ga + 16u, lb + part, idesc, 1u);
+        } else {
             mma_bf16_ts(d_x, ga, lb + 2 * part, idesc, 1u);
             mma_bf16_ts(d_x, ga + 16u, lb + part, idesc, 1u);
             mma_bf16_ts(d_x, ga + 32u, lb, idesc, 1u);
@@ -1166,7 +1178,7 @@ __device__ void run_epilogue(const TcArgs& a, const TcSmem& sm, uint32_t tmem, i
 }
 
 // LIMITED: the waits poll at most a.wait_limit times (the abort-path self-check); otherwise kWaitLimit.
-// NP: BF16 parts per operand (2: three products per entry and chain, 3: six).
+// NP: BF16 parts per operand (2: three or four products per entry and chain, 3: six).
 template <int KERN, bool LIMITED, int NP>
 __global__ void __launch_bounds__(kThreads, 1) k_p2p_tc(const __grid_constant__ TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
