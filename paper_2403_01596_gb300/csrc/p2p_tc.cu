@@ -280,18 +280,25 @@ __device__ __forceinline__ uint32_t pack_bf16(float2 v) {
 // v - w, exactly where w is v's rounding (one packed operation).
 __device__ __forceinline__ float2 residual(float2 v, float2 w) { return __ffma2_rn(w, make_float2(-1.f, -1.f), v); }
 
-// x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.
+// The largest finite BF16 value.  A finite strength above it (up to 0.4 % below the FP32 maximum) would round to infinity,
+// and 0 x inf reaches targets that are not its neighbours; capped, the next part holds the rest of it.
+constexpr float kBf16Max = 3.3895313892515355e38f;
+__device__ __forceinline__ float capped(float x) { return isfinite(x) ? fminf(fmaxf(x, -kBf16Max), kBf16Max) : x; }
+
+// x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.  CAP: any finite x.
+template <bool CAP = false>
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
     const float2 v = make_float2(a, b);
-    hi = pack_bf16(v);
+    hi = pack_bf16(CAP ? make_float2(capped(a), capped(b)) : v);
     lo = pack_bf16(residual(v, unpack_bf16(hi)));
 }
 
 // x = hi + mid + lo with three BF16 parts (each the round-to-nearest of what the
 // previous parts leave), two values per 32-bit word: the parts carry ~24 bits.
+template <bool CAP = false>
 __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
     const float2 v = make_float2(a, b);
-    hi = pack_bf16(v);
+    hi = pack_bf16(CAP ? make_float2(capped(a), capped(b)) : v);
     const float2 r = residual(v, unpack_bf16(hi));
     mid = pack_bf16(r);
     lo = pack_bf16(residual(r, unpack_bf16(mid)));
@@ -302,15 +309,15 @@ __host__ __device__ inline int op_off(int row, int k) {
     return (row >> 3) * kSbo + (k >> 3) * kLbo + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// Splits eight consecutive K elements of one row into NP BF16 parts (2: hi, lo; 3: hi, mid, lo) stored at `off`
+// Splits eight consecutive K elements (strengths) of one row into NP BF16 parts (2: hi, lo; 3: hi, mid, lo) stored at `off`
 // in the images starting at part0, part_bytes apart.
 template <int NP>
 __device__ __forceinline__ void store_parts(unsigned char* part0, int part_bytes, int off, const float (&v)[8]) {
     uint32_t p[NP][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        if constexpr (NP == 2) split2(v[2 * i], v[2 * i + 1], p[0][i], p[1][i]);
-        else split3(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
+        if constexpr (NP == 2) split2<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i]);
+        else split3<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
     }
 #pragma unroll
     for (int q = 0; q < NP; ++q)

@@ -214,9 +214,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.
+// The largest finite BF16 value.  A finite strength above it (up to 0.4 % below the FP32 maximum) would round to infinity,
+// and inf - inf makes NaN of its neighbours' sums; capped, the next part holds the rest of it.
+constexpr float kBf16Max = 3.3895313892515355e38f;
+__device__ __forceinline__ float capped(float x) { return isfinite(x) ? fminf(fmaxf(x, -kBf16Max), kBf16Max) : x; }
+
+// x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.  CAP: any finite x.
+template <bool CAP = false>
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    __nv_bfloat162 h = __floats2bfloat162_rn(CAP ? capped(a) : a, CAP ? capped(b) : b);
     float2 hf = __bfloat1622float2(h);
     __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
     hi = *reinterpret_cast<uint32_t*>(&h);
@@ -225,8 +231,9 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 
 // x = hi + mid + lo with three BF16 parts (each the round-to-nearest of what the
 // previous parts leave), two values per 32-bit word: the parts carry ~24 bits.
+template <bool CAP = false>
 __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    __nv_bfloat162 h = __floats2bfloat162_rn(CAP ? capped(a) : a, CAP ? capped(b) : b);
     const float2 hf = __bfloat1622float2(h);
     const float ra = a - hf.x, rb = b - hf.y;
     __nv_bfloat162 m = __floats2bfloat162_rn(ra, rb);
@@ -251,7 +258,7 @@ __host__ __device__ inline int op_off(int row, int k) {
 
 // Splits n values (n = 1, 2, 4 or 8, consecutive K elements of one row) and
 // stores the hi and lo parts.
-template <int N>
+template <int N, bool CAP>
 __device__ __forceinline__ void store_split(unsigned char* hi, unsigned char* lo, int off, const float (&v)[N]) {
     if constexpr (N == 1) {
         uint16_t h, l;
@@ -260,21 +267,21 @@ __device__ __forceinline__ void store_split(unsigned char* hi, unsigned char* lo
         *reinterpret_cast<uint16_t*>(lo + off) = l;
     } else if constexpr (N == 2) {
         uint32_t h, l;
-        split2(v[0], v[1], h, l);
+        split2<CAP>(v[0], v[1], h, l);
         *reinterpret_cast<uint32_t*>(hi + off) = h;
         *reinterpret_cast<uint32_t*>(lo + off) = l;
     } else if constexpr (N == 4) {
         uint2 h, l;
-        split2(v[0], v[1], h.x, l.x);
-        split2(v[2], v[3], h.y, l.y);
+        split2<CAP>(v[0], v[1], h.x, l.x);
+        split2<CAP>(v[2], v[3], h.y, l.y);
         *reinterpret_cast<uint2*>(hi + off) = h;
         *reinterpret_cast<uint2*>(lo + off) = l;
     } else {
         uint4 h, l;
-        split2(v[0], v[1], h.x, l.x);
-        split2(v[2], v[3], h.y, l.y);
-        split2(v[4], v[5], h.z, l.z);
-        split2(v[6], v[7], h.w, l.w);
+        split2<CAP>(v[0], v[1], h.x, l.x);
+        split2<CAP>(v[2], v[3], h.y, l.y);
+        split2<CAP>(v[4], v[5], h.z, l.z);
+        split2<CAP>(v[6], v[7], h.w, l.w);
         *reinterpret_cast<uint4*>(hi + off) = h;
         *reinterpret_cast<uint4*>(lo + off) = l;
     }
@@ -283,20 +290,20 @@ __device__ __forceinline__ void store_split(unsigned char* hi, unsigned char* lo
 // Splits n values (n = 2, 4 or 8, consecutive K elements of one row) into NP
 // BF16 parts (2: hi, lo; 3: hi, mid, lo) stored at `off` in the images starting
 // at part0, part_bytes apart.
-template <int NP, int N>
+template <int NP, int N, bool CAP = false>
 __device__ __forceinline__ void store_parts(unsigned char* part0, int part_bytes, int off, const float (&v)[N]) {
     if constexpr (NP == 2) {
-        store_split<N>(part0, part0 + part_bytes, off, v);
+        store_split<N, CAP>(part0, part0 + part_bytes, off, v);
     } else if constexpr (N == 1) {
         uint32_t h, m, l;
-        split3(v[0], 0.f, h, m, l);
+        split3<CAP>(v[0], 0.f, h, m, l);
         *reinterpret_cast<uint16_t*>(part0 + off) = (uint16_t)(h & 0xffffu);
         *reinterpret_cast<uint16_t*>(part0 + part_bytes + off) = (uint16_t)(m & 0xffffu);
         *reinterpret_cast<uint16_t*>(part0 + 2 * part_bytes + off) = (uint16_t)(l & 0xffffu);
     } else {
         uint32_t h[N / 2], m[N / 2], l[N / 2];
 #pragma unroll
-        for (int i = 0; i < N / 2; ++i) split3(v[2 * i], v[2 * i + 1], h[i], m[i], l[i]);
+        for (int i = 0; i < N / 2; ++i) split3<CAP>(v[2 * i], v[2 * i + 1], h[i], m[i], l[i]);
         unsigned char* dst[3] = {part0, part0 + part_bytes, part0 + 2 * part_bytes};
         const uint32_t* src[3] = {h, m, l};
 #pragma unroll
@@ -365,8 +372,8 @@ __global__ void __launch_bounds__(128) k_tcb_pack(const float2* __restrict__ lam
         im[e] = v.y;
     }
     unsigned char* img = rec + lb * NP * kPart;
-    store_parts<NP, 8>(img, kPart, op_off(r, 8 * o), re);
-    store_parts<NP, 8>(img, kPart, op_off(64 + r, 8 * o), im);
+    store_parts<NP, 8, true>(img, kPart, op_off(r, 8 * o), re);
+    store_parts<NP, 8, true>(img, kPart, op_off(64 + r, 8 * o), im);
 }
 
 // ------------------------------------------------------------------ main kernel --

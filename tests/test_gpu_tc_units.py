@@ -112,3 +112,45 @@ def test_tiles_in_a_large_plan(n, ng, kernel, path, widths):
         ref = oracle.p2p(pts, lam, lo, h, ng2, k, kernel=kid).reshape(m, nrhs)
         S = oracle.p2p(pts, np.abs(lam).astype(np.complex64), lo, h, ng2, 0.0, kernel=oracle.LAPLACE).real.reshape(m, nrhs)
         assert _worst(out, ref, S) <= DELTA[path], (nrhs, _worst(out, ref, S))
+
+
+# 58 points per box in a cube: a window of 128 targets covers two or three boxes whose neighbourhoods differ, its list
+# holds more than 64 entries (several segments); one box per unit (4 000 points, or wide three parts) next to it
+@pytest.mark.parametrize("path,nrhs,n,ng", [("tc_bf16x3", 17, 42000, 9), ("tc_bf16x3", 64, 42000, 9), ("tc_bf16x3", 80, 42000, 9),
+                                            ("tc_bf16x6", 17, 42000, 9), ("tc_bf16x6", 32, 42000, 9), ("tc_bf16x6", 64, 42000, 9),
+                                            ("tc_bf16x3", 17, 4000, 4), ("tc_bf16x6", 17, 4000, 4)])
+def test_strengths_at_the_ends_of_fp32(path, nrhs, n, ng):
+    """Infinite and NaN strengths make NaN of their own neighbourhood and right-hand side; the largest finite ones, which
+    round to infinity in BF16, give their neighbours what they are worth; every other result is what it was, bit for bit.
+    Points far enough apart (r > 1) that no term overflows."""
+    api = _api()
+    h = 200.0
+    pts = (np.random.default_rng(n).random((n, 3)) * (ng * h)).astype(np.float32)
+    lo, k = (0.0, 0.0, 0.0), 2 * np.pi / 500.0
+    plan = api.Plan(torch.from_numpy(pts).cuda(), lo, h, ng, k, max_nrhs=nrhs)
+    lam = W.strengths(n, nrhs, 8)
+    clean = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+    cell = np.clip(np.floor(pts.astype(np.float64) / h), 0, ng - 1)
+    near = lambda s: np.abs(cell - cell[s]).max(1) <= 1  # noqa: E731
+    nan, huge, top = np.zeros((n, nrhs), bool), np.zeros((n, nrhs), bool), np.finfo(np.float32).max
+    for s, r, v in ((5, 3, np.inf), (1777, 7, np.nan), (1778, 0, complex(0, -np.inf)), (n - 7, 5, -np.inf)):
+        lam[s, r] = v
+        nan[near(s), r] = True
+    for s, r, v in ((9, 1, top), (n - 11, 2, complex(0, -3.397e38)), (n // 2, 11, 3.39e38), (n // 3, nrhs - 1, -top)):
+        d = np.linalg.norm(pts[near(s)].astype(np.float64) - pts[s], axis=1)
+        assert d[d > 0].min() > 1.0
+        lam[s, r] = v
+        huge[near(s), r] = True
+    out = plan.apply(torch.from_numpy(lam).cuda(), path=path).cpu().numpy()
+    assert plan.async_status() == 0
+    assert np.isnan(out.real[nan]).all() and np.isnan(out.imag[nan]).all()
+    rest = ~nan & ~huge
+    assert np.array_equal(out[rest], clean[rest])
+    # the FP32 kernels form the same G (whose phase is rounded in FP32: one pair may be all of a sum here)
+    cols = np.unique(np.flatnonzero(huge.any(0)))
+    ref = plan.apply(torch.from_numpy(lam).cuda(), path="fp32_shared").cpu().numpy()[:, cols].astype(np.complex128)
+    S = oracle.p2p(pts, np.abs(lam[:, cols].astype(np.complex128)).clip(max=top).astype(np.complex64), lo, h, ng, 0.0,
+                   kernel=oracle.LAPLACE).real.reshape(n, -1)
+    at = huge[:, cols]
+    assert np.isfinite(out[:, cols][at]).all()
+    assert (np.abs(out[:, cols][at].astype(np.complex128) - ref[at]) <= DELTA[path] * S[at]).all()
