@@ -88,3 +88,28 @@ def test_tensor_core_abort_path_frees_tensor_memory():
         assert rel(plan.apply(lam_d, path="tc_bf16x3").cpu().numpy()) <= 1e-5
         assert plan.async_status() == C.P2P_OK
     print("tensor-core abort path, status per poll bound:", seen)
+
+
+@pytest.mark.parametrize("path", ["tc_bf16x3", "tc_bf16x6"])
+def test_one_box_tensor_core_abort_path_frees_tensor_memory(path):
+    """The same of the kernel with one target box per unit, which serves plans of fewer than 12 000 points."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_01596_gb300 import _capi as C, api
+    wl = W.Workload("s", W.unit_sphere(8000, 5), (-1, -1, -1), 2 / 19, 19, 15.0, 5)
+    lam = W.strengths(wl.n, 16, 5)
+    ref = oracle.p2p(wl.points, lam, wl.lo, wl.h, wl.ng, wl.k)
+    plan = api.Plan(torch.from_numpy(wl.points).cuda(), wl.lo, wl.h, wl.ng, wl.k, max_nrhs=16)
+    lam_d = torch.from_numpy(lam).cuda()
+
+    def rel(out):
+        return (np.linalg.norm(out - ref, axis=0) / np.linalg.norm(ref, axis=0)).max()
+
+    for polls in (0, 1, 3):
+        C.p2p_diag_tc_wait_limit(plan._plan, polls)
+        out = plan.apply(lam_d, path=path).cpu().numpy()
+        st = plan.async_status()
+        assert st == C.P2P_ERR_TIMEOUT or (polls > 0 and st == C.P2P_OK and rel(out) <= 1e-5)
+        C.p2p_diag_tc_wait_limit(plan._plan, -1)
+        assert rel(plan.apply(lam_d, path=path).cpu().numpy()) <= 1e-5
+        assert plan.async_status() == C.P2P_OK
