@@ -13,8 +13,8 @@
 // G is formed on the CUDA cores in FP32 (rsqrt, sincos), both operands are split
 // x = hi + lo into BF16, and three products (hi.hi + hi.lo + lo.hi, kind::f16,
 // FP32 accumulation in TMEM) keep the product error near 2^-16; with more than 32
-// right-hand sides lo.lo is added as well, which pays for the longer chains there
-// (kSegment).  With NP = 3 parts (hi + mid + lo, ~24 bits) six products take every
+// right-hand sides lo.lo is added as well, which pays for the truncated additions
+// there (kSegment).  With NP = 3 parts (hi + mid + lo, ~24 bits) six products take every
 // p.q with p + q < 3, and the product error is near 2^-24.
 //
 // Why this shape.  G is the MMA's A operand and goes from registers straight into
@@ -55,8 +55,8 @@
 // right-hand sides the small products (all but hi.hi) have accumulators of their
 // own.  The tensor core's FP32 accumulation truncates, ~2^-26 of the accumulator
 // per MMA in the same direction, so chains are kept short: a unit's list is cut
-// into near-equal segments (kSegment, kSegmentWide), and the epilogue adds the
-// segments in FP32.
+// into near-equal segments (kSegment), and the epilogue adds the segments in
+// FP32.
 //
 // Every wait is bounded: a wait that runs out sets the plan's status word and an
 // abort flag; every role then stops, the producer waits (bounded) for the bulk
@@ -91,15 +91,17 @@ constexpr int kSets = 4;               // G sets; set s takes entries s, s + kSe
 // product of an entry is a truncated addition to the one accumulator, and with the three of hi / lo the error came out
 // above that of the split alone even with short segments.  The fourth product, lo.lo, takes the split's own error from 4.4e-6
 // to 3.5e-6, more than those additions cost, and the issuers have time for it (a G set takes ~750 cycles for an entry, its
-// MMAs 384, 512 with the fourth).  Relative L2 error / time, 64 right-hand sides on 200 003 sphere points at 20
-// per box and on the 2^21-point ellipsoid, entries per segment x products:
-//   48 x 3  4.53e-6 331 us, 5.00e-6 3556 us      16 x 3  4.47e-6 401 us, 5.06e-6 4340 us   (split alone 4.4e-6)
-//   48 x 4  3.65e-6 346 us, 3.70e-6 3673 us      64 x 4  3.74e-6 332 us, 3.80e-6 3546 us
-//   96 x 4  3.77e-6 319 us, 3.94e-6 3372 us; at 47 points per box, 40 right-hand sides 4.39e-6 (64 x 4: 3.93e-6)
+// MMAs 384, 512 with the fourth).  Relative L2 error / time with 64 right-hand sides on 200 003 sphere points at 20 per box
+// and on the 2^21-point ellipsoid, and with 40 at 47 points per box, entries per segment x products:
+//   48 x 3  4.53e-6 331 us   5.00e-6 3556 us   4.64e-6
+//   16 x 3  4.47e-6 401 us   5.06e-6 4340 us   4.50e-6
+//   48 x 4  3.65e-6 346 us   3.70e-6 3673 us   3.86e-6
+//   64 x 4  3.74e-6 332 us   3.80e-6 3546 us   3.93e-6; in a cube at 100 per box, where every slot of an entry is a pair,
+//                                              4.98e-6 (one box per unit: 4.87e-6)
 // (Six products per entry would need segments of 6 to 8 entries to be as exact as chains of ~55 additions, and the
 // epilogue's share makes that slower than one box per unit: 2^21-point ellipsoid, 64 right-hand sides 7.4 ms against 6.9.
 // p2p_tc_box.cu takes those calls.)
-constexpr int kSegment = 48, kSegmentWide = 64;
+constexpr int kSegment = 48;
 constexpr int kAColumn = 256;          // first TMEM column of the operand slots
 constexpr int kMmaWarp0 = 1, kScoutWarp = 3, kEpiWarp0 = 4, kGWarp0 = 8;
 constexpr int kWarps = kGWarp0 + 4 * kSets;
@@ -708,8 +710,7 @@ __device__ void run_scout(const TcArgs& a, const TcSmem& sm, int lane) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(P2P_FULL_MASK, cnt, o);
             if (cnt == 0) continue;  // two point sets, no source nearby: the rows keep the zeros written before the launch
-            const int most = a.rhs <= 32 ? kSegment : kSegmentWide;
-            const int segments = (cnt + most - 1) / most;
+            const int segments = (cnt + kSegment - 1) / kSegment;
             h0 = make_int4(b0, t0, nt, cnt);
             h1 = make_int4(off, E, (int)want, (cnt + segments - 1) / segments);
         }
