@@ -470,12 +470,14 @@ P2P_API p2p_status p2p_apply_guarded(const p2p_plan* plan, const void* lambda, v
  * (each plan's own list, heaviest first) form one queue, plan after plan in the
  * order given, and the warps of a persistent grid take turns in it.
  * Giving the plans from smallest to largest leaves the tail to the largest
- * geometry's lightest items.
+ * geometry's lightest items.  With one right-hand side and every plan on the
+ * box-group kernel the queue holds the plans' box groups instead, and the blocks
+ * of the grid take turns in it.
  *
  *   plans           [host] count plan pointers, 1 <= count <= 16; the plans must
  *                          outlive the batch and are applied with nrhs columns
  *   nrhs                   1 .. min over plans of max_nrhs
- *   warps_per_cta          0 (default 8) or 1 .. 16
+ *   warps_per_cta          0 (default 8) or 1 .. 16, which asks for the staged pipeline
  *   workspace       [dev]  at least p2p_batch_workspace_size bytes, 256-byte aligned
  *
  * p2p_batch_create synchronises once (it builds the work queue on the device).
@@ -487,6 +489,8 @@ P2P_API p2p_status p2p_apply_guarded(const p2p_plan* plan, const void* lambda, v
  * lambdas and writes outs every time p2p_batch_graph_launch replays it; update
  * the buffers' contents in place between replays).  A batch shares its plans'
  * staging buffers: do not apply those plans concurrently with the batch.
+ * p2p_batch_info reports the launch that runs: entries of its queue, blocks and
+ * warps per block.
  */
 typedef struct p2p_batch p2p_batch;
 P2P_API p2p_status p2p_batch_workspace_size(const p2p_plan* const* plans, int32_t count, int32_t nrhs,

@@ -249,6 +249,7 @@ P2P_API p2p_status p2p_batch_create(p2p_batch** batch, const p2p_plan* const* pl
     int64_t total = 0;
     p2p_status st = check_plans(plans, count, nrhs, &total);
     if (st != P2P_OK) return st;
+    const bool shaped = warps_per_cta != 0;  // the caller names the staged launch's shape
     if (warps_per_cta == 0) warps_per_cta = 8;
     if (warps_per_cta < 1 || warps_per_cta > 16) return P2P_ERR_INVALID;
     if (!workspace || ((uintptr_t)workspace & 255)) return P2P_ERR_INVALID;
@@ -316,18 +317,16 @@ P2P_API p2p_status p2p_batch_create(p2p_batch** batch, const p2p_plan* const* pl
     }
     b->grid = ctas_per_sm * sms;
     FAIL(cudaMemcpyAsync(L.geoms, host, sizeof(BatchGeom) * count, cudaMemcpyHostToDevice, s), "p2p_batch_create");
+    if (group && !shaped) FAIL(p2p_group_batch_create(&b->group, plans, count, L.group, s), "p2p_batch_create/groups");
     const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (blocks) {
+    if (b->group.grid > 0) {
+        // every row is stored: only two-set outputs (targets in no group's reach) are zeroed
+        for (int g = 0; g < count; ++g) b->io.out_off[g + 1] = b->io.out_off[g] + (plans[g]->two_sets ? plans[g]->n : 0);
+    } else if (blocks) {
         k_batch_order<<<blocks, 256, 0, s>>>(L.geoms, off, L.order);
         FAIL(cudaGetLastError(), "p2p_batch_create/order");
     }
     FAIL(cudaStreamSynchronize(s), "p2p_batch_create");
-    if (group) {
-        FAIL(p2p_group_batch_create(&b->group, plans, count, L.group, s), "p2p_batch_create/groups");
-        if (b->group.grid > 0)  // every row is stored: only two-set outputs (targets in no group's reach) are zeroed
-            for (int g = 0; g < count; ++g)
-                b->io.out_off[g + 1] = b->io.out_off[g] + (plans[g]->two_sets ? plans[g]->n : 0);
-    }
 #undef FAIL
     *batch = b;
     return P2P_OK;
@@ -383,9 +382,10 @@ P2P_API p2p_status p2p_batch_graph_launch(const p2p_batch* batch, p2p_stream_t s
 
 P2P_API p2p_status p2p_batch_info(const p2p_batch* batch, int64_t* work_items, int32_t* grid, int32_t* warps_per_cta) {
     if (!batch) return P2P_ERR_INVALID;
-    if (work_items) *work_items = batch->total;
-    if (grid) *grid = batch->grid;
-    if (warps_per_cta) *warps_per_cta = batch->warps;
+    const bool group = batch->group.grid > 0;
+    if (work_items) *work_items = group ? batch->group.total : batch->total;
+    if (grid) *grid = group ? batch->group.grid : batch->grid;
+    if (warps_per_cta) *warps_per_cta = group ? batch->group.warps : batch->warps;
     return P2P_OK;
 }
 

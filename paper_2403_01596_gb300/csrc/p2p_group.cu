@@ -681,6 +681,7 @@ cudaError_t p2p_group_batch_create(p2p_group_batch* b, const p2p_plan* const* pl
     b->kernel = plans[0]->kernel;
     b->smem = group_smem_bytes(cap, pos_cap);
     b->grid = 0;
+    b->warps = kGroupWarps;
     int dev = 0, sms = 0, optin = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -242,7 +242,7 @@ struct p2p_group_batch {
     unsigned char* geoms;
     size_t geom_bytes, smem;
     void* order;
-    int32_t total, cap, pos_cap, kernel, grid;  // grid 0: not used
+    int32_t total, cap, pos_cap, kernel, grid, warps;  // grid 0: not used
 };
 bool p2p_group_batch_possible(const p2p_plan* const* plans, int32_t count, int32_t nrhs);
 size_t p2p_group_batch_bytes(const p2p_plan* const* plans, int32_t count);

@@ -70,3 +70,23 @@ def test_batched_groups(kernel):
         batch.replay()
         for o, p, l in zip(outs, plans, lams):
             assert torch.equal(o[:, 0], p.apply(l)) and p.async_status() == 0
+
+
+def test_batch_info_reports_the_launch():
+    """A batch on the box-group launch reports its groups, blocks of 8 warps and a grid no larger than the groups; a
+    caller that names the warps per block gets the staged launch of that shape, with the same results."""
+    api = _api()
+    plans, lams = [], []
+    for i, (n, ng) in enumerate([(3000, 6), (1500, 5)]):
+        pts = torch.rand(n, 3, generator=torch.Generator(device="cuda").manual_seed(i), device="cuda")
+        plans.append(api.Plan(pts, (0.0, 0.0, 0.0), 1.0 / ng, ng, 9.0, tuning={"warp_boxes": -2}))
+        lams.append(torch.from_numpy(W.strengths(n, 1, i)).cuda())
+    group = api.Batch(plans)
+    groups = sum(-(-p.num_boxes // 16) for p in plans)
+    assert (group.info["work_items"], group.info["warps_per_cta"]) == (groups, 8) and 0 < group.info["grid"] <= groups
+    staged = api.Batch(plans, warps_per_cta=4)
+    assert staged.info["work_items"] == sum(p.info["work_items"] for p in plans) and staged.info["warps_per_cta"] == 4
+    for o, s, p, l in zip(group.apply(lams), staged.apply(lams), plans, lams):
+        assert torch.equal(o[:, 0], p.apply(l))
+        st = p.structure
+        assert _close(api, p, st.points, st.lo, st.h, st.ng, l, s[:, 0])
