@@ -640,9 +640,8 @@ p2p_status p2p_group_launch(const p2p_plan* p, float2* out, int64_t ld, float k,
 
 // ---------------------------------------------------------------- batches --
 
-// Whether a batch of these plans runs its one right-hand side through the box-group kernel: every plan does so by
-// itself, with one kernel function, and the largest of their buffers still fits three blocks per SM's shared memory
-// as the plans' own do (the launch takes one size for all).
+// Whether a batch of these plans may run its one right-hand side through the box-group kernel: every plan does so by
+// itself, with one kernel function.  p2p_group_batch_create looks at the shapes.
 bool p2p_group_batch_possible(const p2p_plan* const* plans, int32_t count, int32_t nrhs) {
     if (nrhs != 1 || count > kMaxBatchPlans) return false;
     for (int g = 0; g < count; ++g)
@@ -650,14 +649,22 @@ bool p2p_group_batch_possible(const p2p_plan* const* plans, int32_t count, int32
     return true;
 }
 
+// Heaviest box of a batch over its average warp at most, with three and with two blocks per SM.
+constexpr double kEven3 = 2.6, kEven2 = 0.6;
+
 size_t p2p_group_batch_bytes(const p2p_plan* const* plans, int32_t count) {
     int64_t total = 0;
     for (int g = 0; g < count; ++g) total += plans[g]->n_groups;
     return align_up(sizeof(GroupArgs) * kMaxBatchPlans, 256) + align_up((size_t)total * sizeof(int2), 256);
 }
 
-// Fills b from workspace ws (p2p_group_batch_bytes, 256-byte aligned); b->grid is 0 where no block fits.  The copy
-// from `host` is complete when the stream has come this far: the caller synchronises before the arguments leave scope.
+// Fills b from workspace ws (p2p_group_batch_bytes, 256-byte aligned); b->grid is 0 where the staged pipeline is the better
+// launch: the largest buffers of all plans (one size for the launch) leave one block per SM, or the heaviest box, which
+// one warp sweeps alone, is worth more than kEven3 or kEven2 of the launch's average warps.  Plans whose tuning named the kernel keep it.
+// Measured on equal and unequal batches of 1 - 16 spheres, ellipsoids, cubes and spheres with a dense cap, 20 000 -
+// 140 000 points at 12 - 24 per box, box-group / staged by blocks per SM and heaviest box / average warp: three blocks up to 2.6
+// 0.72 - 1.09 (sixteen spheres of 65 537 at 15 per box 0.252 / 0.325 ms), above 1.0 - 2.3; two blocks up to 0.6
+// 0.72 - 1.11, above 0.98 - 4.5 (one cap of 1 000 points and seven spheres of 65 536 points 0.36 / 0.17 ms); one block 2.4 - 15.
 cudaError_t p2p_group_batch_create(p2p_group_batch* b, const p2p_plan* const* plans, int32_t count, void* ws,
                                    cudaStream_t s) {
     GroupArgs host[kMaxBatchPlans];
@@ -695,6 +702,15 @@ cudaError_t p2p_group_batch_create(p2p_group_batch* b, const p2p_plan* const* pl
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGroupWarps * 32, b->smem);
     if (e != cudaSuccess || per_sm == 0) return e;
+    bool asked = false;
+    double pairs = 0.0, heavy = 0.0;
+    for (int g = 0; g < count; ++g) {
+        asked |= plans[g]->group_asked != 0;
+        pairs += (double)plans[g]->pairs;
+        heavy = std::max(heavy, (double)plans[g]->heavy);
+    }
+    const double even = pairs / ((double)per_sm * sms * kGroupWarps);
+    if (!asked && (per_sm < 2 || heavy > (per_sm >= 3 ? kEven3 : kEven2) * even)) return cudaSuccess;
     e = cudaMemcpyAsync(geoms, host, sizeof(GroupArgs) * count, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     k_group_order<<<(unsigned)((b->total + 255) / 256), 256, 0, s>>>(geoms, o, order);

@@ -139,6 +139,8 @@ struct p2p_plan {
     int32_t group_cap;      // largest union (sources): the kernel's coordinate and strength buffers
     int32_t group_pos_cap;  // largest sum of a group's padded list lengths: its position buffer
     int32_t group_grid;     // persistent grid (blocks of 8 warps)
+    int32_t group_asked;    // 1: the caller's tuning named the kernel
+    int64_t pairs, heavy;   // targets x sources of all boxes, and of the heaviest box
     int32_t* g_union;       // [n_groups * kGroupBoxes * 27] union boxes of every group, ascending
     int32_t* g_nunion;      // [n_groups]
     int32_t* g_order;       // [n_groups] groups, heaviest first

@@ -255,6 +255,8 @@ struct ListInfo {
     int32_t packed;            // entries of all lists, each padded to 4
     int32_t items[3];          // work items with the chunk of each candidate tuning
     unsigned int status;       // nonzero: invalid CSR
+    unsigned long long pairs;  // targets x sources of all boxes, and of the heaviest box
+    unsigned long long heavy;
 };
 
 // Per target box: S_b, the length of its source list, and the size of the source box of its own cell (the sources
@@ -315,7 +317,15 @@ __global__ void __launch_bounds__(kThreads)
     const int32_t i2 = __reduce_add_sync(P2P_FULL_MASK, (int32_t)(((int64_t)len + chunk2 - 1) / chunk2));
     const int tails = __popc(__ballot_sync(P2P_FULL_MASK, tail));
     const bool any_bad = __any_sync(P2P_FULL_MASK, bad);
+    unsigned long long pairs = bad ? 0ull : (unsigned long long)own * (unsigned long long)s, heavy = pairs;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        pairs += __shfl_xor_sync(P2P_FULL_MASK, pairs, o);
+        heavy = max(heavy, __shfl_xor_sync(P2P_FULL_MASK, heavy, o));
+    }
     if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&info->pairs, pairs);
+        atomicMax(&info->heavy, heavy);
         atomicMax(&info->max_len, max_len);
         atomicMax(&info->max_box, max_own);
         if (tails) atomicAdd(&info->tails, tails);
@@ -1235,6 +1245,9 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     p->n_groups = 0;
     p->group_cap = 0;
     p->group_pos_cap = 0;
+    p->group_asked = t.warp_boxes == -2;
+    p->pairs = (int64_t)info.pairs;
+    p->heavy = (int64_t)info.heavy;
     if (p->tune.warp_boxes == -2 && (layout != P2P_LAYOUT_INDEXED || nb == 0)) p->tune.warp_boxes = -1;
     int32_t cap[2] = {0, 0};
     if (p->tune.warp_boxes == -2) {

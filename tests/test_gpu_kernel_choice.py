@@ -90,3 +90,24 @@ def test_batch_info_reports_the_launch():
         assert torch.equal(o[:, 0], p.apply(l))
         st = p.structure
         assert _close(api, p, st.points, st.lo, st.h, st.ng, l, s[:, 0])
+
+
+def test_batch_takes_groups_only_where_no_box_decides():
+    """Spheres of ~18 points per box on the box-group kernel by their own choice: one alone has too little work for the
+    boxes that single warps sweep and runs the staged launch, sixteen together the box-group launch; a plan whose tuning
+    names the kernel keeps it."""
+    api = _api()
+    lo, ng = (-1.0, -1.0, -1.0), 16
+    plans, lams = [], []
+    for i in range(16):
+        pts = torch.from_numpy(W.unit_sphere(20000, 4 + i)).cuda()
+        plans.append(api.Plan(pts, lo, 2.0 / ng, ng, 9.0))
+        assert plans[-1].info["tuning"]["warp_boxes"] == -2
+        lams.append(torch.from_numpy(W.strengths(20000, 1, i)).cuda())
+    asked = [api.Plan(plans[0].structure.points, lo, 2.0 / ng, ng, 9.0, tuning={"warp_boxes": -2})]
+    groups = lambda ps: sum(-(-p.num_boxes // 16) for p in ps)  # noqa: E731
+    for ps, own in ((plans[:1], False), (plans, True), (asked, True)):
+        batch = api.Batch(ps)
+        assert batch.info["work_items"] == (groups(ps) if own else sum(p.info["work_items"] for p in ps))
+        for o, p, l in zip(batch.apply(lams[:len(ps)]), ps, lams):
+            assert p.async_status() == 0 and _close(api, p, p.structure.points, lo, 2.0 / ng, ng, l, o[:, 0])
