@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(P2P_PAIR_MAX_THREADS, R == 1 ? P2P_PAIR_MIN_BL
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
     unsigned char* ws = smem_raw + (size_t)warp * warp_smem_bytes(a.chunk, R, a.sym);
-    run_pipeline<R>(ws, a.chunk, a.sym != 0, lane, a.items, a.n_items, (int64_t)blockIdx.x * warps + warp,
+    run_pipeline<R>(ws, a.chunk, a.sym != 0, lane, true, a.items, a.n_items, (int64_t)blockIdx.x * warps + warp,
                     (int64_t)gridDim.x * warps, a.status, [&](const ItemRec&) -> const PairArgs* { return &a; });
 }
 

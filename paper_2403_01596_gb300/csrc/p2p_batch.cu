@@ -10,7 +10,7 @@
 //                   atomics;
 //   k_pair_batched  a persistent grid (resident blocks x SMs) whose warps take
 //                   work items (geometry, box, source chunk) from one combined
-//                   list in turns (p2p_turn).  The list
+//                   list with a fixed stride (one plan: p2p_turn).  The list
 //                   is the plans' own item lists (each heaviest first) one after
 //                   the other in the order the plans were given, so the warps work
 //                   on one geometry's data at a time and the last geometry's light
@@ -99,12 +99,12 @@ __global__ void k_batch_stage(BatchGeom* __restrict__ geoms, const BatchIO io, u
 template <int R>
 __global__ void __launch_bounds__(P2P_PAIR_MAX_THREADS, R == 1 ? P2P_PAIR_MIN_BLOCKS : 1)
     k_pair_batched(const BatchGeom* __restrict__ geoms, const ItemRec* __restrict__ recs, int64_t total, int chunk_max,
-                   int sym_any) {
+                   int sym_any, bool back) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
     unsigned char* ws = smem_raw + (size_t)warp * warp_smem_bytes(chunk_max, R, sym_any != 0);
-    run_pipeline<R>(ws, chunk_max, sym_any != 0, lane, recs, total, (int64_t)blockIdx.x * warps + warp, (int64_t)gridDim.x * warps,
+    run_pipeline<R>(ws, chunk_max, sym_any != 0, lane, back, recs, total, (int64_t)blockIdx.x * warps + warp, (int64_t)gridDim.x * warps,
                     geoms[0].a.status, [&](const ItemRec& r) -> const PairArgs* { return &geoms[r.b].a; });
 }
 
@@ -219,11 +219,11 @@ static p2p_status batch_launch(const p2p_batch* b, const void* const* lambdas, v
     if (group) return p2p_group_batch_launch(&b->group, s);
     const int smem = b->warps * b->warp_bytes;
     if (b->R == 1)
-        k_pair_batched<1><<<b->grid, b->warps * 32, smem, s>>>(b->L.geoms, b->L.order, b->total, b->chunk_max, b->sym_any);
+        k_pair_batched<1><<<b->grid, b->warps * 32, smem, s>>>(b->L.geoms, b->L.order, b->total, b->chunk_max, b->sym_any, b->count == 1);
     else if (b->R == 2)
-        k_pair_batched<2><<<b->grid, b->warps * 32, smem, s>>>(b->L.geoms, b->L.order, b->total, b->chunk_max, b->sym_any);
+        k_pair_batched<2><<<b->grid, b->warps * 32, smem, s>>>(b->L.geoms, b->L.order, b->total, b->chunk_max, b->sym_any, b->count == 1);
     else
-        k_pair_batched<4><<<b->grid, b->warps * 32, smem, s>>>(b->L.geoms, b->L.order, b->total, b->chunk_max, b->sym_any);
+        k_pair_batched<4><<<b->grid, b->warps * 32, smem, s>>>(b->L.geoms, b->L.order, b->total, b->chunk_max, b->sym_any, b->count == 1);
     P2P_CHECK_LAUNCH("p2p_batch_apply/pair");
     return P2P_OK;
 }

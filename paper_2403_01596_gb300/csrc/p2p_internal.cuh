@@ -258,8 +258,12 @@ p2p_status p2p_group_batch_launch(const p2p_group_batch* b, cudaStream_t s);
 // shared memory (start of a kernel's item costs little, the sums of the costs decide): 8 right-hand sides on a
 // 500 000-point shell assembly 423 -> 405 us, 2^20 sphere points at 64 per box 816 -> 811 us.  Not used by the
 // direct and box-group kernels, which were slower with it (2^20-point Laplace plate 79.8 -> 85.8 us, sixteen pieces of
-// 65 536 points 270 -> 286 us): there neighbours in the list share their sources in the L1 or L2.
-__host__ __device__ inline int64_t p2p_turn(int64_t k, int64_t w, int64_t W) { return k * W + ((k & 1) ? W - 1 - w : w); }
+// 65 536 points 270 -> 286 us): there neighbours in the list share their sources in the L1 or L2.  back = false is the
+// fixed stride, for the list of a batch of several plans, one heaviest-first list after the other: four assemblies of
+// 65 537 points at 30 per box 164 us, back and forth 182 (one of 20 001 points: 58 and 54).
+__host__ __device__ inline int64_t p2p_turn(int64_t k, int64_t w, int64_t W, bool back = true) {
+    return k * W + (back && (k & 1) ? W - 1 - w : w);
+}
 
 // Persistent grid sizes of the pair kernel for the plan's kernel, layout and
 // tuning (resident blocks per SM x SMs), one per right-hand-side block width.

@@ -640,7 +640,7 @@ __device__ __forceinline__ ItemRec gather_rec(int32_t v) {
     return r;
 }
 
-// The per-warp pipeline over the items p2p_turn(0, 1, ..., first, stride) of `items`
+// The per-warp pipeline over the items p2p_turn(0, 1, ..., first, stride, back) of `items`
 // (n of them).  `args_of(rec)` points to the PairArgs an item belongs to.  At the
 // top of iteration k the warp holds records k .. k+2 (lane-distributed) and
 // starts loading record k+3; it issues the index copy of item k+2 (index stage
@@ -648,8 +648,8 @@ __device__ __forceinline__ ItemRec gather_rec(int32_t v) {
 // (k+1) % 2), then waits for item k's data and sweeps it.  Every mbarrier wait
 // is bounded.
 template <int R, typename ArgsOf>
-__device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool sym, int lane, const ItemRec* items, int64_t n,
-                                             int64_t first, int64_t stride, unsigned int* status, ArgsOf args_of) {
+__device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool sym, int lane, bool back, const ItemRec* items,
+                                             int64_t n, int64_t first, int64_t stride, unsigned int* status, ArgsOf args_of) {
     const WarpSmem w = warp_smem(ws, chunk, R, sym);
     if (lane == 0) {
 #pragma unroll
@@ -660,12 +660,13 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
     if (first >= n) return;
     uint32_t parity[5] = {0u, 0u, 0u, 0u, 0u};
     bool failed = false;
+    const auto at = [&](int64_t k) { return p2p_turn(k, first, stride, back); };
     // prologue: records 0..2, index copies of items 0 and 1, data of item 0
     int32_t v0 = load_rec_lane(items, first, n, lane);
-    int32_t v1 = load_rec_lane(items, p2p_turn(1, first, stride), n, lane);
-    int32_t v2 = load_rec_lane(items, p2p_turn(2, first, stride), n, lane);
+    int32_t v1 = load_rec_lane(items, at(1), n, lane);
+    int32_t v2 = load_rec_lane(items, at(2), n, lane);
     ItemRec r0 = gather_rec(v0), r1 = gather_rec(v1);
-    const bool has1 = p2p_turn(1, first, stride) < n;
+    const bool has1 = at(1) < n;
     const PairArgs* a0 = args_of(r0);
     const PairArgs* a1 = has1 ? args_of(r1) : nullptr;
     if (lane == 0) {
@@ -680,7 +681,7 @@ __device__ __forceinline__ void run_pipeline(unsigned char* ws, int chunk, bool 
     while (!failed) {
         const int cur = (int)(k & 1), nxt = cur ^ 1;
         const int i0 = (int)(k % 3), i1s = (int)((k + 1) % 3), i2s = (int)((k + 2) % 3);  // index stages
-        const int64_t i2 = p2p_turn(k + 2, first, stride), i3 = p2p_turn(k + 3, first, stride);
+        const int64_t i2 = at(k + 2), i3 = at(k + 3);
         const int32_t v3 = load_rec_lane(items, i3, n, lane);  // consumed two iterations later
         const ItemRec r2 = gather_rec(v2);
         const PairArgs* a2 = i2 < n ? args_of(r2) : nullptr;
