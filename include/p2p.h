@@ -123,18 +123,21 @@ typedef enum {
  * of many targets; the direct kernel gives each warp 1, 2, 4, 8, 16 or 32 whole
  * boxes (32 / warp_boxes lanes each) and reads the sources through the L1, which
  * suits sparse boxes (a few targets each), where a staged item carries too little
- * work for its fixed cost.  0: the plan decides from its mean box occupancy D and
- * its number of boxes (with many boxes the direct kernel with 32 .. 4 boxes per warp
- * up to D = 9, the box-group kernel up to D = 24 on the indexed layout, the staged
- * pipeline above; with few boxes fewer boxes per warp, or the staged pipeline);
+ * work for its fixed cost.  0: the plan decides from its mean box occupancy D, its
+ * number of boxes and its heaviest box (with many boxes the direct kernel with
+ * 32 .. 4 boxes per warp up to D = 9, the box-group kernel up to D = 24 on the indexed
+ * layout, the staged pipeline above; with few boxes fewer boxes per warp, or the
+ * staged pipeline, which alone cuts a box into items, also where one box would
+ * decide the time);
  * -1: the staged pipeline; 1 .. 32: the direct kernel with that many boxes
  * per warp; -2 (indexed layout only): the box-group
  * kernel, in which groups of 16 consecutive target boxes stage the union of their
  * neighbourhoods in shared memory once and every box sweeps its own neighbour
  * boxes inside it (a plan whose largest union exceeds 8 192 sources, or of another
  * layout, runs the staged pipeline instead and reports -1).
- * Multi-RHS applies, the symmetric layout and the batched launch always use the
- * staged pipeline. */
+ * Applies of several right-hand sides and the symmetric layout have kernels of
+ * their own choice; a batch of one right-hand side takes the box-group kernel where
+ * every plan does and the work is spread evenly, else the staged pipeline. */
 typedef struct {
     int32_t chunk;         /* sources staged per work item, multiple of 32, 32..1024 (default 192) */
     int32_t warps_per_cta; /* warps per thread block of the pair kernel, 1..16 (default 8) */

@@ -729,6 +729,23 @@ int32_t auto_warp_boxes(int64_t n, int32_t nb) {
     return d <= 9.0 && nb >= 55000 ? 4 : -2;
 }
 
+// Whether the kernel that auto_warp_boxes names would wait for the heaviest box.  There a box stays on one warp, or on
+// 32 / wb lanes of one, while the staged pipeline cuts it into items, so a cluster in an otherwise even geometry decides
+// the apply, whatever the mean occupancy.  The direct kernel takes ~3.7 ns per pair of a box's share of the warp, the
+// staged one 1.1 - 1.7 ns per box of the plan; the box-group kernel is behind once its heaviest box is worth 2.5 times the
+// average warp and long by itself (24 576 pairs take it ~40 us).  Measured (us), spheres with patches of 3, 6 and 12
+// times the mean density:
+//   direct / staged   25 773 boxes of 3.9 74 / 37, 158 / 38, 413 / 48; 103 990 of 3.8 93 / 115, 194 / 116, 491 / 127;
+//                     259 512 of 3.9 208 / 280, 397 / 281, 1201 / 286; 125 720 of 8.0 386 / 212, 858 / 218, 2453 / 246
+//   group / staged    47 636 boxes of 8.4 101 / 92, 165 / 99, 372 / 132; 10 965 of 9.1 60 / 38, 118 / 51, 352 / 80
+// and clustered assemblies, group / staged: 3 771 boxes of 8 193 / 32, 34 136 of 11.7 434 / 143, 84 640 of 11.8 800 / 335;
+// direct / staged: 123 825 of 8.1 2317 / 332, in the redundant layout with the Laplace kernel 1699 / 234.
+bool heaviest_decides(int32_t wb, const ListInfo& info, int32_t nb, int sms) {
+    const double heavy = (double)info.heavy;
+    if (wb > 0) return heavy * wb > 61.0 / sms * nb + 4096.0;
+    return heavy > 24576.0 && heavy * (24.0 * sms) > 2.5 * (double)info.pairs;
+}
+
 struct PlanLayout {
     p2p_plan p;  // pointers only
     int32_t *n_chunks, *item_off, *padded, *maxes, *list_len, *self_len;
@@ -1222,7 +1239,11 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     // direct kernel: one item per target box (the item-sort scratch is free again)
     p->direct_k = 0;
     if (layout != P2P_LAYOUT_SYMMETRIC && layout != P2P_LAYOUT_REPETITION) {
-        const int32_t wb = t.warp_boxes == 0 ? auto_warp_boxes(n, nb) : t.warp_boxes;
+        int32_t wb = t.warp_boxes;
+        if (wb == 0) {
+            wb = auto_warp_boxes(n, nb);
+            if (wb != -1 && heaviest_decides(wb, info, nb, sms)) wb = -1;
+        }
         p->tune.warp_boxes = wb;
         if (wb > 0) {
             p->direct_k = wb;

@@ -111,3 +111,30 @@ def test_batch_takes_groups_only_where_no_box_decides():
         assert batch.info["work_items"] == (groups(ps) if own else sum(p.info["work_items"] for p in ps))
         for o, p, l in zip(batch.apply(lams[:len(ps)]), ps, lams):
             assert p.async_status() == 0 and _close(api, p, p.structure.points, lo, 2.0 / ng, ng, l, o[:, 0])
+
+
+# a geometry whose mean occupancy names the direct or the box-group kernel, evenly spread and with a dense cap
+@pytest.mark.parametrize("n,ng,cap,radius", [(100_000, 80, 0.0, 0.0), (100_000, 80, 0.01, 0.01), (60_000, 44, 0.0, 0.0),
+                                             (60_000, 44, 0.02, 0.02), (400_000, 160, 0.01, 0.01)])
+@pytest.mark.parametrize("kernel", ["helmholtz", "laplace"])
+@pytest.mark.parametrize("layout", ["indexed", "redundant"])
+def test_heaviest_box(n, ng, cap, radius, kernel, layout):
+    """A plan left to choose takes the staged pipeline where one box holds a cluster, and what its mean occupancy says
+    otherwise; a request is kept either way."""
+    api = _api()
+    pts = W.unit_sphere(n, 7).astype(np.float64)
+    m = int(cap * n)
+    if m:
+        q = np.random.default_rng(8).normal(size=(m, 3)) * radius + [0.0, 0.6, 0.8]
+        pts[:m] = q / np.linalg.norm(q, axis=1, keepdims=True)
+    pts = torch.from_numpy(pts.astype(np.float32)).cuda()
+    lo, h = (-1.0, -1.0, -1.0), 2.0 / ng
+    lam = torch.from_numpy(W.strengths(n, 1, 9)).cuda()
+    plan = api.Plan(pts, lo, h, ng, 2 * np.pi * 0.25 / h, kernel=kernel, layout=layout)
+    even = -2 if ng == 44 and layout == "indexed" else (-1 if ng == 44 else 4)
+    assert plan.info["tuning"]["warp_boxes"] == (-1 if m else even)
+    out = plan.apply(lam)
+    assert plan.async_status() == 0 and _close(api, plan, pts, lo, h, ng, lam, out)
+    if m and n == 60_000:
+        asked = api.Plan(pts, lo, h, ng, plan.k, kernel=kernel, layout=layout, tuning={"warp_boxes": 2})
+        assert asked.info["tuning"]["warp_boxes"] == 2 and _close(api, asked, pts, lo, h, ng, lam, asked.apply(lam))
