@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kBuildThreads)
         }
         if (lane < nm) g_morder[g * kGroupBoxes + rank] = lane;
         if (lane == 0) {
-            keys[g] = cost_key<kCostBits>(cost);
+            keys[g] = cost_key<kFineCostBits>(cost);
             vals[g] = (int32_t)g;
         }
     }
@@ -445,9 +445,64 @@ __device__ __forceinline__ void prefetch_copies(const GroupArgs& a, int32_t g, i
     cp_async_commit();
 }
 
-// One group of a block: warp w takes the group's w-th costliest member, then further members from a shared counter.
-// `top` and `a` are the same arguments; a may be read only after the first barrier (a batch fills it meanwhile).
-// prefetch(): starts the copies of the next group's copy list.
+// Block = one group at a time: warp w takes the group's w-th costliest member, then further members from a
+// shared counter as it finishes.  (The loop is written out here and in sweep_group: through one function the Laplace kernel
+// took 2 - 6 % longer, 233 us to 244 for the 10^6-point cube at 14.5 per box.)
+template <int KERN>
+__global__ void __launch_bounds__(kGroupWarps * 32, P2P_GROUP_MIN_BLOCKS) k_pair_group(const __grid_constant__ GroupArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const GroupSmem sm = group_smem(smem, a.cap, a.pos_cap);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2* red = sm.red + warp * kMaxTT * 32;
+    // the first group's union copies, read ahead into shared memory like every later group's
+    if (blockIdx.x < a.n_groups) prefetch_copies(a, __ldg(a.order + blockIdx.x), sm.ents);
+    for (int64_t gi = blockIdx.x; gi < a.n_groups; gi += gridDim.x) {
+        const int32_t g = __ldg(a.order + gi);
+        const int nu = __ldg(a.g_nunion + g);
+        const int32_t b0 = g * kGroupBoxes;
+        const int nm = min(a.nb - b0, kGroupBoxes);
+        const int32_t* order = a.g_morder + (int64_t)g * kGroupBoxes;
+        const int32_t pos0 = __ldg(a.pk_off + b0), npos = __ldg(a.pk_off + b0 + nm) - pos0;
+        // this group's copy list has arrived, and every warp has finished the previous group
+        cp_async_wait<0>();
+        __syncthreads();
+        // the union: one warp per union box, its sources contiguous in the buffer; the members' position lists
+        // contiguous from the group's first list (every list padded to 4 entries, so 8-byte copies)
+        for (int u = warp; u < nu; u += kGroupWarps) {
+            const int4 c = sm.ents[u];
+            for (int e = lane; e < c.z; e += 32) {
+                cp_async16(sm.sx + c.y + e, a.xs + c.x + e);
+                cp_async8(sm.sl + c.y + e, a.lam + c.x + e);
+            }
+        }
+        for (int e = threadIdx.x; e < npos / 4; e += kGroupWarps * 32)
+            cp_async8(sm.pos + 4 * e, a.g_pos + pos0 + 4 * e);
+        cp_async_commit();
+        // this warp's first member, loaded while the union is staged
+        Member m;
+        const bool has = warp < nm;
+        if (has) load_member(a, b0 + __ldg(order + warp), lane, m);
+        if (threadIdx.x == 0) *sm.next = kGroupWarps;
+        cp_async_wait<0>();
+        __syncthreads();
+        // the next group's copy list, in flight while this group is swept
+        if (gi + gridDim.x < a.n_groups) prefetch_copies(a, __ldg(a.order + gi + gridDim.x), sm.ents);
+        if (has) {
+            sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
+            while (true) {
+                int idx = 0;
+                if (lane == 0) idx = atomicAdd(sm.next, 1);
+                idx = __shfl_sync(P2P_FULL_MASK, idx, 0);
+                if (idx >= nm) break;
+                load_member(a, b0 + __ldg(order + idx), lane, m);
+                sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
+            }
+        }
+    }
+}
+
+// One group of a block of a batch, as in k_pair_group.  `top` and `a` are the same arguments; a may be read only after the
+// first barrier (it is filled meanwhile).  prefetch(): starts the copies of the next group's copy list.
 template <int KERN, typename Prefetch>
 __device__ __forceinline__ void sweep_group(const GroupArgs& top, const GroupArgs& a, int32_t g, const GroupSmem& sm,
                                             Prefetch prefetch) {
@@ -492,19 +547,6 @@ __device__ __forceinline__ void sweep_group(const GroupArgs& top, const GroupArg
             load_member(a, b0 + __ldg(order + idx), lane, m);
             sweep_member<KERN>(a, sm.sx, sm.sl, sm.pos, pos0, red, m, lane);
         }
-    }
-}
-
-template <int KERN>
-__global__ void __launch_bounds__(kGroupWarps * 32, P2P_GROUP_MIN_BLOCKS) k_pair_group(const __grid_constant__ GroupArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const GroupSmem sm = group_smem(smem, a.cap, a.pos_cap);
-    // the first group's union copies, read ahead into shared memory like every later group's
-    if (blockIdx.x < a.n_groups) prefetch_copies(a, __ldg(a.order + blockIdx.x), sm.ents);
-    for (int64_t gi = blockIdx.x; gi < a.n_groups; gi += gridDim.x) {
-        sweep_group<KERN>(a, a, __ldg(a.order + gi), sm, [&]() {
-            if (gi + gridDim.x < a.n_groups) prefetch_copies(a, __ldg(a.order + gi + gridDim.x), sm.ents);
-        });
     }
 }
 
@@ -597,7 +639,7 @@ cudaError_t p2p_group_build(p2p_plan* p, const int32_t* nbr_ptr, const int32_t* 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     bool in_alt = false;
-    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, ng, kCostBits, radix_ws, radix_bytes, s, &in_alt);
+    e = radix_sort_pairs(keys, vals, keys_alt, vals_alt, ng, kFineCostBits, radix_ws, radix_bytes, s, &in_alt);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(p->g_order, in_alt ? vals_alt : vals, (size_t)ng * sizeof(int32_t), cudaMemcpyDeviceToDevice,
                         s);
