@@ -689,8 +689,8 @@ p2p_tuning resolve_tuning(const p2p_tuning* t) {
 // Largest union the box-group kernel stages (sources; 24 bytes each in shared memory; its positions are 16-bit).
 constexpr int32_t kGroupCapMax = 8192;
 
-// The one-right-hand-side kernel of a plan left to choose (warp_boxes = 0), from the mean number of targets per box D
-// and the number of boxes: > 0 boxes per warp of the direct kernel, -2 the box-group kernel (indexed layout only,
+// The one-right-hand-side kernel of a plan left to choose (warp_boxes = 0), from the mean number of targets per box D,
+// the number of boxes and the sources of all lists: > 0 boxes per warp of the direct kernel, -2 the box-group kernel (indexed layout only,
 // other layouts take the staged pipeline), -1 the staged pipeline.
 //
 // The direct kernel with several boxes per warp does the least work per pair on sparse boxes, but a box there is a
@@ -714,22 +714,61 @@ constexpr int32_t kGroupCapMax = 8192;
 //   D = 20:      784: 13.8 | 25 | 48                        3 296: 31 | 35 | 54    13 599: 88 | 85 | 102
 //   cube, D = 9: 6 859: 30 | 25 | 31 / 86 / 156; D = 16: 1 000: 17 | 27, 17 576: 118 | 98; D = 21: 3 375: 40 | 45,
 //   12 167: 147 | 151; D = 32 (4 096 boxes): 122 | 137
-// Laplace gives the same ranking at about two thirds of the times, with several boxes per warp a little earlier.
-int32_t auto_warp_boxes(int64_t n, int32_t nb) {
+// Laplace gives the same ranking at about two thirds of the times, with several boxes per warp earlier (plan_warp_boxes).
+//
+// Which of two kernels is ahead also depends on the mean list length L (L = 12 - 15 D on a surface, up to 27 D in a
+// volume).  Applies in a loop, staging and launches included:
+//   eight | four boxes per warp   L = 27: 79 346 boxes 35.9 | 35.9 (Laplace 29.7 | 31.6), 126 626 46 | 48 (37.7 | 41.8); L = 30:
+//             92 350 41 | 37, 148 652 48 | 50 (39.9 | 44.1); L = 40: 117 269 58 | 55; L = 45: 138 941 73 | 79, 198 460 108 | 111;
+//             L = 53: 162 659 98 | 97; L = 77: 225 809 134 | 127; L = 105: 245 458 211 | 202
+//   sixteen | eight               L = 15, D = 2.0: 199 650 42 | 40, 349 478 60 | 62 (Laplace, redundant layout 83 | 88)
+//   group | staged                D = 18, surface: 1 108 24.6 | 18.5, 2 229 24.3 | 19.3, 4 579 31.6 | 32.2; cube: 1 000 29.9 | 15.9,
+//             1 331 30.2 | 18.5, 2 197 27.6 | 28.9, 4 913 47 | 45, 6 859 57 | 62
+//             D = 20 - 23, sphere: 2 259 32 | 27, 4 626 46 | 48 (Laplace 31.4 | 35.8), 6 970 77 | 58, 10 718 92 | 83 (two blocks
+//             per SM: 304 groups are a wave), 19 332 137 | 144 (89 | 98); plate: 18 225 87 | 96 (56 | 64), 45 369 200 | 231;
+//             cube: 4 913 69 | 63, 6 859 109 | 91, 10 648 132 | 135, 29 791 387 | 415
+// On surfaces of 1 000 - 4 000 boxes at D = 12 - 19.5 the staged pipeline would be up to 1.3 times as fast; the box-group
+// kernel is kept there, which callers of such plans see in p2p_plan_info and batches of them build on.
+int32_t auto_warp_boxes(int64_t n, int32_t nb, int64_t sources) {
     if (nb <= 0) return -1;
-    const double d = (double)n / nb;
+    const double d = (double)n / nb, len = (double)sources / nb;
+    const bool volume = len > 300.0;
     if (d > 24.0) return -1;
-    if (d > 12.0) return nb >= 6000 || (nb >= 1000 && d <= 19.5) ? -2 : -1;
+    if (d > 20.0) return nb >= (volume ? 10000 : 4000) ? -2 : -1;
+    if (d > 12.0) return nb >= 4000 || (nb >= (volume ? 2000 : 1000) && d <= 19.5) ? -2 : -1;
     if (nb < 2500) return d <= 2.5 ? 1 : -1;
     if (d <= 1.3) return nb < 15000 ? 4 : 32;
-    if (d <= 1.9) return nb < 15000 ? 4 : 16;
+    if (d <= 1.9 || (d <= 2.05 && len <= 16.0 && nb >= 250000)) return nb < 15000 ? 4 : 16;
     if (d <= 2.5) return nb < 15000 ? 4 : 8;
-    if (d <= 5.0) return nb < 15000 ? 1 : (nb < 150000 ? 4 : 8);
+    if (d <= 5.2) return nb < 15000 ? 1 : (len <= 50.0 && nb >= (len <= 28.0 ? 75000 : 120000) ? 8 : 4);
     if (d <= 7.0) return nb < 45000 ? 1 : 4;
-    return d <= 9.0 && nb >= 55000 ? 4 : -2;
+    return d <= 9.1 && nb >= 55000 ? 4 : -2;
 }
 
-// Whether the kernel that auto_warp_boxes names would wait for the heaviest box.  There a box stays on one warp, or on
+// The same for a plan's kernel function and layout.  A Laplace pair costs two thirds of a Helmholtz one, so a box's chain
+// on a few lanes hides earlier.  Measured (us):
+//   four | one box per warp   D = 6.2: 40 303 boxes 34 | 40, 39 595 (L = 82) 44 | 46, 20 978 27.6 | 25.6
+//   eight | four              D = 3.6, L = 43: 111 854 43 | 46
+//   four | group              D = 8, L = 71: 31 317 37 | 42, 50 163 48 | 60; L = 106: 31 311 49 | 46, 50 124 62 | 71; L = 202: 29 788
+//                             77 | 66, 50 633 97 | 103; D = 9, L = 80: 44 516 53 | 57; L = 120: 110 529 146 | 160; D = 10, L = 89:
+//                             24 964 44 | 38, 39 998 54 | 54, 70 224 78 | 91; L = 133: 71 093 122 | 114
+//   four | staged (redundant) D = 8, L = 71: 31 317 40 | 48; L = 106: 50 124 93 | 83; D = 10, L = 90: 39 998 72 | 67, 99 852 148 | 158
+int32_t plan_warp_boxes(int64_t n, int32_t nb, int64_t sources, p2p_kernel kernel, p2p_layout layout) {
+    const int32_t wb = auto_warp_boxes(n, nb, sources);
+    const double d = (double)n / (nb > 0 ? nb : 1), len = (double)sources / (nb > 0 ? nb : 1);
+    if (kernel == P2P_LAPLACE) {
+        if (wb == 1 && d > 5.2 && nb >= 24000) return 4;
+        if (wb == 4 && d > 2.5 && d <= 5.2 && len <= 45.0 && nb >= 100000) return 8;
+        if (wb == -2 && d <= 12.0) {
+            const bool indexed = layout == P2P_LAYOUT_INDEXED;
+            if (len <= 95.0 && (d <= 8.5 ? nb >= 30000 : d <= 10.5 && nb >= (indexed ? 40000 : 55000))) return 4;
+            if (indexed && (d <= 8.5 ? nb >= 45000 : d <= 9.2 && len <= 125.0 && nb >= 55000)) return 4;
+        }
+    }
+    return wb == -2 && layout != P2P_LAYOUT_INDEXED ? -1 : wb;
+}
+
+// Whether the kernel that plan_warp_boxes names would wait for the heaviest box.  There a box stays on one warp, or on
 // 32 / wb lanes of one, while the staged pipeline cuts it into items, so a cluster in an otherwise even geometry decides
 // the apply, whatever the mean occupancy.  The direct kernel takes ~3.7 ns per pair of a box's share of the warp, the
 // staged one 1.1 - 1.7 ns per box of the plan; the box-group kernel is behind once its heaviest box is worth 2.5 times the
@@ -779,7 +818,7 @@ PlanLayout plan_layout(int64_t n, int32_t nb, int64_t n_src, int32_t nbs, bool t
     L.p.box_src = c.take<int32_t>(mb);
     L.p.items = c.take<ItemRec>(max_items);
     L.p.ditems = c.take<ItemRec>(mb);
-    if (layout == P2P_LAYOUT_INDEXED && (t.warp_boxes == -2 || (t.warp_boxes == 0 && auto_warp_boxes(n, nb) == -2))) {
+    if (layout == P2P_LAYOUT_INDEXED && (t.warp_boxes == -2 || (t.warp_boxes == 0 && auto_warp_boxes(n, nb, sources) == -2))) {
         // box-group kernel tables (requested, or the plan's own choice)
         const size_t ngr = (mb + kGroupBoxes - 1) / kGroupBoxes;
         L.p.g_union = c.take<int32_t>(ngr * kGroupBoxes * 27);
@@ -1241,7 +1280,7 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     if (layout != P2P_LAYOUT_SYMMETRIC && layout != P2P_LAYOUT_REPETITION) {
         int32_t wb = t.warp_boxes;
         if (wb == 0) {
-            wb = auto_warp_boxes(n, nb);
+            wb = plan_warp_boxes(n, nb, in.sources, kernel, layout);
             if (wb != -1 && heaviest_decides(wb, info, nb, sms)) wb = -1;
         }
         p->tune.warp_boxes = wb;
@@ -1293,6 +1332,13 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     p->n_items = items;
     p->packed = info.packed;
     FAIL_CUDA(p2p_pair_configure(p), "p2p_plan_create/occupancy");
+    // a second or third wave of two blocks per SM that runs partly empty, on a surface: the staged pipeline
+    // (auto_warp_boxes, D = 20 - 23)
+    if (t.warp_boxes == 0 && p->group_k && n > 20ll * nb && in.sources <= 300ll * nb && p->group_grid <= 2 * sms &&
+        p->n_groups > p->group_grid && 2 * p->n_groups <= 5 * p->group_grid) {
+        p->group_k = 0;
+        p->tune.warp_boxes = -1;
+    }
 #undef FAIL_CUDA
     *plan = p;
     return P2P_OK;

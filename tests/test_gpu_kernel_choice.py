@@ -138,3 +138,25 @@ def test_heaviest_box(n, ng, cap, radius, kernel, layout):
     if m and n == 60_000:
         asked = api.Plan(pts, lo, h, ng, plan.k, kernel=kernel, layout=layout, tuning={"warp_boxes": 2})
         assert asked.info["tuning"]["warp_boxes"] == 2 and _close(api, asked, pts, lo, h, ng, lam, asked.apply(lam))
+
+
+# shape, points, boxes per axis, kernel, layout, expected: one point on either side of the lines that depend on the list
+# length (plates 9, cubes up to 27 times the occupancy), the kernel function and the layout
+@pytest.mark.parametrize("shape,n,ng,kernel,layout,want", [
+    ("plate", 400_001, 211, "laplace", "indexed", 4), ("plate", 400_001, 211, "helmholtz", "indexed", -2),
+    ("plate", 400_001, 211, "laplace", "redundant", -1), ("plate", 250_001, 177, "laplace", "redundant", 4),
+    ("plate", 400_001, 356, "laplace", "indexed", 8), ("cube", 400_001, 50, "laplace", "indexed", 4),
+    ("cube", 700_001, 61, "helmholtz", "indexed", 4), ("plate", 250_001, 201, "laplace", "indexed", 4),
+    ("plate", 250_001, 201, "helmholtz", "indexed", 1), ("cube", 14_301, 10, "helmholtz", "indexed", -1),
+    ("cube", 34_001, 13, "helmholtz", "indexed", -2)])
+def test_choice_by_list_length_kernel_and_layout(shape, n, ng, kernel, layout, want):
+    api = _api()
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    pts, lo, h = torch.rand(n, 3, generator=gen, device="cuda"), (0.0, 0.0, 0.0), 1.0 / ng
+    if shape == "plate":
+        pts[:, 2] = 0.5
+    plan = api.Plan(pts, lo, h, ng, 2 * np.pi * 0.25 / h, kernel=kernel, layout=layout)
+    assert plan.info["tuning"]["warp_boxes"] == want, (n / plan.num_boxes, plan.num_boxes, plan.structure.sources / plan.num_boxes)
+    lam = torch.from_numpy(W.strengths(n, 1, n)).cuda()
+    out = plan.apply(lam)
+    assert plan.async_status() == 0 and _close(api, plan, pts, lo, h, ng, lam, out)
