@@ -3,10 +3,12 @@
 For a point set and grid, every candidate configuration is built as a plan on
 the shared box structure and timed with CUDA events on the current stream
 (warm-up, then the median of a few applies).  The winner is cached in a JSON
-file keyed by (GPU name, SM count, kernel, occupancy bucket, nrhs, layouts
-searched), so a later plan for a similar workload on the same GPU reuses it
-without timing.  The occupancy bucket is the power of two nearest to the mean
-number of points per non-empty box.
+file keyed by (GPU name, SM count, kernel, occupancy bucket, box bucket, nrhs,
+layouts searched), so a later plan for a similar workload on the same GPU reuses
+it without timing.  The occupancy bucket is the power of two nearest to the mean
+number of points per non-empty box, the box bucket the power of two nearest to
+the number of boxes: at one occupancy a few thousand boxes and a few hundred
+thousand have different winners.
 
 The cache file defaults to $P2P_AUTOTUNE_CACHE, else
 ~/.cache/p2p_gb300/autotune.json.
@@ -20,8 +22,8 @@ import statistics
 import threading
 
 # staged pipeline (warp_boxes -1) with several chunk / block shapes, the direct kernel with 1 - 32 boxes per warp
-# and the box-group kernel (-2, indexed layout only) (one-RHS applies only; for several RHS a plan runs the staged
-# pipeline whatever warp_boxes says)
+# and the box-group kernel (-2, indexed layout only) (warp_boxes counts for one-RHS applies only; several RHS have a
+# kernel of their own, which takes its source chunks from the tuning, and its warps per block for two RHS on few boxes)
 DEFAULT_CANDIDATES = (
     {"chunk": 192, "warps_per_cta": 8, "target_group": 32, "warp_boxes": -1},
     {"chunk": 128, "warps_per_cta": 8, "target_group": 32, "warp_boxes": -1},
@@ -57,8 +59,12 @@ def occupancy_bucket(n_points: int, num_boxes: int) -> int:
     return int(2 ** round(math.log2(max(d, 1.0))))
 
 
-def cache_key(gpu: str, sms: int, kernel: str, bucket: int, nrhs: int, layouts) -> str:
-    return f"v3|{gpu}|{sms}|{kernel}|d{bucket}|r{nrhs}|{'+'.join(sorted(layouts))}"
+def box_bucket(num_boxes: int) -> int:
+    return int(2 ** round(math.log2(num_boxes))) if num_boxes > 0 else 0
+
+
+def cache_key(gpu: str, sms: int, kernel: str, bucket: int, nrhs: int, layouts, boxes: int = 0) -> str:
+    return f"v4|{gpu}|{sms}|{kernel}|d{bucket}|b{boxes}|r{nrhs}|{'+'.join(sorted(layouts))}"
 
 
 def load_cache(path: str | None = None) -> dict:
@@ -113,7 +119,7 @@ def tune(structure, k: float, kernel: str = "helmholtz", nrhs: int = 1, layouts=
     dev = structure.points.device
     props = torch.cuda.get_device_properties(dev)
     key = cache_key(props.name, props.multi_processor_count, kernel,
-                    occupancy_bucket(structure.n, structure.num_boxes), nrhs, layouts)
+                    occupancy_bucket(structure.n, structure.num_boxes), nrhs, layouts, box_bucket(structure.num_boxes))
     with _lock:
         cache = load_cache(path) if use_cache else {}
     if use_cache and key in cache:

@@ -47,3 +47,9 @@ def test_candidates_are_valid_tunings():
     for cand in T.DEFAULT_CANDIDATES:
         # a valid tuning gives a workspace size; an invalid one raises
         assert C.p2p_plan_workspace_size(1000, 100, 500, 5000, 0, 1, cand) > 0
+
+
+def test_cache_key_separates_box_counts():
+    assert T.box_bucket(131520) == 131072 and T.box_bucket(1000) == 1024 and T.box_bucket(0) == 0
+    keys = {T.cache_key("NVIDIA GB300", 152, "helmholtz", 8, 1, ("indexed",), T.box_bucket(n)) for n in (1800, 60000, 131520)}
+    assert len(keys) == 3
