@@ -47,12 +47,12 @@ constexpr int kBlockRhs = 8;            // right-hand sides per launch at most
 // Warps of an SM: two blocks of 8 at 128 registers, or one of 12 at 168 where that is faster although fewer warps are
 // resident: 8 right-hand sides (which spill at 128) 424 -> 417 us on the 500 000-point assembly and 225 -> 218 us on
 // 300 001 sphere points, the Helmholtz gradient 550 -> 516 us on 500 001 points at 50 per box; the Laplace gradient
-// (107 -> 116 us on 500 001 points at 8) and 3 right-hand sides (71 -> 80 us) are slower with 12.
+// (107 -> 116 us on 500 001 points at 8), the Helmholtz gradient of uneven geometries (p2p_grad_launch) and 3 right-hand
+// sides (71 -> 80 us) are slower with 12.
 struct Shape {
     int warps, blocks;
 };
 __host__ __device__ constexpr Shape multi_shape(int R) { return R == 8 ? Shape{12, 1} : Shape{8, 2}; }
-__host__ __device__ constexpr Shape grad_shape(int kernel) { return kernel == P2P_HELMHOLTZ ? Shape{12, 1} : Shape{8, 2}; }
 
 struct MultiArgs {
     const ItemRec* items;
@@ -497,10 +497,10 @@ __device__ __forceinline__ void run_grad(Stream<2>& st, Place& cur, Place& nxt, 
     __syncwarp();
 }
 
-template <int KERN>
-__global__ void __launch_bounds__(grad_shape(KERN).warps * 32, grad_shape(KERN).blocks)
-    k_grad(const __grid_constant__ MultiArgs a, float* out) {
-    constexpr int kWarps = grad_shape(KERN).warps;
+// WARPS: of a block, 12 (one block per SM) or 8 (two).
+template <int KERN, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, WARPS == 12 ? 1 : 2) k_grad(const __grid_constant__ MultiArgs a, float* out) {
+    constexpr int kWarps = WARPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* ws = reinterpret_cast<float*>(smem_raw) + warp * kGradWarpFloats;
@@ -649,16 +649,25 @@ p2p_status p2p_grad_launch(const p2p_plan* p, const float2* lam, const float2* g
     a.perm = p->perm;
     a.k = p->k;
     a.tg = p->tune.target_group;
-    const Shape shape = grad_shape(p->kernel);
+    // Where the heaviest box is worth more than four of the average warps (32 per SM), the items' turns leave the warps with
+    // its items far behind the others: a grid of sixteen times the resident blocks, whose blocks come as SMs become free.
+    // Helmholtz takes 16 warps per SM there, more of them beside the long ones.  Clustered assemblies, as before the stream /
+    // with 12 warps in turns / here, us: 60 001 points at 10 per box 75 / 73 / 64, at 60 161 / 189 / 148, 300 001 at 10 230 / 249 /
+    // 212, Laplace 150 / 149 / 130.  On even geometries the larger grid only starts more blocks (262 144 sphere points at 16,
+    // Helmholtz with 12 warps 119 -> 127; a cube at 20 176 -> 196).
+    const bool uneven = (double)p->heavy * 32.0 * sms > 4.0 * (double)p->pairs;
+    const bool helm = p->kernel == P2P_HELMHOLTZ, narrow = helm && !uneven;
+    const Shape shape = narrow ? Shape{12, 1} : Shape{8, 2};
     const int64_t blocks = ((int64_t)a.n_items + shape.warps - 1) / shape.warps;
     if (blocks == 0) return P2P_OK;
     const int smem = shape.warps * kGradWarpFloats * (int)sizeof(float);
-    auto kern = p->kernel == P2P_HELMHOLTZ ? k_grad<P2P_HELMHOLTZ> : k_grad<P2P_LAPLACE>;
+    auto kern = narrow ? k_grad<P2P_HELMHOLTZ, 12> : (helm ? k_grad<P2P_HELMHOLTZ, 8> : k_grad<P2P_LAPLACE, 8>);
+    const int64_t grid = std::min<int64_t>(blocks, (int64_t)sms * shape.blocks * (uneven ? 16 : 1));
     if (smem > 48 * 1024)
         P2P_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "p2p_grad_points");
     for (int q = 0; q < nrhs; ++q) {
         a.lam = reinterpret_cast<const float*>(rows + (int64_t)q * p->n);
-        kern<<<(unsigned)std::min<int64_t>(blocks, (int64_t)sms * shape.blocks), shape.warps * 32, smem, s>>>(a, grad);
+        kern<<<(unsigned)grid, shape.warps * 32, smem, s>>>(a, grad);
         P2P_CHECK_LAUNCH("p2p_grad_points/kernel");
     }
     return P2P_OK;

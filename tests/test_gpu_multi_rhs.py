@@ -69,3 +69,28 @@ def test_two_on_both_sides_of_the_kernel_choice(n, ng, flat, kernel, layout):
     assert plan.async_status() == 0
     assert (np.abs(got - ref) <= 2.0 ** -20 * S).all()
     assert (np.abs(got - alone) <= 2.0 ** -19 * S).all()
+
+
+@pytest.mark.parametrize("share,radius", [(0.0, 0.0), (0.3, 0.03)])
+@pytest.mark.parametrize("kernel", ["helmholtz", "laplace"])
+def test_gradient_of_even_and_clustered_geometries(share, radius, kernel):
+    """The coordinate gradient on both launch shapes: points spread over a cube, and with a cluster whose box is worth many
+    average warps.  Tolerance: relative L2 1e-5, as for every FP32 result against the oracle."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_01596_gb300 import api
+    n, ng = 20_000, 11
+    rng = np.random.default_rng(6)
+    pts = rng.random((n, 3))
+    m = int(share * n)
+    pts[:m] = 0.5 + radius * rng.random((m, 3))
+    pts = pts.astype(np.float32)
+    lo, h = (0.0, 0.0, 0.0), 1.0 / ng
+    k = float(np.float32(2 * np.pi * ng / 4)) if kernel == "helmholtz" else 0.0
+    kid = oracle.HELMHOLTZ if kernel == "helmholtz" else oracle.LAPLACE
+    plan = api.Plan(torch.from_numpy(pts).cuda(), lo, h, ng, k, kernel=kernel)
+    lam, g = W.strengths(n, 1, 7), W.strengths(n, 1, 8)
+    got = plan.grad_points(torch.from_numpy(lam).cuda(), torch.from_numpy(g).cuda()).cpu().numpy()
+    assert plan.async_status() == 0
+    ref = oracle.grad_points(pts, lam, g, lo, h, ng, k, kernel=kid)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
