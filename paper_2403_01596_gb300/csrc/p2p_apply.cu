@@ -300,16 +300,19 @@ static p2p_path resolve_path(const p2p_plan* plan, int32_t nrhs, p2p_path path) 
 
 static bool is_tc(p2p_path path) { return path == P2P_PATH_TC_BF16X3 || path == P2P_PATH_TC_BF16X6; }
 // Several right-hand sides on the streamed kernel (p2p_multi.cu): every layout with full source lists, from the sorted
-// strengths.  Two of them stay with the staged pipeline where the plan has few boxes, fewer the more points each holds:
-// one box's chain then decides, and the streamed kernel stages a box's list once per 32 targets.  Measured with two
-// right-hand sides on spheres, streamed / staged, us: 1132 boxes of 7 points 19.5 / 19.5, 2326 of 7 21 / 21, 3850
-// of 7 23 / 25; 499 of 16 30 / 27, 2672 of 16 35 / 40; 620 of 26 30 / 28, 2279 of 29 (Laplace) 43 / 38, 4191 of 29
-// 80 / 92 (Laplace 62 / 69); 1389 of 47 71 / 64 (Laplace 54 / 46), 7156 of 42 233 / 249.  From three right-hand sides on the streamed kernel won
-// everywhere from 8 000 points up (499 boxes of 16 with three: 34 / 42).
+// strengths.  Two of them stay with the staged pipeline where one box's chain decides, since the streamed kernel stages a
+// box's list once per 32 targets: where the plan has few boxes, fewer the more points each holds, and where its heaviest
+// box is worth more than twenty average warps.  Measured with two right-hand sides, streamed / staged, us, on
+// spheres: 1132 boxes of 7 points 19.5 / 19.5, 2326 of 7 21 / 21, 3850 of 7 23 / 25; 499 of 16 30 / 27, 2672 of 16 35 / 40;
+// 620 of 26 30 / 28, 2279 of 29 (Laplace) 43 / 38, 4191 of 29 80 / 92 (Laplace 62 / 69); 1389 of 47 71 / 64 (Laplace 54 / 46),
+// 7156 of 42 233 / 249; on clustered assemblies by heaviest box / average warp: 30 - 40 (70 001 points at 9 to 12 per box)
+// 64 / 57 and 74 / 65 (Laplace 50 / 42 and 58 / 48), 25 (100 001) 75 / 77 and 98 / 94 (59 / 57, 73 / 64), 10 (400 001) 188 / 220
+// and 243 / 263 (139 / 159).  From three right-hand sides on the streamed kernel won everywhere from 8 000 points up (499
+// boxes of 16 with three: 34 / 42).
 static bool is_multi(const p2p_plan* plan, int32_t nrhs, p2p_path path) {
     if (path != P2P_PATH_FP32_SHARED || nrhs < 2) return false;
     if (plan->layout != P2P_LAYOUT_INDEXED && plan->layout != P2P_LAYOUT_REDUNDANT) return false;
-    return nrhs > 2 || (plan->nb >= 2048 && (int64_t)plan->nb * plan->nb >= 80 * plan->n);
+    return nrhs > 2 || (plan->nb >= 2048 && (int64_t)plan->nb * plan->nb >= 80 * plan->n && plan->heavy <= 20 * plan->even);
 }
 static int tc_parts(p2p_path path) { return path == P2P_PATH_TC_BF16X6 ? 3 : 2; }
 // One box per unit (p2p_tc_box.cu) instead of 128 targets: where units of 128 targets are too few for the SMs, and for

@@ -141,6 +141,7 @@ struct p2p_plan {
     int32_t group_grid;     // persistent grid (blocks of 8 warps)
     int32_t group_asked;    // 1: the caller's tuning named the kernel
     int64_t pairs, heavy;   // targets x sources of all boxes, and of the heaviest box
+    int64_t even;           // pairs of the average warp, 32 per SM
     int32_t* g_union;       // [n_groups * kGroupBoxes * 27] union boxes of every group, ascending
     int32_t* g_nunion;      // [n_groups]
     int32_t* g_order;       // [n_groups] groups, heaviest first

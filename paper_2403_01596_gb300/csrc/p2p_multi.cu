@@ -655,7 +655,7 @@ p2p_status p2p_grad_launch(const p2p_plan* p, const float2* lam, const float2* g
     // with 12 warps in turns / here, us: 60 001 points at 10 per box 75 / 73 / 64, at 60 161 / 189 / 148, 300 001 at 10 230 / 249 /
     // 212, Laplace 150 / 149 / 130.  On even geometries the larger grid only starts more blocks (262 144 sphere points at 16,
     // Helmholtz with 12 warps 119 -> 127; a cube at 20 176 -> 196).
-    const bool uneven = (double)p->heavy * 32.0 * sms > 4.0 * (double)p->pairs;
+    const bool uneven = p->heavy > 4 * p->even;
     const bool helm = p->kernel == P2P_HELMHOLTZ, narrow = helm && !uneven;
     const Shape shape = narrow ? Shape{12, 1} : Shape{8, 2};
     const int64_t blocks = ((int64_t)a.n_items + shape.warps - 1) / shape.warps;

@@ -1308,6 +1308,7 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     p->group_asked = t.warp_boxes == -2;
     p->pairs = (int64_t)info.pairs;
     p->heavy = (int64_t)info.heavy;
+    p->even = p->pairs / (32ll * sms);
     if (p->tune.warp_boxes == -2 && (layout != P2P_LAYOUT_INDEXED || nb == 0)) p->tune.warp_boxes = -1;
     int32_t cap[2] = {0, 0};
     if (p->tune.warp_boxes == -2) {

@@ -94,3 +94,29 @@ def test_gradient_of_even_and_clustered_geometries(share, radius, kernel):
     assert plan.async_status() == 0
     ref = oracle.grad_points(pts, lam, g, lo, h, ng, k, kernel=kid)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+
+
+@pytest.mark.parametrize("share", [0.0, 0.3])
+@pytest.mark.parametrize("kernel", ["helmholtz", "laplace"])
+def test_two_with_and_without_a_cluster(share, kernel):
+    """Two right-hand sides on a plan of many boxes, streamed, and with a box that decides the time, staged; same bound."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_01596_gb300 import api
+    n, ng = 30_000, 16
+    rng = np.random.default_rng(9)
+    pts = rng.random((n, 3))
+    m = int(share * n)
+    pts[:m] = 0.5 + 0.02 * rng.random((m, 3))
+    pts = pts.astype(np.float32)
+    lo, h = (0.0, 0.0, 0.0), 1.0 / ng
+    k = float(np.float32(2 * np.pi * ng / 4)) if kernel == "helmholtz" else 0.0
+    kid = oracle.HELMHOLTZ if kernel == "helmholtz" else oracle.LAPLACE
+    plan = api.Plan(torch.from_numpy(pts).cuda(), lo, h, ng, k, kernel=kernel, max_nrhs=2)
+    assert plan.num_boxes >= 2048 and plan.num_boxes ** 2 >= 80 * n
+    lam = W.strengths(n, 2, n).reshape(n, 2)
+    got = plan.apply(torch.from_numpy(lam).cuda()).cpu().numpy()
+    assert plan.async_status() == 0
+    S = oracle.p2p(pts, np.abs(lam).astype(np.complex64), lo, h, ng, 0.0, kernel=oracle.LAPLACE).real.reshape(n, 2)
+    ref = oracle.p2p(pts, lam, lo, h, ng, k, kernel=kid).reshape(n, 2)
+    assert (np.abs(got - ref) <= 2.0 ** -20 * S).all()
