@@ -316,15 +316,23 @@ static bool is_multi(const p2p_plan* plan, int32_t nrhs, p2p_path path) {
 }
 static int tc_parts(p2p_path path) { return path == P2P_PATH_TC_BF16X6 ? 3 : 2; }
 // One box per unit (p2p_tc_box.cu) instead of 128 targets: where units of 128 targets are too few for the SMs, and for
-// three parts with more than 32 right-hand sides per launch, whose chains would have to be too short (kSegment).
+// three parts with more than 32 right-hand sides per launch, whose chains would have to be too short (kSegment).  With long
+// lists and the Helmholtz kernel, where a unit takes longest, a second or third round of the SMs that is nearly empty (152
+// units are 19 456 targets) costs more than it does elsewhere, so the lines lie a little higher.
 // Measured on spheres at 20 points per box, us, 128 targets / one box: hi / lo, 16 right-hand sides, 8 193 points 48 / 39,
 // 16 385 62 / 55, 30 001 73 / 93; 64: 16 385 69 / 56, 30 001 89 / 93 (at 45 per box 117 / 111), 60 001 141 / 157; three
-// parts, 32: 8 193 66 / 52, 16 385 76 / 77, 30 001 99 / 124; 64: 60 001 260 / 227.
+// parts, 32: 8 193 66 / 52, 16 385 76 / 77, 30 001 99 / 124; 64: 60 001 260 / 227.  Long lists, Helmholtz: ellipsoid at 48 per
+// box, 24: 20 001 88 / 77, three parts 12 501 94 / 85; cube at 24 per box, 24: 20 001 95 / 92, 26 001 103 / 96, 33 001 level; 64:
+// 41 001 163 / 138, 47 001 172 / 158, 52 001 level; three parts, 24: 16 001 95 / 86, 20 001 level (at 48 per box 21 501 147 / 137).
 static bool tc_by_box(const p2p_plan* plan, int32_t nrhs, int parts) {
     if (!plan->tcb_gstart) return false;
     const bool wide = p2p_tc_launch_rhs(nrhs) > 32;
-    if (parts == 3) return wide || plan->n < 12000;
-    return plan->n < (wide ? kTcBoxTargets : 20000);
+    if (parts == 3 && wide) return true;
+    const bool dense = plan->kernel == P2P_HELMHOLTZ && plan->sources >= 240ll * plan->nb;
+    const bool volume = plan->sources > 16ll * plan->n;  // 9 - 15 sources per target and point of a box on a surface
+    int64_t limit = parts == 3 ? 12000 : (wide ? kTcBoxTargets : 20000);
+    if (dense) limit = parts == 3 ? (volume ? 22000 : 14000) : (wide ? (volume ? 50000 : limit) : (volume ? 30000 : 22000));
+    return plan->n < limit;
 }
 
 P2P_API p2p_status p2p_apply_stage(const p2p_plan* plan, const void* lambda, int32_t nrhs, int64_t ld, p2p_path path,

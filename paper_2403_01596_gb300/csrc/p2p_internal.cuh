@@ -126,7 +126,7 @@ struct p2p_plan {
     unsigned char* tc_pack; // per-apply group records: BF16 part images of the strengths, source coordinates
     // tensor-core path by single boxes (p2p_tc_box.cu), where p2p_tcb_planned: null otherwise
     int32_t* tcb_gstart;    // [nbs + 1] first 16-source group of every source box
-    int32_t tcb_groups;     // bound of the groups: records of one launch in tc_pack
+    int32_t tcb_groups;     // source groups: records of one launch in tc_pack
     int32_t* tcb_glist_off; // [nb + 1] offsets of the per-box group lists
     int32_t* tcb_glist;     // per box: the groups of its neighbour boxes (ascending box id), padded to four with -1
     int32_t* tcb_gcount;    // [nb] groups in the list of every box (without padding)

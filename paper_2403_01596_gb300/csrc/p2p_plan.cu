@@ -1271,10 +1271,9 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
     }
     if (p->tc_pack)  // n_chunks and padded are free once the items are built
         FAIL_CUDA(p2p_tc_build(p, L.n_chunks, L.padded, L.scan_ws, s), "p2p_plan_create/tc_lists");
-    if (p->tcb_gstart) {
-        p->tcb_groups = (int32_t)(p->n_src / 16 + p->nbs);
+    p->tcb_groups = 0;
+    if (p->tcb_gstart && p->nbs > 0)
         FAIL_CUDA(p2p_tcb_build(p, L.n_chunks, L.scan_ws, s), "p2p_plan_create/tc_box_lists");
-    }
     // direct kernel: one item per target box (the item-sort scratch is free again)
     p->direct_k = 0;
     if (layout != P2P_LAYOUT_SYMMETRIC && layout != P2P_LAYOUT_REPETITION) {
@@ -1317,6 +1316,9 @@ p2p_status plan_create(p2p_plan** plan, const PlanInput& in, p2p_kernel kernel, 
                                   L.radix_bytes, L.maxes, s, cap),
                   "p2p_plan_create/groups");
     }
+    if (p->tcb_gstart && p->nbs > 0)
+        FAIL_CUDA(cudaMemcpyAsync(&p->tcb_groups, p->tcb_gstart + p->nbs, sizeof(int32_t), cudaMemcpyDeviceToHost, s),
+                  "p2p_plan_create/tc_box_groups");
     // the plan is complete when this returns: later calls may use it on any stream
     FAIL_CUDA(cudaStreamSynchronize(s), "p2p_plan_create");
     if (p->tune.warp_boxes == -2) {

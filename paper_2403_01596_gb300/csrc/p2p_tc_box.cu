@@ -341,7 +341,6 @@ __global__ void __launch_bounds__(128) k_tcb_pack(const float2* __restrict__ lam
                                                  int32_t nb, int32_t rb_launch, int64_t chunk_bytes,
                                                  unsigned char* __restrict__ pack) {
     const int g = blockIdx.x, rb = blockIdx.y;
-    if (g >= gstart[nb]) return;  // the grid covers a bound of the groups
     // box of group g: the last c with gstart[c] <= g
     int lo = 0, hi = nb - 1;
     while (lo < hi) {
