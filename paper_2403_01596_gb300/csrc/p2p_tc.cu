@@ -287,6 +287,14 @@ __device__ __forceinline__ float2 residual(float2 v, float2 w) { return __ffma2_
 constexpr float kBf16Max = 3.3895313892515355e38f;
 __device__ __forceinline__ float capped(float x) { return isfinite(x) ? fminf(fmaxf(x, -kBf16Max), kBf16Max) : x; }
 
+// Whether some of eight values would round to infinity in BF16 (or is infinite); splitting them takes the capped form then.
+__device__ __forceinline__ bool any_above(const float (&v)[8]) {
+    float m = fabsf(v[0]);
+#pragma unroll
+    for (int i = 1; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
+    return m > kBf16Max;
+}
+
 // x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.  CAP: any finite x.
 template <bool CAP = false>
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
@@ -313,13 +321,13 @@ __host__ __device__ inline int op_off(int row, int k) {
 
 // Splits eight consecutive K elements (strengths) of one row into NP BF16 parts (2: hi, lo; 3: hi, mid, lo) stored at `off`
 // in the images starting at part0, part_bytes apart.
-template <int NP>
+template <int NP, bool CAP>
 __device__ __forceinline__ void store_parts(unsigned char* part0, int part_bytes, int off, const float (&v)[8]) {
     uint32_t p[NP][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        if constexpr (NP == 2) split2<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i]);
-        else split3<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
+        if constexpr (NP == 2) split2<CAP>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i]);
+        else split3<CAP>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
     }
 #pragma unroll
     for (int q = 0; q < NP; ++q)
@@ -373,8 +381,13 @@ __global__ void __launch_bounds__(128) k_tc_pack(const float2* __restrict__ lam,
         im[e] = v.y;
     }
     if (r < rhs) {
-        store_parts<NP>(rec, image_bytes(rhs), op_off(r, 8 * o), re);
-        store_parts<NP>(rec, image_bytes(rhs), op_off(rhs + r, 8 * o), im);
+        if (any_above(re) || any_above(im)) {
+            store_parts<NP, true>(rec, image_bytes(rhs), op_off(r, 8 * o), re);
+            store_parts<NP, true>(rec, image_bytes(rhs), op_off(rhs + r, 8 * o), im);
+        } else {
+            store_parts<NP, false>(rec, image_bytes(rhs), op_off(r, 8 * o), re);
+            store_parts<NP, false>(rec, image_bytes(rhs), op_off(rhs + r, 8 * o), im);
+        }
     }
     float* xyz = reinterpret_cast<float*>(rec + NP * image_bytes(rhs));
     uint32_t* mark = reinterpret_cast<uint32_t*>(rec + NP * image_bytes(rhs) + kXyzBytes);
@@ -1278,14 +1291,14 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm_check(const float* __restric
             float v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) v[i] = A[(int64_t)row * K + ks * 16 + half * 8 + i];
-            store_parts<2>(a_hi, (int)(a_lo - a_hi), op_off(row, half * 8), v);
+            store_parts<2, false>(a_hi, (int)(a_lo - a_hi), op_off(row, half * 8), v);
         }
         for (int c = tid; c < n * 2; c += 128) {
             const int row = c >> 1, half = c & 1;
             float v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) v[i] = B[(int64_t)row * K + ks * 16 + half * 8 + i];
-            store_parts<2>(b_hi, (int)(b_lo - b_hi), op_off(row, half * 8), v);
+            store_parts<2, false>(b_hi, (int)(b_lo - b_hi), op_off(row, half * 8), v);
         }
         fence_async_smem();
         tc_fence_before();

@@ -219,6 +219,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 constexpr float kBf16Max = 3.3895313892515355e38f;
 __device__ __forceinline__ float capped(float x) { return isfinite(x) ? fminf(fmaxf(x, -kBf16Max), kBf16Max) : x; }
 
+// Whether some of eight values would round to infinity in BF16 (or is infinite); splitting them takes the capped form then.
+__device__ __forceinline__ bool any_above(const float (&v)[8]) {
+    float m = fabsf(v[0]);
+#pragma unroll
+    for (int i = 1; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
+    return m > kBf16Max;
+}
+
 // x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.  CAP: any finite x.
 template <bool CAP = false>
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
@@ -371,8 +379,13 @@ __global__ void __launch_bounds__(128) k_tcb_pack(const float2* __restrict__ lam
         im[e] = v.y;
     }
     unsigned char* img = rec + lb * NP * kPart;
-    store_parts<NP, 8, true>(img, kPart, op_off(r, 8 * o), re);
-    store_parts<NP, 8, true>(img, kPart, op_off(64 + r, 8 * o), im);
+    if (any_above(re) || any_above(im)) {
+        store_parts<NP, 8, true>(img, kPart, op_off(r, 8 * o), re);
+        store_parts<NP, 8, true>(img, kPart, op_off(64 + r, 8 * o), im);
+    } else {
+        store_parts<NP, 8>(img, kPart, op_off(r, 8 * o), re);
+        store_parts<NP, 8>(img, kPart, op_off(64 + r, 8 * o), im);
+    }
 }
 
 // ------------------------------------------------------------------ main kernel --
