@@ -26,7 +26,7 @@
 // keeps, per box, the list of the groups of its neighbour boxes (ascending box
 // id), padded with -1 to a multiple of four entries.
 //
-// Main kernel (k_p2p_tc): persistent, one CTA per SM, units (box, target group)
+// Main kernel (k_p2p_tc_box): persistent, one CTA per SM, units (box, target group)
 // round robin over the CTAs in Morton order (neighbouring CTAs share records in
 // L2).  Warp roles:
 //   warps 0-3    one producer per G set: walks a unit's group list four entries (a quad) at a time and
@@ -37,7 +37,6 @@
 //                block) into the set's own accumulator, committed to the slot's release barrier
 //   warps 24-27  epilogue: sums the sets' accumulators (TMEM -> registers), combines Re/Im through
 //                shared memory and writes out[perm[t]]
-// (with P2P_TC_SETS = 2: two producers, two sets of eight warps, entries taken in pairs)
 // Four independent issue chains (one per set) keep the tensor core fed with the
 // small (N = 2T) MMAs.  With the hi/lo split (units of up to 32 targets) two TMEM
 // buffers alternate between a CTA's units so the epilogue of one unit overlaps
@@ -52,73 +51,25 @@
 // Operands use the canonical K-major layout without swizzle: 8-row x 16-byte
 // core matrices, the two K-adjacent cores of a 16-wide K slice 128 bytes apart
 // (leading byte offset) and 8-row groups 256 bytes apart (stride byte offset).
-#include <cuda_bf16.h>
 #include <math.h>
 
-#include "p2p_internal.cuh"
+#include "p2p_tc_common.cuh"
 
 using namespace p2p_detail;
+using namespace p2p_tc_common;
 
 namespace {
 
-constexpr float kInv4Pi = 0.0795774715459476679f;
-constexpr int kSrcGroup = 16;          // sources per stage (MMA K)
-constexpr int kPart = 4096;            // one BF16 image of a 128 x 16 A operand
-constexpr int kImage = 2 * kPart;      // hi + lo images (the operand self-check)
-constexpr int kLbo = 128, kSbo = 256;  // core-matrix strides (K direction, 8-row groups)
 constexpr int kSetCols = 256;          // TMEM columns of a unit buffer of 32-target units (an accumulator per set)
-// G sets (independent producer -> G -> MMA chains; 2 or 4, the group lists are
-// padded to multiples of 4).  On the 2^21-point ellipsoid at 64 RHS four sets of
-// four warps measured 5.1 ms against 5.3 for two sets of eight with units of up
-// to 64 targets; two sets would also halve the accumulators of the three-part
-// split, whose error grows with the accumulation chains.
-#ifndef P2P_TC_SETS
-#define P2P_TC_SETS 4
-#endif
-constexpr int kSets = P2P_TC_SETS;     // G sets; set s takes list entries s, s + kSets, ... of a unit
+// G sets (independent producer -> G -> MMA chains; the group lists are padded to a
+// multiple of them).  Four sets of four warps rather than two of eight: each set has an
+// accumulator of its own, and the error grows with the length of the accumulation chains.
+constexpr int kSets = 4;               // set s takes list entries s, s + kSets, ... of a unit
 constexpr int kSetWarps = 16 / kSets;  // warps of one G set
 constexpr int kSetThreads = 32 * kSetWarps;
 constexpr int kGWarp0 = kSets, kMmaWarp0 = kGWarp0 + kSetWarps * kSets, kEpiWarp0 = kMmaWarp0 + kSets;
 constexpr int kWarps = kEpiWarp0 + 4;
 constexpr int kThreads = kWarps * 32;
-// A waiting thread is suspended (up to kSuspendNs per poll) until the phase
-// completes, so idle roles do not take issue slots from the working warps.
-// kWaitLimit polls bound every wait to a few seconds at most.
-constexpr uint32_t kSuspendNs = 10000;
-constexpr uint32_t kWaitLimit = 1u << 18;
-constexpr uint32_t kDrainLimit = 1u << 14;
-
-// --------------------------------------------------------------- PTX helpers --
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Shared-memory matrix descriptor: start, leading and stride byte offsets (>> 4),
-// descriptor version 1 at bit 46, no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(kLbo >> 4) << 16) | ((uint64_t)(kSbo >> 4) << 32) |
-           (1ull << 46);
-}
-
-// Instruction descriptor of kind::f16: D f32, A and B bf16, both K-major, N, M = 128.
-__host__ __device__ inline uint32_t idesc_bf16_f32(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
-        : "memory");
-    return done != 0;
-}
 
 // Bounded wait; gives up early once *abort is set.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
@@ -130,49 +81,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // Named barrier 5 for the epilogue warps (0 is __syncthreads).
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 5, 128;" ::: "memory"); }
 // Barrier of the 128 epilogue threads that also ORs a condition over them.
@@ -200,68 +108,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
     for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 32 lanes x 16 consecutive 32-bit columns of TMEM into registers.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// The largest finite BF16 value.  A finite strength above it (up to 0.4 % below the FP32 maximum) would round to infinity,
-// and inf - inf makes NaN of its neighbours' sums; capped, the next part holds the rest of it.
-constexpr float kBf16Max = 3.3895313892515355e38f;
-__device__ __forceinline__ float capped(float x) { return isfinite(x) ? fminf(fmaxf(x, -kBf16Max), kBf16Max) : x; }
-
-// Whether some of eight values would round to infinity in BF16 (or is infinite); splitting them takes the capped form then.
-__device__ __forceinline__ bool any_above(const float (&v)[8]) {
-    float m = fabsf(v[0]);
-#pragma unroll
-    for (int i = 1; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
-    return m > kBf16Max;
-}
-
-// x = hi + lo with hi, lo BF16 (round to nearest), two values per 32-bit word.  CAP: any finite x.
-template <bool CAP = false>
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(CAP ? capped(a) : a, CAP ? capped(b) : b);
-    float2 hf = __bfloat1622float2(h);
-    __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-}
-
-// x = hi + mid + lo with three BF16 parts (each the round-to-nearest of what the
-// previous parts leave), two values per 32-bit word: the parts carry ~24 bits.
-template <bool CAP = false>
-__device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(CAP ? capped(a) : a, CAP ? capped(b) : b);
-    const float2 hf = __bfloat1622float2(h);
-    const float ra = a - hf.x, rb = b - hf.y;
-    __nv_bfloat162 m = __floats2bfloat162_rn(ra, rb);
-    const float2 mf = __bfloat1622float2(m);
-    __nv_bfloat162 l = __floats2bfloat162_rn(ra - mf.x, rb - mf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    mid = *reinterpret_cast<uint32_t*>(&m);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-}
-
 __device__ __forceinline__ void split1(float a, uint16_t& hi, uint16_t& lo) {
     __nv_bfloat16 h = __float2bfloat16_rn(a);
     __nv_bfloat16 l = __float2bfloat16_rn(a - __bfloat162float(h));
     hi = *reinterpret_cast<uint16_t*>(&h);
     lo = *reinterpret_cast<uint16_t*>(&l);
-}
-
-// Byte offset of element (row, k) of a K-major operand with 16-wide K slices.
-__host__ __device__ inline int op_off(int row, int k) {
-    return (row >> 3) * kSbo + (k >> 3) * kLbo + (row & 7) * 16 + (k & 7) * 2;
 }
 
 // Splits n values (n = 1, 2, 4 or 8, consecutive K elements of one row) and
@@ -897,10 +748,11 @@ TcShape tc_shape(int32_t nrhs, int optin, int np) {
     TcShape s;
     s.rb_count = (nrhs + 63) / 64;
     // One accumulator per G set (rb_count blocks x 2T columns) in each unit buffer.  The hi/lo split keeps two
-    // buffers of 32-target units, so the epilogue of one unit overlaps the MMAs of the next.  The three-part
-    // split takes 64-target units in one buffer (all 512 columns): a box of 33 - 64 targets is one unit instead
-    // of two walking the same list, and its six MMAs per stage leave the epilogue's wait a smaller share (the
-    // ellipsoid at 64 RHS: 7.14 ms against 7.64; hi/lo with the same shape 5.46 against 5.11).
+    // buffers of 32-target units, so the epilogue of one unit overlaps the MMAs of the next (plans of up to 40 000
+    // targets; one buffer of 64-target units was 7 % slower).  The three-part split takes 64-target units in one
+    // buffer (all 512 columns): a box of 33 - 64 targets is one unit instead of two walking the same list, and its
+    // six MMAs per stage leave the epilogue's wait a smaller share (the 2^21-point ellipsoid at 64 RHS: 7.14 ms
+    // against 7.64).
     const int units_in_tmem = np == 3 ? 1 : 2;
     s.tg = (2 * kSetCols / (units_in_tmem * 2 * kSets * s.rb_count)) / 8 * 8;
     if (s.tg > 64) s.tg = 64;
@@ -954,9 +806,9 @@ __global__ void k_tcb_list_fill(const int32_t* __restrict__ nbr_ptr, const int32
 
 // RHS blocks of 64 per launch.  One block per launch keeps units of 32 targets
 // (the TMEM accumulators of four G sets x two unit buffers hold 2 T x 64 RHS
-// each); a launch over two blocks must halve the unit to 16 targets and measured
-// 15.4 ms on the 2^21-point ellipsoid at 128 RHS against 2 x 5.2 ms for two
-// launches of one block (G is formed once per launch: its share is small).
+// each); a launch over two blocks must halve the unit to 16 targets and took 1.5
+// times as long as two launches of one block (G is formed once per launch: its
+// share is small).
 constexpr int kRbLaunch = 1;
 
 // Room for the records of either split (sized for three parts), chunk by chunk.
