@@ -92,15 +92,12 @@ constexpr int kSets = 4;               // G sets; set s takes entries s, s + kSe
 //   48 x 3  4.53e-6 331 us   5.00e-6 3556 us   4.64e-6
 //   16 x 3  4.47e-6 401 us   5.06e-6 4340 us   4.50e-6
 //   48 x 4  3.65e-6 346 us   3.70e-6 3673 us   3.86e-6
-//   64 x 4  3.74e-6 332 us   3.80e-6 3546 us   3.93e-6
-// The more of an entry's slots are pairs, the more of its additions count: at 100 points per box 64 entries came out at
-// 4.63e-6 on an ellipsoid and 4.98e-6 in a cube, 48 at 4.21e-6 and 4.44e-6 (one box per unit 4.57e-6, 4.87e-6), and on a clustered
-// assembly at 50 per box at 5.7e-6, 4.6e-6 (5.2e-6).  So wide hi / lo launches take 64 on plans without large boxes.
+//   64 x 4  3.74e-6 332 us   3.80e-6 3546 us   3.93e-6; in a cube at 100 per box, where every slot of an entry is a pair,
+//                                              4.98e-6 (one box per unit: 4.87e-6)
 // (Six products per entry would need segments of 6 to 8 entries to be as exact as chains of ~55 additions, and the
 // epilogue's share makes that slower than one box per unit: 2^21-point ellipsoid, 64 right-hand sides 7.4 ms against 6.9.
 // p2p_tc_box.cu takes those calls.)
-constexpr int kSegment = 48, kSegmentWide = 64;
-constexpr int kWideBox = 96;           // targets of the largest box at most for kSegmentWide
+constexpr int kSegment = 48;
 constexpr int kAColumn = 256;          // first TMEM column of the operand slots
 constexpr int kMmaWarp0 = 1, kScoutWarp = 3, kEpiWarp0 = 4, kGWarp0 = 8;
 constexpr int kWarps = kGWarp0 + 4 * kSets;
@@ -463,7 +460,6 @@ struct TcArgs {
     int32_t rhs;                   // the same rounded up to 8 (R)
     int32_t nb;
     int32_t nblk;
-    int32_t segment;               // entries added up in one accumulator chain at most
     int32_t slot_bytes;
     int32_t slots_log;             // log2 of the record slots (3 or 4)
     int32_t a_slots;               // TMEM operand slots (a power of two, at least kSets)
@@ -594,7 +590,7 @@ __device__ void run_scout(const TcArgs& a, const TcSmem& sm, int lane) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(P2P_FULL_MASK, cnt, o);
             if (cnt == 0) continue;  // two point sets, no source nearby: the rows keep the zeros written before the launch
-            const int segments = (cnt + a.segment - 1) / a.segment;
+            const int segments = (cnt + kSegment - 1) / kSegment;
             h0 = make_int4(b0, t0, nt, cnt);
             h1 = make_int4(off, E, (int)want, (cnt + segments - 1) / segments);
         }
@@ -1319,7 +1315,6 @@ p2p_status p2p_apply_tc(const p2p_plan* plan, float2* out, int32_t nrhs, int64_t
     a.rhs = rhs;
     a.nb = plan->nb;
     a.nblk = p2p_tc_block_count(plan->nb);
-    a.segment = np == 2 && rhs > 32 && plan->max_box <= kWideBox ? kSegmentWide : kSegment;
     a.a_slots = np == 3 ? 4 : 8;  // 48 or 32 columns each in 256
     a.k = adjoint ? -plan->k : plan->k;
     a.status = plan->status;
