@@ -645,7 +645,7 @@ def _rel_l2_cols(x, ref):
 
 def measure_multirhs(scale, steps, samples, free_first=()):
     """The 64-RHS comparison on the 2:1:1 ellipsoid (2^21 points, 188^3 grid, leaf edge 0.2 wavelength):
-    the tensor-core paths (BF16 hi/lo split with 3 MMAs, hi/mid/lo with 6; tcgen05, FP32 accumulation)
+    the tensor-core paths (BF16 hi/lo split with 4 MMAs per 16 sources, hi/mid/lo with 6; tcgen05, FP32 accumulation)
     against the FP32 path with G shared over RHS blocks and the plain per-RHS FP32 path, each timed with CUDA
     events; rel-L2 vs the FP64 oracle per right-hand side and the largest |err| / sum_j |G lambda_j| on
     `samples` sampled targets.  Returns the record (timings, errors, roofline)."""
@@ -698,7 +698,7 @@ def measure_multirhs(scale, steps, samples, free_first=()):
         res[path]["rel_l2_per_rhs"] = [float(v) for v in e]
     f_max = float(peaks.get("sm_max_mhz", 2070.0)) * 1e6
     mufu_peak = props.multi_processor_count * 16 * f_max / 3 / 1e9        # G evaluations per second (G/s)
-    tc_flops = 3 * 8 * P * nrhs                                           # hi.hi + hi.lo + lo.hi, realified complex
+    tc_flops = 3 * 8 * P * nrhs                                           # hi.hi + hi.lo + lo.hi, realified complex; lo.lo not counted
     t_tc = kern_ms * 1e-3                                                 # the pipelined kernel alone
     sizes = torch.diff(plan.structure.box_ptr.long())
     groups = int(((sizes + 15) // 16).sum().item())                      # 16-source groups of the pre-pack

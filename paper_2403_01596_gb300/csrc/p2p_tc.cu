@@ -86,14 +86,14 @@ constexpr int kSets = 4;               // G sets; set s takes entries s, s + kSe
 // 32 right-hand sides) a chain takes one truncated addition per entry.  Wider launches have no TMEM left for that: every
 // product of an entry is a truncated addition to the one accumulator, and with the three of hi / lo the error came out
 // above that of the split alone even with short segments.  The fourth product, lo.lo, takes the split's own error from 4.4e-6
-// to 3.5e-6, more than those additions cost, and the issuers have time for it (a G set takes ~750 cycles for an entry, its
-// MMAs 384, 512 with the fourth).  Relative L2 error / time with 64 right-hand sides on 200 003 sphere points at 20 per box
+// to 3.5e-6, more than those additions cost, and the issuers have time for most of it (a G set takes ~750 cycles for an
+// entry, its MMAs 384, 512 with the fourth).  Relative L2 error / time with 64 right-hand sides on 200 003 sphere points at 20 per box
 // and on the 2^21-point ellipsoid, and with 40 at 47 points per box, entries per segment x products:
 //   48 x 3  4.53e-6 331 us   5.00e-6 3556 us   4.64e-6
 //   16 x 3  4.47e-6 401 us   5.06e-6 4340 us   4.50e-6
 //   48 x 4  3.65e-6 346 us   3.70e-6 3673 us   3.86e-6
 //   64 x 4  3.74e-6 332 us   3.80e-6 3546 us   3.93e-6; in a cube at 100 per box, where every slot of an entry is a pair,
-//                                              4.98e-6 (one box per unit: 4.87e-6)
+//                                              4.98e-6 (one box per unit: 4.87e-6), at 75 per box 4.645e-6 (4.636e-6)
 // (Six products per entry would need segments of 6 to 8 entries to be as exact as chains of ~55 additions, and the
 // epilogue's share makes that slower than one box per unit: 2^21-point ellipsoid, 64 right-hand sides 7.4 ms against 6.9.
 // p2p_tc_box.cu takes those calls.)
